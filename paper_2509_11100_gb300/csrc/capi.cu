@@ -105,6 +105,7 @@ struct relsim_ctx {
     int64_t rcap = 0;
     // GMRES
     int mrest = 30;
+    int solve_rows = 0;        // tile height of the one-launch solve (0: the launches of gmres.cu)
     int64_t nvec = 0;
     double* V = nullptr;
     double* gw = nullptr;
@@ -872,14 +873,32 @@ GmSetup gm_setup(relsim_ctx* c)
     return s;
 }
 
-// b, x = E^n, |b|, r = b - A x, |r|, start of the first cycle
+// b, x = E^n
 template <typename T>
-int solve_prologue(relsim_ctx* c, const GmSetup& S, cudaStream_t s, GmCond outer)
+int solve_rhs(relsim_ctx* c, const GmSetup& S, cudaStream_t s)
 {
     PROF_BEGIN(RELSIM_PROF_RHS);
     CK(rhs<T>((const T*)c->E, (const T*)c->B[c->bcur], (const T*)c->J, c->gb, c->g, s));
     CK(fields_to_vec<T>((const T*)c->E, c->gx, S.n, c->g.df, s));
     PROF_END();
+    return RELSIM_OK;
+}
+
+// the whole solve in one launch (grids that fit: solve.cu)
+template <typename T>
+int solve_launch(relsim_ctx* c, const GmSetup& S, cudaStream_t s, bool tr)
+{
+    PROF_BEGIN(RELSIM_PROF_GMRES_APPLY);
+    CK(gm_solve<T>((const T*)c->M, c->gb, c->gx, S.p, S.q, c->g, c->solve_rows, c->partial, c->gms, c->dpush, tr, s));
+    PROF_END();
+    return RELSIM_OK;
+}
+
+// b, x = E^n, |b|, r = b - A x, |r|, start of the first cycle
+template <typename T>
+int solve_prologue(relsim_ctx* c, const GmSetup& S, cudaStream_t s, GmCond outer)
+{
+    TRY(solve_rhs<T>(c, S, s));
     PROF_BEGIN(RELSIM_PROF_GMRES_ORTHO);
     CK(gm_dots(c->V, S.ldv, 0, c->gb, S.n, c->partial, S.nb, s, c->g.df));
     CK(reduce_partials(c->partial, S.nb, 1, c->dsum, s));
@@ -947,6 +966,8 @@ int solve_reserve(relsim_ctx* c, const GmSetup& S)
     const int nbf = field_grid_blocks(c->g);
     int64_t need = (int64_t)(S.nb > S.nbo ? S.nb : S.nbo) * (S.m + 2);
     if ((int64_t)nbf * 6 > need) need = (int64_t)nbf * 6;
+    if (c->solve_rows && gm_solve_partials(c->g, c->solve_rows, S.m) > need)
+        need = gm_solve_partials(c->g, c->solve_rows, S.m);
     return ensure_partial(c, need);
 }
 
@@ -973,6 +994,14 @@ int head_async(relsim_ctx* c, int k)
     CK(cudaMemcpyAsync(c->ghead + k, c->gms, kGmHead, cudaMemcpyDeviceToHost, c->st));
     CK(cudaMemcpyAsync(c->hpush, c->dpush, sizeof(int), cudaMemcpyDeviceToHost, c->st));
     return RELSIM_OK;
+}
+
+// wait for the one-launch solve's outcome (ghead[0])
+int solve_read(relsim_ctx* c)
+{
+    TRY(head_async(c, 0));
+    CK(cudaStreamSynchronize(c->st));
+    return check_push(c);
 }
 
 // The solve driven from the host: the same kernels as the graph, with the
@@ -1013,8 +1042,14 @@ int solve_impl(relsim_ctx* c, int* iters_out, double* relres_out)
 {
     const GmSetup S = gm_setup(c);
     TRY(solve_reserve(c, S));
-    TRY(solve_prologue<T>(c, S, c->st, GmCond{0, 0}));
-    TRY(gm_drive<T>(c, S, false));
+    if (c->solve_rows) {
+        TRY(solve_rhs<T>(c, S, c->st));
+        TRY(solve_launch<T>(c, S, c->st, false));
+        TRY(solve_read(c));
+    } else {
+        TRY(solve_prologue<T>(c, S, c->st, GmCond{0, 0}));
+        TRY(gm_drive<T>(c, S, false));
+    }
     const GmState h = c->ghead[0];
     if (h.status == kGmNonfinite) return solve_outcome(c, &h, iters_out, relres_out);
     TRY(solve_epilogue<T>(c, c->st));
@@ -1208,6 +1243,11 @@ int capture_into(relsim_ctx* c, cudaStream_t s, cudaGraph_t body, long long* tal
 template <typename T>
 int capture_solve(relsim_ctx* c, const GmSetup& S, StepGraph& G)
 {
+    if (c->solve_rows) {
+        TRY(solve_rhs<T>(c, S, c->st));
+        TRY(solve_launch<T>(c, S, c->st, false));
+        return solve_epilogue<T>(c, c->st);
+    }
     cudaGraph_t top = nullptr;
     TRY(capture_graph(c, c->st, &top));
     cudaGraphConditionalHandle ho;
@@ -1346,14 +1386,19 @@ int adjoint_impl(relsim_ctx* c, const double* gE1, const double* gB1, const doub
     const GmSetup S = gm_setup(c);
     TRY(solve_reserve(c, S));
     CK(adjoint_pre(d1, d2, d3, c->gb, c->g, c->st));
-    CK(gm_dots(c->V, S.ldv, 0, c->gb, S.n, c->partial, S.nb, c->st, c->g.df));
-    CK(reduce_partials(c->partial, S.nb, 1, c->dsum, c->st));
-    CK(gm_begin(c->gms, c->dsum, c->st));
     CK(cudaMemsetAsync(c->gx, 0, sizeof(double) * (size_t)n, c->st));
-    CK(op_residual<T>((const T*)c->M, c->gx, c->gb, S.p.r, c->g, c->partial, c->dpush, c->st, true));
-    CK(reduce_partials(c->partial, S.nbo, 1, c->dsum, c->st));
-    CK(gm_cycle(c->gms, c->dsum, S.p, S.q, GmCond{0, 0}, c->st));
-    TRY(gm_drive<T>(c, S, true));
+    if (c->solve_rows) {
+        TRY(solve_launch<T>(c, S, c->st, true));
+        TRY(solve_read(c));
+    } else {
+        CK(gm_dots(c->V, S.ldv, 0, c->gb, S.n, c->partial, S.nb, c->st, c->g.df));
+        CK(reduce_partials(c->partial, S.nb, 1, c->dsum, c->st));
+        CK(gm_begin(c->gms, c->dsum, c->st));
+        CK(op_residual<T>((const T*)c->M, c->gx, c->gb, S.p.r, c->g, c->partial, c->dpush, c->st, true));
+        CK(reduce_partials(c->partial, S.nbo, 1, c->dsum, c->st));
+        CK(gm_cycle(c->gms, c->dsum, S.p, S.q, GmCond{0, 0}, c->st));
+        TRY(gm_drive<T>(c, S, true));
+    }
     const GmState h = c->ghead[0];
     if (iters) *iters = h.total;
     if (relres) *relres = h.relres;
@@ -2237,6 +2282,13 @@ int relsim_init(const relsim_config* cfg, void* cuda_stream, relsim_ctx** out)
     A(dalloc(c, &c->gb, sizeof(double) * c->nvec));
     A(dalloc(c, &c->dsum, sizeof(double) * 4 * (kMaxRestart + 2)));
     A(dalloc(c, &c->gms, sizeof(GmState)));
+    // (the grid barrier counts its arrivals in 32 bits)
+    if (c->cfg.gmres_maxit <= 1 << 20 &&
+        (cfg->precision == 32 ? gm_solve_rows<float>(c->g, &c->solve_rows)
+                              : gm_solve_rows<double>(c->g, &c->solve_rows)) != cudaSuccess) {
+        r = fail(c, RELSIM_ERR_CUDA, "sizing the solve's launch failed");
+        goto fail_init;
+    }
     if (cudaMemsetAsync(c->gms, 0, sizeof(GmState), c->st) != cudaSuccess) {
         r = fail(c, RELSIM_ERR_CUDA, "cudaMemsetAsync failed");
         goto fail_init;

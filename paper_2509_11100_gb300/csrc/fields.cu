@@ -19,6 +19,7 @@
 
 #include "dfloat.cuh"
 #include "launch.cuh"
+#include "opcore.cuh"
 
 namespace relsim {
 
@@ -44,14 +45,6 @@ __global__ void k_to_double(const T* __restrict__ in, double* out, int64_t n)
     for (int64_t k = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; k < n;
          k += (int64_t)gridDim.x * blockDim.x)
         out[k] = (double)in[k];
-}
-
-// store v (formed in T) in a GMRES vector slot
-template <bool DF, typename T>
-__device__ __forceinline__ void vst(double* v, int64_t k, T val)
-{
-    if constexpr (DF) reinterpret_cast<dfl*>(v)[k] = df_from_f((float)val);
-    else v[k] = (double)val;
 }
 
 // b = E^n + theta dt curl_n B^n - theta dt Jhat
@@ -102,95 +95,11 @@ __global__ void k_df_to_double(const double* __restrict__ in, double* out, int64
         out[k] = df_to_double(reinterpret_cast<const dfl*>(in)[k]);
 }
 
-// Node-local loads of a GMRES vector as T
-template <typename T, bool DF = false>
-__device__ __forceinline__ T vld(const double* v, int64_t k)
-{
-    if constexpr (DF) {
-        const float2 a = __ldg(reinterpret_cast<const float2*>(v) + k);
-        return (T)df_to_f(dfl{a.x, a.y});
-    } else {
-        return (T)__ldg(v + k);
-    }
-}
-__device__ __forceinline__ dfl dld(const double* v, int64_t k)
-{
-    const float2 a = __ldg(reinterpret_cast<const float2*>(v) + k);
-    return dfl{a.x, a.y};
-}
-
-// (curl_n curl_c v) and (M v) at a node from its 3x3 stencil of v,
-// f[k][a][b] = component k at node (i-1+a, j-1+b), and its mass-matrix
-// blocks: Mg = the node's own five blocks M[g][0..4], Mn[o] = the block
-// M[g-o][o+1] of the neighbour g - o for the half offsets o = (1,0), (-1,1),
-// (0,1), (1,1) (M_{g,g-o} = M_{g-o,g}).
-template <typename T, typename P, bool TR>
-__device__ __forceinline__ void op_stencil_t(const T (&f)[3][3][3], P Mg, const P (&Mn)[4], T idx2, T idy2,
-                                           T cc[3], T mv[3])
-{
-    // curl_c at the four centres (i-1+ca+1/2, j-1+cb+1/2)
-    T C[3][2][2];
-#pragma unroll
-    for (int ca = 0; ca < 2; ++ca)
-#pragma unroll
-        for (int cb = 0; cb < 2; ++cb) {
-            T dx[3], dy[3];
-#pragma unroll
-            for (int k = 0; k < 3; ++k) {
-                dx[k] = (f[k][ca + 1][cb] - f[k][ca][cb] + f[k][ca + 1][cb + 1] - f[k][ca][cb + 1]) * idx2;
-                dy[k] = (f[k][ca][cb + 1] - f[k][ca][cb] + f[k][ca + 1][cb + 1] - f[k][ca + 1][cb]) * idy2;
-            }
-            C[0][ca][cb] = dy[2];
-            C[1][ca][cb] = -dx[2];
-            C[2][ca][cb] = dx[1] - dy[0];
-        }
-    // curl_n at the node from the four centres
-    T dx[3], dy[3];
-#pragma unroll
-    for (int k = 0; k < 3; ++k) {
-        dx[k] = (C[k][1][1] - C[k][0][1] + C[k][1][0] - C[k][0][0]) * idx2;
-        dy[k] = (C[k][1][1] - C[k][1][0] + C[k][0][1] - C[k][0][0]) * idy2;
-    }
-    cc[0] = dy[2];
-    cc[1] = -dx[2];
-    cc[2] = dx[1] - dy[0];
-    // M v: own blocks M[g][o] times v(g+o), neighbours' blocks M[g-o][o] times v(g-o);
-    // with TR every 3x3 block is applied transposed (M^T v: the stored block
-    // of the pair (g, g') serves both orders, M_{g'g} = M_{gg'})
-    constexpr int pa[4] = {2, 0, 1, 2}, pb[4] = {1, 2, 2, 2};   // g + o in the stencil
-    constexpr int ma[4] = {0, 2, 1, 0}, mb[4] = {1, 0, 0, 0};   // g - o
-    T r[3] = {T(0), T(0), T(0)};
-#pragma unroll
-    for (int rr = 0; rr < 3; ++rr)
-#pragma unroll
-        for (int s = 0; s < 3; ++s) r[rr] += T(Mg[TR ? s * 3 + rr : rr * 3 + s]) * f[s][1][1];
-#pragma unroll
-    for (int o = 0; o < 4; ++o) {
-        P Mo = Mg + (o + 1) * 9;
-#pragma unroll
-        for (int rr = 0; rr < 3; ++rr)
-#pragma unroll
-            for (int s = 0; s < 3; ++s)
-                r[rr] += T(Mo[TR ? s * 3 + rr : rr * 3 + s]) * f[s][pa[o]][pb[o]] +
-                         T(Mn[o][TR ? s * 3 + rr : rr * 3 + s]) * f[s][ma[o]][mb[o]];
-    }
-    mv[0] = r[0];
-    mv[1] = r[1];
-    mv[2] = r[2];
-}
-
-template <typename T, typename P>
-__device__ __forceinline__ void op_stencil(const T (&f)[3][3][3], P Mg, const P (&Mn)[4], T idx2, T idy2,
-                                           T cc[3], T mv[3])
-{
-    op_stencil_t<T, P, false>(f, Mg, Mn, idx2, idy2, cc, mv);
-}
-
 // the same at node (i,j) straight from global memory (v a GMRES vector,
 // component-major)
 template <typename T, bool DF = false>
 __device__ __forceinline__ void op_parts(const T* __restrict__ M, const double* __restrict__ v, int i,
-                                         int j, const GridP& g, T cc[3], T mv[3])
+                                         int j, const GridP& g, T (&cc)[3], T (&mv)[3])
 {
     const int nx = g.nx, ny = g.ny, nc = g.ncell;
     const int xs[3] = {wrap1(i - 1, nx), i, wrap1(i + 1, nx)};
@@ -228,8 +137,6 @@ __device__ __forceinline__ void op_parts(const T* __restrict__ M, const double* 
 // the residual and the dot products are formed in FP64.
 
 enum { kOpA = 0, kOpResidual = 1, kOpArnoldi = 2 };
-constexpr long long kOpMaxPolls = 1ll << 26;   // bounded mbarrier wait
-constexpr int kOpChunk = 8;                    // dot products reduced per shared-memory pass
 
 // The tile height is a compile-time shape with two instances per form (FP32:
 // 8 rows, or 4; FP64: 4, or 2); the autotuner picks one per context (YY = 0:
@@ -259,40 +166,6 @@ constexpr bool op_buffer_fits()
 static_assert(op_buffer_fits<float, 0>() && op_buffer_fits<float, 4>() && op_buffer_fits<double, 0>() &&
                   op_buffer_fits<double, 2>(),
               "the reduction buffer fits in the mass-matrix tile");
-
-// Dot2 (Ogita, Rump and Oishi, "Accurate sum and dot product", SIAM J. Sci.
-// Comput. 26, 2005) on the FP32 pipe: a running sum s with its error e,
-// each term's product split exactly by TwoProduct and added by TwoSum.
-struct Dot2 {
-    float s = 0.0f, e = 0.0f;
-    // += a b, a double-float, b FP32
-    __device__ __forceinline__ void add(dfl a, float b)
-    {
-        const dfl p = df_two_prod(a.hi, b);
-        const dfl t = df_two_sum(s, p.hi);
-        s = t.hi;
-        e = __fadd_rn(e, __fadd_rn(t.lo, __fmaf_rn(a.lo, b, p.lo)));
-    }
-    // += a b, both double-float
-    __device__ __forceinline__ void add(dfl a, dfl b)
-    {
-        const dfl p = df_two_prod(a.hi, b.hi);
-        const float pe = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
-        const dfl t = df_two_sum(s, p.hi);
-        s = t.hi;
-        e = __fadd_rn(e, __fadd_rn(t.lo, pe));
-    }
-    // -= a b, both double-float
-    __device__ __forceinline__ void sub(dfl a, dfl b)
-    {
-        const dfl p = df_two_prod(a.hi, b.hi);
-        const float pe = __fmaf_rn(a.hi, b.lo, __fmaf_rn(a.lo, b.hi, p.lo));
-        const dfl t = df_two_sum(s, -p.hi);
-        s = t.hi;
-        e = __fadd_rn(e, __fsub_rn(t.lo, pe));
-    }
-    __device__ __forceinline__ dfl value() const { return df_fast_two_sum(s, e); }
-};
 
 template <typename T, int MODE, bool TR, int YY = 0, bool DF = false>
 __global__ void __launch_bounds__(OpTile<T, YY>::threads, sizeof(T) == 4 ? 3 : 2)

@@ -356,6 +356,7 @@ struct GmState {
     int total, restarts, kdim, run, inner, status, zero, pad;
     double cs[kMaxRestart], sn[kMaxRestart], gv[kMaxRestart + 1], y[kMaxRestart];
     double H[(kMaxRestart + 1) * kMaxRestart];
+    unsigned ctl, bar, bar_out;   // the one-launch solve's decision and grid barrier (solve.cu)
 };
 enum { kGmOk = 0, kGmNotConverged = 1, kGmNonfinite = 2 };
 // The fixed pointers the control kernels build launch arguments from.
@@ -400,6 +401,18 @@ cudaError_t reduce_partials_dyn(const double* partial, int nblocks, const GmDyn*
                                 cudaStream_t st);
 cudaError_t gm_update_scale_dyn(const GmDyn* dyn, const double* V, int64_t ldv, int64_t n, cudaStream_t st,
                                 int df);
+
+// ----- solve.cu: the solve in one cooperative launch -----
+// *rows: the tile height to use, 0 if the grid does not fit
+template <typename T>
+cudaError_t gm_solve_rows(GridP g, int* rows);
+// doubles of partial sums it needs (m: the restart length)
+int64_t gm_solve_partials(GridP g, int rows, int m);
+// from b and the first iterate x (GMRES vectors): x, and the outcome in st;
+// p.r and p.V are its work vectors
+template <typename T>
+cudaError_t gm_solve(const T* M, const double* b, double* x, const GmPtrs& p, const GmParams& q, GridP g, int rows,
+                     double* partial, GmState* st, int* err, bool tr, cudaStream_t s);
 
 // ----- diag.cu -----
 // tw[2 (m nx + i) + {0, 1}] = cos, sin of 2 pi ((m i) mod nx) / nx, m < nmodes

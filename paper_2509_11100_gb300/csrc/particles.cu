@@ -134,18 +134,22 @@ struct Unit {
     int j, i0, cn, c0;
 };
 
-__device__ __forceinline__ Unit unit_of(int u, int nx)
+// (uw: the units' width, at most kUnitW)
+__device__ __forceinline__ Unit unit_of(int u, int nx, int uw = kUnitW)
 {
-    const int nseg = (nx + kUnitW - 1) / kUnitW;
+    const int nseg = (nx + uw - 1) / uw;
     Unit r;
     r.j = u / nseg;
-    r.i0 = (u - r.j * nseg) * kUnitW;
-    r.cn = min(kUnitW, nx - r.i0);
+    r.i0 = (u - r.j * nseg) * uw;
+    r.cn = min(uw, nx - r.i0);
     r.c0 = r.j * nx + r.i0;
     return r;
 }
 
-__host__ __device__ __forceinline__ int units_of(int nx, int ny) { return ny * ((nx + kUnitW - 1) / kUnitW); }
+__host__ __device__ __forceinline__ int units_of(int nx, int ny, int uw = kUnitW)
+{
+    return ny * ((nx + uw - 1) / uw);
+}
 
 // B^n on the centres around a unit: [comp][row j-1, j, j+1][col i0-1 .. i0+cn].
 // NTHR threads (tid < NTHR) share the loads; for a warp the loop unrolls so
@@ -1129,7 +1133,7 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
                                                const T* __restrict__ Eth, const T* __restrict__ B,
                                                const T* __restrict__ En, GridP g, T beta, T dt_dx, T dt_dy, T qdt,
                                                T m, double* __restrict__ lsum, const PushDesc<T>* __restrict__ descs,
-                                               int ninst, int total_units)
+                                               int ninst, int total_units, int uw)
 {
     constexpr int W = PushCfg<T>::warps;
     __shared__ int sstart[W][kUnitW + 1];
@@ -1142,7 +1146,7 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     int nx = g.nx, ny = g.ny, nc = g.ncell;
-    const int nunits = BATCH ? total_units : units_of(nx, ny);
+    const int nunits = BATCH ? total_units : units_of(nx, ny, uw);
     const unsigned lt = (1u << lane) - 1u;
     int* ss = sstart[wib];
     PushTile<T>& tl = stile[wib];
@@ -1175,7 +1179,7 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
             ids = dst.id != nullptr;
             u = ug - d.unit0;
         }
-        const Unit un = unit_of(u, nx);
+        const Unit un = unit_of(u, nx, uw);
         unit_setup<T>(un, start, ss, tl, Eth, B, nx, ny, nc, lane);
         if constexpr (PRED) {
             load_tile_E<T, 32>(sen[wib].En, En, un, nx, ny, nc, lane);
@@ -1357,10 +1361,11 @@ template <typename T, bool PRED>
 __global__ void __launch_bounds__(PushCfg<T>::threads, PushCfg<T>::min_blocks)
 k_push_sort(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int32_t* __restrict__ n9,
             int32_t* __restrict__ off9, const T* __restrict__ Eth, const T* __restrict__ B,
-            const T* __restrict__ En, GridP g, T beta, T dt_dx, T dt_dy, T qdt, T m, double* __restrict__ lsum)
+            const T* __restrict__ En, GridP g, T beta, T dt_dx, T dt_dy, T qdt, T m, double* __restrict__ lsum,
+            int uw)
 {
     push_sort_core<T, PRED, false>(src, dst, start, n9, off9, Eth, B, En, g, beta, dt_dx, dt_dy, qdt, m, lsum,
-                                   nullptr, 0, 0);
+                                   nullptr, 0, 0, uw);
 }
 
 // the push of one species over the units of several instances in one launch
@@ -1371,7 +1376,7 @@ k_push_sort_batch(const PushDesc<T>* __restrict__ descs, int ninst, int total_un
     PArrays<T> none;
     memset(&none, 0, sizeof(none));
     push_sort_core<T, PRED, true>(none, none, nullptr, nullptr, nullptr, nullptr, nullptr, nullptr, GridP{}, T(0),
-                                  T(0), T(0), T(0), T(0), nullptr, descs, ninst, total_units);
+                                  T(0), T(0), T(0), T(0), nullptr, descs, ninst, total_units, kUnitW);
 }
 
 // General path (moves of more than one cell): push in place order, write the
@@ -1380,7 +1385,7 @@ template <typename T, bool PRED>
 __global__ void __launch_bounds__(PushCfg<T>::threads, PushCfg<T>::min_blocks)
 k_push_general(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int32_t* __restrict__ key,
                const T* __restrict__ Eth, const T* __restrict__ B, const T* __restrict__ En, GridP g, T beta,
-               T dt_dx, T dt_dy, T qdt, T m, double* __restrict__ lsum)
+               T dt_dx, T dt_dy, T qdt, T m, double* __restrict__ lsum, int uw)
 {
     constexpr int W = PushCfg<T>::warps;
     __shared__ int sstart[W][kUnitW + 1];
@@ -1391,12 +1396,12 @@ k_push_general(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nx = g.nx, ny = g.ny, nc = g.ncell;
-    const int nunits = units_of(nx, ny);
+    const int nunits = units_of(nx, ny, uw);
     int* ss = sstart[wib];
     PushTile<T>& tl = stile[wib];
     T acc[kLedger] = {T(0), T(0), T(0), T(0)};
     for (int u = warp; u < nunits; u += nwarps) {
-        const Unit un = unit_of(u, nx);
+        const Unit un = unit_of(u, nx, uw);
         unit_setup<T>(un, start, ss, tl, Eth, B, nx, ny, nc, lane);
         if constexpr (PRED) {
             load_tile_E<T, 32>(sen[wib].En, En, un, nx, ny, nc, lane);
@@ -1438,7 +1443,7 @@ template <typename T, bool BATCH>
 __device__ __forceinline__ void permute_core(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start_new,
                                              const int32_t* __restrict__ n9, const int32_t* __restrict__ off9,
                                              GridP g, int* __restrict__ err, const PushDesc<T>* __restrict__ descs,
-                                             int ninst, int total_units)
+                                             int ninst, int total_units, int uw)
 {
     __shared__ int scs[8][kUnitW + 1];          // new cell starts of the unit
     __shared__ int srs[8][kUnitW][kNDir];       // run start in src, in run order
@@ -1447,7 +1452,7 @@ __device__ __forceinline__ void permute_core(PArrays<T> src, PArrays<T> dst, con
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     int nx = g.nx, ny = g.ny;
-    const int nunits = BATCH ? total_units : units_of(nx, ny);
+    const int nunits = BATCH ? total_units : units_of(nx, ny, uw);
     bool ids = dst.id != nullptr;
     int* cs = scs[wib];
     for (int ug = warp; ug < nunits; ug += nwarps) {
@@ -1467,7 +1472,7 @@ __device__ __forceinline__ void permute_core(PArrays<T> src, PArrays<T> dst, con
             ids = dst.id != nullptr;
             u = ug - d.unit0;
         }
-        const Unit un = unit_of(u, nx);
+        const Unit un = unit_of(u, nx, uw);
         const int cn = un.cn;
 #pragma unroll
         for (int k0 = 0; k0 <= kUnitW; k0 += 32)
@@ -1555,9 +1560,9 @@ __device__ __forceinline__ void permute_core(PArrays<T> src, PArrays<T> dst, con
 template <typename T>
 __global__ void __launch_bounds__(256)
 k_permute(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start_new, const int32_t* __restrict__ n9,
-          const int32_t* __restrict__ off9, GridP g, int* __restrict__ err)
+          const int32_t* __restrict__ off9, GridP g, int* __restrict__ err, int uw)
 {
-    permute_core<T, false>(src, dst, start_new, n9, off9, g, err, nullptr, 0, 0);
+    permute_core<T, false>(src, dst, start_new, n9, off9, g, err, nullptr, 0, 0, uw);
 }
 
 // the re-sort of one species over the units of several instances
@@ -1567,7 +1572,7 @@ k_permute_batch(const PushDesc<T>* __restrict__ descs, int ninst, int total_unit
 {
     PArrays<T> none;
     memset(&none, 0, sizeof(none));
-    permute_core<T, true>(none, none, nullptr, nullptr, nullptr, GridP{}, nullptr, descs, ninst, total_units);
+    permute_core<T, true>(none, none, nullptr, nullptr, nullptr, GridP{}, nullptr, descs, ninst, total_units, kUnitW);
 }
 
 template <typename T>
@@ -1741,7 +1746,7 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
                const double* __restrict__ gx1, double* __restrict__ gu0, double* __restrict__ gx0,
                double* __restrict__ gE, double* __restrict__ gB, const T* __restrict__ Eth,
                const T* __restrict__ B, GridP g, double beta_d, const T* __restrict__ Eold,
-               double* __restrict__ gEold)
+               double* __restrict__ gEold, int uw)
 {
     using A = T;
     constexpr int W = PushCfg<T>::warps;
@@ -1752,12 +1757,12 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nx = g.nx, ny = g.ny, nc = g.ncell;
-    const int nunits = units_of(nx, ny);
+    const int nunits = units_of(nx, ny, uw);
     int* ss = sstart[wib];
     PushTile<T>& tl = stile[wib];
     const A rdx = A(1.0 / g.dx), rdy = A(1.0 / g.dy), dt = A(g.dt), beta = A(beta_d);
     for (int u = warp; u < nunits; u += nwarps) {
-        const Unit un = unit_of(u, nx);
+        const Unit un = unit_of(u, nx, uw);
         unit_setup<T>(un, start, ss, tl, Eth, B, nx, ny, nc, lane);
         if constexpr (PRED) {
             load_tile_E<T, 32>(sen[wib].En, Eold, un, nx, ny, nc, lane);
@@ -1957,7 +1962,7 @@ __global__ void __launch_bounds__(PushCfg<T>::threads, sizeof(T) == 4 ? 4 : 1)
 k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* __restrict__ gJ,
                   const double* __restrict__ gM, double* __restrict__ gu0, double* __restrict__ gx0,
                   double* __restrict__ gw0, double* __restrict__ gB, const T* __restrict__ B, GridP g, double beta_d,
-                  double cq, const T* __restrict__ Eold, double* __restrict__ gEold)
+                  double cq, const T* __restrict__ Eold, double* __restrict__ gEold, int uw)
 {
     using A = T;
     constexpr int W = PushCfg<T>::warps;
@@ -1968,7 +1973,7 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int nx = g.nx, ny = g.ny, nc = g.ncell;
-    const int nunits = units_of(nx, ny);
+    const int nunits = units_of(nx, ny, uw);
     int* ss = sstart[wib];
     PushTile<T>& tl = stile[wib];
     const A rdx = A(1.0 / g.dx), rdy = A(1.0 / g.dy), beta = A(beta_d);
@@ -1979,7 +1984,7 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
     constexpr int ps[10] = {0, 0, 0, 0, 1, 1, 1, 2, 2, 3};
     constexpr int po[10] = {0, 1, 3, 4, 0, 2, 3, 0, 1, 0};
     for (int u = warp; u < nunits; u += nwarps) {
-        const Unit un = unit_of(u, nx);
+        const Unit un = unit_of(u, nx, uw);
         unit_setup<T>(un, start, ss, tl, B, B, nx, ny, nc, lane);
         if constexpr (PRED) {
             load_tile_E<T, 32>(sen[wib].En, Eold, un, nx, ny, nc, lane);
@@ -2181,10 +2186,24 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
 
 int row_units(GridP g) { return units_of(g.nx, g.ny); }
 
+// The width of the row units of the passes that give a warp a unit (push,
+// re-sort, adjoints): the full 32 cells, halved while that leaves fewer than
+// eight warps per SM in flight (with 16 as the line, eight instances stepped
+// side by side lost 8% to the narrower units' tiles and half-full batches). A unit's warp takes its particles batch after
+// batch, so on a small grid the launch lasts as long as one unit: at 128x64
+// with 32 particles a cell (FP32 form) the push of a species took 65 us on
+// 256 units of 32 cells, 21 us on 2048 of 4 (the re-sort 24 and 7 us).
+int unit_width(GridP g)
+{
+    int uw = kUnitW;
+    while (uw > 2 && units_of(g.nx, g.ny, uw) < 152 * 8) uw /= 2;
+    return uw;
+}
+
 int push_grid_blocks(GridP g, int precision, int cap)
 {
-    return blocks_for(units_of(g.nx, g.ny), precision == 32 ? PushCfg<float>::warps : PushCfg<double>::warps,
-                      cap > 0 ? cap : 152 * 16);
+    return blocks_for(units_of(g.nx, g.ny, unit_width(g)),
+                      precision == 32 ? PushCfg<float>::warps : PushCfg<double>::warps, cap > 0 ? cap : 152 * 16);
 }
 
 template <typename T>
@@ -2255,7 +2274,7 @@ cudaError_t push_sort(PArrays<T> src, PArrays<T> dst, const int32_t* start, int3
     count_launches(1);
     kern<<<lsum_blocks, PushCfg<T>::threads, 0, st>>>(src, dst, start, n9, off9, Eth, B, En, g, beta,
                                                       (T)(g.dt / g.dx), (T)(g.dt / g.dy), (T)(sc.q * g.dt),
-                                                      (T)sc.m, lsum_partial);
+                                                      (T)sc.m, lsum_partial, unit_width(g));
     return cudaGetLastError();
 }
 
@@ -2304,10 +2323,11 @@ cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const double* 
     const int nb = push_grid_blocks(g, sizeof(T) == 4 ? 32 : 64, 152 * 16);
     if (En)
         k_deposit_adjoint<T, true><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gJ, gM, gu0, gx0, gw0, gB, B, g,
-                                                                       beta, sc.q, En, gEn);
+                                                                       beta, sc.q, En, gEn, unit_width(g));
     else
         k_deposit_adjoint<T, false><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gJ, gM, gu0, gx0, gw0, gB, B, g,
-                                                                        beta, sc.q, nullptr, nullptr);
+                                                                        beta, sc.q, nullptr, nullptr,
+                                                                        unit_width(g));
     return cudaGetLastError();
 }
 
@@ -2321,10 +2341,10 @@ cudaError_t push_adjoint(PArrays<T> src, const int32_t* start, const double* gu1
     const int nb = push_grid_blocks(g, sizeof(T) == 4 ? 32 : 64, 152 * 16);
     if (En)
         k_push_adjoint<T, true><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gu1, gx1, gu0, gx0, gE, gB, Eth, B,
-                                                                    g, beta, En, gEn);
+                                                                    g, beta, En, gEn, unit_width(g));
     else
         k_push_adjoint<T, false><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gu1, gx1, gu0, gx0, gE, gB, Eth, B,
-                                                                     g, beta, nullptr, nullptr);
+                                                                     g, beta, nullptr, nullptr, unit_width(g));
     return cudaGetLastError();
 }
 
@@ -2338,7 +2358,7 @@ cudaError_t push_general(PArrays<T> src, PArrays<T> dst, const int32_t* start, i
     count_launches(1);
     kern<<<lsum_blocks, PushCfg<T>::threads, 0, st>>>(src, dst, start, key, Eth, B, En, g, beta,
                                                       (T)(g.dt / g.dx), (T)(g.dt / g.dy), (T)(sc.q * g.dt),
-                                                      (T)sc.m, lsum_partial);
+                                                      (T)sc.m, lsum_partial, unit_width(g));
     return cudaGetLastError();
 }
 
@@ -2347,8 +2367,9 @@ cudaError_t permute(PArrays<T> src, PArrays<T> dst, const int32_t* start_new, co
                     const int32_t* off9, GridP g, int* err, cudaStream_t st)
 {
     count_launches(1);
-    k_permute<T><<<blocks_for(units_of(g.nx, g.ny), 8, 152 * 16), 256, 0, st>>>(src, dst, start_new, n9, off9,
-                                                                             g, err);
+    const int uw = unit_width(g);
+    k_permute<T><<<blocks_for(units_of(g.nx, g.ny, uw), 8, 152 * 16), 256, 0, st>>>(src, dst, start_new, n9, off9, g,
+                                                                                    err, uw);
     return cudaGetLastError();
 }
 

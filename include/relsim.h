@@ -388,7 +388,7 @@ RELSIM_API int relsim_push_adjoint(relsim_ctx* ctx, int species, const double* g
    push's re-sort leaves, so a window of steps chains calls without
    reordering anything. The context is left solved (relsim_push advances
    it). *iters, *rel_residual (may be NULL): the adjoint solve. Device
-   scratch of 10 max_s(n_s) + 7*3*ncell + 45*ncell doubles is kept by the
+   scratch of 10 max_s(n_s) + 90*ncell doubles is kept by the
    context. In a gamma_pred context the chain also runs through the
    predicted Lorentz factor gamma(u^n + beta E^n(x)) of the deposit and the
    push: its dL/dE^n joins the field adjoint's in gE, its dL/du^n and

@@ -64,6 +64,13 @@ __global__ void k_scatter_grad(const int32_t* __restrict__ id, const double* __r
     }
 }
 
+template <typename T>
+__global__ void k_narrow(const double* __restrict__ in, T* __restrict__ out, int64_t n)
+{
+    for (int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; i < n; i += (int64_t)gridDim.x * blockDim.x)
+        out[i] = narrow<T>(in[i]);
+}
+
 // gw[id[i]] += lw[i]
 __global__ void k_scatter_add_w(const int32_t* __restrict__ id, const double* __restrict__ lw, double* __restrict__ gw,
                                 int64_t n)
@@ -115,6 +122,17 @@ cudaError_t scatter_grad(const int32_t* id, const double* lu, const double* lx, 
         k_scatter_grad<false><<<grid_for(n), kThreads, 0, st>>>(id, lu, lx, gu, gx, n);
     return cudaGetLastError();
 }
+
+template <typename T>
+cudaError_t narrow_array(const double* in, T* out, int64_t n, cudaStream_t st)
+{
+    if (n <= 0) return cudaSuccess;
+    count_launches(1);
+    k_narrow<T><<<grid_for(n), kThreads, 0, st>>>(in, out, n);
+    return cudaGetLastError();
+}
+template cudaError_t narrow_array<float>(const double*, float*, int64_t, cudaStream_t);
+template cudaError_t narrow_array<double>(const double*, double*, int64_t, cudaStream_t);
 
 cudaError_t scatter_add_w(const int32_t* id, const double* lw, double* gw, int64_t n, cudaStream_t st)
 {

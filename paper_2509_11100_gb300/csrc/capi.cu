@@ -1423,6 +1423,25 @@ int adjoint_impl(relsim_ctx* c, const double* gE1, const double* gB1, const doub
     return RELSIM_OK;
 }
 
+// the deposit adjoint's gJ and gM in the form's precision: each is read once
+// per particle, so the FP32 form converts them once per node here (as casts
+// in the kernel they were 100 operations a particle on the FP64 pipe)
+template <typename T>
+int narrow_gm(relsim_ctx* c, const double* gJ, const double* gM, T* scratch, const T** nJ, const T** nM)
+{
+    if constexpr (sizeof(T) == 8) {
+        *nJ = gJ;
+        *nM = gM;
+    } else {
+        const int64_t nf = 3 * (int64_t)c->g.ncell, nm = (int64_t)c->g.ncell * kMBlock;
+        CK(narrow_array<T>(gM, scratch, nm, c->st));
+        CK(narrow_array<T>(gJ, scratch + nm, nf, c->st));
+        *nM = scratch;
+        *nJ = scratch + nm;
+    }
+    return RELSIM_OK;
+}
+
 // The adjoint of one species' deposit (k_deposit_adjoint); gB is
 // overwritten with this species' contribution.
 template <typename T>
@@ -1441,9 +1460,13 @@ int deposit_adjoint_impl(relsim_ctx* c, int s, const double* gJ, const double* g
     double* oB = host ? c->stage + nf + nm + 5 * n : gB;
     double* ow = gw0 ? (host ? c->stage + nf + nm + 5 * n + nf : gw0) : nullptr;
     CK(cudaMemsetAsync(oB, 0, sizeof(double) * (size_t)nf, c->st));
-    if (n > 0)
-        CK(deposit_adjoint<T>(arrays<T>(sp, sp.cur), sp.start, dJ, dM, ou, ox, ow, oB, (const T*)c->B[c->bcur], c->g,
+    if (n > 0) {
+        if (sizeof(T) == 4) TRY(ensure_adj(c, (nf + nm + 1) / 2));
+        const T *tJ = nullptr, *tM = nullptr;
+        TRY(narrow_gm<T>(c, dJ, dM, (T*)c->adj, &tJ, &tM));
+        CK(deposit_adjoint<T>(arrays<T>(sp, sp.cur), sp.start, tJ, tM, ou, ox, ow, oB, (const T*)c->B[c->bcur], c->g,
                               SpeciesConst{c->cfg.q[s], c->cfg.m[s]}, c->st));
+    }
     if (host) {
         CK(cudaMemcpyAsync(gu0, ou, sizeof(double) * (size_t)(3 * n), cudaMemcpyDeviceToHost, c->st));
         CK(cudaMemcpyAsync(gx0, ox, sizeof(double) * (size_t)(2 * n), cudaMemcpyDeviceToHost, c->st));
@@ -1500,7 +1523,7 @@ int step_adjoint_impl(relsim_ctx* c, double* gE, double* gB, double* const* gu, 
     const int64_t nf = 3 * (int64_t)c->g.ncell, nm = (int64_t)c->g.ncell * kMBlock;
     int64_t nmax = 0;
     for (int s = 0; s < c->cfg.nspecies; ++s) nmax = c->sp[s].n > nmax ? c->sp[s].n : nmax;
-    TRY(ensure_adj(c, 10 * nmax + 7 * nf + nm));
+    TRY(ensure_adj(c, 10 * nmax + 7 * nf + nm + (nf + nm + 1) / 2));
     double* L = c->adj;           // 5 nmax: a species' gradients in its current order
     double* P = L + 5 * nmax;     // 5 nmax: its push adjoint's dL/du^n, dL/dx^{n+1/2}
     double* sE = P + 5 * nmax;    // dL/dE^{n+theta} of the pushes
@@ -1510,6 +1533,7 @@ int step_adjoint_impl(relsim_ctx* c, double* gE, double* gB, double* const* gu, 
     double* fJ = fB + nf;
     double* fM = fJ + nf;
     double* sEn = fM + nm;        // predicted gbar: dL/dE^n of the pushes and the deposits
+    T* narrowed = (T*)(sEn + nf);   // FP32 form: dL/dM and dL/dJhat in FP32
     const T* Bn = (const T*)c->B[c->bcur];
     // E^n of the predicted gbar (the solve kept it before E^{n+1} replaced it)
     const T* En = c->En ? (const T*)c->En : nullptr;
@@ -1527,13 +1551,15 @@ int step_adjoint_impl(relsim_ctx* c, double* gE, double* gB, double* const* gu, 
     }
     const int fr = adjoint_impl<T>(c, gE, gB, sE, fE, fB, fJ, fM, iters, relres, RELSIM_DEVICE);
     if (fr != RELSIM_OK && fr != RELSIM_ERR_NOT_CONVERGED) return fr;
+    const T *tJ = nullptr, *tM = nullptr;
+    TRY(narrow_gm<T>(c, fJ, fM, narrowed, &tJ, &tM));
     for (int s = 0; s < c->cfg.nspecies; ++s) {
         Species& sp = c->sp[s];
         const int64_t n = sp.n;
         if (n == 0) continue;
         const PArrays<T> a = arrays<T>(sp, sp.cur);
         double* lw = gw && gw[s] ? P : nullptr;   // the push adjoint's output was scattered already
-        CK(deposit_adjoint<T>(a, sp.start, fJ, fM, L, L + 3 * n, lw, sB, Bn, c->g,
+        CK(deposit_adjoint<T>(a, sp.start, tJ, tM, L, L + 3 * n, lw, sB, Bn, c->g,
                               SpeciesConst{c->cfg.q[s], c->cfg.m[s]}, c->st, En, sEn));
         CK(scatter_grad(a.id, L, L + 3 * n, gu[s], gx[s], n, true, c->st));
         if (lw) CK(scatter_add_w(a.id, lw, gw[s], n, c->st));

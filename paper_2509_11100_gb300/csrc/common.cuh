@@ -169,6 +169,57 @@ template <> struct Consts<double> {
     static __device__ __forceinline__ double one_below() { return 0.99999999999999989; }  // 1 - 2^-53
 };
 
+// ---- FP32 <-> FP64 conversions on the integer pipe ----
+// GB300 converts between FP32 and FP64 on its FP64 pipe, which takes a warp's
+// operation in about 64 cycles; a kernel that only carries FP32 values in or
+// out of FP64 arrays is bound by that alone. These give the bits of the casts
+// (round to nearest even; any NaN becomes a quiet one) in about ten integer
+// instructions, with branches for subnormal and non-finite values.
+__device__ __forceinline__ double widen(float a)
+{
+    const unsigned b = __float_as_uint(a), m = b & 0x7fffffffu;
+    unsigned hi = (m >> 3) + 0x38000000u, lo = b << 29;
+    if (m - 0x00800000u >= 0x7f000000u) {
+        if (m >= 0x7f800000u) {
+            hi += 0x38000000u;   // infinite, NaN
+        } else if (m == 0u) {
+            hi = 0u;
+        } else {                 // subnormal: normalised
+            const int n = __clz((int)m) - 8;
+            hi = ((unsigned)(896 - n) << 20) + ((m << n) >> 3);
+            lo = (m << n) << 29;
+        }
+    }
+    return __hiloint2double((int)(hi | (b & 0x80000000u)), (int)lo);
+}
+__device__ __forceinline__ double widen(double a) { return a; }
+
+template <typename T> __device__ __forceinline__ T narrow(double a);
+template <> __device__ __forceinline__ double narrow<double>(double a) { return a; }
+template <> __device__ __forceinline__ float narrow<float>(double a)
+{
+    const unsigned hi = (unsigned)__double2hiint(a), lo = (unsigned)__double2loint(a), m = hi & 0x7fffffffu;
+    // 2^-126 <= |a| < 2^128: the exponent rebased, 29 bits rounded off
+    unsigned q = __funnelshift_r(lo, m - 0x38000000u, 29);
+    const unsigned rest = lo & 0x1fffffffu;
+    q += rest + (q & 1u) > 0x10000000u ? 1u : 0u;
+    if (m - 0x38100000u >= 0x47f00000u - 0x38100000u) {
+        if (m >= 0x47f00000u) {
+            q = m > 0x7ff00000u || (m == 0x7ff00000u && lo != 0u) ? 0x7fffffffu : 0x7f800000u;
+        } else {   // subnormal in FP32 (or zero): units of 2^-149
+            const int s = 926 - (int)(m >> 20);
+            q = 0u;
+            if (s <= 54) {
+                const unsigned long long sig = ((unsigned long long)((m & 0xfffffu) | 0x100000u) << 32) | lo;
+                const unsigned long long r = sig & ((1ull << s) - 1ull), half = 1ull << (s - 1);
+                q = (unsigned)(sig >> s);
+                if (r > half || (r == half && (q & 1u))) ++q;
+            }
+        }
+    }
+    return __uint_as_float(q | (hi & 0x80000000u));
+}
+
 // ---- TMA bulk copies (cp.async.bulk) completing on an mbarrier ----
 // A bulk copy needs 16-byte aligned source and destination addresses and a
 // size that is a multiple of 16 bytes.

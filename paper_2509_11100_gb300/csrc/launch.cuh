@@ -188,6 +188,9 @@ cudaError_t gather_grad(const int32_t* id, const double* gu, const double* gx, d
 cudaError_t scatter_grad(const int32_t* id, const double* lu, const double* lx, double* gu, double* gx, int64_t n,
                          bool add, cudaStream_t st);
 // gw[id[i]] += lw[i]
+// out = in in the form's precision
+template <typename T>
+cudaError_t narrow_array(const double* in, T* out, int64_t n, cudaStream_t st);
 cudaError_t scatter_add_w(const int32_t* id, const double* lw, double* gw, int64_t n, cudaStream_t st);
 // bit 0 of *bad if id[i] or ids[i] is outside [0, n) (flag accumulates)
 cudaError_t check_ids(const int32_t* id, const int32_t* ids, int64_t n, int* bad, cudaStream_t st);
@@ -232,7 +235,7 @@ cudaError_t push_general(PArrays<T> src, PArrays<T> dst, const int32_t* start, i
 // predicted gbar = gamma(u^n + beta E^n(x)) with E^n = En, and dL/dE^n
 // added into gEn.
 template <typename T>
-cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const double* gJ, const double* gM, double* gu0,
+cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const T* gJ, const T* gM, double* gu0,
                             double* gx0, double* gw0, double* gB, const T* B, GridP g, SpeciesConst sc,
                             cudaStream_t st, const T* En = nullptr, double* gEn = nullptr);
 // adjoint of the push with the fields fixed: per particle dL/du^n,

@@ -22,6 +22,51 @@ __device__ __forceinline__ bool is_pow2(double v)
     return frexp(v, &e) == 0.5;
 }
 
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// A finite lattice coordinate into its cell (wrapped into [0, n)) and the
+// offset within it, rounded toward zero in FP32
+template <typename T>
+__device__ __noinline__ void split_cell_wrap(double xs, int n, int& i, T& f)
+{
+    if (xs < 0.0 || xs >= (double)n) xs -= n * floor(xs / n);
+    const double fi = floor(xs);
+    i = (int)fi;
+    if (i >= n) i -= n;
+    if (i < 0) i = 0;
+    f = from_double_rz<T>(xs - fi);
+}
+template <typename T>
+__device__ __forceinline__ void split_cell(double xs, int n, int& i, T& f)
+{
+    if constexpr (sizeof(T) == 4) {
+        // inside the box, on the integer pipe: the coordinate's bits are cut
+        // at the unit place, the fraction's leading 24 are the offset (exact,
+        // then truncated: the same as floor, subtraction and conversion)
+        const unsigned hi = (unsigned)__double2hiint(xs), lo = (unsigned)__double2loint(xs);
+        const int sh = 1075 - (int)(hi >> 20);   // fraction bits of the 53-bit significand (a sign bit: negative)
+        if (sh >= 22 && sh < 100) {
+            const unsigned long long sig = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+            i = sh > 52 ? 0 : (int)(sig >> sh);
+            if (i < n) {
+                const unsigned long long r = sh > 52 ? sig : sig & ((1ull << sh) - 1ull);
+                const int lz = __clzll((long long)r);
+                f = r == 0ull ? 0.0f
+                              : __uint_as_float(((unsigned)(190 - lz - sh) << 23) |
+                                                ((unsigned)((r << lz) >> 40) & 0x7fffffu));
+                return;
+            }
+        } else if ((hi | lo) == 0u) {
+            i = 0;
+            f = 0.0f;
+            return;
+        }
+    }
+    split_cell_wrap<T>(xs, n, i, f);
+}
+
+// (FP32 form: the positions and momenta go from FP64 to FP32 on the integer
+// pipe; on the FP64 pipe about 25 operations a particle bounded the load)
 template <typename T>
 __global__ void k_load_convert(const double* __restrict__ x, const double* __restrict__ u,
                                const double* __restrict__ w, int64_t n, GridP g, PArrays<T> out,
@@ -32,32 +77,29 @@ __global__ void k_load_convert(const double* __restrict__ x, const double* __res
     // a power-of-two cell size scales exactly by its reciprocal (FP64
     // division is costly on this GPU); any other size divides
     const double rdx = 1.0 / g.dx, rdy = 1.0 / g.dy;
-    const bool exact = is_pow2(g.dx) && is_pow2(g.dy);
+    const bool exact = is_pow2(g.dx) && is_pow2(g.dy), unit = is_one(g.dx) && is_one(g.dy);
     for (; p < n; p += stride) {
-        double xs = exact ? x[2 * p] * rdx : x[2 * p] / g.dx;
-        double ys = exact ? x[2 * p + 1] * rdy : x[2 * p + 1] / g.dy;
+        double xs = x[2 * p], ys = x[2 * p + 1];
+        if (!unit) {
+            xs = exact ? xs * rdx : xs / g.dx;
+            ys = exact ? ys * rdy : ys / g.dy;
+        }
         double ux = u[3 * p], uy = u[3 * p + 1], uz = u[3 * p + 2], ww = w[p];
-        if (!isfinite(xs) || !isfinite(ys) || !isfinite(ux) || !isfinite(uy) || !isfinite(uz) ||
-            !isfinite(ww)) {
+        if (!finite_bits(xs) || !finite_bits(ys) || !finite_bits(ux) || !finite_bits(uy) || !finite_bits(uz) ||
+            !finite_bits(ww)) {
             atomicOr(bad, 1);
             xs = ys = 0.0;
         }
-        // periodic wrap into [0, n) (only for positions outside the box),
-        // then split into cell + offset
-        if (xs < 0.0 || xs >= (double)g.nx) xs -= g.nx * floor(xs / g.nx);
-        if (ys < 0.0 || ys >= (double)g.ny) ys -= g.ny * floor(ys / g.ny);
-        double fi = floor(xs), fj = floor(ys);
-        int i = (int)fi, j = (int)fj;
-        if (i >= g.nx) i -= g.nx;
-        if (j >= g.ny) j -= g.ny;
-        if (i < 0) i = 0;
-        if (j < 0) j = 0;
-        out.fx[p] = from_double_rz<T>(xs - fi);
-        out.fy[p] = from_double_rz<T>(ys - fj);
-        out.ux[p] = (T)ux;
-        out.uy[p] = (T)uy;
-        out.uz[p] = (T)uz;
-        out.w[p] = (T)ww;
+        int i, j;
+        T fx, fy;
+        split_cell<T>(xs, g.nx, i, fx);
+        split_cell<T>(ys, g.ny, j, fy);
+        out.fx[p] = fx;
+        out.fy[p] = fy;
+        out.ux[p] = narrow<T>(ux);
+        out.uy[p] = narrow<T>(uy);
+        out.uz[p] = narrow<T>(uz);
+        out.w[p] = narrow<T>(ww);
         key[p] = j * g.nx + i;
         val[p] = (int32_t)p;
     }
@@ -90,7 +132,8 @@ __global__ void k_gather(const int32_t* __restrict__ perm, PArrays<T> src, PArra
     }
 }
 
-// one warp per cell: absolute positions back to FP64
+// one warp per cell: absolute positions back to FP64 (FP32 form: bound by the
+// FP64 pipe, so one addition a coordinate is all that is left on it)
 template <typename T>
 __global__ void k_export(PArrays<T> pa, const int32_t* __restrict__ start, GridP g, double* x,
                          double* u, double* w, int32_t* id)
@@ -98,20 +141,27 @@ __global__ void k_export(PArrays<T> pa, const int32_t* __restrict__ start, GridP
     const int lane = threadIdx.x & 31;
     int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const bool unit = is_one(g.dx) && is_one(g.dy);
     for (int c = warp; c < g.ncell; c += nwarps) {
         int i = c % g.nx, j = c / g.nx;
+        const double id0 = (double)i, jd0 = (double)j;
         int p1 = start[c + 1];
         for (int p = start[c] + lane; p < p1; p += 32) {
             if (x) {
-                x[2 * (int64_t)p] = ((double)i + (double)pa.fx[p]) * g.dx;
-                x[2 * (int64_t)p + 1] = ((double)j + (double)pa.fy[p]) * g.dy;
+                double xs = id0 + widen(pa.fx[p]), ys = jd0 + widen(pa.fy[p]);
+                if (!unit) {
+                    xs *= g.dx;
+                    ys *= g.dy;
+                }
+                x[2 * (int64_t)p] = xs;
+                x[2 * (int64_t)p + 1] = ys;
             }
             if (u) {
-                u[3 * (int64_t)p] = (double)pa.ux[p];
-                u[3 * (int64_t)p + 1] = (double)pa.uy[p];
-                u[3 * (int64_t)p + 2] = (double)pa.uz[p];
+                u[3 * (int64_t)p] = widen(pa.ux[p]);
+                u[3 * (int64_t)p + 1] = widen(pa.uy[p]);
+                u[3 * (int64_t)p + 2] = widen(pa.uz[p]);
             }
-            if (w) w[p] = (double)pa.w[p];
+            if (w) w[p] = widen(pa.w[p]);
             if (id && pa.id) id[p] = pa.id[p];
         }
     }
@@ -1724,7 +1774,7 @@ __device__ __forceinline__ void flush_centres(const A (&gc)[3][3][3], const Runs
 #pragma unroll
             for (int k = 0; k < 3; ++k) {
                 const A s = run_sum(gc[k][r][c], rn);
-                if (rn.head && act) atomicAdd(gB + (int64_t)k * nc + cell, (double)s);
+                if (rn.head && act) atomicAdd(gB + (int64_t)k * nc + cell, widen(s));
             }
         }
     }
@@ -1860,12 +1910,12 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
                 for (int k = 0; k < 3; ++k) u1[k] = A(2) * ub[k] - u0[k];
                 const A g1 = sqrt(A(1) + u1[0] * u1[0] + u1[1] * u1[1] + u1[2] * u1[2]);
                 // backward: x1 = x + dt u1/g1
-                const A gp[3] = {(A)gx1[2 * (int64_t)p], (A)gx1[2 * (int64_t)p + 1], A(0)};
+                const A gp[3] = {narrow<A>(gx1[2 * (int64_t)p]), narrow<A>(gx1[2 * (int64_t)p + 1]), A(0)};
                 const A up = u1[0] * gp[0] + u1[1] * gp[1];
                 A gt[3], gub[3], gu[3], gw[3];
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
-                    gt[k] = (A)gu1[3 * (int64_t)p + k] + dt * (gp[k] / g1 - u1[k] * up / (g1 * g1 * g1));
+                    gt[k] = narrow<A>(gu1[3 * (int64_t)p + k]) + dt * (gp[k] / g1 - u1[k] * up / (g1 * g1 * g1));
                     gub[k] = A(2) * gt[k];
                     gu[k] = -gt[k];
                 }
@@ -1917,9 +1967,9 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
 #pragma unroll
                         for (int c = 0; c < 3; ++c) gc[k][r][c] = Ry[r] * Cx[c] * gBp[k];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) gu0[3 * (int64_t)p + k] = (double)gu[k];
-                gx0[2 * (int64_t)p] = (double)gxp;
-                gx0[2 * (int64_t)p + 1] = (double)gyp;
+                for (int k = 0; k < 3; ++k) gu0[3 * (int64_t)p + k] = widen(gu[k]);
+                gx0[2 * (int64_t)p] = widen(gxp);
+                gx0[2 * (int64_t)p + 1] = widen(gyp);
             }
             // the cell runs' totals: nodes (i, j), (i+1, j), (i, j+1), (i+1, j+1)
             const Runs rn = runs_of(act ? cl : -1, lane);
@@ -1932,7 +1982,7 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
 #pragma unroll
                 for (int k = 0; k < 3; ++k) {
                     const A s = run_sum(gn[q][k], rn);
-                    if (rn.head && act) atomicAdd(gE + (int64_t)k * nc + nodes[q], (double)s);
+                    if (rn.head && act) atomicAdd(gE + (int64_t)k * nc + nodes[q], widen(s));
                 }
             if constexpr (PRED) {
 #pragma unroll
@@ -1940,7 +1990,7 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         const A s = run_sum(go[q][k], rn);
-                        if (rn.head && act) atomicAdd(gEold + (int64_t)k * nc + nodes[q], (double)s);
+                        if (rn.head && act) atomicAdd(gEold + (int64_t)k * nc + nodes[q], widen(s));
                     }
             }
             flush_centres(gc, rn, act, gB, i, j, nx, ny, nc);
@@ -1959,8 +2009,8 @@ k_push_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* 
 // and dL/dx^{n+1/2} (gx0), FP64.
 template <typename T, bool PRED>
 __global__ void __launch_bounds__(PushCfg<T>::threads, sizeof(T) == 4 ? 4 : 1)
-k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const double* __restrict__ gJ,
-                  const double* __restrict__ gM, double* __restrict__ gu0, double* __restrict__ gx0,
+k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const T* __restrict__ gJ,
+                  const T* __restrict__ gM, double* __restrict__ gu0, double* __restrict__ gx0,
                   double* __restrict__ gw0, double* __restrict__ gB, const T* __restrict__ B, GridP g, double beta_d,
                   double cq, const T* __restrict__ Eold, double* __restrict__ gEold, int uw)
 {
@@ -2071,7 +2121,7 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
                 A sJw = A(0), sMw = A(0);   // the same sums per unit weight (J and M are linear in w)
 #pragma unroll
                 for (int k = 0; k < 4; ++k) {
-                    const A gj[3] = {(A)gJ[nodes[k]], (A)gJ[nc + nodes[k]], (A)gJ[2 * (int64_t)nc + nodes[k]]};
+                    const A gj[3] = {ld(gJ + nodes[k]), ld(gJ + nc + nodes[k]), ld(gJ + 2 * (int64_t)nc + nodes[k])};
                     const A f = cJ * Wn[k];
                     A sJ = A(0);
 #pragma unroll
@@ -2089,10 +2139,10 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
                 }
 #pragma unroll
                 for (int pr = 0; pr < 10; ++pr) {
-                    const double* G = gM + nodes[ps[pr]] * kMBlock + po[pr] * 9;
+                    const A* G = gM + nodes[ps[pr]] * kMBlock + po[pr] * 9;
                     A Gv[9];
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) Gv[e] = (A)G[e];
+                    for (int e = 0; e < 9; ++e) Gv[e] = ld(G + e);
                     A s2 = A(0);
 #pragma unroll
                     for (int r = 0; r < 3; ++r)
@@ -2158,10 +2208,10 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
 #pragma unroll
                         for (int c = 0; c < 3; ++c) gc[k][r][c] = Ry[r] * Cx[c] * gBp[k];
 #pragma unroll
-                for (int k = 0; k < 3; ++k) gu0[3 * (int64_t)p + k] = (double)gu[k];
-                gx0[2 * (int64_t)p] = (double)gxp;
-                gx0[2 * (int64_t)p + 1] = (double)gyp;
-                if (gw0) gw0[p] = (double)((cJ0 * sJw + cM0 * sMw) * rgb);
+                for (int k = 0; k < 3; ++k) gu0[3 * (int64_t)p + k] = widen(gu[k]);
+                gx0[2 * (int64_t)p] = widen(gxp);
+                gx0[2 * (int64_t)p + 1] = widen(gyp);
+                if (gw0) gw0[p] = widen((cJ0 * sJw + cM0 * sMw) * rgb);
             }
             const Runs rn = runs_of(act ? cl : -1, lane);
             flush_centres(gc, rn, act, gB, i, j, nx, ny, nc);
@@ -2174,7 +2224,7 @@ k_deposit_adjoint(PArrays<T> src, const int32_t* __restrict__ start, const doubl
 #pragma unroll
                     for (int k = 0; k < 3; ++k) {
                         const A sq = run_sum(go[q][k], rn);
-                        if (rn.head && act) atomicAdd(gEold + (int64_t)k * nc + nodes[q], (double)sq);
+                        if (rn.head && act) atomicAdd(gEold + (int64_t)k * nc + nodes[q], widen(sq));
                     }
             }
         }
@@ -2314,7 +2364,7 @@ cudaError_t permute_batch(const PushDesc<T>* descs, int ninst, int total_units, 
 }
 
 template <typename T>
-cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const double* gJ, const double* gM, double* gu0,
+cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const T* gJ, const T* gM, double* gu0,
                             double* gx0, double* gw0, double* gB, const T* B, GridP g, SpeciesConst sc, cudaStream_t st,
                             const T* En, double* gEn)
 {
@@ -2413,7 +2463,7 @@ cudaError_t spectrum(PArrays<T> p, int64_t n, int variable, const T* edges, int 
     template cudaError_t push_general<T>(PArrays<T>, PArrays<T>, const int32_t*, int32_t*, const T*, \
                                          const T*, const T*, GridP, SpeciesConst, double*, int,      \
                                          cudaStream_t);                                              \
-    template cudaError_t deposit_adjoint<T>(PArrays<T>, const int32_t*, const double*, const double*, \
+    template cudaError_t deposit_adjoint<T>(PArrays<T>, const int32_t*, const T*, const T*, \
                                             double*, double*, double*, double*, const T*, GridP,      \
                                             SpeciesConst, cudaStream_t, const T*, double*);           \
     template cudaError_t push_adjoint<T>(PArrays<T>, const int32_t*, const double*, const double*,   \

@@ -220,6 +220,49 @@ template <> __device__ __forceinline__ float narrow<float>(double a)
     return __uint_as_float(q | (hi & 0x80000000u));
 }
 
+__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
+
+// A finite lattice coordinate into its cell (wrapped into [0, n)) and the
+// offset within it, rounded toward zero in FP32
+template <typename T>
+__device__ __noinline__ void split_cell_wrap(double xs, int n, int& i, T& f)
+{
+    if (xs < 0.0 || xs >= (double)n) xs -= n * floor(xs / n);
+    const double fi = floor(xs);
+    i = (int)fi;
+    if (i >= n) i -= n;
+    if (i < 0) i = 0;
+    f = from_double_rz<T>(xs - fi);
+}
+template <typename T>
+__device__ __forceinline__ void split_cell(double xs, int n, int& i, T& f)
+{
+    if constexpr (sizeof(T) == 4) {
+        // inside the box, on the integer pipe: the coordinate's bits are cut
+        // at the unit place, the fraction's leading 24 are the offset (exact,
+        // then truncated: the same as floor, subtraction and conversion)
+        const unsigned hi = (unsigned)__double2hiint(xs), lo = (unsigned)__double2loint(xs);
+        const int sh = 1075 - (int)(hi >> 20);   // fraction bits of the 53-bit significand (a sign bit: negative)
+        if (sh >= 22 && sh < 100) {
+            const unsigned long long sig = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
+            i = sh > 52 ? 0 : (int)(sig >> sh);
+            if (i < n) {
+                const unsigned long long r = sh > 52 ? sig : sig & ((1ull << sh) - 1ull);
+                const int lz = __clzll((long long)r);
+                f = r == 0ull ? 0.0f
+                              : __uint_as_float(((unsigned)(190 - lz - sh) << 23) |
+                                                ((unsigned)((r << lz) >> 40) & 0x7fffffu));
+                return;
+            }
+        } else if ((hi | lo) == 0u) {
+            i = 0;
+            f = 0.0f;
+            return;
+        }
+    }
+    split_cell_wrap<T>(xs, n, i, f);
+}
+
 // ---- TMA bulk copies (cp.async.bulk) completing on an mbarrier ----
 // A bulk copy needs 16-byte aligned source and destination addresses and a
 // size that is a multiple of 16 bytes.

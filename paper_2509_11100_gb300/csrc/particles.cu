@@ -22,49 +22,6 @@ __device__ __forceinline__ bool is_pow2(double v)
     return frexp(v, &e) == 0.5;
 }
 
-__device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
-
-// A finite lattice coordinate into its cell (wrapped into [0, n)) and the
-// offset within it, rounded toward zero in FP32
-template <typename T>
-__device__ __noinline__ void split_cell_wrap(double xs, int n, int& i, T& f)
-{
-    if (xs < 0.0 || xs >= (double)n) xs -= n * floor(xs / n);
-    const double fi = floor(xs);
-    i = (int)fi;
-    if (i >= n) i -= n;
-    if (i < 0) i = 0;
-    f = from_double_rz<T>(xs - fi);
-}
-template <typename T>
-__device__ __forceinline__ void split_cell(double xs, int n, int& i, T& f)
-{
-    if constexpr (sizeof(T) == 4) {
-        // inside the box, on the integer pipe: the coordinate's bits are cut
-        // at the unit place, the fraction's leading 24 are the offset (exact,
-        // then truncated: the same as floor, subtraction and conversion)
-        const unsigned hi = (unsigned)__double2hiint(xs), lo = (unsigned)__double2loint(xs);
-        const int sh = 1075 - (int)(hi >> 20);   // fraction bits of the 53-bit significand (a sign bit: negative)
-        if (sh >= 22 && sh < 100) {
-            const unsigned long long sig = ((unsigned long long)((hi & 0xfffffu) | 0x100000u) << 32) | lo;
-            i = sh > 52 ? 0 : (int)(sig >> sh);
-            if (i < n) {
-                const unsigned long long r = sh > 52 ? sig : sig & ((1ull << sh) - 1ull);
-                const int lz = __clzll((long long)r);
-                f = r == 0ull ? 0.0f
-                              : __uint_as_float(((unsigned)(190 - lz - sh) << 23) |
-                                                ((unsigned)((r << lz) >> 40) & 0x7fffffu));
-                return;
-            }
-        } else if ((hi | lo) == 0u) {
-            i = 0;
-            f = 0.0f;
-            return;
-        }
-    }
-    split_cell_wrap<T>(xs, n, i, f);
-}
-
 // (FP32 form: the positions and momenta go from FP64 to FP32 on the integer
 // pipe; on the FP64 pipe about 25 operations a particle bounded the load)
 template <typename T>
@@ -299,11 +256,37 @@ __device__ __forceinline__ T gbar_u2(T ux, T uy, T uz, T beta, const T (*sEn)[2]
 }
 
 // reciprocal square root and reciprocal: the hardware approximations in the
-// FP32 form (a few ulp), exact operations in the FP64 form
+// FP32 form (a few ulp). In the FP64 form Newton's iteration from the
+// hardware's FP64 approximations (a relative error e becomes 1.5 e^2 or e^2: two
+// steps from about 2^-20 end at the rounding of the last one): the FP64 pipe
+// takes a warp's operation in about 64 cycles and bounds the FP64 push and
+// deposit, and a square root and a division took it three times as many
+// operations. Values near the ends of the range go the long way.
+__device__ __forceinline__ bool mid_range(double x)   // 2^-900 <= x < 2^900
+{
+    return (unsigned)__double2hiint(x) - ((1023u - 900u) << 20) < (1800u << 20);
+}
 __device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x) { return 1.0 / sqrt(x); }
+__device__ __forceinline__ double rsqrt_t(double x)
+{
+    if (!mid_range(x)) return 1.0 / sqrt(x);
+    double y;
+    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+    const double h = -0.5 * x;
+#pragma unroll
+    for (int k = 0; k < 2; ++k) y = fma(y, fma(h, y * y, 0.5), y);
+    return y;
+}
 __device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rcp_t(double x) { return 1.0 / x; }
+__device__ __forceinline__ double rcp_t(double x)
+{
+    if (!mid_range(x)) return 1.0 / x;
+    double y;
+    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
+#pragma unroll
+    for (int k = 0; k < 2; ++k) y = fma(y, fma(-x, y, 1.0), y);
+    return y;
+}
 
 // The rotation of one particle, shared by the deposit and the push so both
 // see the same alpha: 1/gbar, a = beta B/gbar and 1/(1 + |a|^2).
@@ -372,17 +355,6 @@ struct Moments {
             for (int q = 0; q < 9; ++q) S[k * 9 + q] += t[k] * e[q];
     }
     __device__ __forceinline__ T get(int k, int q) const { return S[k * 9 + q]; }
-    template <int G>
-    __device__ __forceinline__ void group_reduce()
-    {
-#pragma unroll
-        for (int o = G / 2; o >= 1; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 81; ++q) S[q] += __shfl_xor_sync(0xffffffffu, S[q], o);
-#pragma unroll
-            for (int q = 0; q < 12; ++q) Jm[q] += __shfl_xor_sync(0xffffffffu, Jm[q], o);
-        }
-    }
 };
 
 template <>
@@ -425,63 +397,45 @@ struct Moments<float> {
         if (k < 8) return (k & 1) ? Q[k / 2].y : Q[k / 2].x;
         return R;
     }
-    template <int G>
-    __device__ __forceinline__ void group_reduce()
-    {
-#pragma unroll
-        for (int o = G / 2; o >= 1; o >>= 1) {
-#pragma unroll
-            for (int q = 0; q < 36; ++q) {
-                P[q].x += __shfl_xor_sync(0xffffffffu, P[q].x, o);
-                P[q].y += __shfl_xor_sync(0xffffffffu, P[q].y, o);
-            }
-#pragma unroll
-            for (int m = 0; m < 4; ++m) {
-                Q[m].x += __shfl_xor_sync(0xffffffffu, Q[m].x, o);
-                Q[m].y += __shfl_xor_sync(0xffffffffu, Q[m].y, o);
-            }
-            R += __shfl_xor_sync(0xffffffffu, R, o);
-#pragma unroll
-            for (int q = 0; q < 12; ++q) Jm[q] += __shfl_xor_sync(0xffffffffu, Jm[q], o);
-        }
-    }
-    // Reduce-scatter over the 8 lanes of a group (recursive halving, partner
-    // distances 4, 2, 1): afterwards lane gl holds the group sums of the 12
-    // flat values 12 gl .. 12 gl + 11, where lane L's block is S[L][0..8]
-    // followed by S[8][3L..3L+2] (L < 3), Jm[3(L-3)..3(L-3)+2] (3 <= L < 7)
-    // or zeros (L = 7). Each sum pairs the lanes' values in the order the
-    // butterfly of group_reduce does, so the results are the same.
-    __device__ __forceinline__ void reduce_scatter8(int gl, float (&r)[12]) const
-    {
-        float v[96];
-#pragma unroll
-        for (int L = 0; L < 8; ++L) {
-#pragma unroll
-            for (int q = 0; q < 9; ++q) v[12 * L + q] = get(L, q);
-#pragma unroll
-            for (int e = 0; e < 3; ++e)
-                v[12 * L + 9 + e] = L < 3 ? get(8, 3 * L + e) : L < 7 ? Jm[3 * (L - 3) + e] : 0.f;
-        }
-        float h[48];
-        const bool b2 = (gl & 4) != 0, b1 = (gl & 2) != 0, b0 = (gl & 1) != 0;
-#pragma unroll
-        for (int i = 0; i < 48; ++i) {
-            const float keep = b2 ? v[48 + i] : v[i], send = b2 ? v[i] : v[48 + i];
-            h[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
-        }
-        float g[24];
-#pragma unroll
-        for (int i = 0; i < 24; ++i) {
-            const float keep = b1 ? h[24 + i] : h[i], send = b1 ? h[i] : h[24 + i];
-            g[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
-        }
-#pragma unroll
-        for (int i = 0; i < 12; ++i) {
-            const float keep = b0 ? g[12 + i] : g[i], send = b0 ? g[i] : g[12 + i];
-            r[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
-        }
-    }
 };
+
+// Reduce-scatter over the 8 lanes of a group (recursive halving, partner
+// distances 4, 2, 1): afterwards lane gl holds the group sums of the 12
+// flat values 12 gl .. 12 gl + 11, where lane L's block is S[L][0..8]
+// followed by S[8][3L..3L+2] (L < 3), Jm[3(L-3)..3(L-3)+2] (3 <= L < 7)
+// or zeros (L = 7). Each sum pairs the lanes' values in the order the
+// butterfly of group_reduce does, so the results are the same.
+template <typename T>
+__device__ __forceinline__ void reduce_scatter8(const Moments<T>& m, int gl, T (&r)[12])
+{
+    T v[96];
+#pragma unroll
+    for (int L = 0; L < 8; ++L) {
+#pragma unroll
+        for (int q = 0; q < 9; ++q) v[12 * L + q] = m.get(L, q);
+#pragma unroll
+        for (int e = 0; e < 3; ++e)
+            v[12 * L + 9 + e] = L < 3 ? m.get(8, 3 * L + e) : L < 7 ? m.Jm[3 * (L - 3) + e] : T(0);
+    }
+    T h[48];
+    const bool b2 = (gl & 4) != 0, b1 = (gl & 2) != 0, b0 = (gl & 1) != 0;
+#pragma unroll
+    for (int i = 0; i < 48; ++i) {
+        const T keep = b2 ? v[48 + i] : v[i], send = b2 ? v[i] : v[48 + i];
+        h[i] = keep + __shfl_xor_sync(0xffffffffu, send, 4);
+    }
+    T g[24];
+#pragma unroll
+    for (int i = 0; i < 24; ++i) {
+        const T keep = b1 ? h[24 + i] : h[i], send = b1 ? h[i] : h[24 + i];
+        g[i] = keep + __shfl_xor_sync(0xffffffffu, send, 2);
+    }
+#pragma unroll
+    for (int i = 0; i < 12; ++i) {
+        const T keep = b0 ? g[12 + i] : g[i], send = b0 ? g[i] : g[12 + i];
+        r[i] = keep + __shfl_xor_sync(0xffffffffu, send, 1);
+    }
+}
 
 // The node and half offset where the moments S[k][*] of a cell go (k = xx*3
 // + yy): nodes 0..3 = n00, n10, n01, n11; S[4][*] goes to (n00, 4) and also
@@ -874,59 +828,35 @@ __device__ __forceinline__ void deposit_core(const Src& src, int* __restrict__ e
         if (s == nsp - 1) {
             T* const M = src.Mf(ii);
             T* const J = src.Jf(ii);
-            if constexpr (std::is_same<T, float>::value) {
-                static_assert(G == 8, "the FP32 flush scatters over 8 lanes");
-                float r[12];
-                acc.reduce_scatter8(gl, r);
-                if (valid) {
-                    const int i = un.i0 + grp, j = un.j;
-                    const int i1 = wrap1(i + 1, nx), j1 = wrap1(j + 1, ny);
-                    const int n00 = j * nx + i, n10 = j * nx + i1, n01 = j1 * nx + i, n11 = j1 * nx + i1;
-                    // lane gl: S[gl][0..8] to its node and offset (S[4] twice)
-                    const int nd = (kMomNodeBits >> (2 * gl)) & 3, of = (kMomOffBits >> (3 * gl)) & 7;
-                    const int nn = nd == 0 ? n00 : nd == 1 ? n10 : nd == 2 ? n01 : n11;
-                    float* const mk = M + (int64_t)nn * kMBlock + of * 9;
+            static_assert(G == 8, "the flush scatters over 8 lanes");
+            T r[12];
+            reduce_scatter8<T>(acc, gl, r);
+            if (valid) {
+                const int i = un.i0 + grp, j = un.j;
+                const int i1 = wrap1(i + 1, nx), j1 = wrap1(j + 1, ny);
+                const int n00 = j * nx + i, n10 = j * nx + i1, n01 = j1 * nx + i, n11 = j1 * nx + i1;
+                // lane gl: S[gl][0..8] to its node and offset (S[4] twice)
+                const int nd = (kMomNodeBits >> (2 * gl)) & 3, of = (kMomOffBits >> (3 * gl)) & 7;
+                const int nn = nd == 0 ? n00 : nd == 1 ? n10 : nd == 2 ? n01 : n11;
+                T* const mk = M + (int64_t)nn * kMBlock + of * 9;
 #pragma unroll
-                    for (int q = 0; q < 9; ++q) atomicAdd(mk + q, r[q]);
-                    if (gl == 4) {
-                        float* const m4 = M + (int64_t)n10 * kMBlock + 2 * 9;
+                for (int q = 0; q < 9; ++q) atomicAdd(mk + q, r[q]);
+                if (gl == 4) {
+                    T* const m4 = M + (int64_t)n10 * kMBlock + 2 * 9;
 #pragma unroll
-                        for (int q = 0; q < 9; ++q) atomicAdd(m4 + q, r[q]);
-                    }
-                    // the extras: S[8][3gl..3gl+2] (node n11, offset 0) or the
-                    // currents of node gl - 3, components 0..2
-                    if (gl < 3) {
-                        float* const m8 = M + (int64_t)n11 * kMBlock + 3 * gl;
-#pragma unroll
-                        for (int e = 0; e < 3; ++e) atomicAdd(m8 + e, r[9 + e]);
-                    } else if (gl < 7) {
-                        const int a = gl - 3;
-                        const int jn = a == 0 ? n00 : a == 1 ? n10 : a == 2 ? n01 : n11;
-#pragma unroll
-                        for (int e = 0; e < 3; ++e) atomicAdd(J + (int64_t)e * nc + jn, r[9 + e]);
-                    }
+                    for (int q = 0; q < 9; ++q) atomicAdd(m4 + q, r[q]);
                 }
-            } else {
-                acc.template group_reduce<G>();
-                if (valid) {
-                    const int i = un.i0 + grp, j = un.j;
-                    const int i1 = wrap1(i + 1, nx), j1 = wrap1(j + 1, ny);
-                    const int n00 = j * nx + i, n10 = j * nx + i1, n01 = j1 * nx + i, n11 = j1 * nx + i1;
-                    // (destination node, half offset, moment k) of the ten node pairs
-                    const int pn[10] = {n00, n00, n00, n00, n10, n10, n10, n01, n01, n11};
-                    constexpr int po[10] = {0, 1, 3, 4, 0, 2, 3, 0, 1, 0};
-                    constexpr int pk[10] = {0, 3, 1, 4, 6, 4, 7, 2, 5, 8};
+                // the extras: S[8][3gl..3gl+2] (node n11, offset 0) or the
+                // currents of node gl - 3, components 0..2
+                if (gl < 3) {
+                    T* const m8 = M + (int64_t)n11 * kMBlock + 3 * gl;
 #pragma unroll
-                    for (int it = 0; it < 90; ++it) {
-                        if (it % G == gl) {
-                            const int pr = it / 9, q = it % 9;
-                            atomicAdd(M + (int64_t)pn[pr] * kMBlock + po[pr] * 9 + q, acc.get(pk[pr], q));
-                        }
-                    }
-                    const int jn[4] = {n00, n10, n01, n11};
+                    for (int e = 0; e < 3; ++e) atomicAdd(m8 + e, r[9 + e]);
+                } else if (gl < 7) {
+                    const int a = gl - 3;
+                    const int jn = a == 0 ? n00 : a == 1 ? n10 : a == 2 ? n01 : n11;
 #pragma unroll
-                    for (int it = 0; it < 12; ++it)
-                        if ((90 + it) % G == gl) atomicAdd(J + (int64_t)(it % 3) * nc + jn[it / 3], acc.Jm[it]);
+                    for (int e = 0; e < 3; ++e) atomicAdd(J + (int64_t)e * nc + jn, r[9 + e]);
                 }
             }
         }
@@ -2239,20 +2169,23 @@ int row_units(GridP g) { return units_of(g.nx, g.ny); }
 // The width of the row units of the passes that give a warp a unit (push,
 // re-sort, adjoints): the full 32 cells, halved while that leaves fewer than
 // eight warps per SM in flight (with 16 as the line, eight instances stepped
-// side by side lost 8% to the narrower units' tiles and half-full batches). A unit's warp takes its particles batch after
+// side by side lost 8% to the narrower units' tiles and half-full batches), in
+// FP64 fewer than 16 (the FP64 pipe hides the tiles; at 256x128 steps took 3.5
+// ms with 16 and 3.9 with 8). A unit's warp takes its particles batch after
 // batch, so on a small grid the launch lasts as long as one unit: at 128x64
 // with 32 particles a cell (FP32 form) the push of a species took 65 us on
 // 256 units of 32 cells, 21 us on 2048 of 4 (the re-sort 24 and 7 us).
-int unit_width(GridP g)
+int unit_width(GridP g, int precision)
 {
+    const int want = 152 * (precision == 32 ? 8 : 16);
     int uw = kUnitW;
-    while (uw > 2 && units_of(g.nx, g.ny, uw) < 152 * 8) uw /= 2;
+    while (uw > 2 && units_of(g.nx, g.ny, uw) < want) uw /= 2;
     return uw;
 }
 
 int push_grid_blocks(GridP g, int precision, int cap)
 {
-    return blocks_for(units_of(g.nx, g.ny, unit_width(g)),
+    return blocks_for(units_of(g.nx, g.ny, unit_width(g, precision)),
                       precision == 32 ? PushCfg<float>::warps : PushCfg<double>::warps, cap > 0 ? cap : 152 * 16);
 }
 
@@ -2324,7 +2257,7 @@ cudaError_t push_sort(PArrays<T> src, PArrays<T> dst, const int32_t* start, int3
     count_launches(1);
     kern<<<lsum_blocks, PushCfg<T>::threads, 0, st>>>(src, dst, start, n9, off9, Eth, B, En, g, beta,
                                                       (T)(g.dt / g.dx), (T)(g.dt / g.dy), (T)(sc.q * g.dt),
-                                                      (T)sc.m, lsum_partial, unit_width(g));
+                                                      (T)sc.m, lsum_partial, unit_width(g, 8 * (int)sizeof(T)));
     return cudaGetLastError();
 }
 
@@ -2373,11 +2306,11 @@ cudaError_t deposit_adjoint(PArrays<T> src, const int32_t* start, const T* gJ, c
     const int nb = push_grid_blocks(g, sizeof(T) == 4 ? 32 : 64, 152 * 16);
     if (En)
         k_deposit_adjoint<T, true><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gJ, gM, gu0, gx0, gw0, gB, B, g,
-                                                                       beta, sc.q, En, gEn, unit_width(g));
+                                                                       beta, sc.q, En, gEn, unit_width(g, 8 * (int)sizeof(T)));
     else
         k_deposit_adjoint<T, false><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gJ, gM, gu0, gx0, gw0, gB, B, g,
                                                                         beta, sc.q, nullptr, nullptr,
-                                                                        unit_width(g));
+                                                                        unit_width(g, 8 * (int)sizeof(T)));
     return cudaGetLastError();
 }
 
@@ -2391,10 +2324,10 @@ cudaError_t push_adjoint(PArrays<T> src, const int32_t* start, const double* gu1
     const int nb = push_grid_blocks(g, sizeof(T) == 4 ? 32 : 64, 152 * 16);
     if (En)
         k_push_adjoint<T, true><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gu1, gx1, gu0, gx0, gE, gB, Eth, B,
-                                                                    g, beta, En, gEn, unit_width(g));
+                                                                    g, beta, En, gEn, unit_width(g, 8 * (int)sizeof(T)));
     else
         k_push_adjoint<T, false><<<nb, PushCfg<T>::threads, 0, st>>>(src, start, gu1, gx1, gu0, gx0, gE, gB, Eth, B,
-                                                                     g, beta, nullptr, nullptr, unit_width(g));
+                                                                     g, beta, nullptr, nullptr, unit_width(g, 8 * (int)sizeof(T)));
     return cudaGetLastError();
 }
 
@@ -2408,7 +2341,7 @@ cudaError_t push_general(PArrays<T> src, PArrays<T> dst, const int32_t* start, i
     count_launches(1);
     kern<<<lsum_blocks, PushCfg<T>::threads, 0, st>>>(src, dst, start, key, Eth, B, En, g, beta,
                                                       (T)(g.dt / g.dx), (T)(g.dt / g.dy), (T)(sc.q * g.dt),
-                                                      (T)sc.m, lsum_partial, unit_width(g));
+                                                      (T)sc.m, lsum_partial, unit_width(g, 8 * (int)sizeof(T)));
     return cudaGetLastError();
 }
 
@@ -2417,7 +2350,7 @@ cudaError_t permute(PArrays<T> src, PArrays<T> dst, const int32_t* start_new, co
                     const int32_t* off9, GridP g, int* err, cudaStream_t st)
 {
     count_launches(1);
-    const int uw = unit_width(g);
+    const int uw = unit_width(g, 8 * (int)sizeof(T));
     k_permute<T><<<blocks_for(units_of(g.nx, g.ny, uw), 8, 152 * 16), 256, 0, st>>>(src, dst, start_new, n9, off9, g,
                                                                                     err, uw);
     return cudaGetLastError();

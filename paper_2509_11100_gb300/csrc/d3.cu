@@ -146,11 +146,11 @@ __device__ __forceinline__ void corner_weights(T fx, T fy, T fz, T (&W)[8])
     for (int a = 0; a < 8; ++a) W[a] = X[a & 1] * Y[(a >> 1) & 1] * Z[(a >> 2) & 1];
 }
 
-// alpha = (I - [a]x + a a^T)/(1 + |a|^2), a = beta B/gbar (row-major)
+// alpha = (I - [a]x + a a^T)/(1 + |a|^2), a = bg B, bg = beta/gbar (row-major)
 template <typename T>
-__device__ __forceinline__ void alpha3(const T (&Bp)[3], T beta, T gbar, T (&al)[9])
+__device__ __forceinline__ void alpha3(const T (&Bp)[3], T bg, T (&al)[9])
 {
-    const T ax = beta * Bp[0] / gbar, ay = beta * Bp[1] / gbar, az = beta * Bp[2] / gbar;
+    const T ax = bg * Bp[0], ay = bg * Bp[1], az = bg * Bp[2];
     const T ia = T(1) / (T(1) + ax * ax + ay * ay + az * az);
     al[0] = (T(1) + ax * ax) * ia; al[1] = (ax * ay + az) * ia; al[2] = (ax * az - ay) * ia;
     al[3] = (ax * ay - az) * ia; al[4] = (T(1) + ay * ay) * ia; al[5] = (ay * az + ax) * ia;
@@ -162,23 +162,14 @@ __device__ __forceinline__ void alpha3(const T (&Bp)[3], T beta, T gbar, T (&al)
 // shared memory once per segment instead of 24 gathers per particle per field
 
 template <typename T>
-struct Tile3 {
-    T E[3][2][2][33];   // [comp][dy][dz][c]: node (i0 + c, j + dy, k + dz)
+struct Tile3B {
     T B[3][3][3][34];   // [comp][dy][dz][c]: centre (i0 - 1 + c, j - 1 + dy, k - 1 + dz)
 };
-
 template <typename T>
-__device__ __forceinline__ void load_tile3(Tile3<T>& tl, const T* __restrict__ E, const T* __restrict__ B, int i0,
-                                           int cn, int j, int k, const GridP& g, int lane)
+__device__ __forceinline__ void load_tile3B(Tile3B<T>& tl, const T* __restrict__ B, int i0, int cn, int j, int k,
+                                            const GridP& g, int lane)
 {
     const int64_t nc = g.ncell;
-    if (E)
-        for (int q = lane; q < 3 * 2 * 2 * 33; q += 32) {
-            const int c = q % 33, dz = (q / 33) % 2, dy = (q / 66) % 2, comp = q / 132;
-            if (c <= cn)
-                tl.E[comp][dy][dz][c] =
-                    ld(E + comp * nc + node3(wrap1(i0 + c, g.nx), wrap1(j + dy, g.ny), wrap1(k + dz, g.nz), g));
-        }
     for (int q = lane; q < 3 * 3 * 3 * 34; q += 32) {
         const int c = q % 34, dz = (q / 34) % 3, dy = (q / 102) % 3, comp = q / 306;
         if (c <= cn + 1)
@@ -190,7 +181,7 @@ __device__ __forceinline__ void load_tile3(Tile3<T>& tl, const T* __restrict__ E
 
 // B^n at a particle of local cell cl with offsets f, from the tile
 template <typename T>
-__device__ __forceinline__ void tile_B3(const Tile3<T>& tl, int cl, T fx, T fy, T fz, T (&Bp)[3])
+__device__ __forceinline__ void tile_B3(const T (&B)[3][3][3][34], int cl, T fx, T fy, T fz, T (&Bp)[3])
 {
     const bool lx = fx < T(0.5), ly = fy < T(0.5), lz = fz < T(0.5);
     const T tx = lx ? fx + T(0.5) : fx - T(0.5);
@@ -203,110 +194,216 @@ __device__ __forceinline__ void tile_B3(const Tile3<T>& tl, int cl, T fx, T fy, 
     for (int comp = 0; comp < 3; ++comp) {
         T b = T(0);
 #pragma unroll
-        for (int a = 0; a < 8; ++a) b += W[a] * tl.B[comp][y0 + ((a >> 1) & 1)][z0 + ((a >> 2) & 1)][c0 + (a & 1)];
+        for (int a = 0; a < 8; ++a) b += W[a] * B[comp][y0 + ((a >> 1) & 1)][z0 + ((a >> 2) & 1)][c0 + (a & 1)];
         Bp[comp] = b;
     }
+}
+
+// The push's tiles hold every value with its right neighbour, so that the two
+// columns of a gather come in one load: 24 shared loads a particle instead
+// of 48
+template <typename T>
+struct Pair3 {
+    T a, b;
+};
+template <>
+struct __align__(8) Pair3<float> {
+    float a, b;
+};
+template <>
+struct __align__(16) Pair3<double> {
+    double a, b;
+};
+template <typename T>
+struct PairTile3 {
+    Pair3<T> E[3][2][2][32];   // [comp][dy][dz][c]: nodes (i0 + c, j + dy, k + dz) and (i0 + c + 1, ..)
+    Pair3<T> B[3][3][3][33];   // [comp][dy][dz][c]: centres (i0 - 1 + c, j - 1 + dy, k - 1 + dz) and (i0 + c, ..)
+    __device__ __forceinline__ void gather_E(int cl, T fx, T fy, T fz, T (&E3)[3]) const
+    {
+        T W[8];
+        corner_weights(fx, fy, fz, W);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            T e = T(0);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const Pair3<T> q = E[c][a & 1][a >> 1][cl];
+                e += W[2 * a] * q.a;
+                e += W[2 * a + 1] * q.b;
+            }
+            E3[c] = e;
+        }
+    }
+    __device__ __forceinline__ void gather_B(int cl, T fx, T fy, T fz, T (&Bp)[3]) const
+    {
+        const bool lx = fx < T(0.5), ly = fy < T(0.5), lz = fz < T(0.5);
+        const T tx = lx ? fx + T(0.5) : fx - T(0.5);
+        const T ty = ly ? fy + T(0.5) : fy - T(0.5);
+        const T tz = lz ? fz + T(0.5) : fz - T(0.5);
+        const int c0 = lx ? cl : cl + 1, y0 = ly ? 0 : 1, z0 = lz ? 0 : 1;
+        T W[8];
+        corner_weights(tx, ty, tz, W);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            T e = T(0);
+#pragma unroll
+            for (int a = 0; a < 4; ++a) {
+                const Pair3<T> q = B[c][y0 + (a & 1)][z0 + (a >> 1)][c0];
+                e += W[2 * a] * q.a;
+                e += W[2 * a + 1] * q.b;
+            }
+            Bp[c] = e;
+        }
+    }
+};
+
+template <typename T>
+__device__ __forceinline__ void load_pairs3(PairTile3<T>& tl, const T* __restrict__ E, const T* __restrict__ B, int i0,
+                                            int cn, int j, int k, const GridP& g, int lane)
+{
+    const int64_t nc = g.ncell;
+    // a lane a column, the rows in turn (a column's right neighbour is the
+    // next lane's value but for the last)
+    const int ca = wrap1(i0 + min(lane, cn - 1), g.nx), cb = wrap1(i0 + min(lane, cn - 1) + 1, g.nx);
+    const int cz = wrap1(i0 - 1, g.nx);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) {
+        const int64_t row = node3(0, wrap1(j + (r & 1), g.ny), wrap1(k + (r >> 1), g.nz), g);
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (lane < cn) tl.E[c][r & 1][r >> 1][lane] = Pair3<T>{ld(E + c * nc + row + ca), ld(E + c * nc + row + cb)};
+    }
+#pragma unroll
+    for (int r = 0; r < 9; ++r) {
+        const int64_t row = node3(0, wrap1(j - 1 + r % 3, g.ny), wrap1(k - 1 + r / 3, g.nz), g);
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+            if (lane < cn)
+                tl.B[c][r % 3][r / 3][lane + 1] = Pair3<T>{ld(B + c * nc + row + ca), ld(B + c * nc + row + cb)};
+            if (lane == 0) tl.B[c][r % 3][r / 3][0] = Pair3<T>{ld(B + c * nc + row + cz), ld(B + c * nc + row + ca)};
+        }
+    }
+    __syncwarp();
 }
 
 // ---------------------------------------------------------------------------
 // deposit
 
+// A warp takes a row segment of cells and, batch after batch, 32 particles of
+// it whatever cell and species they belong to: each lane forms one particle's
+// weights, c alpha and current and stages them in shared memory (the lanes are
+// full whatever the cells hold); then the warp runs over the staged particles,
+// and lane k adds to the 9 sums of one of the cell's 27 moments
+//   S[xx][yy][zz][e] = sum_p XX YY ZZ c_p alpha_e,   XX in (X0^2, X0 X1, X1^2), ..
+// (the 36 corner pairs take 27 distinct weight products), two particles per
+// paired FP32 FMA. When a cell is done, its 36 blocks go to M from shared
+// memory in address order, so that a warp's additions fall in few sectors, and
+// the moments of the cell's upper x face start the next cell's lower face
+// instead of being added to memory twice.
+//
+// Bound by issue. Before, each lane owned one or two of the 36 pairs, a cell's
+// own batches were often half empty, and each lane added its blocks by itself:
+// 61 warp instructions a particle, 11.5 ms on 256x128x128 with 32 particles a
+// cell (FP32 form), 0.23 ms on 64x32x32.
 template <typename T>
 struct DepCfg3 {
     static constexpr int warps = sizeof(T) == 4 ? 4 : 2;   // static shared memory < 48 KB
 };
-constexpr int kStage3 = 22;   // staged values per particle (20, padded to an even stride for paired loads)
+constexpr int kMom3 = 27;
+constexpr int kItems3 = 36 * 9;        // a cell's additions to M
+constexpr int kFace3 = 26 * 9;         // those not on the upper x face
+// staged values of a particle: c alpha, XX YY, ZZ, corner weights, current
+enum { kS3E = 0, kS3XY = 9, kS3Z = 18, kS3W = 21, kS3V = 29, kS3N = 32 };
 
-// a pair block's 9 sums; in FP32 as four pairs and one, accumulated with
-// the paired FMA (one instruction for two sums)
+// the staged particles of a warp: FP32 two by two, (value of particle 2r,
+// value of particle 2r + 1), rows 16-byte aligned
 template <typename T>
-struct PairAcc {
-    T v[9];
-    __device__ __forceinline__ void zero()
+struct Stage3 {
+    T v[32][kS3N + 1];
+    __device__ __forceinline__ void put(int t, int k, T a) { v[t][k] = a; }
+};
+template <>
+struct Stage3<float> {
+    static constexpr int row = 2 * kS3N + 4;
+    float v[16][row];
+    __device__ __forceinline__ void put(int t, int k, float a) { v[t >> 1][2 * k + (t & 1)] = a; }
+    __device__ __forceinline__ float2 get2(int r, int k) const { return *reinterpret_cast<const float2*>(&v[r][2 * k]); }
+};
+
+// a lane's sums of one moment and one current value over a cell
+template <typename T>
+struct Acc3 {
+    T m[9], j;
+    __device__ __forceinline__ void start(const T (&v)[9], T vj)
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] = T(0);
+        for (int e = 0; e < 9; ++e) m[e] = v[e];
+        j = vj;
     }
-    __device__ __forceinline__ void add(T w, const T* al)
+    __device__ __forceinline__ void add(const Stage3<T>& st, int t0, int t1, int k1, int k2, int ja, int jc)
     {
+        for (int t = t0; t < t1; ++t) {
+            const T w = st.v[t][kS3XY + k1] * st.v[t][kS3Z + k2];
 #pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] += w * al[e];
+            for (int e = 0; e < 9; ++e) m[e] += w * st.v[t][kS3E + e];
+            j += st.v[t][kS3W + ja] * st.v[t][kS3V + jc];
+        }
     }
-    __device__ __forceinline__ void get(T (&o)[9]) const
+    __device__ __forceinline__ void get(T (&v)[9], T& vj) const
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) o[e] = v[e];
+        for (int e = 0; e < 9; ++e) v[e] = m[e];
+        vj = j;
     }
 };
 template <>
-struct PairAcc<float> {
-    float2 v2[4];
-    float v8;
-    __device__ __forceinline__ void zero()
+struct Acc3<float> {
+    float2 m[9], j;   // even and odd staged particles apart
+    __device__ __forceinline__ void start(const float (&v)[9], float vj)
     {
 #pragma unroll
-        for (int k = 0; k < 4; ++k) v2[k] = make_float2(0.f, 0.f);
-        v8 = 0.f;
+        for (int e = 0; e < 9; ++e) m[e] = make_float2(v[e], 0.f);
+        j = make_float2(vj, 0.f);
     }
-    // al: 8-byte aligned row of the 9 staged values
-    __device__ __forceinline__ void add(float w, const float2 (&al2)[4], float al8)
+    // EDGE: the row holds a particle of another cell (its weights are left out)
+    template <bool EDGE>
+    __device__ __forceinline__ void row(const Stage3<float>& st, int r, int t0, int t1, int k1, int k2, int ja, int jc)
     {
-        const float2 ww = make_float2(w, w);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v2[k] = __ffma2_rn(ww, al2[k], v2[k]);
-        v8 = fmaf(w, al8, v8);
-    }
-    __device__ __forceinline__ void get(float (&o)[9]) const
-    {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            o[2 * k] = v2[k].x;
-            o[2 * k + 1] = v2[k].y;
+        const float2 xy = st.get2(r, kS3XY + k1), z = st.get2(r, kS3Z + k2);
+        float2 w = make_float2(xy.x * z.x, xy.y * z.y), wj = st.get2(r, kS3W + ja);
+        if (EDGE) {
+            if (2 * r < t0) w.x = wj.x = 0.f;
+            if (2 * r + 1 >= t1) w.y = wj.y = 0.f;
         }
-        o[8] = v8;
+        const float4* e4 = reinterpret_cast<const float4*>(&st.v[r][0]);
+#pragma unroll
+        for (int h = 0; h < 4; ++h) {
+            const float4 q = e4[h];
+            m[2 * h] = __ffma2_rn(w, make_float2(q.x, q.y), m[2 * h]);
+            m[2 * h + 1] = __ffma2_rn(w, make_float2(q.z, q.w), m[2 * h + 1]);
+        }
+        m[8] = __ffma2_rn(w, st.get2(r, kS3E + 8), m[8]);
+        j = __ffma2_rn(wj, st.get2(r, kS3V + jc), j);
+    }
+    __device__ __forceinline__ void add(const Stage3<float>& st, int t0, int t1, int k1, int k2, int ja, int jc)
+    {
+        int r = t0 >> 1;
+        const int r1 = t1 >> 1;   // rows r0 .. r1-1 are whole but for the first
+        if (t0 & 1) {
+            row<true>(st, r, t0, t1, k1, k2, ja, jc);
+            ++r;
+        }
+#pragma unroll 2
+        for (; r < r1; ++r) row<false>(st, r, t0, t1, k1, k2, ja, jc);
+        if ((t1 & 1) && r == r1) row<true>(st, r, t0, t1, k1, k2, ja, jc);
+    }
+    __device__ __forceinline__ void get(float (&v)[9], float& vj) const
+    {
+#pragma unroll
+        for (int e = 0; e < 9; ++e) v[e] = m[e].x + m[e].y;
+        vj = j.x + j.y;
     }
 };
-
-// a 3x3 block added to the stored block at dst (offset index hs): in FP32
-// as paired atomics (8-byte aligned pairs: the block starts on an even float
-// when hs is even, as 126 per node is even), halving the atomic operations
-__device__ __forceinline__ void add_block9(float* dst, const float (&v)[9], int hs)
-{
-    // constant indices in both branches keep v in registers
-    if (hs & 1) {
-        atomicAdd(dst, v[0]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            atomicAdd(reinterpret_cast<float2*>(dst + 1 + 2 * e), make_float2(v[1 + 2 * e], v[2 + 2 * e]));
-    } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            atomicAdd(reinterpret_cast<float2*>(dst + 2 * e), make_float2(v[2 * e], v[2 * e + 1]));
-        atomicAdd(dst + 8, v[8]);
-    }
-}
-__device__ __forceinline__ void add_block9(double* dst, const double (&v)[9], int)
-{
-#pragma unroll
-    for (int e = 0; e < 9; ++e) atomicAdd(dst + e, v[e]);
-}
-
-// flush a cell's pair block: the block of pair (a, b) is stored at corner a
-// with the offset b - a when that offset is in the stored half, else at
-// corner b with a - b
-template <typename T>
-__device__ __forceinline__ void flush_pair3(T* M, int a, int b, const T (&acc)[9], int i, int j, int k, GridP g)
-{
-    const int di = (b & 1) - (a & 1), dj = ((b >> 1) & 1) - ((a >> 1) & 1), dk = ((b >> 2) & 1) - ((a >> 2) & 1);
-    int hs = half3(di, dj, dk), at = a;
-    if (hs < 0) {
-        hs = half3(-di, -dj, -dk);
-        at = b;
-    }
-    const int64_t gn =
-        node3(wrap1(i + (at & 1), g.nx), wrap1(j + ((at >> 1) & 1), g.ny), wrap1(k + ((at >> 2) & 1), g.nz), g);
-    add_block9(M + gn * kMBlock3 + hs * 9, acc, hs);
-}
 
 // the 36 unordered corner pairs (a <= b) of a cell, pair q
 __device__ __forceinline__ void pair_of(int q, int& a, int& b)
@@ -319,122 +416,177 @@ __device__ __forceinline__ void pair_of(int q, int& a, int& b)
     }
     b = a + r;
 }
+// where pair q's block is stored (corner at, offset index hs: at corner a
+// with the offset b - a when that is in the stored half, else at b with
+// a - b), its moment, and its place in the order (upper x face last, then by
+// corner and offset)
+__device__ __forceinline__ void pair_block(int q, int& at, int& hs, int& mom, int& place)
+{
+    int a, b;
+    pair_of(q, a, b);
+    const int di = (b & 1) - (a & 1), dj = ((b >> 1) & 1) - ((a >> 1) & 1), dk = ((b >> 2) & 1) - ((a >> 2) & 1);
+    hs = half3(di, dj, dk);
+    at = a;
+    if (hs < 0) {
+        hs = half3(-di, -dj, -dk);
+        at = b;
+    }
+    mom = ((a >> 2 & 1) + (b >> 2 & 1)) * 9 + ((a & 1) + (b & 1)) * 3 + (a >> 1 & 1) + (b >> 1 & 1);
+    place = ((a & b & 1) * 8 + at) * kHalf3 + hs;
+}
 
 template <typename T>
 __global__ void __launch_bounds__(32 * DepCfg3<T>::warps)
-k_deposit3(DepositSpecies<T> ds, FzArrays<T> fz, const T* __restrict__ B, T* __restrict__ M, T* __restrict__ J,
-           GridP g)
+k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__ FzArrays<T> fz,
+           const T* __restrict__ B, T* __restrict__ M, T* __restrict__ J,
+           GridP g, int uw)
 {
     constexpr int kW = DepCfg3<T>::warps;
-    __shared__ __align__(16) T sh[kW][32][kStage3];
-    __shared__ Tile3<T> stl[kW];
+    __shared__ __align__(16) Stage3<T> sst[kW];
+    __shared__ Tile3B<T> stl[kW];
+    __shared__ T smom[kW][kMom3 * 9];   // a cell's moments, for the additions
+    __shared__ int64_t snode[kW][8];    // its corners' nodes
+    __shared__ unsigned item[kItems3];  // an addition: corner << 16 | place in the node's blocks << 8 | moment value
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    for (int q = threadIdx.x; q < 36; q += blockDim.x) {
+        int at, hs, mom, place, rank = 0;
+        pair_block(q, at, hs, mom, place);
+        for (int o = 0; o < 36; ++o) {
+            int at2, hs2, mom2, place2;
+            pair_block(o, at2, hs2, mom2, place2);
+            rank += place2 < place ? 1 : 0;
+        }
+        for (int e = 0; e < 9; ++e)
+            item[rank * 9 + e] = (unsigned)at << 16 | (unsigned)(hs * 9 + e) << 8 | (unsigned)(mom * 9 + e);
+    }
+    __syncthreads();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int nseg = (g.nx + 31) / 32;
+    const int nseg = (g.nx + uw - 1) / uw;
     const int64_t nunits = (int64_t)nseg * g.ny * g.nz;
-    T (*st)[kStage3] = sh[wib];
-    // the pairs this lane owns (q0 = lane, q1 = lane + 32 for lanes 0..3) and
-    // the current component it owns (lanes 4..27: corner (lane-4)/3, component (lane-4)%3)
-    int a0, b0, a1 = 0, b1 = 0;
-    pair_of(lane, a0, b0);
-    const bool two = lane < 4;
-    if (two) pair_of(lane + 32, a1, b1);
-    const bool ownj = lane >= 4 && lane < 28;
-    const int ja = ownj ? (lane - 4) / 3 : 0, jc = ownj ? (lane - 4) % 3 : 0;
+    const int nsp = ds.nsp, gcells = 32 / nsp;   // cells whose (cell, species) ranges fit the lanes
+    Stage3<T>& st = sst[wib];
+    // the moment this lane sums (lanes 0 .. 26: ZZ, XX, YY) and the current
+    // value (lanes 0 .. 23: corner, component)
+    const int k1 = lane < kMom3 ? lane % 9 : 0, k2 = lane < kMom3 ? lane / 9 : 0;
+    const int ja = lane < 24 ? lane / 3 : 0, jc = lane < 24 ? lane % 3 : 0;
+    const bool low = lane < kMom3 && k1 < 3;   // a moment of the lower x face
     for (int64_t u = warp; u < nunits; u += nwarps) {
-        const int i0 = (int)(u % nseg) * 32;
+        const int i0 = (int)(u % nseg) * uw;
         const int jk = (int)(u / nseg);
         const int j = jk % g.ny, k = jk / g.ny;
-        const int cn = min(32, g.nx - i0);
+        const int cn = min(uw, g.nx - i0);
         __syncwarp();
-        load_tile3<T>(stl[wib], nullptr, B, i0, cn, j, k, g, lane);
-        for (int cl = 0; cl < cn; ++cl) {
-            const int i = i0 + cl;
-            const int64_t c = node3(i, j, k, g);
-            PairAcc<T> acc0, acc1;
-            acc0.zero();
-            acc1.zero();
-            T accj = T(0);
-            // the cell's particles of all species as one list (cum[s] = the
-            // first list index of species s), staged 32 at a time
-            // (fully unrolled over the species so the tables stay in registers)
-            int cum[kMaxSpecies + 1], pst[kMaxSpecies];
-            cum[0] = 0;
-#pragma unroll
-            for (int s = 0; s < kMaxSpecies; ++s) {
-                pst[s] = s < ds.nsp ? ds.start[s][c] : 0;
-                cum[s + 1] = cum[s] + (s < ds.nsp ? ds.start[s][c + 1] - pst[s] : 0);
+        load_tile3B<T>(stl[wib], B, i0, cn, j, k, g, lane);
+        Acc3<T> acc;
+        {
+            const T zero[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
+            acc.start(zero, T(0));
+        }
+        bool carry = false;   // the previous cell left sums on this cell's lower face
+        for (int cg = 0; cg < cn; cg += gcells) {
+            // the particles of up to gcells cells as one list: lane l holds
+            // the range of cell l / nsp, species l % nsp
+            const int gc0 = min(gcells, cn - cg);
+            int first = 0, cnt = 0;
+            if (lane < gc0 * nsp) {
+                const int64_t c = node3(i0 + cg + lane / nsp, j, k, g);
+                const int32_t* sp = ds.start[lane % nsp];
+                first = sp[c];
+                cnt = sp[c + 1] - first;
             }
-            const int total = cum[kMaxSpecies];
-            if (total == 0) continue;
-            for (int q0 = 0; q0 < total; q0 += 32) {
-                const int t = q0 + lane;
-                if (t < total) {
-                    int s = 0, p = pst[0] + t;
+            int incl = cnt;
 #pragma unroll
-                    for (int q = 1; q < kMaxSpecies; ++q)
-                        if (t >= cum[q] && cum[q + 1] > cum[q]) {
-                            s = q;
-                            p = pst[q] + (t - cum[q]);
-                        }
+            for (int o = 1; o < 32; o <<= 1) {
+                const int up = __shfl_up_sync(0xffffffffu, incl, o);
+                if (lane >= o) incl += up;
+            }
+            const int total = __shfl_sync(0xffffffffu, incl, 31);
+            const int base = first - (incl - cnt);   // particle = base + list index
+            int cl = 0;                              // the cell the warp is adding up
+            int cend = __shfl_sync(0xffffffffu, incl, nsp - 1);
+            for (int w0 = 0; cl < gc0; w0 += 32) {   // (every pass ends cells or takes 32 particles)
+                const int t = w0 + lane;
+                // the range the lane's particle lies in (all lanes search)
+                int seg = 0;
+#pragma unroll
+                for (int o = 16; o > 0; o >>= 1)
+                    if (__shfl_sync(0xffffffffu, incl, seg + o - 1) <= t) seg += o;
+                const int p = __shfl_sync(0xffffffffu, base, seg) + t;
+                if (t < total) {
+                    const int s = seg % nsp, pc = cg + seg / nsp;
                     const T fx = ld(ds.fx[s] + p), fy = ld(ds.fy[s] + p), fzz = ld(fz.fz[s] + p);
                     const T ux = ld(ds.ux[s] + p), uy = ld(ds.uy[s] + p), uz = ld(ds.uz[s] + p);
                     const T wt = ld(ds.w[s] + p);
                     T W[8], Bp[3], al[9];
                     corner_weights(fx, fy, fzz, W);
-                    tile_B3(stl[wib], cl, fx, fy, fzz, Bp);
-                    const T gbar = sqrt(T(1) + ux * ux + uy * uy + uz * uz);
-                    alpha3(Bp, ds.beta[s], gbar, al);
-                    const T cM = wt * ds.cM[s] / gbar, cJ = wt * ds.cJ[s] / gbar;
+                    tile_B3(stl[wib].B, pc, fx, fy, fzz, Bp);
+                    const T ig = T(1) / sqrt(T(1) + ux * ux + uy * uy + uz * uz);
+                    alpha3(Bp, ds.beta[s] * ig, al);
+                    const T cM = wt * ds.cM[s] * ig, cJ = wt * ds.cJ[s] * ig;
+                    const T X[3] = {(T(1) - fx) * (T(1) - fx), (T(1) - fx) * fx, fx * fx};
+                    const T Y[3] = {(T(1) - fy) * (T(1) - fy), (T(1) - fy) * fy, fy * fy};
 #pragma unroll
-                    for (int a = 0; a < 8; ++a) st[lane][a] = W[a];
+                    for (int e = 0; e < 9; ++e) st.put(lane, kS3E + e, cM * al[e]);
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) st[lane][8 + e] = cM * al[e];
+                    for (int e = 0; e < 9; ++e) st.put(lane, kS3XY + e, X[e / 3] * Y[e % 3]);
+                    st.put(lane, kS3Z, (T(1) - fzz) * (T(1) - fzz));
+                    st.put(lane, kS3Z + 1, (T(1) - fzz) * fzz);
+                    st.put(lane, kS3Z + 2, fzz * fzz);
+#pragma unroll
+                    for (int a = 0; a < 8; ++a) st.put(lane, kS3W + a, W[a]);
 #pragma unroll
                     for (int r = 0; r < 3; ++r)
-                        st[lane][17 + r] = cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz);
+                        st.put(lane, kS3V + r, cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz));
+                } else {
+#pragma unroll
+                    for (int q = 0; q < kS3N; ++q) st.put(lane, q, T(0));
                 }
                 __syncwarp();
-                const int m = min(32, total - q0);
-                for (int t2 = 0; t2 < m; ++t2) {
-                    const T wab = st[t2][a0] * st[t2][b0];
-                    const T w1 = two ? st[t2][a1] * st[t2][b1] : T(0);
-                    if constexpr (sizeof(T) == 4) {
-                        float2 al2[4];
-                        const float2* r2 = reinterpret_cast<const float2*>(&st[t2][8]);
+                const int wend = min(w0 + 32, total);
+                int pos = w0;
+                while (cl < gc0) {
+                    const int upto = min(cend, wend);
+                    if (upto > pos) acc.add(st, pos - w0, upto - w0, k1, k2, ja, jc);
+                    pos = max(pos, upto);
+                    if (cend > wend) break;   // the cell goes on in the next batch
+                    // the cell is done
+                    const int before = cl == 0 ? 0 : __shfl_sync(0xffffffffu, incl, cl * nsp - 1);
+                    const bool last = cg + cl == cn - 1;
+                    T v[9], vj;
+                    acc.get(v, vj);
+                    if (carry || cend > before) {
+                        if (lane < kMom3)
 #pragma unroll
-                        for (int q = 0; q < 4; ++q) al2[q] = r2[q];
-                        const float al8 = st[t2][16];
-                        acc0.add(wab, al2, al8);
-                        if (two) acc1.add(w1, al2, al8);
-                    } else {
-                        T al[9];
-#pragma unroll
-                        for (int e = 0; e < 9; ++e) al[e] = st[t2][8 + e];
-                        acc0.add(wab, al);
-                        if (two) acc1.add(w1, al);
+                            for (int e = 0; e < 9; ++e) smom[wib][lane * 9 + e] = v[e];
+                        const int i = i0 + cg + cl;
+                        const int64_t nd = node3(wrap1(i + (lane & 1), g.nx), wrap1(j + ((lane >> 1) & 1), g.ny),
+                                                 wrap1(k + ((lane >> 2) & 1), g.nz), g);
+                        if (lane < 8) snode[wib][lane] = nd;
+                        __syncwarp();
+                        const int nit = last ? kItems3 : kFace3;
+                        for (int it = lane; it < nit; it += 32) {
+                            const unsigned q = item[it];
+                            atomicAdd(M + snode[wib][q >> 16] * kMBlock3 + ((q >> 8) & 255u), smom[wib][q & 255u]);
+                        }
+                        if (lane < 24 && (last || (ja & 1) == 0))
+                            atomicAdd(J + (int64_t)jc * g.ncell + snode[wib][ja], vj);
+                        __syncwarp();
+                        carry = !last;
                     }
-                    if (ownj) accj += st[t2][ja] * st[t2][17 + jc];
+                    // the upper x face's sums start the next cell's lower face
+                    T n9[9];
+#pragma unroll
+                    for (int e = 0; e < 9; ++e) {
+                        const T up = __shfl_down_sync(0xffffffffu, v[e], 6);
+                        n9[e] = low && !last ? up : T(0);
+                    }
+                    const T upj = __shfl_down_sync(0xffffffffu, vj, 3);
+                    acc.start(n9, lane < 24 && (ja & 1) == 0 && !last ? upj : T(0));
+                    ++cl;
+                    if (cl < gc0) cend = __shfl_sync(0xffffffffu, incl, cl * nsp + nsp - 1);
                 }
                 __syncwarp();
-            }
-            // flush: the block of pair (a, b) is stored at corner a with the
-            // offset b - a when that offset is in the stored half, else at
-            // corner b with a - b
-            {
-                T v[9];
-                acc0.get(v);
-                flush_pair3(M, a0, b0, v, i, j, k, g);
-                if (two) {
-                    acc1.get(v);
-                    flush_pair3(M, a1, b1, v, i, j, k, g);
-                }
-            }
-            if (ownj) {
-                const int64_t gn = node3(wrap1(i + (ja & 1), g.nx), wrap1(j + ((ja >> 1) & 1), g.ny),
-                                         wrap1(k + ((ja >> 2) & 1), g.nz), g);
-                atomicAdd(J + (int64_t)jc * g.ncell + gn, accj);
             }
         }
     }
@@ -773,7 +925,11 @@ k_work3(const T* __restrict__ M, const T* __restrict__ J, const T* __restrict__ 
 // ---------------------------------------------------------------------------
 // push
 
-constexpr int kPushWarps3 = 4;
+// warps of a block: static shared memory below 48 KB
+template <typename T>
+struct PushCfg3 {
+    static constexpr int warps = sizeof(T) == 4 ? 4 : 2;
+};
 
 // The explicit push with E^{n+theta} and B^n at x^{n+1/2}: ubar = alpha (u +
 // beta E), u^{n+1} = 2 ubar - u^n, x^{n+3/2} = x^{n+1/2} + dt u^{n+1}/gamma^{n+1}
@@ -785,114 +941,132 @@ constexpr int kPushWarps3 = 4;
 // atomic per new cell and warp: the lanes with equal keys found by
 // match-any), for the unstable counting sort that follows.
 template <typename T>
-__global__ void __launch_bounds__(32 * kPushWarps3)
+__global__ void __launch_bounds__(32 * PushCfg3<T>::warps)
 k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict__ dfz,
         const int32_t* __restrict__ start, int32_t* __restrict__ key, int32_t* __restrict__ rank,
         int32_t* __restrict__ count, const T* __restrict__ Eth, const T* __restrict__ B, GridP g, T beta, T qdt,
-        T m, double* __restrict__ lsum)
+        T m, double* __restrict__ lsum, int uw)
 {
-    __shared__ int sst[kPushWarps3][33];
-    __shared__ Tile3<T> stl[kPushWarps3];
+    __shared__ int sst[PushCfg3<T>::warps][33];
+    __shared__ PairTile3<T> stl[PushCfg3<T>::warps];
     __shared__ double red[32 * 4];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int nseg = (g.nx + 31) / 32;
+    const int nseg = (g.nx + uw - 1) / uw;
     const int64_t nunits = (int64_t)nseg * g.ny * g.nz;
     int* ss = sst[wib];
-    const T dt = gc<T>(g).dt, rdx = gc<T>(g).rdx, rdy = gc<T>(g).rdy, rdz = gc<T>(g).rdz;
+    const PairTile3<T>& tl = stl[wib];
+    const T dtx = gc<T>(g).dt * gc<T>(g).rdx, dty = gc<T>(g).dt * gc<T>(g).rdy, dtz = gc<T>(g).dt * gc<T>(g).rdz;
     T acc[4] = {T(0), T(0), T(0), T(0)};
+    // a batch whose slots are still on their way: its particle, the lanes that
+    // share its new cell, and (the first of them) what the count was
+    int wait_p = -1, wait_base = 0;
+    unsigned wait_peers = 0u;
+    auto settle = [&]() {
+        const int b = __shfl_sync(0xffffffffu, wait_base, wait_peers ? __ffs(wait_peers) - 1 : lane);
+        if (wait_p >= 0) rank[wait_p] = b + __popc(wait_peers & ((1u << lane) - 1u));
+        wait_p = -1;
+    };
     for (int64_t u = warp; u < nunits; u += nwarps) {
-        const int i0 = (int)(u % nseg) * 32;
+        const int i0 = (int)(u % nseg) * uw;
         const int jk = (int)(u / nseg);
         const int j = jk % g.ny, k = jk / g.ny;
-        const int cn = min(32, g.nx - i0);
+        const int cn = min(uw, g.nx - i0);
         const int64_t c0 = node3(i0, j, k, g);
         __syncwarp();
         if (lane <= cn) ss[lane] = start[c0 + lane];
         if (lane == 0 && cn == 32) ss[32] = start[c0 + 32];
-        load_tile3<T>(stl[wib], Eth, B, i0, cn, j, k, g, lane);
-        const Tile3<T>& tl = stl[wib];
+        load_pairs3<T>(stl[wib], Eth, B, i0, cn, j, k, g, lane);
         const int P0 = ss[0], P1 = ss[cn];
         int cl = 0;
+        // the next batch is loaded while this one is pushed
+        T nfx = T(0), nfy = T(0), nfz = T(0), nux = T(0), nuy = T(0), nuz = T(0), nw = T(0);
+        auto fetch = [&](int q) {
+            if (q < P1) {
+                nfx = ld(src.fx + q);
+                nfy = ld(src.fy + q);
+                nfz = ld(sfz + q);
+                nux = ld(src.ux + q);
+                nuy = ld(src.uy + q);
+                nuz = ld(src.uz + q);
+                nw = ld(src.w + q);
+            }
+        };
+        fetch(P0 + lane);
         for (int p0 = P0; p0 < P1; p0 += 32) {
             const int p = p0 + lane;
             const bool act = p < P1;
+            const T fx = nfx, fy = nfy, fz = nfz, ux = nux, uy = nuy, uz = nuz, w = nw;
+            fetch(p + 32);
             int newkey = -1 - lane;   // distinct for idle lanes
             if (act) {
-            while (ss[cl + 1] <= p) ++cl;
-            const int i = i0 + cl;
-            const T fx = ld(src.fx + p), fy = ld(src.fy + p), fz = ld(sfz + p);
-            const T ux = ld(src.ux + p), uy = ld(src.uy + p), uz = ld(src.uz + p), w = ld(src.w + p);
-            T W[8];
-            corner_weights(fx, fy, fz, W);
-            T E[3];
+                while (ss[cl + 1] <= p) ++cl;
+                T E[3], Bp[3];
+                tl.gather_E(cl, fx, fy, fz, E);
+                tl.gather_B(cl, fx, fy, fz, Bp);
+                const T u02 = ux * ux + uy * uy + uz * uz;
+                const T g0 = sqrt(T(1) + u02), ig0 = T(1) / g0;
+                const T bg = beta * ig0, ax = bg * Bp[0], ay = bg * Bp[1], az = bg * Bp[2];
+                const T sa = T(1) / (T(1) + ax * ax + ay * ay + az * az);
+                const T wx = ux + beta * E[0], wy = uy + beta * E[1], wz = uz + beta * E[2];
+                const T wa = wx * ax + wy * ay + wz * az;
+                const T ubx = sa * (wx + (wy * az - wz * ay) + wa * ax);
+                const T uby = sa * (wy + (wz * ax - wx * az) + wa * ay);
+                const T ubz = sa * (wz + (wx * ay - wy * ax) + wa * az);
+                const T u1x = T(2) * ubx - ux, u1y = T(2) * uby - uy, u1z = T(2) * ubz - uz;
+                const T u12 = u1x * u1x + u1y * u1y + u1z * u1z;
+                const T g1 = sqrt(T(1) + u12), ig1 = T(1) / g1;
+                const T t[3] = {fx + dtx * (u1x * ig1), fy + dty * (u1y * ig1), fz + dtz * (u1z * ig1)};
+                const int nn[3] = {g.nx, g.ny, g.nz}, cc[3] = {i0 + cl, j, k};
+                T fn[3];
+                int cnew[3];
 #pragma unroll
-            for (int c = 0; c < 3; ++c) {
-                T e = T(0);
-#pragma unroll
-                for (int a = 0; a < 8; ++a) e += W[a] * tl.E[c][(a >> 1) & 1][(a >> 2) & 1][cl + (a & 1)];
-                E[c] = e;
-            }
-            T Bp[3];
-            tile_B3(tl, cl, fx, fy, fz, Bp);
-            const T u02 = ux * ux + uy * uy + uz * uz;
-            const T g0 = sqrt(T(1) + u02);
-            const T ax = beta * Bp[0] / g0, ay = beta * Bp[1] / g0, az = beta * Bp[2] / g0;
-            const T sa = T(1) / (T(1) + ax * ax + ay * ay + az * az);
-            const T wx = ux + beta * E[0], wy = uy + beta * E[1], wz = uz + beta * E[2];
-            const T wa = wx * ax + wy * ay + wz * az;
-            const T ubx = sa * (wx + (wy * az - wz * ay) + wa * ax);
-            const T uby = sa * (wy + (wz * ax - wx * az) + wa * ay);
-            const T ubz = sa * (wz + (wx * ay - wy * ax) + wa * az);
-            const T u1x = T(2) * ubx - ux, u1y = T(2) * uby - uy, u1z = T(2) * ubz - uz;
-            const T u12 = u1x * u1x + u1y * u1y + u1z * u1z;
-            const T g1 = sqrt(T(1) + u12);
-            const T t[3] = {fx + dt * rdx * (u1x / g1), fy + dt * rdy * (u1y / g1), fz + dt * rdz * (u1z / g1)};
-            const int nn[3] = {g.nx, g.ny, g.nz}, cc[3] = {i, j, k};
-            T fn[3];
-            int cnew[3];
-#pragma unroll
-            for (int a = 0; a < 3; ++a) {
-                const T fl = floor(t[a]);
-                int sh = (int)fl;
-                T f = t[a] - fl;
-                if (f >= T(1)) { f -= T(1); sh += 1; }
-                fn[a] = f;
-                int q = (cc[a] + sh) % nn[a];
-                if (q < 0) q += nn[a];
-                cnew[a] = q;
-            }
-            dst.fx[p] = fn[0];
-            dst.fy[p] = fn[1];
-            dfz[p] = fn[2];
-            dst.ux[p] = u1x;
-            dst.uy[p] = u1y;
-            dst.uz[p] = u1z;
-            dst.w[p] = w;
-            if (dst.id) dst.id[p] = src.id[p];
-            newkey = (int32_t)node3(cnew[0], cnew[1], cnew[2], g);
-            key[p] = newkey;
-            // ledger: g0 - g1 = (u0 - u1).(u0 + u1)/(g0 + g1)
-            const T ue = ubx * E[0] + uby * E[1] + ubz * E[2];
-            const T du = (ux - u1x) * (ux + u1x) + (uy - u1y) * (uy + u1y) + (uz - u1z) * (uz + u1z);
-            const T igs = T(1) / (g0 + g1);
-            acc[0] -= w * m * du * igs;
-            acc[1] += qdt * w * ue / g0;
-            acc[2] += qdt * w * ue * du * igs * igs / g0;
-            acc[3] += w * m * u12 / (g1 + T(1));
+                for (int a = 0; a < 3; ++a) {
+                    const T fl = floor(t[a]);
+                    int sh = (int)fl;
+                    T f = t[a] - fl;
+                    if (f >= T(1)) { f -= T(1); sh += 1; }
+                    fn[a] = f;
+                    int q = cc[a] + sh;
+                    if ((unsigned)q >= (unsigned)nn[a]) {   // across the box: any distance
+                        q %= nn[a];
+                        if (q < 0) q += nn[a];
+                    }
+                    cnew[a] = q;
+                }
+                dst.fx[p] = fn[0];
+                dst.fy[p] = fn[1];
+                dfz[p] = fn[2];
+                dst.ux[p] = u1x;
+                dst.uy[p] = u1y;
+                dst.uz[p] = u1z;
+                dst.w[p] = w;
+                if (dst.id) dst.id[p] = src.id[p];
+                newkey = (int32_t)node3(cnew[0], cnew[1], cnew[2], g);
+                key[p] = newkey;
+                // ledger: g0 - g1 = (u0 - u1).(u0 + u1)/(g0 + g1)
+                const T ue = ubx * E[0] + uby * E[1] + ubz * E[2];
+                const T du = (ux - u1x) * (ux + u1x) + (uy - u1y) * (uy + u1y) + (uz - u1z) * (uz + u1z);
+                const T igs = T(1) / (g0 + g1), wk = qdt * w * ue * ig0;
+                acc[0] -= w * m * du * igs;
+                acc[1] += wk;
+                acc[2] += wk * du * igs * igs;
+                acc[3] += w * m * u12 / (g1 + T(1));
             }
             if (rank) {
+                settle();   // the last batch's slots have had this one's time to arrive
                 const unsigned peers = __match_any_sync(0xffffffffu, newkey);
-                const int leader = __ffs(peers) - 1;
-                int base = 0;
-                if (act && lane == leader) base = atomicAdd(count + newkey, __popc(peers));
-                base = __shfl_sync(0xffffffffu, base, leader);
-                if (act) rank[p] = base + __popc(peers & ((1u << lane) - 1u));
+                wait_peers = peers;
+                if (act) {
+                    wait_p = p;
+                    if ((peers & ((1u << lane) - 1u)) == 0u) wait_base = atomicAdd(count + newkey, __popc(peers));
+                }
             }
         }
         __syncwarp();
     }
+    if (rank) settle();
     double v[4], o[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = (double)acc[q];
@@ -902,22 +1076,49 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict
         for (int q = 0; q < 4; ++q) lsum[(int64_t)blockIdx.x * 4 + q] = o[q];
 }
 
-// the counting sort's placement: particle p to start[key[p]] + rank[p]
+// the counting sort's placement: particle p to start[key[p]] + rank[p]. Four
+// particles a thread: each waits on a chain of loads (key, start, then the
+// stores), and one at a time left the kernel bound by that wait
 template <typename T>
-__global__ void k_place3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict__ dfz,
-                         const int32_t* __restrict__ key, const int32_t* __restrict__ rank,
-                         const int32_t* __restrict__ start, int64_t n)
+__global__ void __launch_bounds__(256)
+k_place3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict__ dfz,
+         const int32_t* __restrict__ key, const int32_t* __restrict__ rank, const int32_t* __restrict__ start,
+         int64_t n)
 {
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t q = (int64_t)start[key[p]] + rank[p];
-        dst.fx[q] = src.fx[p];
-        dst.fy[q] = src.fy[p];
-        if (dfz) dfz[q] = sfz[p];   // null for 2D particles
-        dst.ux[q] = src.ux[p];
-        dst.uy[q] = src.uy[p];
-        dst.uz[q] = src.uz[p];
-        dst.w[q] = src.w[p];
-        if (dst.id) dst.id[q] = src.id[p];
+    constexpr int U = 4;
+    for (int64_t b = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; b < n; b += (int64_t)gridDim.x * (256 * U)) {
+        int64_t q[U], p[U];
+        int kk[U], rr[U];
+#pragma unroll
+        for (int v = 0; v < U; ++v) {
+            p[v] = b + 256 * v;
+            const bool in = p[v] < n;
+            kk[v] = in ? ld(key + p[v]) : 0;
+            rr[v] = in ? ld(rank + p[v]) : 0;
+            if (!in) p[v] = -1;
+        }
+#pragma unroll
+        for (int v = 0; v < U; ++v) q[v] = (int64_t)ld(start + kk[v]) + rr[v];
+        // one array at a time: its U loads in flight, then its stores
+        auto move = [&](const T* a, T* o) {
+            T x[U];
+#pragma unroll
+            for (int v = 0; v < U; ++v) x[v] = p[v] >= 0 ? ld(a + p[v]) : T(0);
+#pragma unroll
+            for (int v = 0; v < U; ++v)
+                if (p[v] >= 0) o[q[v]] = x[v];
+        };
+        move(src.fx, dst.fx);
+        move(src.fy, dst.fy);
+        if (dfz) move(sfz, dfz);   // null for 2D particles
+        move(src.ux, dst.ux);
+        move(src.uy, dst.uy);
+        move(src.uz, dst.uz);
+        move(src.w, dst.w);
+        if (dst.id)
+#pragma unroll
+            for (int v = 0; v < U; ++v)
+                if (p[v] >= 0) dst.id[q[v]] = src.id[p[v]];
     }
 }
 
@@ -952,14 +1153,24 @@ cudaError_t export_particles3(PArrays<T> p, const T* fz, const int32_t* start, G
     return cudaGetLastError();
 }
 
+// the width of the row segments a warp takes: 32 cells, halved while that
+// leaves fewer than eight warps per SM
+static int unit_width3(GridP g)
+{
+    int uw = 32;
+    while (uw > 4 && (int64_t)((g.nx + uw - 1) / uw) * g.ny * g.nz < 152 * 8) uw /= 2;
+    return uw;
+}
+
 template <typename T>
 cudaError_t deposit3(const DepositSpecies<T>& ds, const FzArrays<T>& fz, const T* B, T* M, T* J, GridP g,
                      cudaStream_t st, int blocks)
 {
-    const int64_t units = (int64_t)((g.nx + 31) / 32) * g.ny * g.nz;
+    const int uw = unit_width3(g);
+    const int64_t units = (int64_t)((g.nx + uw - 1) / uw) * g.ny * g.nz;
     count_launches(1);
     k_deposit3<T><<<grid3(units, DepCfg3<T>::warps, blocks > 0 ? blocks : 152 * 8), 32 * DepCfg3<T>::warps, 0, st>>>(
-        ds, fz, B, M, J, g);
+        ds, fz, B, M, J, g, uw);
     return cudaGetLastError();
 }
 
@@ -998,8 +1209,9 @@ cudaError_t field_update3(const double* x, const T* M, const T* J, T* Eth, T* E,
 
 int push_blocks3(GridP g, int cap)
 {
-    const int64_t units = (int64_t)((g.nx + 31) / 32) * g.ny * g.nz;
-    return (int)grid3(units, kPushWarps3, cap > 0 ? cap : 152 * 16);
+    const int uw = unit_width3(g);
+    const int64_t units = (int64_t)((g.nx + uw - 1) / uw) * g.ny * g.nz;
+    return (int)grid3(units, PushCfg3<float>::warps, cap > 0 ? cap : 152 * 16);
 }
 
 template <typename T>
@@ -1008,9 +1220,9 @@ cudaError_t push3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const in
                   int nblocks, cudaStream_t st)
 {
     count_launches(1);
-    k_push3<T><<<nblocks, 32 * kPushWarps3, 0, st>>>(src, sfz, dst, dfz, start, key, rank, count, Eth, B, g,
+    k_push3<T><<<nblocks, 32 * PushCfg3<T>::warps, 0, st>>>(src, sfz, dst, dfz, start, key, rank, count, Eth, B, g,
                                                        (T)(sc.q * g.dt / (2.0 * sc.m)), (T)(sc.q * g.dt), (T)sc.m,
-                                                       lsum);
+                                                       lsum, unit_width3(g));
     return cudaGetLastError();
 }
 
@@ -1020,7 +1232,7 @@ cudaError_t place3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const i
 {
     if (n <= 0) return cudaSuccess;
     count_launches(1);
-    k_place3<T><<<grid3(n, 256, 152 * 32), 256, 0, st>>>(src, sfz, dst, dfz, key, rank, start, n);
+    k_place3<T><<<grid3(n, 256 * 4, 152 * 32), 256, 0, st>>>(src, sfz, dst, dfz, key, rank, start, n);
     return cudaGetLastError();
 }
 

@@ -950,7 +950,7 @@ int solve_epilogue(relsim_ctx* c, cudaStream_t s)
     CK(cudaMemcpyAsync(c->dled + kLedgerLen - 2, c->dled + 3, 2 * sizeof(double), cudaMemcpyDeviceToDevice, s));
     // the predicted-gamma push needs E^n after E^{n+1} has replaced it
     if (c->En) CK(cudaMemcpyAsync(c->En, c->E, c->esz * 3 * (size_t)c->g.ncell, cudaMemcpyDeviceToDevice, s));
-    const int nbf = field_grid_blocks(c->g);
+    const int nbf = field_grid_blocks(c->g, c->prec);
     PROF_BEGIN(RELSIM_PROF_FIELD_UPDATE);
     CK(field_update<T>(c->gx, (const T*)c->M, (const T*)c->J, (T*)c->Eth, (T*)c->E, (const T*)c->B[c->bcur],
                        (T*)c->B[1 - c->bcur], c->g, c->partial, nbf, s));
@@ -963,7 +963,7 @@ int solve_epilogue(relsim_ctx* c, cudaStream_t s)
 // capture must not allocate)
 int solve_reserve(relsim_ctx* c, const GmSetup& S)
 {
-    const int nbf = field_grid_blocks(c->g);
+    const int nbf = field_grid_blocks(c->g, c->prec);
     int64_t need = (int64_t)(S.nb > S.nbo ? S.nb : S.nbo) * (S.m + 2);
     if ((int64_t)nbf * 6 > need) need = (int64_t)nbf * 6;
     if (c->solve_rows && gm_solve_partials(c->g, c->solve_rows, S.m) > need)

@@ -10,17 +10,15 @@
 //
 // Kernels:
 //   k_load3, k_gather3, k_export3   load, re-sort gather, read-back
-//   k_deposit3   warp per row segment of cells; for each cell the lanes stage
-//                their particles' weights, c alpha and c alpha u / gbar in
-//                shared memory, then each lane accumulates the node pairs it
-//                owns over the cell's particles in registers and flushes them
-//                once per cell (FP32 or FP64 atomics)
-//   k_op3        the operator A = I + (theta dt)^2 curl_n curl_c + theta dt M,
-//                one thread per node, in the three modes of the 2D operator
+//   k_deposit3   warp per row segment of cells: its particles staged in shared
+//                memory 32 at a time, the lanes sum the 27 distinct weight
+//                products of a cell's node pairs
+//   k_op3        the operator A = I + (theta dt)^2 curl_n curl_c + theta dt M on
+//                32 x 2 x 2-node tiles, in the three modes of the 2D operator
 //   k_rhs3, k_field_update3   the right-hand side, the field update with the
-//                field ledger terms
-//   k_push3      warp per row segment, the push with the cell change of the
-//                general path (any move length), followed by the radix sort
+//                field ledger terms (on the operator's tiles)
+//   k_push3      warp per row segment, the push with each particle's new cell
+//                and its slot there (any move length); k_place3 places them
 #include "launch.cuh"
 
 namespace relsim {
@@ -56,11 +54,17 @@ __global__ void k_load3(const double* __restrict__ x, const double* __restrict__
                         int64_t n, GridP g, PArrays<T> out, T* __restrict__ ofz, int32_t* __restrict__ key,
                         int32_t* __restrict__ val, int* bad)
 {
+    const bool unit = is_one(g.dx) && is_one(g.dy) && is_one(g.dz);
     for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p < n; p += (int64_t)gridDim.x * blockDim.x) {
-        double s[3] = {x[3 * p] / g.dx, x[3 * p + 1] / g.dy, x[3 * p + 2] / g.dz};
+        double s[3] = {x[3 * p], x[3 * p + 1], x[3 * p + 2]};
+        if (!unit) {
+            s[0] /= g.dx;
+            s[1] /= g.dy;
+            s[2] /= g.dz;
+        }
         const double ux = u[3 * p], uy = u[3 * p + 1], uz = u[3 * p + 2], ww = w[p];
-        if (!isfinite(s[0]) || !isfinite(s[1]) || !isfinite(s[2]) || !isfinite(ux) || !isfinite(uy) ||
-            !isfinite(uz) || !isfinite(ww)) {
+        if (!finite_bits(s[0]) || !finite_bits(s[1]) || !finite_bits(s[2]) || !finite_bits(ux) || !finite_bits(uy) ||
+            !finite_bits(uz) || !finite_bits(ww)) {
             atomicOr(bad, 1);
             s[0] = s[1] = s[2] = 0.0;
         }
@@ -68,22 +72,14 @@ __global__ void k_load3(const double* __restrict__ x, const double* __restrict__
         int c[3];
         T f[3];
 #pragma unroll
-        for (int a = 0; a < 3; ++a) {
-            if (s[a] < 0.0 || s[a] >= (double)nn[a]) s[a] -= nn[a] * floor(s[a] / nn[a]);
-            const double fl = floor(s[a]);
-            int ci = (int)fl;
-            if (ci >= nn[a]) ci -= nn[a];
-            if (ci < 0) ci = 0;
-            c[a] = ci;
-            f[a] = from_double_rz<T>(s[a] - fl);
-        }
+        for (int a = 0; a < 3; ++a) split_cell<T>(s[a], nn[a], c[a], f[a]);
         out.fx[p] = f[0];
         out.fy[p] = f[1];
         ofz[p] = f[2];
-        out.ux[p] = (T)ux;
-        out.uy[p] = (T)uy;
-        out.uz[p] = (T)uz;
-        out.w[p] = (T)ww;
+        out.ux[p] = narrow<T>(ux);
+        out.uy[p] = narrow<T>(uy);
+        out.uz[p] = narrow<T>(uz);
+        out.w[p] = narrow<T>(ww);
         key[p] = (int32_t)node3(c[0], c[1], c[2], g);
         val[p] = (int32_t)p;
     }
@@ -114,21 +110,29 @@ __global__ void k_export3(PArrays<T> pa, const T* __restrict__ fz, const int32_t
     const int lane = threadIdx.x & 31;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
+    const bool unit = is_one(g.dx) && is_one(g.dy) && is_one(g.dz);
     for (int c = warp; c < g.ncell; c += nwarps) {
         const int i = c % g.nx, j = (c / g.nx) % g.ny, k = c / (g.nx * g.ny);
+        const double id0 = (double)i, jd0 = (double)j, kd0 = (double)k;
         const int p1 = start[c + 1];
         for (int p = start[c] + lane; p < p1; p += 32) {
             if (x) {
-                x[3 * (int64_t)p] = ((double)i + (double)pa.fx[p]) * g.dx;
-                x[3 * (int64_t)p + 1] = ((double)j + (double)pa.fy[p]) * g.dy;
-                x[3 * (int64_t)p + 2] = ((double)k + (double)fz[p]) * g.dz;
+                double xs = id0 + widen(pa.fx[p]), ys = jd0 + widen(pa.fy[p]), zs = kd0 + widen(fz[p]);
+                if (!unit) {
+                    xs *= g.dx;
+                    ys *= g.dy;
+                    zs *= g.dz;
+                }
+                x[3 * (int64_t)p] = xs;
+                x[3 * (int64_t)p + 1] = ys;
+                x[3 * (int64_t)p + 2] = zs;
             }
             if (u) {
-                u[3 * (int64_t)p] = (double)pa.ux[p];
-                u[3 * (int64_t)p + 1] = (double)pa.uy[p];
-                u[3 * (int64_t)p + 2] = (double)pa.uz[p];
+                u[3 * (int64_t)p] = widen(pa.ux[p]);
+                u[3 * (int64_t)p + 1] = widen(pa.uy[p]);
+                u[3 * (int64_t)p + 2] = widen(pa.uz[p]);
             }
-            if (w) w[p] = (double)pa.w[p];
+            if (w) w[p] = widen(pa.w[p]);
             if (id && pa.id) id[p] = pa.id[p];
         }
     }
@@ -312,8 +316,9 @@ struct DepCfg3 {
 constexpr int kMom3 = 27;
 constexpr int kItems3 = 36 * 9;        // a cell's additions to M
 constexpr int kFace3 = 26 * 9;         // those not on the upper x face
-// staged values of a particle: c alpha, XX YY, ZZ, corner weights, current
-enum { kS3E = 0, kS3XY = 9, kS3Z = 18, kS3W = 21, kS3V = 29, kS3N = 32 };
+// staged values of a particle: c alpha (rows of four), XX YY, corner weights
+// (lower, upper z face), ZZ, current
+enum { kS3E = 0, kS3XY = 12, kS3W = 22, kS3Z = 30, kS3V = 33, kS3N = 36 };
 
 // the staged particles of a warp: FP32 two by two, (value of particle 2r,
 // value of particle 2r + 1), rows 16-byte aligned
@@ -324,84 +329,124 @@ struct Stage3 {
 };
 template <>
 struct Stage3<float> {
-    static constexpr int row = 2 * kS3N + 4;
+    static constexpr int row = 2 * kS3N + 4;   // (an odd number of 16-byte pieces)
     float v[16][row];
     __device__ __forceinline__ void put(int t, int k, float a) { v[t >> 1][2 * k + (t & 1)] = a; }
     __device__ __forceinline__ float2 get2(int r, int k) const { return *reinterpret_cast<const float2*>(&v[r][2 * k]); }
+    // two neighbouring values (k even)
+    __device__ __forceinline__ void get4(int r, int k, float2& a, float2& b) const
+    {
+        const float4 q = *reinterpret_cast<const float4*>(&v[r][2 * k]);
+        a = make_float2(q.x, q.y);
+        b = make_float2(q.z, q.w);
+    }
 };
 
-// a lane's sums of one moment and one current value over a cell
+// A lane's sums over a cell: lanes 0..26 are three groups of nine that take
+// the staged rows in turn; a group's lane (zz, er) sums the nine moments
+// (XX, YY) of its ZZ for row er of alpha, and at zz = 0 and 2 component er of
+// the current at the four corners of the lower and upper z face. (What a
+// staged row costs is the bytes a lane loads, also where all lanes load the
+// same ones: a tile of 9 products x 3 entries takes a third of the shared-
+// memory traffic of one product x 9 entries in each lane.)
 template <typename T>
 struct Acc3 {
-    T m[9], j;
-    __device__ __forceinline__ void start(const T (&v)[9], T vj)
+    T m[9][3], j[4];
+    __device__ __forceinline__ void clear()
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) m[e] = v[e];
-        j = vj;
+        for (int k = 0; k < 9; ++k)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) m[k][e] = T(0);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = T(0);
     }
-    __device__ __forceinline__ void add(const Stage3<T>& st, int t0, int t1, int k1, int k2, int ja, int jc)
+    // staged particles t0 .. t1-1, every third from the grp-th of the batch
+    __device__ __forceinline__ void add(const Stage3<T>& st, int t0, int t1, int grp, int zz, int er)
     {
-        for (int t = t0; t < t1; ++t) {
-            const T w = st.v[t][kS3XY + k1] * st.v[t][kS3Z + k2];
+        for (int t = t0 + (grp + 3 - t0 % 3) % 3; t < t1; t += 3) {
+            const T* r = st.v[t];
+            const T z = r[kS3Z + zz];
+            T e[3];
 #pragma unroll
-            for (int e = 0; e < 9; ++e) m[e] += w * st.v[t][kS3E + e];
-            j += st.v[t][kS3W + ja] * st.v[t][kS3V + jc];
+            for (int q = 0; q < 3; ++q) e[q] = z * r[kS3E + 4 * er + q];
+#pragma unroll
+            for (int k = 0; k < 9; ++k) {
+                const T w = r[kS3XY + k];
+#pragma unroll
+                for (int q = 0; q < 3; ++q) m[k][q] += w * e[q];
+            }
+            const T v = r[kS3V + er];
+#pragma unroll
+            for (int c = 0; c < 4; ++c) j[c] += r[kS3W + 2 * zz + c] * v;
         }
     }
-    __device__ __forceinline__ void get(T (&v)[9], T& vj) const
+    __device__ __forceinline__ T moment(int k, int e) const { return m[k][e]; }
+    __device__ __forceinline__ T current(int c) const { return j[c]; }
+    // the upper x face's sums become the next cell's lower face's
+    __device__ __forceinline__ void carry()
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] = m[e];
-        vj = j;
+        for (int k = 0; k < 9; ++k)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) m[k][e] = k < 3 ? m[k + 6][e] : T(0);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = (c & 1) == 0 ? j[c + 1] : T(0);
     }
 };
 template <>
 struct Acc3<float> {
-    float2 m[9], j;   // even and odd staged particles apart
-    __device__ __forceinline__ void start(const float (&v)[9], float vj)
+    float2 m[9][3], j[4];   // even and odd staged particles apart
+    __device__ __forceinline__ void clear()
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) m[e] = make_float2(v[e], 0.f);
-        j = make_float2(vj, 0.f);
-    }
-    // EDGE: the row holds a particle of another cell (its weights are left out)
-    template <bool EDGE>
-    __device__ __forceinline__ void row(const Stage3<float>& st, int r, int t0, int t1, int k1, int k2, int ja, int jc)
-    {
-        const float2 xy = st.get2(r, kS3XY + k1), z = st.get2(r, kS3Z + k2);
-        float2 w = make_float2(xy.x * z.x, xy.y * z.y), wj = st.get2(r, kS3W + ja);
-        if (EDGE) {
-            if (2 * r < t0) w.x = wj.x = 0.f;
-            if (2 * r + 1 >= t1) w.y = wj.y = 0.f;
-        }
-        const float4* e4 = reinterpret_cast<const float4*>(&st.v[r][0]);
+        for (int k = 0; k < 9; ++k)
 #pragma unroll
-        for (int h = 0; h < 4; ++h) {
-            const float4 q = e4[h];
-            m[2 * h] = __ffma2_rn(w, make_float2(q.x, q.y), m[2 * h]);
-            m[2 * h + 1] = __ffma2_rn(w, make_float2(q.z, q.w), m[2 * h + 1]);
-        }
-        m[8] = __ffma2_rn(w, st.get2(r, kS3E + 8), m[8]);
-        j = __ffma2_rn(wj, st.get2(r, kS3V + jc), j);
+            for (int e = 0; e < 3; ++e) m[k][e] = make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = make_float2(0.f, 0.f);
     }
-    __device__ __forceinline__ void add(const Stage3<float>& st, int t0, int t1, int k1, int k2, int ja, int jc)
+    __device__ __forceinline__ void add(const Stage3<float>& st, int t0, int t1, int grp, int zz, int er)
     {
-        int r = t0 >> 1;
-        const int r1 = t1 >> 1;   // rows r0 .. r1-1 are whole but for the first
-        if (t0 & 1) {
-            row<true>(st, r, t0, t1, k1, k2, ja, jc);
-            ++r;
+        const int r0 = t0 >> 1, r1 = (t1 + 1) >> 1;
+        for (int r = r0 + (grp + 3 - r0 % 3) % 3; r < r1; r += 3) {
+            float2 z = st.get2(r, kS3Z + zz), v = st.get2(r, kS3V + er);
+            // a row at the cell's ends may hold a particle of another cell
+            if (2 * r < t0) z.x = v.x = 0.f;
+            if (2 * r + 1 >= t1) z.y = v.y = 0.f;
+            float2 e[3], a, b;
+            st.get4(r, kS3E + 4 * er, a, b);
+            e[0] = __fmul2_rn(z, a);
+            e[1] = __fmul2_rn(z, b);
+            e[2] = __fmul2_rn(z, st.get2(r, kS3E + 4 * er + 2));
+#pragma unroll
+            for (int k = 0; k < 9; k += 2) {
+                if (k < 8) st.get4(r, kS3XY + k, a, b);
+                else a = st.get2(r, kS3XY + k);
+#pragma unroll
+                for (int q = 0; q < 3; ++q) {
+                    m[k][q] = __ffma2_rn(a, e[q], m[k][q]);
+                    if (k < 8) m[k + 1][q] = __ffma2_rn(b, e[q], m[k + 1][q]);
+                }
+            }
+#pragma unroll
+            for (int c = 0; c < 4; c += 2) {
+                st.get4(r, kS3W + 2 * zz + c, a, b);
+                j[c] = __ffma2_rn(a, v, j[c]);
+                j[c + 1] = __ffma2_rn(b, v, j[c + 1]);
+            }
         }
-#pragma unroll 2
-        for (; r < r1; ++r) row<false>(st, r, t0, t1, k1, k2, ja, jc);
-        if ((t1 & 1) && r == r1) row<true>(st, r, t0, t1, k1, k2, ja, jc);
     }
-    __device__ __forceinline__ void get(float (&v)[9], float& vj) const
+    __device__ __forceinline__ float moment(int k, int e) const { return m[k][e].x + m[k][e].y; }
+    __device__ __forceinline__ float current(int c) const { return j[c].x + j[c].y; }
+    __device__ __forceinline__ void carry()
     {
 #pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] = m[e].x + m[e].y;
-        vj = j.x + j.y;
+        for (int k = 0; k < 9; ++k)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) m[k][e] = k < 3 ? m[k + 6][e] : make_float2(0.f, 0.f);
+#pragma unroll
+        for (int c = 0; c < 4; ++c) j[c] = (c & 1) == 0 ? j[c + 1] : make_float2(0.f, 0.f);
     }
 };
 
@@ -444,7 +489,8 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
     constexpr int kW = DepCfg3<T>::warps;
     __shared__ __align__(16) Stage3<T> sst[kW];
     __shared__ Tile3B<T> stl[kW];
-    __shared__ T smom[kW][kMom3 * 9];   // a cell's moments, for the additions
+    __shared__ T smom[kW][3][kMom3 * 9];   // a cell's moments (the three groups'), for the additions
+    __shared__ T scur[kW][3][24];          // and its currents: corner, component
     __shared__ int64_t snode[kW][8];    // its corners' nodes
     __shared__ unsigned item[kItems3];  // an addition: corner << 16 | place in the node's blocks << 8 | moment value
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
@@ -466,11 +512,8 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
     const int64_t nunits = (int64_t)nseg * g.ny * g.nz;
     const int nsp = ds.nsp, gcells = 32 / nsp;   // cells whose (cell, species) ranges fit the lanes
     Stage3<T>& st = sst[wib];
-    // the moment this lane sums (lanes 0 .. 26: ZZ, XX, YY) and the current
-    // value (lanes 0 .. 23: corner, component)
-    const int k1 = lane < kMom3 ? lane % 9 : 0, k2 = lane < kMom3 ? lane / 9 : 0;
-    const int ja = lane < 24 ? lane / 3 : 0, jc = lane < 24 ? lane % 3 : 0;
-    const bool low = lane < kMom3 && k1 < 3;   // a moment of the lower x face
+    const bool own = lane < 27;
+    const int grp = own ? lane / 9 : 0, zz = own ? lane / 3 % 3 : 0, er = own ? lane % 3 : 0;
     for (int64_t u = warp; u < nunits; u += nwarps) {
         const int i0 = (int)(u % nseg) * uw;
         const int jk = (int)(u / nseg);
@@ -479,10 +522,7 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
         __syncwarp();
         load_tile3B<T>(stl[wib], B, i0, cn, j, k, g, lane);
         Acc3<T> acc;
-        {
-            const T zero[9] = {T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0), T(0)};
-            acc.start(zero, T(0));
-        }
+        acc.clear();
         bool carry = false;   // the previous cell left sums on this cell's lower face
         for (int cg = 0; cg < cn; cg += gcells) {
             // the particles of up to gcells cells as one list: lane l holds
@@ -527,7 +567,7 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
                     const T X[3] = {(T(1) - fx) * (T(1) - fx), (T(1) - fx) * fx, fx * fx};
                     const T Y[3] = {(T(1) - fy) * (T(1) - fy), (T(1) - fy) * fy, fy * fy};
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) st.put(lane, kS3E + e, cM * al[e]);
+                    for (int e = 0; e < 9; ++e) st.put(lane, kS3E + 4 * (e / 3) + e % 3, cM * al[e]);
 #pragma unroll
                     for (int e = 0; e < 9; ++e) st.put(lane, kS3XY + e, X[e / 3] * Y[e % 3]);
                     st.put(lane, kS3Z, (T(1) - fzz) * (T(1) - fzz));
@@ -547,42 +587,46 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
                 int pos = w0;
                 while (cl < gc0) {
                     const int upto = min(cend, wend);
-                    if (upto > pos) acc.add(st, pos - w0, upto - w0, k1, k2, ja, jc);
+                    if (upto > pos && own) acc.add(st, pos - w0, upto - w0, grp, zz, er);
                     pos = max(pos, upto);
                     if (cend > wend) break;   // the cell goes on in the next batch
                     // the cell is done
                     const int before = cl == 0 ? 0 : __shfl_sync(0xffffffffu, incl, cl * nsp - 1);
                     const bool last = cg + cl == cn - 1;
-                    T v[9], vj;
-                    acc.get(v, vj);
                     if (carry || cend > before) {
-                        if (lane < kMom3)
+                        if (own) {
+                            T* const o = smom[wib][grp] + zz * 81 + er * 3;
 #pragma unroll
-                            for (int e = 0; e < 9; ++e) smom[wib][lane * 9 + e] = v[e];
+                            for (int k = 0; k < 9; ++k)
+                                if (k < 6 || last)
+#pragma unroll
+                                    for (int e = 0; e < 3; ++e) o[k * 9 + e] = acc.moment(k, e);
+                            if (zz != 1)
+#pragma unroll
+                                for (int c = 0; c < 4; ++c) scur[wib][grp][(zz * 2 + c) * 3 + er] = acc.current(c);
+                        }
                         const int i = i0 + cg + cl;
                         const int64_t nd = node3(wrap1(i + (lane & 1), g.nx), wrap1(j + ((lane >> 1) & 1), g.ny),
                                                  wrap1(k + ((lane >> 2) & 1), g.nz), g);
                         if (lane < 8) snode[wib][lane] = nd;
                         __syncwarp();
                         const int nit = last ? kItems3 : kFace3;
+                        const T* sm = &smom[wib][0][0];
                         for (int it = lane; it < nit; it += 32) {
-                            const unsigned q = item[it];
-                            atomicAdd(M + snode[wib][q >> 16] * kMBlock3 + ((q >> 8) & 255u), smom[wib][q & 255u]);
+                            const unsigned q = item[it], v = q & 255u;
+                            atomicAdd(M + snode[wib][q >> 16] * kMBlock3 + ((q >> 8) & 255u),
+                                      sm[v] + sm[kMom3 * 9 + v] + sm[2 * kMom3 * 9 + v]);
                         }
+                        const int ja = lane / 3, jc = lane % 3;
                         if (lane < 24 && (last || (ja & 1) == 0))
-                            atomicAdd(J + (int64_t)jc * g.ncell + snode[wib][ja], vj);
+                            atomicAdd(J + (int64_t)jc * g.ncell + snode[wib][ja],
+                                      scur[wib][0][lane] + scur[wib][1][lane] + scur[wib][2][lane]);
                         __syncwarp();
                         carry = !last;
                     }
                     // the upper x face's sums start the next cell's lower face
-                    T n9[9];
-#pragma unroll
-                    for (int e = 0; e < 9; ++e) {
-                        const T up = __shfl_down_sync(0xffffffffu, v[e], 6);
-                        n9[e] = low && !last ? up : T(0);
-                    }
-                    const T upj = __shfl_down_sync(0xffffffffu, vj, 3);
-                    acc.start(n9, lane < 24 && (ja & 1) == 0 && !last ? upj : T(0));
+                    if (last) acc.clear();
+                    else acc.carry();
                     ++cl;
                     if (cl < gc0) cend = __shfl_sync(0xffffffffu, incl, cl * nsp + nsp - 1);
                 }
@@ -596,9 +640,153 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
 // the implicit operator, the right-hand side and the field update
 
 enum { k3A = 0, k3Residual = 1, k3Arnoldi = 2 };
-constexpr int kOpX3 = 32, kOpY3 = 4, kOpZ3 = 2;
-constexpr int kOpT3 = kOpX3 * kOpY3 * kOpZ3;
 constexpr int kOpChunk3 = 8;
+
+// the differences along each axis of three components at the 8 corners
+// f(comp, a, b, c) of a cube, averaged over its 4 edges, as a curl: a cell
+// from its nodes, or a node from the cells around it
+template <typename T, typename F>
+__device__ __forceinline__ void curl_cell3(F f, T rx, T ry, T rz, T (&C)[3])
+{
+    T d[3][3];   // d[axis][comp]
+#pragma unroll
+    for (int comp = 0; comp < 3; ++comp) {
+        T sx = T(0), sy = T(0), sz = T(0);
+#pragma unroll
+        for (int e1 = 0; e1 < 2; ++e1)
+#pragma unroll
+            for (int e2 = 0; e2 < 2; ++e2) {
+                sx += f(comp, 1, e1, e2) - f(comp, 0, e1, e2);
+                sy += f(comp, e1, 1, e2) - f(comp, e1, 0, e2);
+                sz += f(comp, e1, e2, 1) - f(comp, e1, e2, 0);
+            }
+        d[0][comp] = sx * rx;
+        d[1][comp] = sy * ry;
+        d[2][comp] = sz * rz;
+    }
+    C[0] = d[1][2] - d[2][1];
+    C[1] = d[2][0] - d[0][2];
+    C[2] = d[0][1] - d[1][0];
+}
+
+// The operator's tiles: 32 x 2 x 2 nodes (FP64: 32 x 2 x 1), one thread a
+// node. The tile's own mass-matrix rows (16 KB a row of 32 nodes in FP32) come
+// into shared memory by asynchronous copies, all in flight together, while
+// the input is staged; read straight from global memory (504 bytes from lane
+// to lane) every load of a block touched 32 lines, and the operator was bound
+// by their latency: 1.28 ms an application on 256x128x128 (FP32 form).
+template <typename T>
+struct Op3 {
+    static constexpr int X = 32, Y = 2, Z = sizeof(T) == 4 ? 2 : 1, threads = X * Y * Z;
+    struct Shared {
+        T Mm[Z * Y][X * kMBlock3];              // own blocks, row z Y + y
+        T v[3][Z + 2][Y + 2][X + 2];            // the input on the 1-node halo
+        T C[3][Z + 1][Y + 1][X + 1];            // its curl on the cells around the tile's nodes
+    };
+    static_assert(sizeof(Shared) >= sizeof(double) * kOpChunk3 * threads, "the dot products reuse it");
+};
+// a block's tile and this thread's node
+template <typename T>
+struct At3 {
+    int i0, j0, k0, tw, th, td, tx, ty, tz, i, j, k;
+    bool active;
+    int64_t gidx;
+    __device__ __forceinline__ explicit At3(const GridP& g)
+    {
+        using O = Op3<T>;
+        const int nx = (g.nx + O::X - 1) / O::X, ny = (g.ny + O::Y - 1) / O::Y;
+        const int bx = blockIdx.x % nx, by = (blockIdx.x / nx) % ny, bz = blockIdx.x / (nx * ny);
+        i0 = bx * O::X;
+        j0 = by * O::Y;
+        k0 = bz * O::Z;
+        tw = min(O::X, g.nx - i0);
+        th = min(O::Y, g.ny - j0);
+        td = min(O::Z, g.nz - k0);
+        tx = threadIdx.x % O::X;
+        ty = (threadIdx.x / O::X) % O::Y;
+        tz = threadIdx.x / (O::X * O::Y);
+        i = i0 + tx;
+        j = j0 + ty;
+        k = k0 + tz;
+        active = tx < tw && ty < th && tz < td;
+        gidx = active ? node3(i, j, k, g) : 0;
+    }
+};
+
+// start the copies of the tile's mass-matrix rows (16 bytes each where the
+// rows are aligned to that, else 8)
+template <typename T>
+__device__ __forceinline__ void fetch_rows3(typename Op3<T>::Shared& S, const T* __restrict__ M, const At3<T>& t,
+                                            const GridP& g)
+{
+    using O = Op3<T>;
+    const bool wide = ((int64_t)g.nx * kMBlock3 * sizeof(T)) % 16 == 0;
+    const int n = t.tw * kMBlock3 * (int)sizeof(T) / (wide ? 16 : 8);
+#pragma unroll
+    for (int r = 0; r < O::Y * O::Z; ++r) {
+        const int y = r % O::Y, z = r / O::Y;
+        if (y >= t.th || z >= t.td) continue;
+        const char* src = reinterpret_cast<const char*>(M + node3(t.i0, t.j0 + y, t.k0 + z, g) * kMBlock3);
+        char* dst = reinterpret_cast<char*>(&S.Mm[r][0]);
+        if (wide)
+            for (int q = threadIdx.x; q < n; q += O::threads) cp_async16(dst + 16 * q, src + 16 * q);
+        else
+            for (int q = threadIdx.x; q < n; q += O::threads) cp_async8(dst + 8 * q, src + 8 * q);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// the input (FP64) on the tile's halo in T, times s, and its curl on the
+// cells around the tile's nodes (each formed once); the rows' copies land
+template <typename T, bool SCALED>
+__device__ __forceinline__ void stage_input3(typename Op3<T>::Shared& S, const double* __restrict__ in, T s,
+                                             const At3<T>& t, const GridP& g)
+{
+    using O = Op3<T>;
+    constexpr int HX = O::X + 2, HY = O::Y + 2, HZ = O::Z + 2;
+    const int64_t nc = g.ncell;
+    const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
+    const int ga = wrap1(min(t.i0 - 1 + lane, 2 * g.nx - 1), g.nx), gb = wrap1(min(t.i0 + 31 + lane, 2 * g.nx - 1), g.nx);
+    // a warp a row of 34 (a lane a column, the last two by two lanes), four
+    // rows of loads in flight
+    constexpr int rows = 3 * HZ * HY, W = O::threads / 32;
+    for (int r0 = wid; r0 < rows; r0 += 4 * W) {
+        double a[4], b[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = min(r0 + v * W, rows - 1), comp = r / (HZ * HY), zz = (r / HY) % HZ, yy = r % HY;
+            const int gj = wrap1(min(t.j0 - 1 + yy, 2 * g.ny - 1), g.ny), gk = wrap1(min(t.k0 - 1 + zz, 2 * g.nz - 1), g.nz);
+            const double* row = in + comp * nc + node3(0, gj, gk, g);
+            a[v] = __ldg(row + ga);
+            b[v] = lane < 2 ? __ldg(row + gb) : 0.0;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = r0 + v * W;
+            if (r >= rows) break;
+            T* o = &S.v[0][0][0][0] + r * HX;
+            T x = narrow<T>(a[v]);
+            if (SCALED) x *= s;
+            o[lane] = x;
+            if (lane < 2) {
+                T y = narrow<T>(b[v]);
+                if (SCALED) y *= s;
+                o[32 + lane] = y;
+            }
+        }
+    }
+    __syncthreads();
+    const T rx = gc<T>(g).qdx, ry = gc<T>(g).qdy, rz = gc<T>(g).qdz;
+    for (int q = threadIdx.x; q < (O::Z + 1) * (O::Y + 1) * (O::X + 1); q += O::threads) {
+        const int c = q % (O::X + 1), y = (q / (O::X + 1)) % (O::Y + 1), z = q / ((O::X + 1) * (O::Y + 1));
+        T C[3];
+        curl_cell3<T>([&](int comp, int p, int o, int w) { return S.v[comp][z + w][y + o][c + p]; }, rx, ry, rz, C);
+#pragma unroll
+        for (int comp = 0; comp < 3; ++comp) S.C[comp][z][y][c] = C[comp];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+}
 
 // the offset of stored block h (0..13)
 __device__ __forceinline__ void half_offset3(int h, int& di, int& dj, int& dk)
@@ -608,105 +796,105 @@ __device__ __forceinline__ void half_offset3(int h, int& di, int& dj, int& dk)
     else { di = (h - 5) % 3 - 1; dj = (h - 5) / 3 - 1; dk = 1; }
 }
 
-// (curl_n curl_c v) at a node from v on its 3x3x3 neighbourhood,
-// f(comp, a, b, c) = component comp at node (i-1+a, j-1+b, k-1+c)
-template <typename T, typename F>
-__device__ __forceinline__ void curlcurl3(F f, T rdx4, T rdy4, T rdz4, T (&out)[3])
+// a stored block (9 values; even: the row starts on a pair of T) in registers
+__device__ __forceinline__ void block3(const float* p, int h, float (&m)[9])
 {
-    // curl_c at the 8 cells around the node: cell (ci, cj, ck) spans local
-    // nodes ci..ci+1, cj..cj+1, ck..ck+1 (ci = 0: the cell i-1)
-    T C[3][2][2][2];
+    if (h & 1) {
+        m[0] = p[0];
 #pragma unroll
-    for (int ci = 0; ci < 2; ++ci)
+        for (int e = 0; e < 4; ++e) {
+            const float2 q = *reinterpret_cast<const float2*>(p + 1 + 2 * e);
+            m[1 + 2 * e] = q.x;
+            m[2 + 2 * e] = q.y;
+        }
+    } else {
 #pragma unroll
-        for (int cj = 0; cj < 2; ++cj)
-#pragma unroll
-            for (int ck = 0; ck < 2; ++ck) {
-                T d[3][3];   // d[axis][comp]
-#pragma unroll
-                for (int comp = 0; comp < 3; ++comp) {
-                    T sx = T(0), sy = T(0), sz = T(0);
-#pragma unroll
-                    for (int e1 = 0; e1 < 2; ++e1)
-#pragma unroll
-                        for (int e2 = 0; e2 < 2; ++e2) {
-                            sx += f(comp, ci + 1, cj + e1, ck + e2) - f(comp, ci, cj + e1, ck + e2);
-                            sy += f(comp, ci + e1, cj + 1, ck + e2) - f(comp, ci + e1, cj, ck + e2);
-                            sz += f(comp, ci + e1, cj + e2, ck + 1) - f(comp, ci + e1, cj + e2, ck);
-                        }
-                    d[0][comp] = sx * rdx4;
-                    d[1][comp] = sy * rdy4;
-                    d[2][comp] = sz * rdz4;
-                }
-                C[0][ci][cj][ck] = d[1][2] - d[2][1];
-                C[1][ci][cj][ck] = d[2][0] - d[0][2];
-                C[2][ci][cj][ck] = d[0][1] - d[1][0];
-            }
-    // curl_n at the node from the 8 cells
-    T d[3][3];
-#pragma unroll
-    for (int comp = 0; comp < 3; ++comp) {
-        T sx = T(0), sy = T(0), sz = T(0);
-#pragma unroll
-        for (int e1 = 0; e1 < 2; ++e1)
-#pragma unroll
-            for (int e2 = 0; e2 < 2; ++e2) {
-                sx += C[comp][1][e1][e2] - C[comp][0][e1][e2];
-                sy += C[comp][e1][1][e2] - C[comp][e1][0][e2];
-                sz += C[comp][e1][e2][1] - C[comp][e1][e2][0];
-            }
-        d[0][comp] = sx * rdx4;
-        d[1][comp] = sy * rdy4;
-        d[2][comp] = sz * rdz4;
+        for (int e = 0; e < 4; ++e) {
+            const float2 q = *reinterpret_cast<const float2*>(p + 2 * e);
+            m[2 * e] = q.x;
+            m[2 * e + 1] = q.y;
+        }
+        m[8] = p[8];
     }
-    out[0] = d[1][2] - d[2][1];
-    out[1] = d[2][0] - d[0][2];
-    out[2] = d[0][1] - d[1][0];
+}
+__device__ __forceinline__ void block3(const double* p, int, double (&m)[9])
+{
+#pragma unroll
+    for (int e = 0; e < 9; ++e) m[e] = p[e];
 }
 
-// (M v) at node (i, j, k): its own 14 stored blocks times v at g + d(h), and
-// the 13 neighbours' blocks M[g - d(h)][h] times v at g - d(h); with TR each
-// block applied transposed
-template <typename T, bool TR, typename F>
-__device__ __forceinline__ void mv3(const T* __restrict__ M, int i, int j, int k, const GridP& g, F f, T (&out)[3])
+// (M v) at the thread's node: its own 14 stored blocks times v at g + d(h),
+// and the 13 neighbours' blocks M[g - d(h)][h] times v at g - d(h) (from the
+// tile where they lie in it, else from global memory); with TR each block
+// applied transposed
+template <typename T, bool TR>
+__device__ __forceinline__ void mv3(const typename Op3<T>::Shared& S, const T* __restrict__ M, const At3<T>& t,
+                                    const GridP& g, T (&out)[3])
 {
+    using O = Op3<T>;
     T r[3] = {T(0), T(0), T(0)};
-    const T* Mg = M + node3(i, j, k, g) * kMBlock3;
+    const T* Mg = &S.Mm[t.tz * O::Y + t.ty][t.tx * kMBlock3];
+    auto add = [&](const T (&m)[9], int di, int dj, int dk) {
+        T vv[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) vv[s] = S.v[s][t.tz + 1 + dk][t.ty + 1 + dj][t.tx + 1 + di];
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr)
+#pragma unroll
+            for (int s = 0; s < 3; ++s) r[rr] += m[TR ? s * 3 + rr : rr * 3 + s] * vv[s];
+    };
+    auto neighbour = [&](int h, T (&m)[9]) {
+        int di, dj, dk;
+        half_offset3(h, di, dj, dk);
+        const int x = t.tx - di, y = t.ty - dj, z = t.tz - dk;
+        const T* Mn = x >= 0 && x < t.tw && y >= 0 && y < t.th && z >= 0
+                          ? &S.Mm[z * O::Y + y][x * kMBlock3]
+                          : M + node3(wrap1(t.i - di, g.nx), wrap1(t.j - dj, g.ny), wrap1(t.k - dk, g.nz), g) * kMBlock3;
+        block3(Mn + h * 9, h, m);
+    };
+    // the neighbours' blocks three at a time (h = 2..4, 5..7, 8..10, 11..13),
+    // each three on their way while the blocks before them are added
+    T nb[2][3][9];
+#pragma unroll
+    for (int q = 0; q < 3; ++q) neighbour(2 + q, nb[0][q]);
 #pragma unroll
     for (int h = 0; h < kHalf3; ++h) {
         int di, dj, dk;
         half_offset3(h, di, dj, dk);
-        const T* Mo = Mg + h * 9;
-        T vv[3];
+        T m[9];
+        block3(Mg + h * 9, h, m);
+        add(m, di, dj, dk);
+    }
 #pragma unroll
-        for (int s = 0; s < 3; ++s) vv[s] = f(s, 1 + di, 1 + dj, 1 + dk);
+    for (int n = 0; n < 4; ++n) {
 #pragma unroll
-        for (int rr = 0; rr < 3; ++rr)
+        for (int q = 0; q < 3; ++q)
+            if (n < 3) neighbour(2 + 3 * (n + 1) + q, nb[(n + 1) & 1][q]);
 #pragma unroll
-            for (int s = 0; s < 3; ++s) r[rr] += ld(Mo + (TR ? s * 3 + rr : rr * 3 + s)) * vv[s];
-        if (h == 0) continue;
-        const T* Mn = M + node3(wrap1(i - di, g.nx), wrap1(j - dj, g.ny), wrap1(k - dk, g.nz), g) * kMBlock3 + h * 9;
-#pragma unroll
-        for (int s = 0; s < 3; ++s) vv[s] = f(s, 1 - di, 1 - dj, 1 - dk);
-#pragma unroll
-        for (int rr = 0; rr < 3; ++rr)
-#pragma unroll
-            for (int s = 0; s < 3; ++s) r[rr] += ld(Mn + (TR ? s * 3 + rr : rr * 3 + s)) * vv[s];
+        for (int q = 0; q < 3; ++q) {
+            int di, dj, dk;
+            half_offset3(2 + 3 * n + q, di, dj, dk);
+            add(nb[n & 1][q], -di, -dj, -dk);
+        }
+    }
+    {
+        T m[9];
+        neighbour(1, m);
+        add(m, -1, 0, 0);
     }
     out[0] = r[0];
     out[1] = r[1];
     out[2] = r[2];
 }
 
-// The operator on tiles of 32 x 4 x 2 nodes, the input staged in T on the
-// tile's 1-node halo (one FP64 load and conversion per staged value); the
-// modes and the per-block partial sums are those of the 2D operator:
+// The operator; the modes and the per-block partial sums are those of the 2D
+// operator:
 //   A:        out = in + B in
 //   Residual: out = b - (in + B in), partial |out|^2
 //   Arnoldi:  v = s in (to vj when vj is not null), out = B v, partials
 //             <out, V_q> (q < nv), <out, v>, <out, out>
 template <typename T, int MODE, bool TR>
-__global__ void __launch_bounds__(kOpT3)
+__global__ void __launch_bounds__(Op3<T>::threads, 3)
 k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const double* __restrict__ b,
       double* __restrict__ out, double* __restrict__ vj, const double* __restrict__ V, int64_t ldv, int nv, GridP g,
       double* __restrict__ partial, const GmDyn* __restrict__ dyn)
@@ -719,76 +907,66 @@ k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const do
         out = dyn->out;
         nv = dyn->nv;
     }
-    constexpr int HX = kOpX3 + 2, HY = kOpY3 + 2, HZ = kOpZ3 + 2;
-    __shared__ T sv[3][HZ][HY][HX];
-    __shared__ double buf[kOpChunk3][kOpT3];
-    const int nx = g.nx, ny = g.ny, nz = g.nz;
+    using O = Op3<T>;
+    extern __shared__ __align__(128) unsigned char op3_smem[];
+    typename O::Shared& S = *reinterpret_cast<typename O::Shared*>(op3_smem);
+    const At3<T> t(g);
     const int64_t nc = g.ncell;
-    const int tx_n = (nx + kOpX3 - 1) / kOpX3, ty_n = (ny + kOpY3 - 1) / kOpY3;
-    const int bx = blockIdx.x % tx_n, by = (blockIdx.x / tx_n) % ty_n, bz = blockIdx.x / (tx_n * ty_n);
-    const int i0 = bx * kOpX3, j0 = by * kOpY3, k0 = bz * kOpZ3;
-    const int tid = threadIdx.x, tx = tid % kOpX3, ty = (tid / kOpX3) % kOpY3, tz = tid / (kOpX3 * kOpY3);
-    const int i = i0 + tx, j = j0 + ty, k = k0 + tz;
-    const bool active = i < nx && j < ny && k < nz;
-    const int64_t gidx = active ? node3(i, j, k, g) : 0;
-    const T sT = (T)s;
-    for (int q = tid; q < 3 * HZ * HY * HX; q += kOpT3) {
-        const int comp = q / (HZ * HY * HX), rem = q % (HZ * HY * HX);
-        const int zz = rem / (HY * HX), yy = (rem / HX) % HY, xx = rem % HX;
-        const int gi = wrap1(min(i0 - 1 + xx, 2 * nx - 1), nx), gj = wrap1(min(j0 - 1 + yy, 2 * ny - 1), ny);
-        const int gk = wrap1(min(k0 - 1 + zz, 2 * nz - 1), nz);
-        T val = (T)__ldg(in + comp * nc + node3(gi, gj, gk, g));
-        if (MODE == k3Arnoldi) val *= sT;
-        sv[comp][zz][yy][xx] = val;
-    }
-    __syncthreads();
+    const int tid = threadIdx.x;
+    fetch_rows3<T>(S, M, t, g);
     double own[3] = {0.0, 0.0, 0.0}, wv[3] = {0.0, 0.0, 0.0};
-    if (active) {
+    if (t.active) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            own[c] = __ldg(in + c * nc + gidx);
+            own[c] = __ldg(in + c * nc + t.gidx);
             if (MODE == k3Arnoldi && !is_one(s)) own[c] *= s;
         }
-        auto f = [&](int comp, int a, int bb, int cc) -> T { return sv[comp][tz + cc][ty + bb][tx + a]; };
+    }
+    if (MODE == k3Arnoldi) stage_input3<T, true>(S, in, (T)s, t, g);
+    else stage_input3<T, false>(S, in, T(1), t, g);
+    if (t.active) {
         T cc3[3], mv[3];
-        curlcurl3<T>(f, gc<T>(g).qdx, gc<T>(g).qdy, gc<T>(g).qdz, cc3);
-        mv3<T, TR>(M, i, j, k, g, f, mv);
+        curl_cell3<T>([&](int comp, int p, int o, int w) { return S.C[comp][t.tz + w][t.ty + o][t.tx + p]; },
+                      gc<T>(g).qdx, gc<T>(g).qdy, gc<T>(g).qdz, cc3);
+        mv3<T, TR>(S, M, t, g, mv);
         const T td = gc<T>(g).td;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double bv = (double)(td * td * cc3[c] + td * mv[c]);
+            const double bv = widen(td * td * cc3[c] + td * mv[c]);
             if (MODE == k3A) wv[c] = own[c] + bv;
-            else if (MODE == k3Residual) wv[c] = b[c * nc + gidx] - (own[c] + bv);
+            else if (MODE == k3Residual) wv[c] = b[c * nc + t.gidx] - (own[c] + bv);
             else wv[c] = bv;
-            out[c * nc + gidx] = wv[c];
-            if (MODE == k3Arnoldi && vj) vj[c * nc + gidx] = own[c];
+            out[c * nc + t.gidx] = wv[c];
+            if (MODE == k3Arnoldi && vj) vj[c * nc + t.gidx] = own[c];
         }
     }
     if (MODE == k3A) return;
     const int nq = MODE == k3Residual ? 1 : nv + 2;
     const int lane = tid & 31, wid = tid >> 5;
+    double* buf = reinterpret_cast<double*>(op3_smem);   // [kOpChunk3][threads]
+    __syncthreads();   // the tile is no longer read
     for (int q0 = 0; q0 < nq; q0 += kOpChunk3) {
         const int kc = min(kOpChunk3, nq - q0);
         for (int c = 0; c < kc; ++c) {
             const int q = q0 + c;
             double d = 0.0;
-            if (active) {
+            if (t.active) {
                 if (MODE == k3Residual || q == nv + 1) d = wv[0] * wv[0] + wv[1] * wv[1] + wv[2] * wv[2];
                 else if (q == nv) d = wv[0] * own[0] + wv[1] * own[1] + wv[2] * own[2];
                 else {
-                    const double* Vq = V + (int64_t)q * ldv + gidx;
+                    const double* Vq = V + (int64_t)q * ldv + t.gidx;
                     d = wv[0] * __ldg(Vq) + wv[1] * __ldg(Vq + nc) + wv[2] * __ldg(Vq + 2 * nc);
                 }
             }
-            buf[c][tid] = d;
+            buf[c * O::threads + tid] = d;
         }
         __syncthreads();
-        for (int c = wid; c < kc; c += kOpT3 / 32) {
-            double t = 0.0;
+        for (int c = wid; c < kc; c += O::threads / 32) {
+            double sum = 0.0;
 #pragma unroll
-            for (int m = 0; m < kOpT3 / 32; ++m) t += buf[c][m * 32 + lane];
-            t = warp_sum(t);
-            if (lane == 0) partial[(int64_t)blockIdx.x * nq + q0 + c] = t;
+            for (int m = 0; m < O::threads / 32; ++m) sum += buf[c * O::threads + m * 32 + lane];
+            sum = warp_sum(sum);
+            if (lane == 0) partial[(int64_t)blockIdx.x * nq + q0 + c] = sum;
         }
         __syncthreads();
     }
@@ -831,95 +1009,59 @@ __global__ void k_rhs3(const T* __restrict__ E, const T* __restrict__ B, const T
 constexpr int kFieldLedger3 = 6;
 
 // E^{n+theta} (FP64 solution) -> Eth, E^{n+1}, B^{n+1} of cell (i,j,k) and the
-// field ledger terms 0..4 (as the 2D field update); term 5 (the work) by
-// k_work3 from Eth in T
+// field ledger terms, on the operator's tiles: the solution is staged in T
+// once for the curl, the work and the update (as two kernels it was converted
+// at every one of a node's 24 uses, on the FP64 pipe, and M was read from
+// global memory: 1.7 ms on 256x128x128, FP32 form). Term 5 is the work
+// dt dV (Jhat + M E^{n+theta}) . E^{n+theta}.
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_field_update3(const double* __restrict__ x, T* __restrict__ Eth, T* __restrict__ E, const T* __restrict__ B0,
-                T* __restrict__ B1, GridP g, double* __restrict__ partial)
+__global__ void __launch_bounds__(Op3<T>::threads, 3)
+k_field_update3(const double* __restrict__ x, const T* __restrict__ M, const T* __restrict__ J, T* __restrict__ Eth,
+                T* __restrict__ E, const T* __restrict__ B0, T* __restrict__ B1, GridP g, double* __restrict__ partial)
 {
-    __shared__ double red[32 * 5];
+    using O = Op3<T>;
+    extern __shared__ __align__(128) unsigned char op3_smem[];
+    typename O::Shared& S = *reinterpret_cast<typename O::Shared*>(op3_smem);
+    const At3<T> t(g);
     const int64_t nc = g.ncell;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if (gidx < nc) {
-        const int i = (int)(gidx % g.nx), j = (int)((gidx / g.nx) % g.ny), k = (int)(gidx / ((int64_t)g.nx * g.ny));
-        const T th = gc<T>(g).theta, hdV = gc<T>(g).hdV;
+    fetch_rows3<T>(S, M, t, g);
+    stage_input3<T, false>(S, x, T(1), t, g);
+    T acc[kFieldLedger3] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    if (t.active) {
+        const T th = gc<T>(g).theta, hdV = gc<T>(g).hdV, dt = gc<T>(g).dt;
+        T mv[3], wk = T(0);
+        mv3<T, false>(S, M, t, g, mv);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const T et = (T)x[c * nc + gidx];
-            const T e0 = E[c * nc + gidx];
+            const T et = S.v[c][t.tz + 1][t.ty + 1][t.tx + 1];
+            const T e0 = E[c * nc + t.gidx];
             const T e1 = (et - (T(1) - th) * e0) / th;
-            Eth[c * nc + gidx] = et;
-            E[c * nc + gidx] = e1;
+            Eth[c * nc + t.gidx] = et;
+            E[c * nc + t.gidx] = e1;
             acc[0] += hdV * (e1 - e0) * (e1 + e0);
             acc[2] += (e1 - e0) * (e1 - e0);
             acc[3] += hdV * e1 * e1;
-        }
-        const int ii[2] = {i, wrap1(i + 1, g.nx)}, jj[2] = {j, wrap1(j + 1, g.ny)}, kk[2] = {k, wrap1(k + 1, g.nz)};
-        T d[3][3];
-#pragma unroll
-        for (int comp = 0; comp < 3; ++comp) {
-            T sx = T(0), sy = T(0), sz = T(0);
-#pragma unroll
-            for (int e1 = 0; e1 < 2; ++e1)
-#pragma unroll
-                for (int e2 = 0; e2 < 2; ++e2) {
-                    sx += (T)x[comp * nc + node3(ii[1], jj[e1], kk[e2], g)] - (T)x[comp * nc + node3(ii[0], jj[e1], kk[e2], g)];
-                    sy += (T)x[comp * nc + node3(ii[e1], jj[1], kk[e2], g)] - (T)x[comp * nc + node3(ii[e1], jj[0], kk[e2], g)];
-                    sz += (T)x[comp * nc + node3(ii[e1], jj[e2], kk[1], g)] - (T)x[comp * nc + node3(ii[e1], jj[e2], kk[0], g)];
-                }
-            d[0][comp] = sx * gc<T>(g).qdx;
-            d[1][comp] = sy * gc<T>(g).qdy;
-            d[2][comp] = sz * gc<T>(g).qdz;
-        }
-        const T curl[3] = {d[1][2] - d[2][1], d[2][0] - d[0][2], d[0][1] - d[1][0]};
-        const T dt = gc<T>(g).dt;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const T b0 = B0[c * nc + gidx];
-            const T b1 = b0 - dt * curl[c];
-            B1[c * nc + gidx] = b1;
+            wk += (J[c * nc + t.gidx] + mv[c]) * et;
+            // the cell's upper nodes: its curl is the one after the node's in x, y and z
+            const T b0 = B0[c * nc + t.gidx];
+            const T b1 = b0 - dt * S.C[c][t.tz + 1][t.ty + 1][t.tx + 1];
+            B1[c * nc + t.gidx] = b1;
             acc[1] += hdV * (b1 - b0) * (b1 + b0);
             acc[2] += (b1 - b0) * (b1 - b0);
             acc[4] += hdV * b1 * b1;
         }
         acc[2] *= gc<T>(g).thdV;
+        acc[5] = gc<T>(g).dtdV * wk;
     }
-    double v[5], o[5];
+    double* red = reinterpret_cast<double*>(op3_smem);
+    __syncthreads();   // the tile is no longer read
+    double v[kFieldLedger3], o[kFieldLedger3];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) v[q] = (double)acc[q];
-    block_sum<5>(v, red, o);
+    for (int q = 0; q < kFieldLedger3; ++q) v[q] = (double)acc[q];
+    block_sum<kFieldLedger3>(v, red, o);
     if (threadIdx.x == 0)
 #pragma unroll
-        for (int q = 0; q < 5; ++q) partial[(int64_t)blockIdx.x * kFieldLedger3 + q] = o[q];
-}
-
-// ledger term 5: dt dV (Jhat + M E^{n+theta}) . E^{n+theta}, with the same
-// blocks as k_field_update3
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_work3(const T* __restrict__ M, const T* __restrict__ J, const T* __restrict__ Eth, GridP g,
-        double* __restrict__ partial)
-{
-    __shared__ double red[32];
-    const int64_t nc = g.ncell;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    T wk = T(0);
-    if (gidx < nc) {
-        const int i = (int)(gidx % g.nx), j = (int)((gidx / g.nx) % g.ny), k = (int)(gidx / ((int64_t)g.nx * g.ny));
-        auto f = [&](int comp, int a, int b, int c) -> T {
-            return ld(Eth + comp * nc + node3(wrap1(i - 1 + a, g.nx), wrap1(j - 1 + b, g.ny), wrap1(k - 1 + c, g.nz), g));
-        };
-        T mv[3];
-        mv3<T, false>(M, i, j, k, g, f, mv);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) wk += (J[c * nc + gidx] + mv[c]) * Eth[c * nc + gidx];
-        wk *= gc<T>(g).dtdV;
-    }
-    double v[1] = {(double)wk}, o[1];
-    block_sum<1>(v, red, o);
-    if (threadIdx.x == 0) partial[(int64_t)blockIdx.x * kFieldLedger3 + 5] = o[0];
+        for (int q = 0; q < kFieldLedger3; ++q) partial[(int64_t)blockIdx.x * kFieldLedger3 + q] = o[q];
 }
 
 // ---------------------------------------------------------------------------
@@ -1099,22 +1241,19 @@ k_place3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restric
         }
 #pragma unroll
         for (int v = 0; v < U; ++v) q[v] = (int64_t)ld(start + kk[v]) + rr[v];
-        // one array at a time: its U loads in flight, then its stores
-        auto move = [&](const T* a, T* o) {
-            T x[U];
+        // (plain loads: read-only ones the compiler moves past the stores)
+        const T* const in[7] = {src.fx, src.fy, sfz, src.ux, src.uy, src.uz, src.w};
+        T* const out[7] = {dst.fx, dst.fy, dfz, dst.ux, dst.uy, dst.uz, dst.w};
+        T x[7][U];
 #pragma unroll
-            for (int v = 0; v < U; ++v) x[v] = p[v] >= 0 ? ld(a + p[v]) : T(0);
+        for (int a = 0; a < 7; ++a)
+#pragma unroll
+            for (int v = 0; v < U; ++v) x[a][v] = p[v] >= 0 && in[a] ? in[a][p[v]] : T(0);
+#pragma unroll
+        for (int a = 0; a < 7; ++a)
 #pragma unroll
             for (int v = 0; v < U; ++v)
-                if (p[v] >= 0) o[q[v]] = x[v];
-        };
-        move(src.fx, dst.fx);
-        move(src.fy, dst.fy);
-        if (dfz) move(sfz, dfz);   // null for 2D particles
-        move(src.ux, dst.ux);
-        move(src.uy, dst.uy);
-        move(src.uz, dst.uz);
-        move(src.w, dst.w);
+                if (p[v] >= 0 && out[a]) out[a][q[v]] = x[a][v];   // (no third offset for 2D particles)
         if (dst.id)
 #pragma unroll
             for (int v = 0; v < U; ++v)
@@ -1174,18 +1313,24 @@ cudaError_t deposit3(const DepositSpecies<T>& ds, const FzArrays<T>& fz, const T
     return cudaGetLastError();
 }
 
-int op_blocks3(GridP g)
+template <typename T>
+static int tiles3(const GridP& g)
 {
-    return ((g.nx + kOpX3 - 1) / kOpX3) * ((g.ny + kOpY3 - 1) / kOpY3) * ((g.nz + kOpZ3 - 1) / kOpZ3);
+    using O = Op3<T>;
+    return ((g.nx + O::X - 1) / O::X) * ((g.ny + O::Y - 1) / O::Y) * ((g.nz + O::Z - 1) / O::Z);
 }
+int op_blocks3(GridP g, int precision) { return precision == 32 ? tiles3<float>(g) : tiles3<double>(g); }
 
 template <typename T, int MODE, bool TR>
 cudaError_t launch_op3(const T* M, const double* in, double sc, const double* b, double* out, double* vj,
                        const double* V, int64_t ldv, int nv, GridP g, double* partial, cudaStream_t st,
                        const GmDyn* dyn)
 {
+    const int smem = (int)sizeof(typename Op3<T>::Shared);
+    const cudaError_t e = cudaFuncSetAttribute(k_op3<T, MODE, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
     count_launches(1);
-    k_op3<T, MODE, TR><<<op_blocks3(g), kOpT3, 0, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial, dyn);
+    k_op3<T, MODE, TR><<<tiles3<T>(g), Op3<T>::threads, smem, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial, dyn);
     return cudaGetLastError();
 }
 
@@ -1201,9 +1346,11 @@ template <typename T>
 cudaError_t field_update3(const double* x, const T* M, const T* J, T* Eth, T* E, const T* B0, T* B1, GridP g,
                           double* partial, int nblocks, cudaStream_t st)
 {
-    count_launches(2);
-    k_field_update3<T><<<nblocks, 256, 0, st>>>(x, Eth, E, B0, B1, g, partial);
-    k_work3<T><<<nblocks, 256, 0, st>>>(M, J, Eth, g, partial);
+    const int smem = (int)sizeof(typename Op3<T>::Shared);
+    const cudaError_t e = cudaFuncSetAttribute(k_field_update3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
+    k_field_update3<T><<<nblocks, Op3<T>::threads, smem, st>>>(x, M, J, Eth, E, B0, B1, g, partial);
     return cudaGetLastError();
 }
 

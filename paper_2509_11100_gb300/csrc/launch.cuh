@@ -132,7 +132,7 @@ cudaError_t export_particles3(PArrays<T> p, const T* fz, const int32_t* start, G
 template <typename T>
 cudaError_t deposit3(const DepositSpecies<T>& ds, const FzArrays<T>& fz, const T* B, T* M, T* J, GridP g,
                      cudaStream_t st, int blocks = 0);   // blocks 0: at most 8 per SM
-int op_blocks3(GridP g);
+int op_blocks3(GridP g, int precision);
 template <typename T, int MODE, bool TR>
 cudaError_t launch_op3(const T* M, const double* in, double sc, const double* b, double* out, double* vj,
                        const double* V, int64_t ldv, int nv, GridP g, double* partial, cudaStream_t st,
@@ -305,7 +305,7 @@ cudaError_t mass_to_double(const T* M, const T* J, double* Md, double* Jd, GridP
 template <typename T>
 cudaError_t mass_from_double(const double* Md, const double* Jd, T* M, T* J, GridP g, int* bad,
                              cudaStream_t st);
-int field_grid_blocks(GridP g);
+int field_grid_blocks(GridP g, int precision);
 
 // GMRES vector kernels: FP64 vectors, or double-float ones when df (the
 // sums and dot products then come out in FP64 per block)

@@ -14,10 +14,9 @@
 //   k_deposit_q   warp per row segment of cells, the segment's B staged in
 //                 shared memory; per cell the particles of all species staged
 //                 in four groups by the half of the cell they sit in (each
-//                 group touches a fixed 3 x 3 of the cell's 4 x 4 nodes); per
-//                 group each lane sums up to 2 of the 45 node pairs of 3 x 3
-//                 nodes with paired FP32 FMAs and adds them to the cell's 106
-//                 pair sums in shared memory, flushed once per cell
+//                 group touches a fixed 3 x 3 of the cell's 4 x 4 nodes), the
+//                 lanes sum the groups' 36 weight products; a ring of four
+//                 node columns in shared memory collects the cells' sums
 //   k_op_q        the operator on 32 x 8-node tiles, the input staged on a
 //                 2-node halo, the 25 blocks per node from global memory, the
 //                 modes and partial dot products of the other operators
@@ -64,37 +63,21 @@ __device__ __forceinline__ void quad3(T d, T (&w)[3])
     w[2] = T(0.5) * b * b;
 }
 
-// the weights on the 4 nodes i-1 .. i+2 of the axis (one of them zero)
-template <typename T>
-__device__ __forceinline__ void node4(T f, T (&w4)[4])
-{
-    T w[3];
-    const bool hi = f >= T(0.5);
-    quad3(hi ? f - T(1) : f, w);
-    w4[0] = hi ? T(0) : w[0];
-    w4[1] = hi ? w[0] : w[1];
-    w4[2] = hi ? w[1] : w[2];
-    w4[3] = hi ? w[2] : T(0);
-}
-
 // field tiles of a row segment (cells i0 .. i0+cn-1 of row j)
 template <typename T>
-struct TileQ {
-    T E[3][4][kQX + 3];   // node (i0 - 1 + c, j - 1 + r)
+struct TileBq {
     T B[3][3][kQX + 2];   // centre (i0 - 1 + c, j - 1 + r)
+};
+template <typename T>
+struct TileQ : TileBq<T> {
+    T E[3][4][kQX + 3];   // node (i0 - 1 + c, j - 1 + r)
 };
 
 template <typename T>
-__device__ __forceinline__ void load_tileq(TileQ<T>& tl, const T* __restrict__ E, const T* __restrict__ B, int i0,
-                                           int cn, int j, const GridP& g, int lane)
+__device__ __forceinline__ void load_tileBq(TileBq<T>& tl, const T* __restrict__ B, int i0, int cn, int j,
+                                            const GridP& g, int lane)
 {
     const int nc = g.ncell;
-    if (E)
-        for (int q = lane; q < 3 * 4 * (kQX + 3); q += 32) {
-            const int c = q % (kQX + 3), r = (q / (kQX + 3)) % 4, comp = q / (4 * (kQX + 3));
-            if (c <= cn + 2)
-                tl.E[comp][r][c] = ld(E + comp * nc + wrap1(j - 1 + r, g.ny) * g.nx + wrap1(i0 - 1 + c, g.nx));
-        }
     for (int q = lane; q < 3 * 3 * (kQX + 2); q += 32) {
         const int c = q % (kQX + 2), r = (q / (kQX + 2)) % 3, comp = q / (3 * (kQX + 2));
         if (c <= cn + 1)
@@ -103,10 +86,23 @@ __device__ __forceinline__ void load_tileq(TileQ<T>& tl, const T* __restrict__ E
     __syncwarp();
 }
 
+template <typename T>
+__device__ __forceinline__ void load_tileq(TileQ<T>& tl, const T* __restrict__ E, const T* __restrict__ B, int i0,
+                                           int cn, int j, const GridP& g, int lane)
+{
+    const int nc = g.ncell;
+    for (int q = lane; q < 3 * 4 * (kQX + 3); q += 32) {
+            const int c = q % (kQX + 3), r = (q / (kQX + 3)) % 4, comp = q / (4 * (kQX + 3));
+            if (c <= cn + 2)
+                tl.E[comp][r][c] = ld(E + comp * nc + wrap1(j - 1 + r, g.ny) * g.nx + wrap1(i0 - 1 + c, g.nx));
+        }
+    load_tileBq<T>(tl, B, i0, cn, j, g, lane);
+}
+
 // B^n at a particle of local cell cl: centres cl-1 .. cl+1 (tile columns
 // cl .. cl+2), rows j-1 .. j+1
 template <typename T>
-__device__ __forceinline__ void tile_Bq(const TileQ<T>& tl, int cl, T fx, T fy, T (&Bp)[3])
+__device__ __forceinline__ void tile_Bq(const T (&B)[3][3][kQX + 2], int cl, T fx, T fy, T (&Bp)[3])
 {
     T wx[3], wy[3];
     quad3(fx - T(0.5), wx);
@@ -115,17 +111,20 @@ __device__ __forceinline__ void tile_Bq(const TileQ<T>& tl, int cl, T fx, T fy, 
     for (int comp = 0; comp < 3; ++comp) {
         T b = T(0);
 #pragma unroll
-        for (int r = 0; r < 3; ++r)
+        for (int r = 0; r < 3; ++r) {
+            T br = T(0);
 #pragma unroll
-            for (int c = 0; c < 3; ++c) b += wy[r] * wx[c] * tl.B[comp][r][cl + c];
+            for (int c = 0; c < 3; ++c) br += wx[c] * B[comp][r][cl + c];
+            b += wy[r] * br;
+        }
         Bp[comp] = b;
     }
 }
 
 template <typename T>
-__device__ __forceinline__ void alphaq(const T (&Bp)[3], T beta, T gbar, T (&al)[9])
+__device__ __forceinline__ void alphaq(const T (&Bp)[3], T bg, T (&al)[9])   // bg = beta/gbar
 {
-    const T ax = beta * Bp[0] / gbar, ay = beta * Bp[1] / gbar, az = beta * Bp[2] / gbar;
+    const T ax = bg * Bp[0], ay = bg * Bp[1], az = bg * Bp[2];
     const T ia = T(1) / (T(1) + ax * ax + ay * ay + az * az);
     al[0] = (T(1) + ax * ax) * ia; al[1] = (ax * ay + az) * ia; al[2] = (ax * az - ay) * ia;
     al[3] = (ax * ay - az) * ia; al[4] = (T(1) + ay * ay) * ia; al[5] = (ay * az + ax) * ia;
@@ -135,312 +134,303 @@ __device__ __forceinline__ void alphaq(const T (&Bp)[3], T beta, T gbar, T (&al)
 // ---------------------------------------------------------------------------
 // deposit
 
-constexpr int kPairsQ = 106;  // node pairs of the 4 x 4 union at most two apart per axis
-
+// A warp takes a row segment of cells; a cell's particles are staged 32 at a
+// time, grouped by the half of the cell they sit in along x and y (hx, hy):
+// a group touches the same 3 x 3 frame of the cell's 4 x 4 nodes. Along an
+// axis the frame's node pairs have six weight products, so a particle adds
+// c alpha_e to 36 products; 27 lanes each sum 2 x 2 of them for one row of
+// alpha (4 products x 3 entries, two particles per paired FP32 FMA), per
+// group in registers over the cell. A cell's sums then go to the union's
+// products in shared memory, held by the column of their left node in a ring
+// of four columns: the next cell's union is this one's moved by a column, so
+// only the column that falls out is added to M, its 37 blocks in address
+// order (the sums of the others grow on).
+//
+// Bound by issue. Before, each lane owned node pairs (45 a group, 106 a
+// cell), a group's sums went through shared memory every 32 particles and
+// all 106 blocks of every cell went to M: 81 warp instructions a particle,
+// 1.85 ms on 512x256 with 128 particles a cell (FP32 form).
 template <typename T>
 struct DepCfgQ {
-    static constexpr int warps = sizeof(T) == 4 ? 4 : 2;
-    static constexpr int min_blocks = sizeof(T) == 4 ? 4 : 1;   // FP32: at most 128 registers
+    static constexpr int warps = sizeof(T) == 4 ? 4 : 2;   // static shared memory below 48 KB
 };
 
+// what a lane adds at once: FP32 two particles, FP64 one
 template <typename T>
-struct AccQ {
-    T v[9];
-    __device__ __forceinline__ void zero()
+struct Pk;
+template <>
+struct Pk<float> {
+    using V = float2;
+    static constexpr int n = 2;
+    static __device__ __forceinline__ V zero() { return make_float2(0.f, 0.f); }
+    static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
+    static __device__ __forceinline__ float sum(V a) { return a.x + a.y; }
+    // two neighbouring staged values (16-byte aligned)
+    static __device__ __forceinline__ void two(const V* p, V& a, V& b)
     {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] = T(0);
-    }
-    __device__ __forceinline__ void add(T w, const T* row)
-    {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) v[e] += w * row[e];
-    }
-    __device__ __forceinline__ void get(T (&o)[9]) const
-    {
-#pragma unroll
-        for (int e = 0; e < 9; ++e) o[e] = v[e];
+        const float4 q = *reinterpret_cast<const float4*>(p);
+        a = make_float2(q.x, q.y);
+        b = make_float2(q.z, q.w);
     }
 };
 template <>
-struct AccQ<float> {
-    float2 v2[4];
-    float v8;
-    __device__ __forceinline__ void zero()
+struct Pk<double> {
+    using V = double;
+    static constexpr int n = 1;
+    static __device__ __forceinline__ V zero() { return 0.0; }
+    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
+    static __device__ __forceinline__ V fma(V a, V b, V c) { return a * b + c; }
+    static __device__ __forceinline__ double sum(V a) { return a; }
+    static __device__ __forceinline__ void two(const V* p, V& a, V& b)
     {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v2[k] = make_float2(0.f, 0.f);
-        v8 = 0.f;
-    }
-    __device__ __forceinline__ void add(float w, const float* row)   // row 8-byte aligned
-    {
-        const float2 ww = make_float2(w, w);
-        const float2* r2 = reinterpret_cast<const float2*>(row);
-#pragma unroll
-        for (int k = 0; k < 4; ++k) v2[k] = __ffma2_rn(ww, r2[k], v2[k]);
-        v8 = fmaf(w, row[8], v8);
-    }
-    __device__ __forceinline__ void get(float (&o)[9]) const
-    {
-#pragma unroll
-        for (int k = 0; k < 4; ++k) {
-            o[2 * k] = v2[k].x;
-            o[2 * k + 1] = v2[k].y;
-        }
-        o[8] = v8;
+        a = p[0];
+        b = p[1];
     }
 };
 
-// a 3x3 block added to the stored block at dst; in FP32 as paired atomics on
-// 8-byte aligned pairs (odd: dst starts on an odd float, as 117 values per
-// node and 9 per block are odd), constant indices in both branches
-__device__ __forceinline__ void add_block9q(float* dst, const float (&v)[9], int odd)
-{
-    if (odd) {
-        atomicAdd(dst, v[0]);
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            atomicAdd(reinterpret_cast<float2*>(dst + 1 + 2 * e), make_float2(v[1 + 2 * e], v[2 + 2 * e]));
-    } else {
-#pragma unroll
-        for (int e = 0; e < 4; ++e)
-            atomicAdd(reinterpret_cast<float2*>(dst + 2 * e), make_float2(v[2 * e], v[2 * e + 1]));
-        atomicAdd(dst + 8, v[8]);
-    }
-}
-__device__ __forceinline__ void add_block9q(double* dst, const double (&v)[9], int)
-{
-#pragma unroll
-    for (int e = 0; e < 9; ++e) atomicAdd(dst + e, v[e]);
-}
+// staged values of a particle: the six x and six y products, c alpha (rows of
+// four), the frame's nine weights, the current
+enum { kQXX = 0, kQYY = 6, kQE = 12, kQW = 24, kQV = 33, kQN = 36, kQRow = 38 };
+template <typename T>
+struct StageQ {
+    typename Pk<T>::V v[32 / Pk<T>::n + 4][kQRow];   // a group starts on a row of its own
+    __device__ __forceinline__ void put(int row, int at, int k, T a) { reinterpret_cast<T*>(&v[row][k])[at] = a; }
+};
 
-// the q-th pair (a <= b, node index 4 y + x in the 4 x 4 union, at most two
-// apart per axis)
-__device__ __forceinline__ void pair_q(int q, int& a, int& b)
+// the union's products: [column of the left node, a ring of four][dx][row c,
+// dy: 3 c + dy][entry]
+constexpr int kUY = 90;                 // values of one (column, dx)
+constexpr int kUCol = 3 * kUY;          // and of a column
+constexpr int kItemsQ = 37 * 9;         // additions to M of a column
+
+// block q (0 .. 36) that holds a column's products: the node it is stored at
+// (col columns right of the left node, union row), its offset index and the
+// product's place (dx, 3 c + dy)
+__device__ __forceinline__ void column_block(int q, int& col, int& row, int& hs, int& dx, int& yt)
 {
     int n = 0;
-    a = b = 0;
-    for (int aa = 0; aa < 16; ++aa)
-        for (int bb = aa; bb < 16; ++bb) {
-            const int dx = (bb & 3) - (aa & 3), dy = (bb >> 2) - (aa >> 2);
-            if (dx > 2 || dx < -2 || dy > 2) continue;
-            if (n == q) {
-                a = aa;
-                b = bb;
-            }
-            ++n;
-        }
+    col = row = hs = dx = yt = 0;
+    for (int x = 0; x < 3; ++x)
+        for (int c = 0; c < 4; ++c)
+            for (int dy = 0; dy < 3 && c + dy < 4; ++dy)
+                for (int way = 0; way < (x > 0 && dy > 0 ? 2 : 1); ++way) {
+                    // way 0: nodes (0, c) and (x, c + dy); 1: (x, c) and (0, c + dy)
+                    if (n++ != q) continue;
+                    col = way ? x : 0;
+                    row = c;
+                    hs = halfq(way ? -x : x, dy);
+                    dx = x;
+                    yt = 3 * c + dy;
+                }
 }
 
 template <typename T>
-__device__ __forceinline__ void flush_q_vals(T* M, int a, int b, const T (&v)[9], int i, int j, const GridP& g)
+__global__ void __launch_bounds__(32 * DepCfgQ<T>::warps)
+k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ B, T* __restrict__ M,
+            T* __restrict__ J, GridP g, int uw)
 {
-    const int di = (b & 3) - (a & 3), dj = (b >> 2) - (a >> 2);
-    int hs = halfq(di, dj), at = a;
-    if (hs < 0) {
-        hs = halfq(-di, -dj);
-        at = b;
-    }
-    const int64_t gn = (int64_t)wrap1(j - 1 + (at >> 2), g.ny) * g.nx + wrap1(i - 1 + (at & 3), g.nx);
-    add_block9q(M + gn * kMBlockQ + hs * 9, v, (int)((gn + hs) & 1));
-}
-
-template <typename T>
-__global__ void __launch_bounds__(32 * DepCfgQ<T>::warps, DepCfgQ<T>::min_blocks)
-k_deposit_q(DepositSpecies<T> ds, const T* __restrict__ B, T* __restrict__ M, T* __restrict__ J, GridP g)
-{
-    // The particles of a cell are taken in four groups by the half of the
-    // cell they sit in along x and y (hx, hy): a group's particles touch the
-    // same 3 x 3 nodes, the union nodes (x + hx, y + hy) of the frame nodes
-    // x, y = 0..2. Each lane owns frame pairs lane and lane + 32 of the 45
-    // pairs of a frame and frame current component lane (of 27), sums a
-    // group's particles in registers and adds the sums to the cell's union
-    // accumulators in shared memory (one owner per entry and group); the
-    // union sums are flushed to M and Jhat once per cell.
     constexpr int kW = DepCfgQ<T>::warps;
-    constexpr int kSt = 22;   // 9 frame weights, pad, 9 c alpha at 10, 3 currents at 19
-    __shared__ __align__(16) T sh[kW][32][kSt];
-    __shared__ __align__(16) T um[kW][kPairsQ][9];
-    __shared__ T uj[kW][48];
-    __shared__ TileQ<T> stl[kW];
+    using P = Pk<T>;
+    using V = typename P::V;
+    __shared__ __align__(16) StageQ<T> sst[kW];
+    __shared__ T sum_[kW][4 * kUCol];
+    __shared__ T sumj[kW][4][12];       // currents: [column][3 row + component]
+    __shared__ TileBq<T> stl[kW];
+    __shared__ int snode[kW][12];       // nodes (col, row) of a column's additions
+    __shared__ unsigned item[kItemsQ];  // node << 20 | place in its blocks << 10 | value in the column
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
+    for (int q = threadIdx.x; q < 37; q += blockDim.x) {
+        int col, row, hs, dx, yt, rank = 0;
+        column_block(q, col, row, hs, dx, yt);
+        for (int o = 0; o < 37; ++o) {
+            int c2, r2, h2, d2, y2;
+            column_block(o, c2, r2, h2, d2, y2);
+            rank += (c2 * 4 + r2) * kHalfQ + h2 < (col * 4 + row) * kHalfQ + hs ? 1 : 0;
+        }
+        for (int e = 0; e < 9; ++e)
+            item[rank * 9 + e] = (unsigned)(col * 4 + row) << 20 | (unsigned)(hs * 9 + e) << 10 |
+                                 (unsigned)(dx * kUY + yt * 9 + e);
+    }
+    for (int q = lane; q < 4 * kUCol; q += 32) sum_[wib][q] = T(0);
+    for (int q = lane; q < 48; q += 32) (&sumj[wib][0][0])[q] = T(0);
+    __syncthreads();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int nseg = (g.nx + kQX - 1) / kQX;
+    const int nseg = (g.nx + uw - 1) / uw;
     const int nunits = nseg * g.ny;
-    T (*st)[kSt] = sh[wib];
-    T (*U)[9] = um[wib];
-    T* UJ = uj[wib];
-    // this lane's frame pairs (a <= b in the frame order 3 y + x)
-    int fa[2] = {0, 0}, fb[2] = {0, 0};
-#pragma unroll
-    for (int t = 0; t < 2; ++t) {
-        const int q = lane + 32 * t;
-        int n = 0;
-        for (int a = 0; a < 9; ++a)
-            for (int b = a; b < 9; ++b) {
-                if (n == q) {
-                    fa[t] = a;
-                    fb[t] = b;
-                }
-                ++n;
-            }
-    }
-    const bool two = lane + 32 < 45;
-    // their union pair index per group
-    int uq[2][4];
-#pragma unroll
-    for (int t = 0; t < 2; ++t)
-#pragma unroll
-        for (int gq = 0; gq < 4; ++gq) {
-            const int hx = gq & 1, hy = gq >> 1;
-            const int ua = 4 * (fa[t] / 3 + hy) + fa[t] % 3 + hx, ub = 4 * (fb[t] / 3 + hy) + fb[t] % 3 + hx;
-            int n = 0, found = 0;
-            for (int a = 0; a < 16; ++a)
-                for (int b = a; b < 16; ++b) {
-                    const int dx = (b & 3) - (a & 3), dy = (b >> 2) - (a >> 2);
-                    if (dx > 2 || dx < -2 || dy > 2) continue;
-                    if (a == ua && b == ub) found = n;
-                    ++n;
-                }
-            uq[t][gq] = found;
-        }
-    // the union pairs this lane flushes
-    int pa[4], pb[4];
-#pragma unroll
-    for (int t = 0; t < 4; ++t) {
-        const int q = lane + 32 * t;
-        if (q < kPairsQ) pair_q(q, pa[t], pb[t]);
-        else pa[t] = pb[t] = 0;
-    }
-    const bool ownj = lane < 27;
-    const int jf = lane / 3, jc = lane % 3;   // frame node and component
-    for (int q = lane; q < kPairsQ * 9; q += 32) (&U[0][0])[q] = T(0);
-    for (int q = lane; q < 48; q += 32) UJ[q] = T(0);
+    StageQ<T>& st = sst[wib];
+    T* const U = sum_[wib];
+    // this lane's products (x types 2 xg, 2 xg + 1, y types 2 yg, 2 yg + 1),
+    // row of alpha, and current (frame node, component)
+    const bool own = lane < 27;
+    const int er = own ? lane % 3 : 0, yg = own ? lane / 3 % 3 : 0, xg = own ? lane / 9 : 0;
+    const int jf = own ? lane / 3 : 0, jc = own ? lane % 3 : 0;
+    // pair type t of the frame's axis: its lower node and the distance
+    auto low_of = [](int t) { return t < 3 ? 0 : (t < 5 ? 1 : 2); };
+    auto dist_of = [](int t) { return t < 3 ? t : (t < 5 ? t - 3 : 0); };
+    const int xl[2] = {low_of(2 * xg), low_of(2 * xg + 1)}, xd[2] = {dist_of(2 * xg), dist_of(2 * xg + 1)};
+    const int yo[2] = {(3 * low_of(2 * yg) + dist_of(2 * yg)) * 9 + 3 * er,
+                       (3 * low_of(2 * yg + 1) + dist_of(2 * yg + 1)) * 9 + 3 * er};
     for (int u = warp; u < nunits; u += nwarps) {
-        const int i0 = (u % nseg) * kQX, j = u / nseg;
-        const int cn = min(kQX, g.nx - i0);
+        const int i0 = (u % nseg) * uw, j = u / nseg;
+        const int cn = min(uw, g.nx - i0);
         __syncwarp();
-        load_tileq<T>(stl[wib], nullptr, B, i0, cn, j, g, lane);
-        for (int cl = 0; cl < cn; ++cl) {
+        load_tileBq<T>(stl[wib], B, i0, cn, j, g, lane);
+        int live = 0;   // columns of the ring that hold sums
+        for (int cl = 0; cl < cn + 3; ++cl) {   // the last three: only the columns left over
             const int i = i0 + cl;
-            const int c = j * g.nx + i;
             int cum[kMaxSpecies + 1], pst[kMaxSpecies];
             cum[0] = 0;
 #pragma unroll
             for (int s = 0; s < kMaxSpecies; ++s) {
-                pst[s] = s < ds.nsp ? ds.start[s][c] : 0;
-                cum[s + 1] = cum[s] + (s < ds.nsp ? ds.start[s][c + 1] - pst[s] : 0);
+                pst[s] = 0;
+                cum[s + 1] = cum[s];
+                if (cl < cn && s < ds.nsp) {
+                    pst[s] = ds.start[s][j * g.nx + i];
+                    cum[s + 1] += ds.start[s][j * g.nx + i + 1] - pst[s];
+                }
             }
             const int total = cum[kMaxSpecies];
-            if (total == 0) continue;
-            for (int q0 = 0; q0 < total; q0 += 32) {
-                const int t = q0 + lane;
-                const bool act = t < total;
-                int grp = -1;
-                T row[kSt];
-                if (act) {
+            if (total > 0) {
+                T acc[4][12], accj[4];   // per group
+#pragma unroll
+                for (int gq = 0; gq < 4; ++gq) {
+                    accj[gq] = T(0);
+#pragma unroll
+                    for (int e = 0; e < 12; ++e) acc[gq][e] = T(0);
+                }
+                for (int q0 = 0; q0 < total; q0 += 32) {
+                    const int t = q0 + lane;
+                    const bool act = t < total;
+                    T fx = T(0), fy = T(0);
                     int s = 0, p = pst[0] + t;
+                    if (act) {
 #pragma unroll
-                    for (int q = 1; q < kMaxSpecies; ++q)
-                        if (t >= cum[q] && cum[q + 1] > cum[q]) {
-                            s = q;
-                            p = pst[q] + (t - cum[q]);
-                        }
-                    const T fx = ld(ds.fx[s] + p), fy = ld(ds.fy[s] + p);
-                    const T ux = ld(ds.ux[s] + p), uy = ld(ds.uy[s] + p), uz = ld(ds.uz[s] + p);
-                    const T wt = ld(ds.w[s] + p);
+                        for (int q = 1; q < kMaxSpecies; ++q)
+                            if (t >= cum[q] && cum[q + 1] > cum[q]) {
+                                s = q;
+                                p = pst[q] + (t - cum[q]);
+                            }
+                        fx = ld(ds.fx[s] + p);
+                        fy = ld(ds.fy[s] + p);
+                    }
                     const int hx = fx >= T(0.5), hy = fy >= T(0.5);
-                    grp = 2 * hy + hx;
-                    T wx[3], wy[3], Bp[3], al[9];
-                    quad3(hx ? fx - T(1) : fx, wx);
-                    quad3(hy ? fy - T(1) : fy, wy);
-                    tile_Bq(stl[wib], cl, fx, fy, Bp);
-                    const T gbar = sqrt(T(1) + ux * ux + uy * uy + uz * uz);
-                    alphaq(Bp, ds.beta[s], gbar, al);
-                    const T cM = wt * ds.cM[s] / gbar, cJ = wt * ds.cJ[s] / gbar;
+                    const int grp = act ? 2 * hy + hx : -1;
+                    // rows of the groups, and this particle's place
+                    int gr[5], row = 0, at = 0;
+                    gr[0] = 0;
 #pragma unroll
-                    for (int r = 0; r < 3; ++r)
+                    for (int gq = 0; gq < 4; ++gq) {
+                        const unsigned bal = __ballot_sync(0xffffffffu, grp == gq);
+                        const int cnt = __popc(bal), place = __popc(bal & ((1u << lane) - 1u));
+                        gr[gq + 1] = gr[gq] + (cnt + P::n - 1) / P::n;
+                        if (grp == gq) {
+                            row = gr[gq] + place / P::n;
+                            at = place % P::n;
+                        }
+                        if (P::n == 2 && (cnt & 1)) {   // the row's other half
+                            st.put(gr[gq + 1] - 1, 1, lane, T(0));
+                            if (lane < kQN - 32) st.put(gr[gq + 1] - 1, 1, 32 + lane, T(0));
+                        }
+                    }
+                    if (act) {
+                        const T ux = ld(ds.ux[s] + p), uy = ld(ds.uy[s] + p), uz = ld(ds.uz[s] + p);
+                        const T wt = ld(ds.w[s] + p);
+                        T wx[3], wy[3], Bp[3], al[9];
+                        quad3(hx ? fx - T(1) : fx, wx);
+                        quad3(hy ? fy - T(1) : fy, wy);
+                        tile_Bq(stl[wib].B, cl, fx, fy, Bp);
+                        const T ig = T(1) / sqrt(T(1) + ux * ux + uy * uy + uz * uz);
+                        alphaq(Bp, ds.beta[s] * ig, al);
+                        const T cM = wt * ds.cM[s] * ig, cJ = wt * ds.cJ[s] * ig;
+                        int n = 0;
 #pragma unroll
-                        for (int c2 = 0; c2 < 3; ++c2) row[3 * r + c2] = wy[r] * wx[c2];
-                    row[9] = T(0);
+                        for (int a = 0; a < 3; ++a)
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) row[10 + e] = cM * al[e];
+                            for (int b2 = a; b2 < 3; ++b2) {
+                                st.put(row, at, kQXX + n, wx[a] * wx[b2]);
+                                st.put(row, at, kQYY + n, wy[a] * wy[b2]);
+                                ++n;
+                            }
 #pragma unroll
-                    for (int r = 0; r < 3; ++r)
-                        row[19 + r] = cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz);
+                        for (int e = 0; e < 9; ++e) st.put(row, at, kQE + 4 * (e / 3) + e % 3, cM * al[e]);
+#pragma unroll
+                        for (int r = 0; r < 3; ++r)
+#pragma unroll
+                            for (int c2 = 0; c2 < 3; ++c2) st.put(row, at, kQW + 3 * r + c2, wy[r] * wx[c2]);
+#pragma unroll
+                        for (int r = 0; r < 3; ++r)
+                            st.put(row, at, kQV + r,
+                                   cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz));
+                    }
+                    __syncwarp();
+#pragma unroll
+                    for (int gq = 0; gq < 4; ++gq) {
+                        if (gr[gq + 1] == gr[gq]) continue;   // warp-uniform
+                        V a[12], aj = P::zero();
+#pragma unroll
+                        for (int e = 0; e < 12; ++e) a[e] = P::zero();
+                        for (int r = gr[gq]; r < gr[gq + 1]; ++r) {
+                            const V* rw = st.v[r];
+                            V x0, x1, y0, y1, e0, e1;
+                            P::two(rw + kQXX + 2 * xg, x0, x1);
+                            P::two(rw + kQYY + 2 * yg, y0, y1);
+                            P::two(rw + kQE + 4 * er, e0, e1);
+                            const V e2 = rw[kQE + 4 * er + 2];
+                            const V w[4] = {P::mul(x0, y0), P::mul(x1, y0), P::mul(x0, y1), P::mul(x1, y1)};
+#pragma unroll
+                            for (int q = 0; q < 4; ++q) {
+                                a[3 * q] = P::fma(w[q], e0, a[3 * q]);
+                                a[3 * q + 1] = P::fma(w[q], e1, a[3 * q + 1]);
+                                a[3 * q + 2] = P::fma(w[q], e2, a[3 * q + 2]);
+                            }
+                            aj = P::fma(rw[kQW + jf], rw[kQV + jc], aj);
+                        }
+#pragma unroll
+                        for (int e = 0; e < 12; ++e) acc[gq][e] += P::sum(a[e]);
+                        accj[gq] += P::sum(aj);
+                    }
+                    __syncwarp();
                 }
-                // staging rows grouped by g (ballot prefix sums)
-                unsigned bal[4];
-                int gb[5];
-                gb[0] = 0;
+                // the cell's sums into the union's products (distinct entries
+                // per lane within a group)
 #pragma unroll
                 for (int gq = 0; gq < 4; ++gq) {
-                    bal[gq] = __ballot_sync(0xffffffffu, grp == gq);
-                    gb[gq + 1] = gb[gq] + __popc(bal[gq]);
-                }
-                if (act) {
-                    int r = 0;
+                    const int hx = gq & 1, hy = gq >> 1;
+                    if (own) {
 #pragma unroll
-                    for (int gq = 0; gq < 4; ++gq)
-                        if (grp == gq) r = gb[gq] + __popc(bal[gq] & ((1u << lane) - 1u));
+                        for (int q = 0; q < 4; ++q) {
+                            T* const o = U + ((cl + xl[q & 1] + hx) & 3) * kUCol + xd[q & 1] * kUY + yo[q >> 1] + 27 * hy;
 #pragma unroll
-                    for (int e = 0; e < kSt; ++e) st[r][e] = row[e];
-                }
-                __syncwarp();
-#pragma unroll
-                for (int gq = 0; gq < 4; ++gq) {
-                    if (gb[gq + 1] == gb[gq]) continue;   // warp-uniform
-                    AccQ<T> a0, a1;
-                    a0.zero();
-                    a1.zero();
-                    T aj = T(0);
-                    for (int r = gb[gq]; r < gb[gq + 1]; ++r) {
-                        const T* rw = st[r];
-                        a0.add(rw[fa[0]] * rw[fb[0]], rw + 10);
-                        if (two) a1.add(rw[fa[1]] * rw[fb[1]], rw + 10);
-                        if (ownj) aj += rw[jf] * rw[19 + jc];
-                    }
-                    // into the union accumulators (distinct entries per lane)
-                    T v[9];
-                    a0.get(v);
-#pragma unroll
-                    for (int e = 0; e < 9; ++e) U[uq[0][gq]][e] += v[e];
-                    if (two) {
-                        a1.get(v);
-#pragma unroll
-                        for (int e = 0; e < 9; ++e) U[uq[1][gq]][e] += v[e];
-                    }
-                    if (ownj) {
-                        const int hx = gq & 1, hy = gq >> 1;
-                        UJ[3 * (4 * (jf / 3 + hy) + jf % 3 + hx) + jc] += aj;
+                            for (int e = 0; e < 3; ++e) o[e] += acc[gq][3 * q + e];
+                        }
+                        sumj[wib][(cl + jf % 3 + hx) & 3][3 * (jf / 3 + hy) + jc] += accj[gq];
                     }
                     __syncwarp();   // another lane may own these entries in the next group
                 }
+                live = 4;
+            }
+            // the column of nodes i - 1 is complete
+            if (live > 0) {
+                if (lane < 12)
+                    snode[wib][lane] = wrap1(j - 1 + (lane & 3), g.ny) * g.nx + wrap1(i - 1 + (lane >> 2), g.nx);
                 __syncwarp();
-            }
-            // flush the cell's union sums and clear them
-#pragma unroll
-            for (int t2 = 0; t2 < 4; ++t2) {
-                const int q = lane + 32 * t2;
-                if (q < kPairsQ) {
-                    T v[9];
-#pragma unroll
-                    for (int e = 0; e < 9; ++e) {
-                        v[e] = U[q][e];
-                        U[q][e] = T(0);
-                    }
-                    flush_q_vals(M, pa[t2], pb[t2], v, i, j, g);
+                T* const C = U + (cl & 3) * kUCol;
+                for (int it = lane; it < kItemsQ; it += 32) {
+                    const unsigned q = item[it];
+                    atomicAdd(M + (int64_t)snode[wib][q >> 20] * kMBlockQ + ((q >> 10) & 1023u), C[q & 1023u]);
                 }
+                if (lane < 12) {
+                    T& vj = sumj[wib][cl & 3][lane];
+                    atomicAdd(J + (int64_t)(lane % 3) * g.ncell + snode[wib][lane / 3], vj);
+                    vj = T(0);
+                }
+                __syncwarp();
+                for (int q = lane; q < kUCol; q += 32) C[q] = T(0);
+                __syncwarp();
+                --live;
             }
-            for (int q = lane; q < 48; q += 32) {
-                const T val = UJ[q];
-                UJ[q] = T(0);
-                const int un = q / 3, comp = q % 3;
-                const int64_t gn = (int64_t)wrap1(j - 1 + (un >> 2), g.ny) * g.nx + wrap1(i - 1 + (un & 3), g.nx);
-                if (val != T(0)) atomicAdd(J + (int64_t)comp * g.ncell + gn, val);
-            }
-            __syncwarp();
         }
     }
 }
@@ -699,7 +689,7 @@ template <typename T>
 __global__ void __launch_bounds__(32 * kPushWarpsQ)
 k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int32_t* __restrict__ key,
          int32_t* __restrict__ rank, int32_t* __restrict__ count, const T* __restrict__ Eth, const T* __restrict__ B,
-         GridP g, T beta, T qdt, T m, double* __restrict__ lsum)
+         GridP g, T beta, T qdt, T m, double* __restrict__ lsum, int uw)
 {
     __shared__ int sst[kPushWarpsQ][kQX + 1];
     __shared__ TileQ<T> stl[kPushWarpsQ];
@@ -707,14 +697,23 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int nseg = (g.nx + kQX - 1) / kQX;
+    const int nseg = (g.nx + uw - 1) / uw;
     const int nunits = nseg * g.ny;
     int* ss = sst[wib];
-    const T dt = gc<T>(g).dt, rdx = gc<T>(g).rdx, rdy = gc<T>(g).rdy;
+    const T dtx = gc<T>(g).dt * gc<T>(g).rdx, dty = gc<T>(g).dt * gc<T>(g).rdy;
     T acc[4] = {T(0), T(0), T(0), T(0)};
+    // a batch whose slots are still on their way: its particle, the lanes that
+    // share its new cell, and (the first of them) what the count was
+    int wait_p = -1, wait_base = 0;
+    unsigned wait_peers = 0u;
+    auto settle = [&]() {
+        const int b = __shfl_sync(0xffffffffu, wait_base, wait_peers ? __ffs(wait_peers) - 1 : lane);
+        if (wait_p >= 0) rank[wait_p] = b + __popc(wait_peers & ((1u << lane) - 1u));
+        wait_p = -1;
+    };
     for (int u = warp; u < nunits; u += nwarps) {
-        const int i0 = (u % nseg) * kQX, j = u / nseg;
-        const int cn = min(kQX, g.nx - i0);
+        const int i0 = (u % nseg) * uw, j = u / nseg;
+        const int cn = min(uw, g.nx - i0);
         const int c0 = j * g.nx + i0;
         __syncwarp();
         if (lane <= cn) ss[lane] = start[c0 + lane];
@@ -723,33 +722,50 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
         const TileQ<T>& tl = stl[wib];
         const int P0 = ss[0], P1 = ss[cn];
         int cl = 0;
+        // the next batch is loaded while this one is pushed
+        T nfx = T(0), nfy = T(0), nux = T(0), nuy = T(0), nuz = T(0), nw = T(0);
+        auto fetch = [&](int q) {
+            if (q < P1) {
+                nfx = ld(src.fx + q);
+                nfy = ld(src.fy + q);
+                nux = ld(src.ux + q);
+                nuy = ld(src.uy + q);
+                nuz = ld(src.uz + q);
+                nw = ld(src.w + q);
+            }
+        };
+        fetch(P0 + lane);
         for (int p0 = P0; p0 < P1; p0 += 32) {
             const int p = p0 + lane;
             const bool act = p < P1;
+            const T fx = nfx, fy = nfy, ux = nux, uy = nuy, uz = nuz, w = nw;
+            fetch(p + 32);
             int newkey = -1 - lane;
             if (act) {
                 while (ss[cl + 1] <= p) ++cl;
-                const int i = i0 + cl;
-                const T fx = ld(src.fx + p), fy = ld(src.fy + p);
-                const T ux = ld(src.ux + p), uy = ld(src.uy + p), uz = ld(src.uz + p), w = ld(src.w + p);
-                T wx[4], wy[4];
-                node4(fx, wx);
-                node4(fy, wy);
+                // E from the particle's own 3 x 3 nodes of the cell's 4 x 4
+                const int hx = fx >= T(0.5), hy = fy >= T(0.5);
+                T wx[3], wy[3];
+                quad3(hx ? fx - T(1) : fx, wx);
+                quad3(hy ? fy - T(1) : fy, wy);
                 T E[3];
 #pragma unroll
                 for (int c = 0; c < 3; ++c) {
                     T e = T(0);
 #pragma unroll
-                    for (int r = 0; r < 4; ++r)
+                    for (int r = 0; r < 3; ++r) {
+                        T er = T(0);
 #pragma unroll
-                        for (int cc = 0; cc < 4; ++cc) e += wy[r] * wx[cc] * tl.E[c][r][cl + cc];
+                        for (int cc = 0; cc < 3; ++cc) er += wx[cc] * tl.E[c][r + hy][cl + cc + hx];
+                        e += wy[r] * er;
+                    }
                     E[c] = e;
                 }
                 T Bp[3];
-                tile_Bq(tl, cl, fx, fy, Bp);
+                tile_Bq(tl.B, cl, fx, fy, Bp);
                 const T u02 = ux * ux + uy * uy + uz * uz;
-                const T g0 = sqrt(T(1) + u02);
-                const T ax = beta * Bp[0] / g0, ay = beta * Bp[1] / g0, az = beta * Bp[2] / g0;
+                const T g0 = sqrt(T(1) + u02), ig0 = T(1) / g0;
+                const T bg = beta * ig0, ax = bg * Bp[0], ay = bg * Bp[1], az = bg * Bp[2];
                 const T sa = T(1) / (T(1) + ax * ax + ay * ay + az * az);
                 const T wxv = ux + beta * E[0], wyv = uy + beta * E[1], wzv = uz + beta * E[2];
                 const T wa = wxv * ax + wyv * ay + wzv * az;
@@ -758,9 +774,9 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
                 const T ubz = sa * (wzv + (wxv * ay - wyv * ax) + wa * az);
                 const T u1x = T(2) * ubx - ux, u1y = T(2) * uby - uy, u1z = T(2) * ubz - uz;
                 const T u12 = u1x * u1x + u1y * u1y + u1z * u1z;
-                const T g1 = sqrt(T(1) + u12);
-                const T t[2] = {fx + dt * rdx * (u1x / g1), fy + dt * rdy * (u1y / g1)};
-                const int nn[2] = {g.nx, g.ny}, cc0[2] = {i, j};
+                const T g1 = sqrt(T(1) + u12), ig1 = T(1) / g1;
+                const T t[2] = {fx + dtx * (u1x * ig1), fy + dty * (u1y * ig1)};
+                const int nn[2] = {g.nx, g.ny}, cc0[2] = {i0 + cl, j};
                 T fn[2];
                 int cnew[2];
 #pragma unroll
@@ -770,8 +786,11 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
                     T f = t[a] - fl;
                     if (f >= T(1)) { f -= T(1); sh += 1; }
                     fn[a] = f;
-                    int q = (cc0[a] + sh) % nn[a];
-                    if (q < 0) q += nn[a];
+                    int q = cc0[a] + sh;
+                    if ((unsigned)q >= (unsigned)nn[a]) {   // across the box: any distance
+                        q %= nn[a];
+                        if (q < 0) q += nn[a];
+                    }
                     cnew[a] = q;
                 }
                 dst.fx[p] = fn[0];
@@ -785,21 +804,23 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
                 key[p] = newkey;
                 const T ue = ubx * E[0] + uby * E[1] + ubz * E[2];
                 const T du = (ux - u1x) * (ux + u1x) + (uy - u1y) * (uy + u1y) + (uz - u1z) * (uz + u1z);
-                const T igs = T(1) / (g0 + g1);
+                const T igs = T(1) / (g0 + g1), wk = qdt * w * ue * ig0;
                 acc[0] -= w * m * du * igs;
-                acc[1] += qdt * w * ue / g0;
-                acc[2] += qdt * w * ue * du * igs * igs / g0;
+                acc[1] += wk;
+                acc[2] += wk * du * igs * igs;
                 acc[3] += w * m * u12 / (g1 + T(1));
             }
+            settle();   // the last batch's slots have had this one's time to arrive
             const unsigned peers = __match_any_sync(0xffffffffu, newkey);
-            const int leader = __ffs(peers) - 1;
-            int base = 0;
-            if (act && lane == leader) base = atomicAdd(count + newkey, __popc(peers));
-            base = __shfl_sync(0xffffffffu, base, leader);
-            if (act) rank[p] = base + __popc(peers & ((1u << lane) - 1u));
+            wait_peers = peers;
+            if (act) {
+                wait_p = p;
+                if ((peers & ((1u << lane) - 1u)) == 0u) wait_base = atomicAdd(count + newkey, __popc(peers));
+            }
         }
         __syncwarp();
     }
+    settle();
     double v[4], o[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = (double)acc[q];
@@ -811,13 +832,24 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
 
 }  // namespace
 
+// the width of the row segments a warp takes: 32 cells, halved (to 8 at
+// least: a segment adds three columns at its end) while that leaves fewer
+// than eight warps per SM
+static int unit_width_q(GridP g)
+{
+    int uw = kQX;
+    while (uw > 8 && ((g.nx + uw - 1) / uw) * g.ny < 152 * 8) uw /= 2;
+    return uw;
+}
+
 template <typename T>
 cudaError_t deposit_q(const DepositSpecies<T>& ds, const T* B, T* M, T* J, GridP g, cudaStream_t st, int blocks)
 {
-    const int units = ((g.nx + kQX - 1) / kQX) * g.ny;
+    const int uw = unit_width_q(g);
+    const int units = ((g.nx + uw - 1) / uw) * g.ny;
     count_launches(1);
     k_deposit_q<T><<<gridq(units, DepCfgQ<T>::warps, blocks > 0 ? blocks : 152 * 8), 32 * DepCfgQ<T>::warps, 0, st>>>(
-        ds, B, M, J, g);
+        ds, B, M, J, g, uw);
     return cudaGetLastError();
 }
 
@@ -845,7 +877,8 @@ cudaError_t field_update_q(const double* x, const T* M, const T* J, T* Eth, T* E
 
 int push_blocks_q(GridP g, int cap)
 {
-    const int64_t units = (int64_t)((g.nx + kQX - 1) / kQX) * g.ny;
+    const int uw = unit_width_q(g);
+    const int64_t units = (int64_t)((g.nx + uw - 1) / uw) * g.ny;
     return (int)gridq(units, kPushWarpsQ, cap > 0 ? cap : 152 * 16);
 }
 
@@ -857,7 +890,7 @@ cudaError_t push_q(PArrays<T> src, PArrays<T> dst, const int32_t* start, int32_t
     count_launches(1);
     k_push_q<T><<<nblocks, 32 * kPushWarpsQ, 0, st>>>(src, dst, start, key, rank, count, Eth, B, g,
                                                         (T)(sc.q * g.dt / (2.0 * sc.m)), (T)(sc.q * g.dt), (T)sc.m,
-                                                        lsum);
+                                                        lsum, unit_width_q(g));
     return cudaGetLastError();
 }
 

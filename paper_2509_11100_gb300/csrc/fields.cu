@@ -824,12 +824,13 @@ int grid_for(int64_t n, int threads, int cap)
 int field_grid_blocks(GridP g, int precision)
 {
     if (g.dim == 3) return op_blocks3(g, precision);
+    if (g.shape == 2) return op_blocks_q(g, precision);
     return grid_for(g.ncell, kFieldThreads, 1 << 30);
 }
 int op_blocks(GridP g, int precision)
 {
     if (g.dim == 3) return op_blocks3(g, precision);
-    if (g.shape == 2) return op_blocks_q(g);
+    if (g.shape == 2) return op_blocks_q(g, precision);
     const int X = 32, Y = g.op_y > 0 ? g.op_y : (precision == 32 ? OpTile<float>::Y : OpTile<double>::Y);
     return ((g.nx + X - 1) / X) * ((g.ny + Y - 1) / Y);
 }

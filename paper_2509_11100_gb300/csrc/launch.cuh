@@ -156,7 +156,7 @@ cudaError_t place3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const i
 template <typename T>
 cudaError_t deposit_q(const DepositSpecies<T>& ds, const T* B, T* M, T* J, GridP g, cudaStream_t st,
                       int blocks = 0);   // blocks 0: at most 8 per SM
-int op_blocks_q(GridP g);
+int op_blocks_q(GridP g, int precision);
 template <typename T, int MODE, bool TR>
 cudaError_t launch_op_q(const T* M, const double* in, double sc, const double* b, double* out, double* vj,
                         const double* V, int64_t ldv, int nv, GridP g, double* partial, cudaStream_t st,

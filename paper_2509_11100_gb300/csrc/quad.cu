@@ -17,13 +17,14 @@
 //                 group touches a fixed 3 x 3 of the cell's 4 x 4 nodes), the
 //                 lanes sum the groups' 36 weight products; a ring of four
 //                 node columns in shared memory collects the cells' sums
-//   k_op_q        the operator on 32 x 8-node tiles, the input staged on a
-//                 2-node halo, the 25 blocks per node from global memory, the
+//   k_op_q        the operator on 32 x 4-node tiles, the tile's mass-matrix
+//                 rows and the input on a 2-node halo in shared memory, the
 //                 modes and partial dot products of the other operators
-//   k_field_update_q, k_work_q   the field update and the ledger terms
+//   k_field_update_q   the field update and the ledger terms on the same tiles
 //   k_push_q      warp per row segment with E and B tiles, the push, the new
 //                 cell and its slot for the counting sort (k_place3 places)
 #include "launch.cuh"
+#include "opcore.cuh"
 
 namespace relsim {
 namespace {
@@ -439,68 +440,177 @@ k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ 
 // the operator and the field update
 
 enum { kqA = 0, kqResidual = 1, kqArnoldi = 2 };
-constexpr int kOpXq = 32, kOpYq = 8, kOpTq = kOpXq * kOpYq;
 constexpr int kOpChunkq = 8;
 
-// (curl_n curl_c v) at a node from v on its 3 x 3 neighbourhood,
-// f(comp, a, b) = component comp at node (i-1+a, j-1+b)
-template <typename T, typename F>
-__device__ __forceinline__ void curlcurl_q(F f, T rdx2, T rdy2, T (&out)[3])
-{
-    T C[3][2][2];
-#pragma unroll
-    for (int ci = 0; ci < 2; ++ci)
-#pragma unroll
-        for (int cj = 0; cj < 2; ++cj) {
-            T dxf[3], dyf[3];
-#pragma unroll
-            for (int comp = 0; comp < 3; ++comp) {
-                dxf[comp] = (f(comp, ci + 1, cj) - f(comp, ci, cj) + f(comp, ci + 1, cj + 1) - f(comp, ci, cj + 1)) * rdx2;
-                dyf[comp] = (f(comp, ci, cj + 1) - f(comp, ci, cj) + f(comp, ci + 1, cj + 1) - f(comp, ci + 1, cj)) * rdy2;
-            }
-            C[0][ci][cj] = dyf[2];
-            C[1][ci][cj] = -dxf[2];
-            C[2][ci][cj] = dxf[1] - dyf[0];
-        }
-    T dxn[3], dyn[3];
-#pragma unroll
-    for (int comp = 0; comp < 3; ++comp) {
-        dxn[comp] = (C[comp][1][1] - C[comp][0][1] + C[comp][1][0] - C[comp][0][0]) * rdx2;
-        dyn[comp] = (C[comp][1][1] - C[comp][1][0] + C[comp][0][1] - C[comp][0][0]) * rdy2;
+// The operator's tiles: 32 x 4 nodes (FP64: 32 x 2), one thread a node. The
+// tile's own mass-matrix rows (15 KB a row in FP32) come into shared memory
+// by asynchronous copies while the input is staged; read straight from global
+// memory (468 bytes from lane to lane) every load of a block touched 32
+// lines: 48 us an application on 512x256 (FP32 form).
+template <typename T>
+struct OpQ {
+    static constexpr int X = 32, Y = sizeof(T) == 4 ? 4 : 2, threads = X * Y;
+    struct Shared {
+        T Mm[Y][X * kMBlockQ];          // own blocks
+        T v[3][Y + 4][X + 4];           // the input on the 2-node halo
+        T C[3][Y + 1][X + 1];           // its curl on the centres around the tile's nodes
+    };
+    static_assert(sizeof(Shared) >= sizeof(double) * kOpChunkq * threads, "the dot products reuse it");
+};
+// a block's tile and this thread's node
+template <typename T>
+struct AtQ {
+    int i0, j0, tw, th, tx, ty, i, j;
+    bool active;
+    int64_t gidx;
+    __device__ __forceinline__ explicit AtQ(const GridP& g)
+    {
+        using O = OpQ<T>;
+        const int nx = (g.nx + O::X - 1) / O::X;
+        i0 = (blockIdx.x % nx) * O::X;
+        j0 = (blockIdx.x / nx) * O::Y;
+        tw = min(O::X, g.nx - i0);
+        th = min(O::Y, g.ny - j0);
+        tx = threadIdx.x % O::X;
+        ty = threadIdx.x / O::X;
+        i = i0 + tx;
+        j = j0 + ty;
+        active = tx < tw && ty < th;
+        gidx = active ? (int64_t)j * g.nx + i : 0;
     }
-    out[0] = dyn[2];
-    out[1] = -dxn[2];
-    out[2] = dxn[1] - dyn[0];
+};
+
+// start the copies of the tile's mass-matrix rows (16 bytes each where the
+// rows are aligned to that, else 4)
+template <typename T>
+__device__ __forceinline__ void fetch_rowsq(typename OpQ<T>::Shared& S, const T* __restrict__ M, const AtQ<T>& t,
+                                            const GridP& g)
+{
+    using O = OpQ<T>;
+    const bool wide = ((int64_t)g.nx * kMBlockQ * sizeof(T)) % 16 == 0;
+    const int n = t.tw * kMBlockQ * (int)sizeof(T) / (wide ? 16 : 4);
+#pragma unroll
+    for (int y = 0; y < O::Y; ++y) {
+        if (y >= t.th) continue;
+        const char* src = reinterpret_cast<const char*>(M + ((int64_t)(t.j0 + y) * g.nx + t.i0) * kMBlockQ);
+        char* dst = reinterpret_cast<char*>(&S.Mm[y][0]);
+        if (wide)
+            for (int q = threadIdx.x; q < n; q += O::threads) cp_async16(dst + 16 * q, src + 16 * q);
+        else
+            for (int q = threadIdx.x; q < n; q += O::threads) cp_async4(dst + 4 * q, src + 4 * q);
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
 }
 
-// (M v) at node (i, j): own 13 stored blocks times v at g + d(h), the 12
-// neighbours' blocks M[g - d(h)][h] times v at g - d(h); f(comp, a, b) = v
-// at node (i-2+a, j-2+b); with TR each block transposed
-template <typename T, bool TR, typename F>
-__device__ __forceinline__ void mv_q(const T* __restrict__ M, int i, int j, const GridP& g, F f, T (&out)[3])
+// the input (FP64) on the tile's halo in T, times s, and its curl on the
+// centres around the tile's nodes (each formed once); the rows' copies land
+template <typename T, bool SCALED>
+__device__ __forceinline__ void stage_inputq(typename OpQ<T>::Shared& S, const double* __restrict__ in, T s,
+                                             const AtQ<T>& t, const GridP& g)
+{
+    using O = OpQ<T>;
+    constexpr int HX = O::X + 4, HY = O::Y + 4;
+    const int64_t nc = g.ncell;
+    const int lane = threadIdx.x % 32, wid = threadIdx.x / 32;
+    // a lane a column, the last four by four lanes; positions past the tile's
+    // last used column or row are clamped (unused); four rows in flight
+    const int ga = wrap1(min(t.i0 - 2 + lane, 2 * g.nx - 1), g.nx), gb = wrap1(min(t.i0 + 30 + lane, 2 * g.nx - 1), g.nx);
+    constexpr int rows = 3 * HY, W = O::threads / 32;
+    for (int r0 = wid; r0 < rows; r0 += 4 * W) {
+        double a[4], b[4];
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = min(r0 + v * W, rows - 1), comp = r / HY, yy = r % HY;
+            const int gj = wrap1(min(t.j0 - 2 + yy, 2 * g.ny - 1), g.ny);
+            const double* row = in + comp * nc + (int64_t)gj * g.nx;
+            a[v] = __ldg(row + ga);
+            b[v] = lane < 4 ? __ldg(row + gb) : 0.0;
+        }
+#pragma unroll
+        for (int v = 0; v < 4; ++v) {
+            const int r = r0 + v * W;
+            if (r >= rows) break;
+            T* o = &S.v[0][0][0] + r * HX;
+            T x = narrow<T>(a[v]);
+            if (SCALED) x *= s;
+            o[lane] = x;
+            if (lane < 4) {
+                T y = narrow<T>(b[v]);
+                if (SCALED) y *= s;
+                o[32 + lane] = y;
+            }
+        }
+    }
+    __syncthreads();
+    const T rx = gc<T>(g).hdx, ry = gc<T>(g).hdy;
+    for (int q = threadIdx.x; q < (O::Y + 1) * (O::X + 1); q += O::threads) {
+        const int c = q % (O::X + 1), y = q / (O::X + 1);
+        T C[3];
+        op_curl_c<T>([&](int comp, int p, int o) { return S.v[comp][y + 1 + o][c + 1 + p]; }, rx, ry, C);
+#pragma unroll
+        for (int comp = 0; comp < 3; ++comp) S.C[comp][y][c] = C[comp];
+    }
+    asm volatile("cp.async.wait_all;" ::: "memory");
+    __syncthreads();
+}
+
+// (M v) at the thread's node: its own 13 stored blocks times v at g + d(h),
+// the 12 neighbours' blocks M[g - d(h)][h] times v at g - d(h) (from the tile
+// where they lie in it, else from global memory); with TR each block
+// transposed
+template <typename T, bool TR>
+__device__ __forceinline__ void mv_q(const typename OpQ<T>::Shared& S, const T* __restrict__ M, const AtQ<T>& t,
+                                     const GridP& g, T (&out)[3])
 {
     T r[3] = {T(0), T(0), T(0)};
-    const T* Mg = M + ((int64_t)j * g.nx + i) * kMBlockQ;
+    const T* Mg = &S.Mm[t.ty][t.tx * kMBlockQ];
+    auto add = [&](const T* m, int di, int dj) {
+        T vv[3];
+#pragma unroll
+        for (int s = 0; s < 3; ++s) vv[s] = S.v[s][t.ty + 2 + dj][t.tx + 2 + di];
+#pragma unroll
+        for (int rr = 0; rr < 3; ++rr)
+#pragma unroll
+            for (int s = 0; s < 3; ++s) r[rr] += m[TR ? s * 3 + rr : rr * 3 + s] * vv[s];
+    };
+    auto neighbour = [&](int h, T (&m)[9]) {
+        int di, dj;
+        halfq_offset(h, di, dj);
+        const int x = t.tx - di, y = t.ty - dj;
+        const T* Mn = x >= 0 && x < t.tw && y >= 0
+                          ? &S.Mm[y][x * kMBlockQ]
+                          : M + ((int64_t)wrap1(t.j - dj, g.ny) * g.nx + wrap1(t.i - di, g.nx)) * kMBlockQ;
+#pragma unroll
+        for (int e = 0; e < 9; ++e) m[e] = Mn[h * 9 + e];
+    };
+    // the neighbours' blocks five at a time (h = 3..7, 8..12), each five on
+    // their way while the blocks before them are added
+    T nb[2][5][9];
+#pragma unroll
+    for (int q = 0; q < 5; ++q) neighbour(3 + q, nb[0][q]);
 #pragma unroll
     for (int h = 0; h < kHalfQ; ++h) {
         int di, dj;
         halfq_offset(h, di, dj);
-        const T* Mo = Mg + h * 9;
-        T vv[3];
+        add(Mg + h * 9, di, dj);
+    }
 #pragma unroll
-        for (int s = 0; s < 3; ++s) vv[s] = f(s, 2 + di, 2 + dj);
+    for (int n = 0; n < 2; ++n) {
 #pragma unroll
-        for (int rr = 0; rr < 3; ++rr)
+        for (int q = 0; q < 5; ++q)
+            if (n == 0) neighbour(8 + q, nb[1][q]);
 #pragma unroll
-            for (int s = 0; s < 3; ++s) r[rr] += ld(Mo + (TR ? s * 3 + rr : rr * 3 + s)) * vv[s];
-        if (h == 0) continue;
-        const T* Mn = M + ((int64_t)wrap1(j - dj, g.ny) * g.nx + wrap1(i - di, g.nx)) * kMBlockQ + h * 9;
+        for (int q = 0; q < 5; ++q) {
+            int di, dj;
+            halfq_offset(3 + 5 * n + q, di, dj);
+            add(nb[n][q], -di, -dj);
+        }
+    }
 #pragma unroll
-        for (int s = 0; s < 3; ++s) vv[s] = f(s, 2 - di, 2 - dj);
-#pragma unroll
-        for (int rr = 0; rr < 3; ++rr)
-#pragma unroll
-            for (int s = 0; s < 3; ++s) r[rr] += ld(Mn + (TR ? s * 3 + rr : rr * 3 + s)) * vv[s];
+    for (int h = 1; h < 3; ++h) {
+        T m[9];
+        neighbour(h, m);
+        add(m, -h, 0);
     }
     out[0] = r[0];
     out[1] = r[1];
@@ -508,7 +618,7 @@ __device__ __forceinline__ void mv_q(const T* __restrict__ M, int i, int j, cons
 }
 
 template <typename T, int MODE, bool TR>
-__global__ void __launch_bounds__(kOpTq)
+__global__ void __launch_bounds__(OpQ<T>::threads, 3)
 k_op_q(const T* __restrict__ M, const double* __restrict__ in, double s, const double* __restrict__ b,
        double* __restrict__ out, double* __restrict__ vj, const double* __restrict__ V, int64_t ldv, int nv, GridP g,
        double* __restrict__ partial, const GmDyn* __restrict__ dyn)
@@ -521,75 +631,66 @@ k_op_q(const T* __restrict__ M, const double* __restrict__ in, double s, const d
         out = dyn->out;
         nv = dyn->nv;
     }
-    constexpr int HX = kOpXq + 4, HY = kOpYq + 4;
-    __shared__ T sv[3][HY][HX];
-    __shared__ double buf[kOpChunkq][kOpTq];
-    const int nx = g.nx, ny = g.ny;
+    using O = OpQ<T>;
+    extern __shared__ __align__(128) unsigned char opq_smem[];
+    typename O::Shared& S = *reinterpret_cast<typename O::Shared*>(opq_smem);
+    const AtQ<T> t(g);
     const int64_t nc = g.ncell;
-    const int tx_n = (nx + kOpXq - 1) / kOpXq;
-    const int i0 = (blockIdx.x % tx_n) * kOpXq, j0 = (blockIdx.x / tx_n) * kOpYq;
-    const int tid = threadIdx.x, tx = tid % kOpXq, ty = tid / kOpXq;
-    const int i = i0 + tx, j = j0 + ty;
-    const bool active = i < nx && j < ny;
-    const int64_t gidx = active ? (int64_t)j * nx + i : 0;
-    const T sT = (T)s;
-    for (int q = tid; q < 3 * HY * HX; q += kOpTq) {
-        const int comp = q / (HY * HX), rem = q % (HY * HX), yy = rem / HX, xx = rem % HX;
-        // positions past the tile's last used column/row are clamped (unused)
-        const int gi = wrap1(min(i0 - 2 + xx, 2 * nx - 1), nx), gj = wrap1(min(j0 - 2 + yy, 2 * ny - 1), ny);
-        T val = (T)__ldg(in + comp * nc + (int64_t)gj * nx + gi);
-        if (MODE == kqArnoldi) val *= sT;
-        sv[comp][yy][xx] = val;
-    }
-    __syncthreads();
+    const int tid = threadIdx.x;
+    fetch_rowsq<T>(S, M, t, g);
     double own[3] = {0.0, 0.0, 0.0}, wv[3] = {0.0, 0.0, 0.0};
-    if (active) {
+    if (t.active) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            own[c] = __ldg(in + c * nc + gidx);
+            own[c] = __ldg(in + c * nc + t.gidx);
             if (MODE == kqArnoldi && !is_one(s)) own[c] *= s;
         }
-        auto f1 = [&](int comp, int a, int bb) -> T { return sv[comp][ty + 1 + bb][tx + 1 + a]; };
-        auto f2 = [&](int comp, int a, int bb) -> T { return sv[comp][ty + bb][tx + a]; };
+    }
+    if (MODE == kqArnoldi) stage_inputq<T, true>(S, in, (T)s, t, g);
+    else stage_inputq<T, false>(S, in, T(1), t, g);
+    if (t.active) {
         T cc[3], mv[3];
-        curlcurl_q<T>(f1, gc<T>(g).hdx, gc<T>(g).hdy, cc);
-        mv_q<T, TR>(M, i, j, g, f2, mv);
+        op_curl_n<T>([&](int comp, int p, int o) { return S.C[comp][t.ty + o][t.tx + p]; }, gc<T>(g).hdx, gc<T>(g).hdy,
+                     cc);
+        mv_q<T, TR>(S, M, t, g, mv);
         const T td = gc<T>(g).td;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const double bv = (double)(td * td * cc[c] + td * mv[c]);
+            const double bv = widen(td * td * cc[c] + td * mv[c]);
             if (MODE == kqA) wv[c] = own[c] + bv;
-            else if (MODE == kqResidual) wv[c] = b[c * nc + gidx] - (own[c] + bv);
+            else if (MODE == kqResidual) wv[c] = b[c * nc + t.gidx] - (own[c] + bv);
             else wv[c] = bv;
-            out[c * nc + gidx] = wv[c];
-            if (MODE == kqArnoldi && vj) vj[c * nc + gidx] = own[c];
+            out[c * nc + t.gidx] = wv[c];
+            if (MODE == kqArnoldi && vj) vj[c * nc + t.gidx] = own[c];
         }
     }
     if (MODE == kqA) return;
     const int nq = MODE == kqResidual ? 1 : nv + 2;
     const int lane = tid & 31, wid = tid >> 5;
+    double* buf = reinterpret_cast<double*>(opq_smem);   // [kOpChunkq][threads]
+    __syncthreads();   // the tile is no longer read
     for (int q0 = 0; q0 < nq; q0 += kOpChunkq) {
         const int kc = min(kOpChunkq, nq - q0);
         for (int c = 0; c < kc; ++c) {
             const int q = q0 + c;
             double d = 0.0;
-            if (active) {
+            if (t.active) {
                 if (MODE == kqResidual || q == nv + 1) d = wv[0] * wv[0] + wv[1] * wv[1] + wv[2] * wv[2];
                 else if (q == nv) d = wv[0] * own[0] + wv[1] * own[1] + wv[2] * own[2];
                 else {
-                    const double* Vq = V + (int64_t)q * ldv + gidx;
+                    const double* Vq = V + (int64_t)q * ldv + t.gidx;
                     d = wv[0] * __ldg(Vq) + wv[1] * __ldg(Vq + nc) + wv[2] * __ldg(Vq + 2 * nc);
                 }
             }
-            buf[c][tid] = d;
+            buf[c * O::threads + tid] = d;
         }
         __syncthreads();
-        for (int c = wid; c < kc; c += kOpTq / 32) {
-            double t = 0.0;
+        for (int c = wid; c < kc; c += O::threads / 32) {
+            double sum = 0.0;
 #pragma unroll
-            for (int mm = 0; mm < kOpTq / 32; ++mm) t += buf[c][mm * 32 + lane];
-            t = warp_sum(t);
-            if (lane == 0) partial[(int64_t)blockIdx.x * nq + q0 + c] = t;
+            for (int mm = 0; mm < O::threads / 32; ++mm) sum += buf[c * O::threads + mm * 32 + lane];
+            sum = warp_sum(sum);
+            if (lane == 0) partial[(int64_t)blockIdx.x * nq + q0 + c] = sum;
         }
         __syncthreads();
     }
@@ -597,87 +698,57 @@ k_op_q(const T* __restrict__ M, const double* __restrict__ in, double s, const d
 
 constexpr int kFieldLedgerQ = 6;
 
-// E^{n+theta} -> Eth, E^{n+1}, B^{n+1} of cell (i, j) and the ledger terms
-// 0..4 of the 2D field update; term 5 (the work) by k_work_q
+// E^{n+theta} -> Eth, E^{n+1}, B^{n+1} of cell (i, j) and the ledger terms of
+// the 2D field update, on the operator's tiles (term 5: the work dt dV
+// (Jhat + M E^{n+theta}) . E^{n+theta})
 template <typename T>
-__global__ void __launch_bounds__(256)
-k_field_update_q(const double* __restrict__ x, T* __restrict__ Eth, T* __restrict__ E, const T* __restrict__ B0,
-                 T* __restrict__ B1, GridP g, double* __restrict__ partial)
+__global__ void __launch_bounds__(OpQ<T>::threads, 3)
+k_field_update_q(const double* __restrict__ x, const T* __restrict__ M, const T* __restrict__ J, T* __restrict__ Eth,
+                 T* __restrict__ E, const T* __restrict__ B0, T* __restrict__ B1, GridP g, double* __restrict__ partial)
 {
-    __shared__ double red[32 * 5];
+    using O = OpQ<T>;
+    extern __shared__ __align__(128) unsigned char opq_smem[];
+    typename O::Shared& S = *reinterpret_cast<typename O::Shared*>(opq_smem);
+    const AtQ<T> t(g);
     const int64_t nc = g.ncell;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    T acc[5] = {T(0), T(0), T(0), T(0), T(0)};
-    if (gidx < nc) {
-        const int i = (int)(gidx % g.nx), j = (int)(gidx / g.nx);
-        const T th = gc<T>(g).theta, hdV = gc<T>(g).hdV;
+    fetch_rowsq<T>(S, M, t, g);
+    stage_inputq<T, false>(S, x, T(1), t, g);
+    T acc[kFieldLedgerQ] = {T(0), T(0), T(0), T(0), T(0), T(0)};
+    if (t.active) {
+        const T th = gc<T>(g).theta, hdV = gc<T>(g).hdV, dt = gc<T>(g).dt;
+        T mv[3], wk = T(0);
+        mv_q<T, false>(S, M, t, g, mv);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
-            const T et = (T)x[c * nc + gidx];
-            const T e0 = E[c * nc + gidx];
+            const T et = S.v[c][t.ty + 2][t.tx + 2];
+            const T e0 = E[c * nc + t.gidx];
             const T e1 = (et - (T(1) - th) * e0) / th;
-            Eth[c * nc + gidx] = et;
-            E[c * nc + gidx] = e1;
+            Eth[c * nc + t.gidx] = et;
+            E[c * nc + t.gidx] = e1;
             acc[0] += hdV * (e1 - e0) * (e1 + e0);
             acc[2] += (e1 - e0) * (e1 - e0);
             acc[3] += hdV * e1 * e1;
-        }
-        const int i1 = wrap1(i + 1, g.nx), j1 = wrap1(j + 1, g.ny);
-        const int64_t n00 = (int64_t)j * g.nx + i, n10 = (int64_t)j * g.nx + i1;
-        const int64_t n01 = (int64_t)j1 * g.nx + i, n11 = (int64_t)j1 * g.nx + i1;
-        const T idx2 = gc<T>(g).hdx, idy2 = gc<T>(g).hdy;
-        T dxE[3], dyE[3];
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const T a = (T)x[c * nc + n00], bq = (T)x[c * nc + n10], cq = (T)x[c * nc + n01], d = (T)x[c * nc + n11];
-            dxE[c] = (bq - a + d - cq) * idx2;
-            dyE[c] = (cq - a + d - bq) * idy2;
-        }
-        const T curl[3] = {dyE[2], -dxE[2], dxE[1] - dyE[0]};
-        const T dt = gc<T>(g).dt;
-#pragma unroll
-        for (int c = 0; c < 3; ++c) {
-            const T b0 = B0[c * nc + gidx];
-            const T b1 = b0 - dt * curl[c];
-            B1[c * nc + gidx] = b1;
+            wk += (J[c * nc + t.gidx] + mv[c]) * et;
+            // the cell's curl is that of the centre after the node's in x and y
+            const T b0 = B0[c * nc + t.gidx];
+            const T b1 = b0 - dt * S.C[c][t.ty + 1][t.tx + 1];
+            B1[c * nc + t.gidx] = b1;
             acc[1] += hdV * (b1 - b0) * (b1 + b0);
             acc[2] += (b1 - b0) * (b1 - b0);
             acc[4] += hdV * b1 * b1;
         }
         acc[2] *= gc<T>(g).thdV;
+        acc[5] = gc<T>(g).dtdV * wk;
     }
-    double v[5], o[5];
+    double* red = reinterpret_cast<double*>(opq_smem);
+    __syncthreads();   // the tile is no longer read
+    double v[kFieldLedgerQ], o[kFieldLedgerQ];
 #pragma unroll
-    for (int q = 0; q < 5; ++q) v[q] = (double)acc[q];
-    block_sum<5>(v, red, o);
+    for (int q = 0; q < kFieldLedgerQ; ++q) v[q] = (double)acc[q];
+    block_sum<kFieldLedgerQ>(v, red, o);
     if (threadIdx.x == 0)
 #pragma unroll
-        for (int q = 0; q < 5; ++q) partial[(int64_t)blockIdx.x * kFieldLedgerQ + q] = o[q];
-}
-
-template <typename T>
-__global__ void __launch_bounds__(256)
-k_work_q(const T* __restrict__ M, const T* __restrict__ J, const T* __restrict__ Eth, GridP g,
-         double* __restrict__ partial)
-{
-    __shared__ double red[32];
-    const int64_t nc = g.ncell;
-    const int64_t gidx = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
-    T wk = T(0);
-    if (gidx < nc) {
-        const int i = (int)(gidx % g.nx), j = (int)(gidx / g.nx);
-        auto f = [&](int comp, int a, int b) -> T {
-            return ld(Eth + comp * nc + (int64_t)wrap1(j - 2 + b, g.ny) * g.nx + wrap1(i - 2 + a, g.nx));
-        };
-        T mv[3];
-        mv_q<T, false>(M, i, j, g, f, mv);
-#pragma unroll
-        for (int c = 0; c < 3; ++c) wk += (J[c * nc + gidx] + mv[c]) * Eth[c * nc + gidx];
-        wk *= gc<T>(g).dtdV;
-    }
-    double v[1] = {(double)wk}, o[1];
-    block_sum<1>(v, red, o);
-    if (threadIdx.x == 0) partial[(int64_t)blockIdx.x * kFieldLedgerQ + 5] = o[0];
+        for (int q = 0; q < kFieldLedgerQ; ++q) partial[(int64_t)blockIdx.x * kFieldLedgerQ + q] = o[q];
 }
 
 // ---------------------------------------------------------------------------
@@ -853,15 +924,25 @@ cudaError_t deposit_q(const DepositSpecies<T>& ds, const T* B, T* M, T* J, GridP
     return cudaGetLastError();
 }
 
-int op_blocks_q(GridP g) { return ((g.nx + kOpXq - 1) / kOpXq) * ((g.ny + kOpYq - 1) / kOpYq); }
+template <typename T>
+static int tiles_q(const GridP& g)
+{
+    using O = OpQ<T>;
+    return ((g.nx + O::X - 1) / O::X) * ((g.ny + O::Y - 1) / O::Y);
+}
+int op_blocks_q(GridP g, int precision) { return precision == 32 ? tiles_q<float>(g) : tiles_q<double>(g); }
 
 template <typename T, int MODE, bool TR>
 cudaError_t launch_op_q(const T* M, const double* in, double sc, const double* b, double* out, double* vj,
                         const double* V, int64_t ldv, int nv, GridP g, double* partial, cudaStream_t st,
                         const GmDyn* dyn)
 {
+    const int smem = (int)sizeof(typename OpQ<T>::Shared);
+    const cudaError_t e = cudaFuncSetAttribute(k_op_q<T, MODE, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
     count_launches(1);
-    k_op_q<T, MODE, TR><<<op_blocks_q(g), kOpTq, 0, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial, dyn);
+    k_op_q<T, MODE, TR><<<tiles_q<T>(g), OpQ<T>::threads, smem, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial,
+                                                                      dyn);
     return cudaGetLastError();
 }
 
@@ -869,9 +950,11 @@ template <typename T>
 cudaError_t field_update_q(const double* x, const T* M, const T* J, T* Eth, T* E, const T* B0, T* B1, GridP g,
                            double* partial, int nblocks, cudaStream_t st)
 {
-    count_launches(2);
-    k_field_update_q<T><<<nblocks, 256, 0, st>>>(x, Eth, E, B0, B1, g, partial);
-    k_work_q<T><<<nblocks, 256, 0, st>>>(M, J, Eth, g, partial);
+    const int smem = (int)sizeof(typename OpQ<T>::Shared);
+    const cudaError_t e = cudaFuncSetAttribute(k_field_update_q<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    if (e != cudaSuccess) return e;
+    count_launches(1);
+    k_field_update_q<T><<<nblocks, OpQ<T>::threads, smem, st>>>(x, M, J, Eth, E, B0, B1, g, partial);
     return cudaGetLastError();
 }
 

@@ -72,6 +72,8 @@ struct StepGraph {
     uint64_t gen = 0;
     int bcur = -1;
     int32_t* start[kMaxSpecies] = {};
+    int64_t n[kMaxSpecies] = {};   // particles and current buffer of each species
+    int cur[kMaxSpecies] = {};
     long long k_static = 0, k_cycle = 0, k_iter = 0;   // kernels outside the loops, per cycle, per iteration
 };
 
@@ -124,7 +126,7 @@ struct relsim_ctx {
     GmState* ghead = nullptr;  // pinned host, two read-back slots (heads only)
     // step graphs (two layouts alternate from step to step)
     StepGraph sg[2];
-    uint64_t gen = 1;          // bumped whenever a buffer or the loaded state changes
+    uint64_t gen = 1;          // bumped whenever a buffer or a launch shape changes
     bool graph_off = false;    // a capture failed: host-driven steps from then on
     std::string graph_why;     // why
     int dep_blocks = 0;        // launch shapes chosen by relsim_autotune (0: defaults)
@@ -1311,13 +1313,29 @@ int capture_step(relsim_ctx* c, StepGraph& G)
     if (r != RELSIM_OK) return r;
     G.gen = c->gen;
     G.bcur = c->bcur;
-    for (int s = 0; s < kMaxSpecies; ++s) G.start[s] = c->sp[s].start;
+    for (int s = 0; s < kMaxSpecies; ++s) {
+        G.start[s] = c->sp[s].start;
+        G.n[s] = c->sp[s].n;
+        G.cur[s] = c->sp[s].cur;
+    }
     return RELSIM_OK;
+}
+
+// captured on the context's buffers and counts (of either step parity). A
+// load of as many particles into the same buffers leaves them as they are, so
+// a run that reloads states (the segments of a differentiable window) keeps
+// its graphs; captured anew at every load they cost about a millisecond each
+bool graph_current(const relsim_ctx* c, const StepGraph& G)
+{
+    if (!G.exec || G.gen != c->gen) return false;
+    for (int s = 0; s < kMaxSpecies; ++s)
+        if (G.n[s] != c->sp[s].n || G.cur[s] != c->sp[s].cur) return false;
+    return true;
 }
 
 bool graph_matches(const relsim_ctx* c, const StepGraph& G)
 {
-    if (!G.exec || G.gen != c->gen || G.bcur != c->bcur) return false;
+    if (!graph_current(c, G) || G.bcur != c->bcur) return false;
     for (int s = 0; s < kMaxSpecies; ++s)
         if (G.start[s] != c->sp[s].start) return false;
     return true;
@@ -1333,7 +1351,7 @@ int step_graph(relsim_ctx* c, relsim_energy* ledger, int* status)
         if (graph_matches(c, g)) G = &g;
     if (!G) {
         // replace the slot not matching the other parity's layout
-        G = &c->sg[c->sg[0].exec && c->sg[0].gen == c->gen && c->sg[0].bcur != c->bcur ? 1 : 0];
+        G = &c->sg[graph_current(c, c->sg[0]) && c->sg[0].bcur != c->bcur ? 1 : 0];
         if (capture_step<T>(c, *G) != RELSIM_OK) {
             c->graph_off = true;
             c->graph_why = c->err;
@@ -1683,6 +1701,8 @@ struct SharedKey {
     uint64_t gen = 0;
     int bcur = -1;
     int32_t* start[kMaxSpecies] = {};
+    int64_t n[kMaxSpecies] = {};
+    int cur[kMaxSpecies] = {};
 };
 
 struct relsim_shared {
@@ -1814,7 +1834,11 @@ int shared_capture(relsim_shared* sb, int k)
             SharedKey& q = sb->key[k][i];
             q.gen = sb->c[i]->gen;
             q.bcur = sb->c[i]->bcur;
-            for (int s = 0; s < kMaxSpecies; ++s) q.start[s] = sb->c[i]->sp[s].start;
+            for (int s = 0; s < kMaxSpecies; ++s) {
+                q.start[s] = sb->c[i]->sp[s].start;
+                q.n[s] = sb->c[i]->sp[s].n;
+                q.cur[s] = sb->c[i]->sp[s].cur;
+            }
         }
     }
     return r;
@@ -1831,7 +1855,8 @@ int shared_slot(const relsim_shared* sb)
             const relsim_ctx* c = sb->c[i];
             const SharedKey& q = sb->key[k][i];
             ok = q.gen == c->gen && q.bcur == c->bcur && graph_eligible(c);
-            for (int s = 0; s < kMaxSpecies && ok; ++s) ok = q.start[s] == c->sp[s].start;
+            for (int s = 0; s < kMaxSpecies && ok; ++s)
+                ok = q.start[s] == c->sp[s].start && q.n[s] == c->sp[s].n && q.cur[s] == c->sp[s].cur;
         }
         if (ok) return k;
     }
@@ -2422,7 +2447,6 @@ int relsim_load_particles(relsim_ctx* c, int species, int64_t n, const double* x
                           const double* w, int where)
 {
     if (!c) return RELSIM_ERR_INVALID_ARG;
-    ++c->gen;
     if (species < 0 || species >= c->cfg.nspecies)
         return fail(c, RELSIM_ERR_INVALID_ARG, "species %d out of range", species);
     if (n < 0 || n > 2147483647LL) return fail(c, RELSIM_ERR_INVALID_ARG, "bad particle count %lld", (long long)n);
@@ -2440,7 +2464,6 @@ int relsim_load_particles(relsim_ctx* c, int species, int64_t n, const double* x
 int relsim_set_fields(relsim_ctx* c, const double* E, const double* B, int where)
 {
     if (!c) return RELSIM_ERR_INVALID_ARG;
-    ++c->gen;
     if (where != RELSIM_HOST && where != RELSIM_DEVICE) return fail(c, RELSIM_ERR_INVALID_ARG, "bad where");
     if (c->state == kSolved) c->bcur = 1 - c->bcur;   // the solved fields become current
     int r = DISPATCH(set_fields_impl, c, E, B, where);
@@ -2482,7 +2505,6 @@ int relsim_load_particles_native(relsim_ctx* c, int species, int64_t n, const in
                                  const void* u, const void* w, const int32_t* id, int where)
 {
     if (!c) return RELSIM_ERR_INVALID_ARG;
-    ++c->gen;
     if (species < 0 || species >= c->cfg.nspecies)
         return fail(c, RELSIM_ERR_INVALID_ARG, "species %d out of range", species);
     if (n < 0 || n > 2147483647LL) return fail(c, RELSIM_ERR_INVALID_ARG, "bad particle count %lld", (long long)n);
@@ -2575,7 +2597,6 @@ int relsim_set_mass_matrix(relsim_ctx* c, const double* M, const double* J, int 
 {
     if (!c || !M || !J) return RELSIM_ERR_INVALID_ARG;
     if (where != RELSIM_HOST && where != RELSIM_DEVICE) return fail(c, RELSIM_ERR_INVALID_ARG, "bad where");
-    ++c->gen;
     if (c->state == kEmpty) return fail(c, RELSIM_ERR_BAD_STATE, "context not initialised");
     if (c->state == kSolved) return fail(c, RELSIM_ERR_BAD_STATE, "push the solved step first");
     const int64_t nm = (int64_t)c->g.ncell * mblock_of(c->g), nj = 3 * (int64_t)c->g.ncell;

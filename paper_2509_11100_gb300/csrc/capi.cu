@@ -414,19 +414,25 @@ int load_impl(relsim_ctx* c, int s, int64_t n, const double* x, const double* u,
         else
             CK(load_convert<T>(dx, du, dw, n, c->g, tmp, c->rk[0], c->rv[0], c->dflag, c->st));
         CK(keys_unsorted(c->rk[0], n, c->dflag, c->st));
+        CK(histogram_keys(c->rk[0], n, c->count_new, c->g.ncell, c->st));
+        CK(cells_above(c->count_new, c->g.ncell, c->dflag, c->st));
+        CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp,
+                              c->st));
         PROF_END();
         CK(cudaMemcpyAsync(c->hflag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
         CK(cudaStreamSynchronize(c->st));
         if (*c->hflag & 1) return fail(c, RELSIM_ERR_NONFINITE, "non-finite value in particles");
         PROF_BEGIN(RELSIM_PROF_LOAD);
-        const int32_t* keys = c->rk[0];
         if (*c->hflag & 2) {
             // the stable sort by cell, then the particles gathered in that order
-            bool in1 = false;
-            CK(radix_sort_pairs(c->rk[0], c->rv[0], c->rk[1], c->rv[1], n, c->key_bits, c->rtmp, &in1,
-                                c->st));
-            keys = c->rk[in1 ? 1 : 0];
-            const int32_t* perm = c->rv[in1 ? 1 : 0];
+            const int32_t* perm = c->rv[1];
+            if (*c->hflag & 8) {   // crowded cells
+                bool in1 = false;
+                CK(radix_sort_pairs(c->rk[0], c->rv[0], c->rk[1], c->rv[1], n, c->key_bits, c->rtmp, &in1, c->st));
+                perm = c->rv[in1 ? 1 : 0];
+            } else {
+                CK(stable_cell_order(c->rk[0], n, sp.start, c->g.ncell, c->count_new, c->rk[1], c->rv[1], c->st));
+            }
             if (D == 3)
                 CK(gather_particles3<T>(perm, tmp, (const T*)sp.a[1][6], dst, (T*)sp.a[0][6], n, true, c->st));
             else
@@ -438,9 +444,6 @@ int load_impl(relsim_ctx* c, int s, int64_t n, const double* x, const double* u,
             if (tmp.id)
                 CK(cudaMemcpyAsync(tmp.id, c->rv[0], sizeof(int32_t) * (size_t)n, cudaMemcpyDeviceToDevice, c->st));
         }
-        CK(histogram_keys(keys, n, c->count_new, c->g.ncell, c->st));
-        CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp,
-                              c->st));
         PROF_END();
     }
     // kinetic energy of the loaded species -> ledger slot K1

@@ -905,7 +905,7 @@ int solve_prologue(relsim_ctx* c, const GmSetup& S, cudaStream_t s, GmCond outer
 {
     TRY(solve_rhs<T>(c, S, s));
     PROF_BEGIN(RELSIM_PROF_GMRES_ORTHO);
-    CK(gm_dots(c->V, S.ldv, 0, c->gb, S.n, c->partial, S.nb, s, c->g.df));
+    CK(gm_norm2(c->gb, S.n, c->partial, S.nb, s, c->g.df));
     CK(reduce_partials(c->partial, S.nb, 1, c->dsum, s));
     CK(gm_begin(c->gms, c->dsum, s));
     CK(gm_zero_x(c->gms, c->gx, S.n, s));
@@ -926,9 +926,8 @@ int arnoldi_body(relsim_ctx* c, const GmSetup& S, cudaStream_t s, GmCond inner, 
     CK(op_arnoldi_dyn<T>((const T*)c->M, &c->gms->dyn, c->V, S.ldv, c->g, c->partial, c->dpush, s, tr));
     PROF_END();
     PROF_BEGIN(RELSIM_PROF_GMRES_ORTHO);
-    CK(reduce_partials_dyn(c->partial, S.nbo, &c->gms->dyn, S.m + 2, s));
-    CK(gm_update_scale_dyn(&c->gms->dyn, c->V, S.ldv, S.n, s, c->g.df));
-    CK(gm_tail(c->gms, S.p, S.q, inner, s));
+    CK(reduce_partials_dyn(c->partial, S.nbo, c->gms, S.m, s));
+    CK(gm_update_scale_dyn(c->gms, S.p, S.q, inner, S.n, s, c->g.df));
     PROF_END();
     return RELSIM_OK;
 }
@@ -938,7 +937,7 @@ template <typename T>
 int cycle_end(relsim_ctx* c, const GmSetup& S, cudaStream_t s, GmCond outer, bool tr = false)
 {
     PROF_BEGIN(RELSIM_PROF_GMRES_ORTHO);
-    CK(gm_finish_cycle(c->gms, c->gx, c->V, S.ldv, S.n, S.m, s, c->g.df));
+    CK(gm_combine_dev(c->gx, c->V, S.ldv, &c->gms->kdim, c->gms->y, S.n, s, c->g.df));
     PROF_END();
     PROF_BEGIN(RELSIM_PROF_GMRES_APPLY);
     CK(op_residual<T>((const T*)c->M, c->gx, c->gb, S.p.r, c->g, c->partial, c->dpush, s, tr));
@@ -1412,7 +1411,7 @@ int adjoint_impl(relsim_ctx* c, const double* gE1, const double* gB1, const doub
         TRY(solve_launch<T>(c, S, c->st, true));
         TRY(solve_read(c));
     } else {
-        CK(gm_dots(c->V, S.ldv, 0, c->gb, S.n, c->partial, S.nb, c->st, c->g.df));
+        CK(gm_norm2(c->gb, S.n, c->partial, S.nb, c->st, c->g.df));
         CK(reduce_partials(c->partial, S.nb, 1, c->dsum, c->st));
         CK(gm_begin(c->gms, c->dsum, c->st));
         CK(op_residual<T>((const T*)c->M, c->gx, c->gb, S.p.r, c->g, c->partial, c->dpush, c->st, true));

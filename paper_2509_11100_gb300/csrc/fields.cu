@@ -18,6 +18,7 @@
 #include <atomic>
 
 #include "dfloat.cuh"
+#include "gmtail.cuh"
 #include "launch.cuh"
 #include "opcore.cuh"
 
@@ -521,51 +522,28 @@ __global__ void k_mass_from_double(const double* __restrict__ Md, const double* 
 // by Dot2 / Sum2-style compensation on the FP32 pipe
 
 constexpr int kGmThreads = 256;
-constexpr int kDotChunk = 8;
-
 template <bool DF>
 __global__ void __launch_bounds__(kGmThreads)
-k_gm_dots(const double* __restrict__ V, int64_t ldv, int k0, int kc, const double* __restrict__ w,
-          int64_t n, double* __restrict__ partial, int stride, bool with_ww)
+k_gm_norm2(const double* __restrict__ w, int64_t n, double* __restrict__ partial)
 {
-    __shared__ double red[32 * (kDotChunk + 1)];
-    double out[kDotChunk + 1];
+    __shared__ double red[32];
+    double out[1];
     if constexpr (DF) {
-        Dot2 acc[kDotChunk + 1];
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
+        Dot2 acc;
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
             const dfl we = dld(w, e);
-#pragma unroll
-            for (int c = 0; c < kDotChunk; ++c) {
-                if (c >= kc) break;
-                acc[c].add(dld(V + (int64_t)(k0 + c) * ldv, e), we);
-            }
-            if (with_ww) acc[kDotChunk].add(we, we);
+            acc.add(we, we);
         }
-        dfl v[kDotChunk + 1];
-#pragma unroll
-        for (int c = 0; c <= kDotChunk; ++c) v[c] = acc[c].value();
-        df_block_sum<kDotChunk + 1>(v, reinterpret_cast<dfl*>(red), out);
+        dfl v[1] = {acc.value()};
+        df_block_sum<1>(v, reinterpret_cast<dfl*>(red), out);
     } else {
-        double acc[kDotChunk + 1];
-#pragma unroll
-        for (int c = 0; c <= kDotChunk; ++c) acc[c] = 0.0;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            const double we = w[e];
-#pragma unroll
-            for (int c = 0; c < kDotChunk; ++c) {
-                if (c >= kc) break;   // a branch: no predicated-off FP64 work
-                acc[c] += V[(int64_t)(k0 + c) * ldv + e] * we;
-            }
-            if (with_ww) acc[kDotChunk] += we * we;
-        }
-        block_sum<kDotChunk + 1>(acc, red, out);
+        double acc = 0.0;
+        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x)
+            acc += w[e] * w[e];
+        double v[1] = {acc};
+        block_sum<1>(v, red, out);
     }
-    if (threadIdx.x == 0) {
-        for (int c = 0; c < kc; ++c) partial[(int64_t)blockIdx.x * stride + k0 + c] = out[c];
-        if (with_ww) partial[(int64_t)blockIdx.x * stride + stride - 1] = out[kDotChunk];
-    }
+    if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
 }
 
 constexpr int kGmChunk = 8;   // basis vectors per group of independent loads
@@ -594,95 +572,36 @@ __device__ __forceinline__ dfl df_sub_combination(dfl w, const dfl* hs, const do
     return d.value();
 }
 
+// v_{k} = (w - sum_{c<k} h_c V_c)/hn with hn^2 = <w,w> - sum h_c^2 (h and <w,w>
+// from the dot-product sums hw = [h_0 .. h_{k-1}, <w,w>]; every block forms hn
+// itself), on nblk blocks of which this is the blk-th
 template <bool DF>
-__global__ void __launch_bounds__(kGmThreads)
-k_gm_update(double* __restrict__ w, const double* __restrict__ V, int64_t ldv, int k,
-            const double* __restrict__ h, int64_t n, double* __restrict__ partial)
-{
-    __shared__ double hs[kMaxRestart + 1];
-    __shared__ double red[32];
-    for (int c = threadIdx.x; c < k; c += blockDim.x) {
-        if constexpr (DF) reinterpret_cast<dfl*>(hs)[c] = df_from_double(h[c]);
-        else hs[c] = h[c];
-    }
-    __syncthreads();
-    double out[1];
-    if constexpr (DF) {
-        Dot2 acc;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            const dfl s = df_sub_combination(dld(w, e), reinterpret_cast<const dfl*>(hs), V, ldv, k, e, -1.f);
-            reinterpret_cast<dfl*>(w)[e] = s;
-            acc.add(s, s);
-        }
-        dfl v[1] = {acc.value()};
-        df_block_sum<1>(v, reinterpret_cast<dfl*>(red), out);
-    } else {
-        double acc = 0.0;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            double s = w[e];
-            for (int c0 = 0; c0 < k; c0 += kGmChunk) {
-                const int kc = min(kGmChunk, k - c0);
-                double vv[kGmChunk];
-#pragma unroll
-                for (int c = 0; c < kGmChunk; ++c) vv[c] = c < kc ? __ldg(V + (int64_t)(c0 + c) * ldv + e) : 0.0;
-#pragma unroll
-                for (int c = 0; c < kGmChunk; ++c) {
-                    if (c >= kc) break;   // a branch: no predicated-off FP64 work
-                    s -= hs[c0 + c] * vv[c];
-                }
-            }
-            w[e] = s;
-            acc += s * s;
-        }
-        double v[1] = {acc};
-        block_sum<1>(v, red, out);
-    }
-    if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
-}
-
-// Arnoldi update with the normalisation fused: v_{k} = (w - sum_{c<k} h_c V_c)/hn
-// with hn^2 = <w,w> - sum h_c^2 (h and <w,w> from the dot-product sums hw =
-// [h_0 .. h_{k-1}, <w,w>]; every block forms hn itself).
-template <bool DF>
-__global__ void __launch_bounds__(kGmThreads)
-k_gm_update_scale(const double* __restrict__ w, const double* __restrict__ V, int64_t ldv, int k,
-                  const double* __restrict__ hw, double* __restrict__ vout, int64_t n,
-                  const GmDyn* __restrict__ dyn)
+__device__ __forceinline__ void update_scale(const double* __restrict__ w, const double* __restrict__ V, int64_t ldv,
+                                             int k, const double* __restrict__ hw, double* __restrict__ vout, int64_t n,
+                                             int blk, int nblk)
 {
     __shared__ double hs[kMaxRestart + 1];
     __shared__ double inv;
-    if (dyn) {
-        if (!dyn->live) return;
-        w = dyn->out;
-        k = dyn->nv + 1;
-        hw = dyn->ds;
-        vout = const_cast<double*>(V) + (int64_t)k * ldv;
-    }
     for (int c = threadIdx.x; c < k; c += blockDim.x) {
         if constexpr (DF) reinterpret_cast<dfl*>(hs)[c] = df_from_double(hw[c]);
         else hs[c] = hw[c];
     }
     if (threadIdx.x == 0) {
-        double h2 = hw[k];
-        for (int c = 0; c < k; ++c) h2 -= hw[c] * hw[c];
-        const double iv = h2 > 0.0 ? 1.0 / sqrt(h2) : 0.0;
+        const double h2 = gm_rest2(hw, k - 1);
+        const double iv = h2 > 0.0 ? rsqrt(h2) : 0.0;
         if constexpr (DF) *reinterpret_cast<dfl*>(&inv) = df_from_double(iv);
         else inv = iv;
     }
     __syncthreads();
     if constexpr (DF) {
         const dfl sc = *reinterpret_cast<const dfl*>(&inv);
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
+        for (int64_t e = (int64_t)blk * blockDim.x + threadIdx.x; e < n; e += (int64_t)nblk * blockDim.x) {
             const dfl s = df_sub_combination(dld(w, e), reinterpret_cast<const dfl*>(hs), V, ldv, k, e, -1.f);
             reinterpret_cast<dfl*>(vout)[e] = df_mul(s, sc);
         }
     } else {
         const double sc = inv;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
+        for (int64_t e = (int64_t)blk * blockDim.x + threadIdx.x; e < n; e += (int64_t)nblk * blockDim.x) {
             double s = w[e];
             for (int c0 = 0; c0 < k; c0 += kGmChunk) {
                 const int kc = min(kGmChunk, k - c0);
@@ -700,50 +619,55 @@ k_gm_update_scale(const double* __restrict__ w, const double* __restrict__ V, in
     }
 }
 
-template <bool DF>
-__global__ void k_gm_scale(double* dst, const double* __restrict__ src, double s, int64_t n)
-{
-    if constexpr (DF) {
-        const dfl sd = df_from_double(s);
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x)
-            reinterpret_cast<dfl*>(dst)[e] = df_mul(dld(src, e), sd);
-    } else {
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x)
-            dst[e] = src[e] * s;
-    }
-}
-
+// The basis update of the running iteration (arguments in st->cur, which the
+// reduction kept there: the tail writes the next iteration's into st->dyn
+// while other blocks still read these). Block 0 runs the tail.
 template <bool DF>
 __global__ void __launch_bounds__(kGmThreads)
-k_gm_sub(double* r, const double* __restrict__ b, const double* __restrict__ Ax, int64_t n,
-         double* partial)
+k_gm_update_tail(GmState* __restrict__ st, GmPtrs p, GmParams q, cudaGraphConditionalHandle cond, int has_cond, int64_t n)
 {
-    __shared__ double red[32];
-    double out[1];
-    if constexpr (DF) {
-        Dot2 acc;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            const dfl s = df_sub(dld(b, e), dld(Ax, e));
-            reinterpret_cast<dfl*>(r)[e] = s;
-            acc.add(s, s);
+    const GmDyn& cur = st->cur;
+    if (blockIdx.x != 0) {
+        if (cur.live) {
+            const int k = cur.nv + 1;
+            update_scale<DF>(cur.out, p.V, p.ldv, k, cur.ds, p.V + (int64_t)k * p.ldv, n, blockIdx.x - 1, gridDim.x - 1);
         }
-        dfl v[1] = {acc.value()};
-        df_block_sum<1>(v, reinterpret_cast<dfl*>(red), out);
-    } else {
-        double acc = 0.0;
-        for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n;
-             e += (int64_t)gridDim.x * blockDim.x) {
-            double s = b[e] - Ax[e];
-            r[e] = s;
-            acc += s * s;
-        }
-        double v[1] = {acc};
-        block_sum<1>(v, red, out);
+        return;
     }
-    if (threadIdx.x == 0) partial[blockIdx.x] = out[0];
+    if (threadIdx.x >= 32) return;
+    const int lane = threadIdx.x;
+    int go = 0, kd = 0, status = kGmOk;
+    const int j = cur.nv, live = cur.live;
+    if (live) {
+        const double* hj = cur.ds;
+        const double hn2 = gm_rest2(hj, j);
+        const int total = st->total + 1;
+        __syncwarp();
+        gm_tail_warp(GmTail{st->H, st->cs, st->sn, st->gv, st->rinv, st->y, q.m}, hj, j, hn2,
+                     hn2 > 0.0 ? rsqrt(hn2) : 0.0, q.tol * st->bnorm, total, q.maxit, lane, go, kd, status);
+        if (lane == 0) {
+            st->total = total;
+            st->kdim = kd;
+            if (status != kGmOk) {
+                st->status = status;
+                st->run = 0;
+            }
+        }
+    }
+    if (lane != 0) return;
+    GmDyn& d = st->dyn;
+    if (go) {
+        const int jn = j + 1;
+        d.in = p.V + (int64_t)jn * p.ldv;
+        d.vj = nullptr;
+        d.out = jn % 2 == 0 ? p.w0 : p.r;
+        d.ds = jn % 2 == 0 ? p.ds0 : p.ds1;
+        d.s = 1.0;
+        d.nv = jn;
+    }
+    d.live = go;
+    st->inner = go;
+    if (has_cond) cudaGraphSetConditional(cond, go);
 }
 
 template <bool DF>
@@ -782,14 +706,16 @@ __global__ void k_gm_combine(double* x, const double* __restrict__ V, int64_t ld
 
 // out[s] = sum_b partial[b*nsums + s], fixed order (deterministic)
 __global__ void k_reduce_partials(const double* __restrict__ partial, int nblocks, int nsums,
-                                  double* out, const GmDyn* __restrict__ dyn)
+                                  double* out, GmState* __restrict__ st)
 {
     __shared__ double red[32];
     const int s = blockIdx.x;
-    if (dyn) {
-        if (!dyn->live) return;
-        nsums = dyn->nv + 2;
-        out = dyn->ds;
+    if (st) {
+        const GmDyn& dyn = st->dyn;
+        if (s == 0 && threadIdx.x == 0) st->cur = dyn;
+        if (!dyn.live) return;
+        nsums = dyn.nv + 2;
+        out = dyn.ds;
         if (s >= nsums) return;
     }
     // the loads of a thread's strided partials issued together (U in
@@ -1023,80 +949,29 @@ cudaError_t mass_from_double(const double* Md, const double* Jd, T* M, T* J, Gri
     return cudaGetLastError();
 }
 
-cudaError_t gm_dots(const double* V, int64_t ldv, int k, const double* w, int64_t n,
-                    double* partial, int nblocks, cudaStream_t st, int df)
+cudaError_t gm_norm2(const double* w, int64_t n, double* partial, int nblocks, cudaStream_t st, int df)
 {
-    // partial row stride k+1: k dots then w.w
-    for (int k0 = 0; k0 < k || k0 == 0; k0 += kDotChunk) {
-        int kc = k - k0 < kDotChunk ? k - k0 : kDotChunk;
-        if (kc < 0) kc = 0;
-        count_launches(1);
-        if (df) k_gm_dots<true><<<nblocks, kGmThreads, 0, st>>>(V, ldv, k0, kc, w, n, partial, k + 1, k0 == 0);
-        else k_gm_dots<false><<<nblocks, kGmThreads, 0, st>>>(V, ldv, k0, kc, w, n, partial, k + 1, k0 == 0);
-        if (k0 + kDotChunk >= k) break;
-    }
+    count_launches(1);
+    if (df) k_gm_norm2<true><<<nblocks, kGmThreads, 0, st>>>(w, n, partial);
+    else k_gm_norm2<false><<<nblocks, kGmThreads, 0, st>>>(w, n, partial);
     return cudaGetLastError();
 }
 
-cudaError_t gm_update(double* w, const double* V, int64_t ldv, int k, const double* h, int64_t n,
-                      double* partial, int nblocks, cudaStream_t st, int df)
+
+
+cudaError_t gm_update_scale_dyn(GmState* st, const GmPtrs& p, const GmParams& q, GmCond cond, int64_t n, cudaStream_t s,
+                                int df)
 {
     count_launches(1);
-    if (df) k_gm_update<true><<<nblocks, kGmThreads, 0, st>>>(w, V, ldv, k, h, n, partial);
-    else k_gm_update<false><<<nblocks, kGmThreads, 0, st>>>(w, V, ldv, k, h, n, partial);
+    const int nb = grid_for(n, kGmThreads, 152 * 8) + 1;
+    const auto h = (cudaGraphConditionalHandle)cond.h;
+    if (df) k_gm_update_tail<true><<<nb, kGmThreads, 0, s>>>(st, p, q, h, cond.has, n);
+    else k_gm_update_tail<false><<<nb, kGmThreads, 0, s>>>(st, p, q, h, cond.has, n);
     return cudaGetLastError();
 }
 
-cudaError_t gm_update_scale(const double* w, const double* V, int64_t ldv, int k, const double* hw,
-                            double* vout, int64_t n, cudaStream_t st, int df)
-{
-    count_launches(1);
-    if (df)
-        k_gm_update_scale<true><<<grid_for(n, kGmThreads, 152 * 8), kGmThreads, 0, st>>>(w, V, ldv, k, hw, vout, n,
-                                                                                        nullptr);
-    else
-        k_gm_update_scale<false><<<grid_for(n, kGmThreads, 152 * 8), kGmThreads, 0, st>>>(w, V, ldv, k, hw, vout, n,
-                                                                                         nullptr);
-    return cudaGetLastError();
-}
 
-cudaError_t gm_update_scale_dyn(const GmDyn* dyn, const double* V, int64_t ldv, int64_t n, cudaStream_t st, int df)
-{
-    count_launches(1);
-    if (df)
-        k_gm_update_scale<true><<<grid_for(n, kGmThreads, 152 * 8), kGmThreads, 0, st>>>(nullptr, V, ldv, 0, nullptr,
-                                                                                        nullptr, n, dyn);
-    else
-        k_gm_update_scale<false><<<grid_for(n, kGmThreads, 152 * 8), kGmThreads, 0, st>>>(nullptr, V, ldv, 0,
-                                                                                         nullptr, nullptr, n, dyn);
-    return cudaGetLastError();
-}
 
-cudaError_t gm_scale(double* dst, const double* src, double s, int64_t n, cudaStream_t st, int df)
-{
-    count_launches(1);
-    if (df) k_gm_scale<true><<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(dst, src, s, n);
-    else k_gm_scale<false><<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(dst, src, s, n);
-    return cudaGetLastError();
-}
-
-cudaError_t gm_sub(double* r, const double* b, const double* Ax, int64_t n, double* partial,
-                   int nblocks, cudaStream_t st, int df)
-{
-    count_launches(1);
-    if (df) k_gm_sub<true><<<nblocks, kGmThreads, 0, st>>>(r, b, Ax, n, partial);
-    else k_gm_sub<false><<<nblocks, kGmThreads, 0, st>>>(r, b, Ax, n, partial);
-    return cudaGetLastError();
-}
-
-cudaError_t gm_combine(double* x, const double* V, int64_t ldv, int k, const double* y, int64_t n,
-                       cudaStream_t st, int df)
-{
-    count_launches(1);
-    if (df) k_gm_combine<true><<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(x, V, ldv, k, y, n, nullptr);
-    else k_gm_combine<false><<<grid_for(n, 256, 152 * 16), 256, 0, st>>>(x, V, ldv, k, y, n, nullptr);
-    return cudaGetLastError();
-}
 
 cudaError_t gm_combine_dev(double* x, const double* V, int64_t ldv, const int* k, const double* y, int64_t n,
                            cudaStream_t st, int df)
@@ -1115,11 +990,10 @@ cudaError_t reduce_partials(const double* partial, int nblocks, int nsums, doubl
     return cudaGetLastError();
 }
 
-cudaError_t reduce_partials_dyn(const double* partial, int nblocks, const GmDyn* dyn, int maxsums,
-                                cudaStream_t st)
+cudaError_t reduce_partials_dyn(const double* partial, int nblocks, GmState* st, int m, cudaStream_t s)
 {
     count_launches(1);
-    k_reduce_partials<<<maxsums, 256, 0, st>>>(partial, nblocks, 0, nullptr, dyn);
+    k_reduce_partials<<<m + 2, 256, 0, s>>>(partial, nblocks, 0, nullptr, st);
     return cudaGetLastError();
 }
 

@@ -4,10 +4,12 @@
 // The Arnoldi process runs on B = A - I with an FP64 Krylov basis (double-
 // float pairs in the FP32 form of the 2D scheme with linear shapes). Its
 // heavy kernels (operator with fused dot products, their reduction, the
-// fused basis update) are in fields.cu; the single-thread kernels here keep
-// the small dense part on the device: the Hessenberg column, the Givens
-// rotations, the residual estimate, the stop tests, the triangular solve
-// for the update, and the launch arguments of the next iteration (GmDyn).
+// fused basis update) are in fields.cu; the small dense part stays on the
+// device too: the Hessenberg column, the Givens rotations, the residual
+// estimate, the stop tests and the triangular solve (gmtail.cuh) run on one
+// warp of an extra block of the basis update, hidden behind it (as a launch
+// of its own on one thread the tail took 7 us an iteration), and leave the
+// launch arguments of the next iteration (GmDyn).
 // With nothing left for the host to decide between iterations, the whole
 // solve can run as a CUDA graph whose loops are conditional while nodes
 // (the kernels set the loop conditions), or be driven from the host.
@@ -50,6 +52,7 @@ __global__ void k_gm_cycle(GmState* st, const double* __restrict__ sums, GmPtrs 
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     int run = 0;
+    if (st->run) st->restarts += 1;   // a cycle has ended
     if (st->status == kGmOk) {
         const double beta = sqrt(sums[0]);
         if (!isfinite(beta)) {
@@ -67,7 +70,6 @@ __global__ void k_gm_cycle(GmState* st, const double* __restrict__ sums, GmPtrs 
             } else {
                 run = 1;
                 st->gv[0] = beta;
-                for (int k = 1; k <= q.m; ++k) st->gv[k] = 0.0;
                 st->kdim = 0;
                 GmDyn& d = st->dyn;
                 d.in = p.r;      // v_0 = r / beta, written to V_0 by iteration 0
@@ -89,84 +91,6 @@ __global__ void k_gm_arm(const GmState* __restrict__ st, cudaGraphConditionalHan
 {
     if (threadIdx.x != 0 || blockIdx.x != 0) return;
     if (has_cond) cudaGraphSetConditional(cond, st->run);
-}
-
-__global__ void k_gm_tail(GmState* st, GmPtrs p, GmParams q, cudaGraphConditionalHandle cond, int has_cond)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    GmDyn& d = st->dyn;
-    int inner = 0;
-    if (d.live) {
-        const int j = d.nv, m = q.m;
-        const double* hj = d.ds;
-        const double ww = hj[j + 1];
-        double hn2 = ww;
-        for (int i = 0; i <= j; ++i) hn2 -= hj[i] * hj[i];
-        st->total += 1;
-        if (!isfinite(hn2)) {
-            st->status = kGmNonfinite;
-            st->kdim = 0;
-            st->run = 0;
-        } else if (j > 0 && hn2 < 1e-4 * ww) {
-            st->kdim = j;   // end the cycle without column j; restart from the true residual
-        } else {
-            double* H = st->H;
-            double* cs = st->cs;
-            double* sn = st->sn;
-            double* gv = st->gv;
-            const double hn = sqrt(hn2 > 0.0 ? hn2 : 0.0);
-            for (int i = 0; i <= j; ++i) H[i * m + j] = hj[i];
-            H[j * m + j] += 1.0;   // A = I + B
-            H[(j + 1) * m + j] = hn;
-            for (int i = 0; i < j; ++i) {
-                const double t = cs[i] * H[i * m + j] + sn[i] * H[(i + 1) * m + j];
-                H[(i + 1) * m + j] = -sn[i] * H[i * m + j] + cs[i] * H[(i + 1) * m + j];
-                H[i * m + j] = t;
-            }
-            const double a = H[j * m + j], b = H[(j + 1) * m + j];
-            const double r = hypot(a, b);
-            cs[j] = r == 0.0 ? 1.0 : a / r;
-            sn[j] = r == 0.0 ? 0.0 : b / r;
-            H[j * m + j] = r;
-            H[(j + 1) * m + j] = 0.0;
-            gv[j + 1] = -sn[j] * gv[j];
-            gv[j] = cs[j] * gv[j];
-            st->kdim = j + 1;
-            const bool stop = fabs(gv[j + 1]) <= q.tol * st->bnorm || st->total >= q.maxit || hn == 0.0 ||
-                              j + 1 >= m;
-            if (!stop) {
-                const int jn = j + 1;
-                inner = 1;
-                d.in = p.V + (int64_t)jn * p.ldv;
-                d.vj = nullptr;
-                d.out = jn % 2 == 0 ? p.w0 : p.r;
-                d.ds = jn % 2 == 0 ? p.ds0 : p.ds1;
-                d.s = 1.0;
-                d.nv = jn;
-            }
-        }
-    }
-    d.live = inner;
-    st->inner = inner;
-    if (has_cond) cudaGraphSetConditional(cond, inner);
-}
-
-// back substitution R y = g over the finished cycle's kdim columns
-__global__ void k_gm_solve_y(GmState* st, int m)
-{
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
-    if (!st->run) {
-        st->kdim = 0;
-        return;
-    }
-    const int kdim = st->kdim;
-    const double* H = st->H;
-    for (int i = kdim - 1; i >= 0; --i) {
-        double s = st->gv[i];
-        for (int k = i + 1; k < kdim; ++k) s -= H[i * m + k] * st->y[k];
-        st->y[i] = H[i * m + i] != 0.0 ? s / H[i * m + i] : 0.0;
-    }
-    st->restarts += 1;
 }
 
 }  // namespace
@@ -198,23 +122,6 @@ cudaError_t gm_arm(const GmState* st, GmCond cond, cudaStream_t s)
     count_launches(1);
     k_gm_arm<<<1, 32, 0, s>>>(st, (cudaGraphConditionalHandle)cond.h, cond.has);
     return cudaGetLastError();
-}
-
-cudaError_t gm_tail(GmState* st, GmPtrs p, GmParams q, GmCond cond, cudaStream_t s)
-{
-    count_launches(1);
-    k_gm_tail<<<1, 32, 0, s>>>(st, p, q, (cudaGraphConditionalHandle)cond.h, cond.has);
-    return cudaGetLastError();
-}
-
-cudaError_t gm_finish_cycle(GmState* st, double* x, const double* V, int64_t ldv, int64_t n, int m,
-                            cudaStream_t s, int df)
-{
-    count_launches(1);
-    k_gm_solve_y<<<1, 32, 0, s>>>(st, m);
-    cudaError_t e = cudaGetLastError();
-    if (e != cudaSuccess) return e;
-    return gm_combine_dev(x, V, ldv, &st->kdim, st->y, n, s, df);
 }
 
 }  // namespace relsim

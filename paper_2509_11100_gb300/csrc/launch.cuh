@@ -315,18 +315,7 @@ int field_grid_blocks(GridP g, int precision);
 
 // GMRES vector kernels: FP64 vectors, or double-float ones when df (the
 // sums and dot products then come out in FP64 per block)
-cudaError_t gm_dots(const double* V, int64_t ldv, int k, const double* w, int64_t n,
-                    double* partial, int nblocks, cudaStream_t st, int df);     // k dots + w.w
-cudaError_t gm_update(double* w, const double* V, int64_t ldv, int k, const double* h,
-                      int64_t n, double* partial, int nblocks, cudaStream_t st, int df);  // w -= V h; |w|^2
-cudaError_t gm_scale(double* dst, const double* src, double s, int64_t n, cudaStream_t st, int df);
-// vout = (w - V h)/hn with hn^2 = hw[k] - |h|^2, h = hw[0..k-1]
-cudaError_t gm_update_scale(const double* w, const double* V, int64_t ldv, int k, const double* hw,
-                            double* vout, int64_t n, cudaStream_t st, int df);
-cudaError_t gm_sub(double* r, const double* b, const double* Ax, int64_t n, double* partial,
-                   int nblocks, cudaStream_t st, int df);                      // r = b - Ax; |r|^2
-cudaError_t gm_combine(double* x, const double* V, int64_t ldv, int k, const double* y,
-                       int64_t n, cudaStream_t st, int df);                    // x += V y
+cudaError_t gm_norm2(const double* w, int64_t n, double* partial, int nblocks, cudaStream_t st, int df);   // w.w
 cudaError_t gm_combine_dev(double* x, const double* V, int64_t ldv, const int* k, const double* y,
                            int64_t n, cudaStream_t st, int df);                // x += V y, k read on the device
 cudaError_t reduce_partials(const double* partial, int nblocks, int nsums, double* out,
@@ -365,6 +354,8 @@ struct GmState {
     int total, restarts, kdim, run, inner, status, zero, pad;
     double cs[kMaxRestart], sn[kMaxRestart], gv[kMaxRestart + 1], y[kMaxRestart];
     double H[(kMaxRestart + 1) * kMaxRestart];
+    double rinv[kMaxRestart];     // 1/H[i][i]
+    GmDyn cur;                    // dyn as the running iteration's reduction found it
     unsigned ctl, bar, bar_out;   // the one-launch solve's decision and grid barrier (solve.cu)
 };
 enum { kGmOk = 0, kGmNotConverged = 1, kGmNonfinite = 2 };
@@ -395,20 +386,17 @@ cudaError_t gm_zero_x(const GmState* st, double* x, int64_t n, cudaStream_t s);
 cudaError_t gm_cycle(GmState* st, const double* sums, GmPtrs p, GmParams q, GmCond cond, cudaStream_t s);
 // sets the Arnoldi-loop condition to the state's "run"
 cudaError_t gm_arm(const GmState* st, GmCond cond, cudaStream_t s);
-// after iteration j's sums: Hessenberg column, Givens rotation, residual
-// estimate, stop test, launch arguments of iteration j + 1; sets the
-// Arnoldi-loop condition
-cudaError_t gm_tail(GmState* st, GmPtrs p, GmParams q, GmCond cond, cudaStream_t s);
-// y from the triangular system of the finished cycle; x += V y
-cudaError_t gm_finish_cycle(GmState* st, double* x, const double* V, int64_t ldv, int64_t n, int m,
-                            cudaStream_t s, int df);
 // Arnoldi iteration kernels reading their arguments from dyn
 template <typename T>
 cudaError_t op_arnoldi_dyn(const T* M, const GmDyn* dyn, const double* V, int64_t ldv, GridP g,
                            double* partial, int* err, cudaStream_t st, bool tr = false);
-cudaError_t reduce_partials_dyn(const double* partial, int nblocks, const GmDyn* dyn, int maxsums,
-                                cudaStream_t st);
-cudaError_t gm_update_scale_dyn(const GmDyn* dyn, const double* V, int64_t ldv, int64_t n, cudaStream_t st,
+// the iteration's sums (m: the restart length, so m + 2 sums at most); keeps
+// the iteration's arguments in st->cur
+cudaError_t reduce_partials_dyn(const double* partial, int nblocks, GmState* st, int m, cudaStream_t s);
+// v_{j+1} of the running iteration, and beside it the iteration's tail
+// (gmtail.cuh) with the launch arguments of iteration j + 1; sets the
+// Arnoldi-loop condition
+cudaError_t gm_update_scale_dyn(GmState* st, const GmPtrs& p, const GmParams& q, GmCond cond, int64_t n, cudaStream_t s,
                                 int df);
 
 // ----- solve.cu: the solve in one cooperative launch -----

@@ -20,6 +20,7 @@
 // iteration, stop tests, restart rule and arithmetic per vector element as
 // the launches it replaces; only the order of the dot products' partial
 // sums differs.
+#include "gmtail.cuh"
 #include "launch.cuh"
 #include "opcore.cuh"
 
@@ -347,78 +348,11 @@ k_gm_solve(const __grid_constant__ SolveArgs<T> a)
 
     int total = 0, restarts = 0, status = kGmOk, kdim = 0;   // the same in every thread of every block
     double bn = 0.0;
-    // The tail of iteration j, by one warp of block 0: Hessenberg column,
-    // Givens rotations, residual estimate, stop test, and at a cycle's end
-    // the back substitution. The lanes form the products of the earlier
-    // rotations with the column together; only the chain through them is
-    // serial (one multiply-add a rotation: an FP64 operation takes a warp
-    // about 64 cycles, on one thread the tail took 5000).
+    // the tail of iteration j, by one warp of block 0
     auto tail = [&](int j) {
-        double* H = a.st->H;
-        const int m = a.m;
-        const double ww = sums[j + 1], hn2 = shn2;
-        int go = 0, kd = 0, stt = kGmOk;
-        if (!isfinite(hn2)) {
-            stt = kGmNonfinite;
-        } else if (j > 0 && hn2 < 1e-4 * ww) {
-            kd = j;   // end the cycle without column j; restart from the true residual
-        } else {
-            const double hn = hn2 > 0.0 ? hn2 * srn : 0.0;
-            double t = sums[0];
-            if (j == 0) t += 1.0;   // A = I + B
-            for (int i0s = 0; i0s < j; i0s += 32) {
-                const int i = i0s + lane, kc = min(32, j - i0s);
-                double p = 0.0, q = 0.0, c = 0.0, tm = 0.0;
-                if (i < j) {
-                    double nxt = sums[i + 1];
-                    if (i + 1 == j) nxt += 1.0;
-                    c = cs[i];
-                    p = c * nxt;
-                    q = sn[i] * nxt;
-                }
-                for (int k = 0; k < kc; ++k) {
-                    if (lane == k) tm = t;
-                    t = -sn[i0s + k] * t + __shfl_sync(0xffffffffu, p, k);
-                }
-                if (i < j) H[i * m + j] = c * tm + q;
-            }
-            // one reciprocal square root for the rotation; where the squares
-            // would leave the range, hypot and divisions
-            const double r2 = t * t + hn * hn;
-            double r, ri, c1, s1;
-            if (r2 > 1e-200 && r2 < 1e200) {
-                ri = rsqrt(r2);
-                r = r2 * ri;
-                c1 = t * ri;
-                s1 = hn * ri;
-            } else {
-                r = hypot(t, hn);
-                ri = r == 0.0 ? 0.0 : 1.0 / r;
-                c1 = r == 0.0 ? 1.0 : t / r;
-                s1 = r == 0.0 ? 0.0 : hn / r;
-            }
-            const double g0 = gv[j], g1 = -s1 * g0;
-            __syncwarp();
-            if (lane == 0) {
-                cs[j] = c1;
-                sn[j] = s1;
-                rinv[j] = ri;
-                H[j * m + j] = r;
-                gv[j + 1] = g1;
-                gv[j] = c1 * g0;
-            }
-            kd = j + 1;
-            go = !(fabs(g1) <= a.tol * bn || total >= a.maxit || hn == 0.0 || j + 1 >= m);
-        }
-        __syncwarp();
-        if (!go)   // R y = g over the finished cycle's columns: y_i, then its column off the others
-            for (int i = kd - 1; i >= 0; --i) {
-                const double y = gv[i] * rinv[i];
-                __syncwarp();
-                for (int k = lane; k < i; k += 32) gv[k] -= H[k * m + i] * y;
-                if (lane == 0) a.st->y[i] = y;
-                __syncwarp();
-            }
+        int go, kd, stt;
+        gm_tail_warp(GmTail{a.st->H, cs, sn, gv, rinv, a.st->y, a.m}, sums, j, shn2, srn, a.tol * bn, total, a.maxit,
+                     lane, go, kd, stt);
         if (lane == 0)
             *(volatile unsigned*)&a.st->ctl = (unsigned)go | (unsigned)stt << 8 | (unsigned)kd << 16;
     };
@@ -545,13 +479,7 @@ k_gm_solve(const __grid_constant__ SolveArgs<T> a)
                 grid_sums(a.partial, nq);
                 if (tid < nq) hs[tid] = W::from(sums[tid]);
                 if (tid == 0) {
-                    double h2 = sums[j + 1], h3 = 0.0;   // two chains: every FP64 operation waits for the last
-                    for (int c = 0; c + 1 <= j; c += 2) {
-                        h2 -= sums[c] * sums[c];
-                        h3 -= sums[c + 1] * sums[c + 1];
-                    }
-                    if (j % 2 == 0) h2 -= sums[j] * sums[j];
-                    h2 += h3;
+                    const double h2 = gm_rest2(sums, j);
                     shn2 = h2;
                     srn = h2 > 0.0 ? rsqrt(h2) : 0.0;
                     scale = W::from(srn);

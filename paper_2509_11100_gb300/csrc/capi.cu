@@ -39,6 +39,8 @@ constexpr int kLedgerLen = kLedgerField + kLedgerSpecies * kMaxSpecies + 2;   //
 struct Species {
     int64_t n = 0, cap = 0;
     void* a[2][7] = {};   // fx, fy, ux, uy, uz, w (and fz in 3D) of buffer 0 and 1
+    void* slab[2] = {};   // the one allocation that holds them (3D and quadratic shapes)
+    size_t stride = 0;    // elements from array to array in it
     int32_t* id[2] = {nullptr, nullptr};
     int cur = 0;
     int32_t* start = nullptr;
@@ -284,6 +286,20 @@ PArrays<T> arrays(Species& s, int buf)
     return p;
 }
 
+// a buffer of the species as records (record_sort forms): four, two and one
+// array's room
+template <typename T>
+PRecords<T> records(Species& s, int buf)
+{
+    T* base = (T*)s.slab[buf];
+    PRecords<T> r;
+    r.a = (PRecA<T>*)base;
+    r.b = (PRecB<T>*)(base + 4 * s.stride);
+    r.fz = s.a[buf][6] ? base + 6 * s.stride : nullptr;
+    r.id = s.id[buf];
+    return r;
+}
+
 int ensure_stage(relsim_ctx* c, int64_t ndoubles)
 {
     if (ndoubles <= c->stage_cap) return RELSIM_OK;
@@ -334,6 +350,20 @@ int ensure_partial(relsim_ctx* c, int64_t n)
     return RELSIM_OK;
 }
 
+// the forms whose re-sort is a counting sort of pushed records (PRecords):
+// their species' arrays lie in one allocation per buffer, slot after slot
+bool record_sort(const relsim_ctx* c) { return c->g.dim == 3 || c->g.shape == 2; }
+
+void free_arrays(Species& sp, int b)
+{
+    if (sp.slab[b]) {
+        dfree(sp.slab[b]);
+        for (void*& a : sp.a[b]) a = nullptr;
+    }
+    for (void*& a : sp.a[b]) dfree(a);
+    dfree(sp.id[b]);
+}
+
 int ensure_species(relsim_ctx* c, int s, int64_t n)
 {
     Species& sp = c->sp[s];
@@ -342,14 +372,17 @@ int ensure_species(relsim_ctx* c, int s, int64_t n)
         TRY(dalloc(c, &sp.start_alt, sizeof(int32_t) * (size_t)(c->g.ncell + 1)));
     }
     if (n <= sp.cap) return RELSIM_OK;
-    for (int b = 0; b < 2; ++b) {
-        for (int k = 0; k < 7; ++k) dfree(sp.a[b][k]);
-        dfree(sp.id[b]);
-    }
+    for (int b = 0; b < 2; ++b) free_arrays(sp, b);
     sp.cap = 0;
     const int narr = c->g.dim == 3 ? 7 : 6;
+    sp.stride = ((size_t)n + 8 + 63) / 64 * 64;   // (every array 256-byte aligned)
     for (int b = 0; b < 2; ++b) {
-        for (int k = 0; k < narr; ++k) TRY(dalloc(c, &sp.a[b][k], c->esz * (size_t)(n + 8)));
+        if (record_sort(c)) {
+            TRY(dalloc(c, &sp.slab[b], c->esz * sp.stride * narr));
+            for (int k = 0; k < narr; ++k) sp.a[b][k] = (char*)sp.slab[b] + c->esz * sp.stride * k;
+        } else {
+            for (int k = 0; k < narr; ++k) TRY(dalloc(c, &sp.a[b][k], c->esz * (size_t)(n + 8)));
+        }
         // 8 elements of slack: bulk copies round a range out to 16 bytes
         if (c->cfg.track_ids) TRY(dalloc(c, &sp.id[b], sizeof(int32_t) * (size_t)(n + 8)));
     }
@@ -772,11 +805,11 @@ int autotune_impl(relsim_ctx* c, relsim_tuning* out)
                 if (!lin2)
                     CK(cudaMemsetAsync(c->count_new, 0, sizeof(int32_t) * (size_t)(c->g.ncell + 1), c->st));
                 if (c->g.dim == 3)
-                    CK(push3<T>(src, (T*)sp.a[sp.cur][6], dst, (T*)sp.a[1 - sp.cur][6], sp.start, c->rk[0], c->rv[0],
+                    CK(push3<T>(src, (T*)sp.a[sp.cur][6], records<T>(sp, 1 - sp.cur), sp.start, c->rk[0], c->rv[0],
                                 c->count_new, E, B, c->g, sc, c->partial, nbp, c->st));
                 else if (c->g.shape == 2)
-                    CK(push_q<T>(src, dst, sp.start, c->rk[0], c->rv[0], c->count_new, E, B, c->g, sc, c->partial,
-                                 nbp, c->st));
+                    CK(push_q<T>(src, records<T>(sp, 1 - sp.cur), sp.start, c->rk[0], c->rv[0], c->count_new, E, B,
+                                 c->g, sc, c->partial, nbp, c->st));
                 else
                     CK(push_sort<T>(src, dst, sp.start, c->n9, c->off9, E, B, c->En ? E : nullptr, c->g, sc,
                                     c->partial, nbp, c->dpush, c->st));
@@ -1108,15 +1141,15 @@ int push_enqueue(relsim_ctx* c)
             // depends on it beyond rounding; ids follow the particles)
             TRY(ensure_radix(c, sp.n));
             T* sfz = (T*)sp.a[sp.cur][6];
-            T* dfz = (T*)sp.a[1 - sp.cur][6];
+            const PRecords<T> rec = records<T>(sp, 1 - sp.cur);
             PROF_BEGIN(RELSIM_PROF_GENERAL_SORT);
             CK(cudaMemcpyAsync(led, led + 4, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
             CK(cudaMemsetAsync(c->count_new, 0, sizeof(int32_t) * (size_t)(c->g.ncell + 1), c->st));
-            CK(push3<T>(src, sfz, dst, dfz, sp.start, c->rk[0], c->rv[0], c->count_new, Eth, B, c->g, sc, c->partial,
-                        nbp, c->st));
+            CK(push3<T>(src, sfz, rec, sp.start, c->rk[0], c->rv[0], c->count_new, Eth, B, c->g, sc, c->partial, nbp,
+                        c->st));
             CK(reduce_partials(c->partial, nbp, kLedgerSpecies - 1, led + 1, c->st));
             CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp, c->st));
-            CK(place3<T>(dst, dfz, src, sfz, c->rk[0], c->rv[0], sp.start, sp.n, c->st));
+            CK(place3<T>(rec, src, sfz, c->rk[0], c->rv[0], sp.start, c->rv[1], sp.n, c->st));
             PROF_END();
         } else if (c->g.shape == 2) {
             // quadratic shapes: the push with each particle's new cell and
@@ -1125,11 +1158,12 @@ int push_enqueue(relsim_ctx* c)
             PROF_BEGIN(RELSIM_PROF_GENERAL_SORT);
             CK(cudaMemcpyAsync(led, led + 4, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
             CK(cudaMemsetAsync(c->count_new, 0, sizeof(int32_t) * (size_t)(c->g.ncell + 1), c->st));
-            CK(push_q<T>(src, dst, sp.start, c->rk[0], c->rv[0], c->count_new, Eth, B, c->g, sc, c->partial, nbp,
+            const PRecords<T> rec = records<T>(sp, 1 - sp.cur);
+            CK(push_q<T>(src, rec, sp.start, c->rk[0], c->rv[0], c->count_new, Eth, B, c->g, sc, c->partial, nbp,
                          c->st));
             CK(reduce_partials(c->partial, nbp, kLedgerSpecies - 1, led + 1, c->st));
             CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp, c->st));
-            CK(place3<T>(dst, nullptr, src, nullptr, c->rk[0], c->rv[0], sp.start, sp.n, c->st));
+            CK(place3<T>(rec, src, nullptr, c->rk[0], c->rv[0], sp.start, c->rv[1], sp.n, c->st));
             PROF_END();
         } else if (c->fast_sort) {
             // push, each old cell written back grouped by move direction
@@ -2410,10 +2444,7 @@ void relsim_destroy(relsim_ctx* c)
     cudaStreamSynchronize(c->st);
     for (int s = 0; s < kMaxSpecies; ++s) {
         Species& sp = c->sp[s];
-        for (int b = 0; b < 2; ++b) {
-            for (int k = 0; k < 7; ++k) dfree(sp.a[b][k]);
-            dfree(sp.id[b]);
-        }
+        for (int b = 0; b < 2; ++b) free_arrays(sp, b);
         dfree(sp.start);
         dfree(sp.start_alt);
     }

@@ -18,7 +18,8 @@
 //   k_rhs3, k_field_update3   the right-hand side, the field update with the
 //                field ledger terms (on the operator's tiles)
 //   k_push3      warp per row segment, the push with each particle's new cell
-//                and its slot there (any move length); k_place3 places them
+//                and its slot there (any move length), written as records;
+//                k_places and k_place3 sort them
 #include "launch.cuh"
 
 namespace relsim {
@@ -1078,13 +1079,13 @@ struct PushCfg3 {
 // as a cell shift plus offsets; the pushed particle goes to the same index
 // of dst with its new cell in key. Ledger sums per block: dK, work,
 // mismatch, K1 (as the 2D push). Warp per row segment of up to 32 cells, the
-// lanes over the segment's particles. With rank non-null each particle also
-// takes a slot among its new cell's particles, rank[p] = count[key]++ (one
-// atomic per new cell and warp: the lanes with equal keys found by
-// match-any), for the unstable counting sort that follows.
+// lanes over the segment's particles. Each particle also takes a slot among
+// its new cell's particles, rank[p] = count[key]++ (one atomic per new cell
+// and warp: the lanes with equal keys found by match-any), for the unstable
+// counting sort that follows.
 template <typename T>
 __global__ void __launch_bounds__(32 * PushCfg3<T>::warps)
-k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict__ dfz,
+k_push3(PArrays<T> src, const T* __restrict__ sfz, PRecords<T> dst,
         const int32_t* __restrict__ start, int32_t* __restrict__ key, int32_t* __restrict__ rank,
         int32_t* __restrict__ count, const T* __restrict__ Eth, const T* __restrict__ B, GridP g, T beta, T qdt,
         T m, double* __restrict__ lsum, int uw)
@@ -1177,13 +1178,9 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict
                     }
                     cnew[a] = q;
                 }
-                dst.fx[p] = fn[0];
-                dst.fy[p] = fn[1];
-                dfz[p] = fn[2];
-                dst.ux[p] = u1x;
-                dst.uy[p] = u1y;
-                dst.uz[p] = u1z;
-                dst.w[p] = w;
+                dst.a[p] = PRecA<T>{fn[0], fn[1], u1x, u1y};
+                dst.b[p] = PRecB<T>{u1z, w};
+                dst.fz[p] = fn[2];
                 if (dst.id) dst.id[p] = src.id[p];
                 newkey = (int32_t)node3(cnew[0], cnew[1], cnew[2], g);
                 key[p] = newkey;
@@ -1196,19 +1193,17 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict
                 acc[2] += wk * du * igs * igs;
                 acc[3] += w * m * u12 / (g1 + T(1));
             }
-            if (rank) {
-                settle();   // the last batch's slots have had this one's time to arrive
-                const unsigned peers = __match_any_sync(0xffffffffu, newkey);
-                wait_peers = peers;
-                if (act) {
-                    wait_p = p;
-                    if ((peers & ((1u << lane) - 1u)) == 0u) wait_base = atomicAdd(count + newkey, __popc(peers));
-                }
+            settle();   // the last batch's slots have had this one's time to arrive
+            const unsigned peers = __match_any_sync(0xffffffffu, newkey);
+            wait_peers = peers;
+            if (act) {
+                wait_p = p;
+                if ((peers & ((1u << lane) - 1u)) == 0u) wait_base = atomicAdd(count + newkey, __popc(peers));
             }
         }
         __syncwarp();
     }
-    if (rank) settle();
+    settle();
     double v[4], o[4];
 #pragma unroll
     for (int q = 0; q < 4; ++q) v[q] = (double)acc[q];
@@ -1218,46 +1213,73 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict
         for (int q = 0; q < 4; ++q) lsum[(int64_t)blockIdx.x * 4 + q] = o[q];
 }
 
-// the counting sort's placement: particle p to start[key[p]] + rank[p]. Four
-// particles a thread: each waits on a chain of loads (key, start, then the
-// stores), and one at a time left the kernel bound by that wait
-template <typename T>
+// The counting sort's placement in two passes: where each particle goes
+// (perm[start[key[p]] + rank[p]] = p), then the particles in their new order,
+// each record's pieces read where they lie and the arrays written in order.
+// About half of the particles change cell, so one side of the sort goes to
+// sectors of its own: written from arrays to arrays that was seven or eight
+// scattered 4-byte stores a particle, 3.15 ms a species on 256x128x128 with
+// 16 particles a cell (FP32 form, 67 million with ids). Now one scattered store and four
+// loads of whole pieces, 0.31 + 1.22 ms (3.7 TB/s of algorithmic bytes, bound
+// by sectors used in part). Both run several particles a thread: each waits on a
+// chain of loads.
 __global__ void __launch_bounds__(256)
-k_place3(PArrays<T> src, const T* __restrict__ sfz, PArrays<T> dst, T* __restrict__ dfz,
-         const int32_t* __restrict__ key, const int32_t* __restrict__ rank, const int32_t* __restrict__ start,
-         int64_t n)
+k_places(const int32_t* __restrict__ key, const int32_t* __restrict__ rank, const int32_t* __restrict__ start,
+         int32_t* __restrict__ perm, int64_t n)
 {
     constexpr int U = 4;
     for (int64_t b = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; b < n; b += (int64_t)gridDim.x * (256 * U)) {
-        int64_t q[U], p[U];
         int kk[U], rr[U];
 #pragma unroll
         for (int v = 0; v < U; ++v) {
-            p[v] = b + 256 * v;
-            const bool in = p[v] < n;
-            kk[v] = in ? ld(key + p[v]) : 0;
-            rr[v] = in ? ld(rank + p[v]) : 0;
-            if (!in) p[v] = -1;
+            const int64_t p = b + 256 * v;
+            kk[v] = p < n ? ld(key + p) : 0;
+            rr[v] = p < n ? ld(rank + p) : 0;
         }
 #pragma unroll
-        for (int v = 0; v < U; ++v) q[v] = (int64_t)ld(start + kk[v]) + rr[v];
-        // (plain loads: read-only ones the compiler moves past the stores)
-        const T* const in[7] = {src.fx, src.fy, sfz, src.ux, src.uy, src.uz, src.w};
-        T* const out[7] = {dst.fx, dst.fy, dfz, dst.ux, dst.uy, dst.uz, dst.w};
-        T x[7][U];
+        for (int v = 0; v < U; ++v) kk[v] = ld(start + kk[v]);
 #pragma unroll
-        for (int a = 0; a < 7; ++a)
+        for (int v = 0; v < U; ++v) {
+            const int64_t p = b + 256 * v;
+            if (p < n) perm[(int64_t)kk[v] + rr[v]] = (int32_t)p;
+        }
+    }
+}
+
+constexpr int kPlace3 = 4;   // particles a thread
+template <typename T>
+__global__ void __launch_bounds__(256)
+k_place3(PRecords<T> src, PArrays<T> dst, T* __restrict__ dfz, const int32_t* __restrict__ perm, int64_t n)
+{
+    constexpr int U = kPlace3;
+    for (int64_t b = (int64_t)blockIdx.x * (256 * U) + threadIdx.x; b < n; b += (int64_t)gridDim.x * (256 * U)) {
+        int p[U];
 #pragma unroll
-            for (int v = 0; v < U; ++v) x[a][v] = p[v] >= 0 && in[a] ? in[a][p[v]] : T(0);
+        for (int v = 0; v < U; ++v) p[v] = b + 256 * v < n ? ld(perm + b + 256 * v) : 0;
+        PRecA<T> ra[U];
+        PRecB<T> rb[U];
+        T rz[U];
+        int ri[U];
 #pragma unroll
-        for (int a = 0; a < 7; ++a)
+        for (int v = 0; v < U; ++v) {
+            ra[v] = src.a[p[v]];
+            rb[v] = src.b[p[v]];
+            rz[v] = dfz ? src.fz[p[v]] : T(0);   // (no third offset for 2D particles)
+            ri[v] = src.id ? src.id[p[v]] : 0;
+        }
 #pragma unroll
-            for (int v = 0; v < U; ++v)
-                if (p[v] >= 0 && out[a]) out[a][q[v]] = x[a][v];   // (no third offset for 2D particles)
-        if (dst.id)
-#pragma unroll
-            for (int v = 0; v < U; ++v)
-                if (p[v] >= 0) dst.id[q[v]] = src.id[p[v]];
+        for (int v = 0; v < U; ++v) {
+            const int64_t q = b + 256 * v;
+            if (q >= n) continue;
+            dst.fx[q] = ra[v].fx;
+            dst.fy[q] = ra[v].fy;
+            dst.ux[q] = ra[v].ux;
+            dst.uy[q] = ra[v].uy;
+            dst.uz[q] = rb[v].uz;
+            dst.w[q] = rb[v].w;
+            if (dfz) dfz[q] = rz[v];
+            if (dst.id) dst.id[q] = ri[v];
+        }
     }
 }
 
@@ -1362,24 +1384,25 @@ int push_blocks3(GridP g, int cap)
 }
 
 template <typename T>
-cudaError_t push3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const int32_t* start, int32_t* key,
-                  int32_t* rank, int32_t* count, const T* Eth, const T* B, GridP g, SpeciesConst sc, double* lsum,
-                  int nblocks, cudaStream_t st)
+cudaError_t push3(PArrays<T> src, const T* sfz, PRecords<T> dst, const int32_t* start, int32_t* key, int32_t* rank,
+                  int32_t* count, const T* Eth, const T* B, GridP g, SpeciesConst sc, double* lsum, int nblocks,
+                  cudaStream_t st)
 {
     count_launches(1);
-    k_push3<T><<<nblocks, 32 * PushCfg3<T>::warps, 0, st>>>(src, sfz, dst, dfz, start, key, rank, count, Eth, B, g,
+    k_push3<T><<<nblocks, 32 * PushCfg3<T>::warps, 0, st>>>(src, sfz, dst, start, key, rank, count, Eth, B, g,
                                                        (T)(sc.q * g.dt / (2.0 * sc.m)), (T)(sc.q * g.dt), (T)sc.m,
                                                        lsum, unit_width3(g));
     return cudaGetLastError();
 }
 
 template <typename T>
-cudaError_t place3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const int32_t* key, const int32_t* rank,
-                   const int32_t* start, int64_t n, cudaStream_t st)
+cudaError_t place3(PRecords<T> src, PArrays<T> dst, T* dfz, const int32_t* key, const int32_t* rank,
+                   const int32_t* start, int32_t* perm, int64_t n, cudaStream_t st)
 {
     if (n <= 0) return cudaSuccess;
-    count_launches(1);
-    k_place3<T><<<grid3(n, 256 * 4, 152 * 32), 256, 0, st>>>(src, sfz, dst, dfz, key, rank, start, n);
+    count_launches(2);
+    k_places<<<grid3(n, 256 * 4, 152 * 32), 256, 0, st>>>(key, rank, start, perm, n);
+    k_place3<T><<<grid3(n, 256 * kPlace3, 152 * 32), 256, 0, st>>>(src, dst, dfz, perm, n);
     return cudaGetLastError();
 }
 
@@ -1395,10 +1418,10 @@ cudaError_t place3(PArrays<T> src, const T* sfz, PArrays<T> dst, T* dfz, const i
     template cudaError_t rhs3<T>(const T*, const T*, const T*, double*, GridP, cudaStream_t);                      \
     template cudaError_t field_update3<T>(const double*, const T*, const T*, T*, T*, const T*, T*, GridP, double*, \
                                           int, cudaStream_t);                                                      \
-    template cudaError_t push3<T>(PArrays<T>, const T*, PArrays<T>, T*, const int32_t*, int32_t*, int32_t*,        \
-                                  int32_t*, const T*, const T*, GridP, SpeciesConst, double*, int, cudaStream_t);  \
-    template cudaError_t place3<T>(PArrays<T>, const T*, PArrays<T>, T*, const int32_t*, const int32_t*,           \
-                                   const int32_t*, int64_t, cudaStream_t);                                         \
+    template cudaError_t push3<T>(PArrays<T>, const T*, PRecords<T>, const int32_t*, int32_t*, int32_t*, int32_t*, \
+                                  const T*, const T*, GridP, SpeciesConst, double*, int, cudaStream_t);            \
+    template cudaError_t place3<T>(PRecords<T>, PArrays<T>, T*, const int32_t*, const int32_t*, const int32_t*,    \
+                                   int32_t*, int64_t, cudaStream_t);                                               \
     template cudaError_t launch_op3<T, 0, false>(const T*, const double*, double, const double*, double*, double*, \
                                                  const double*, int64_t, int, GridP, double*, cudaStream_t,        \
                                                  const GmDyn*);                                                    \

@@ -22,7 +22,7 @@
 //                 modes and partial dot products of the other operators
 //   k_field_update_q   the field update and the ledger terms on the same tiles
 //   k_push_q      warp per row segment with E and B tiles, the push, the new
-//                 cell and its slot for the counting sort (k_place3 places)
+//                 cell and its slot for the counting sort (k_places, k_place3)
 #include "launch.cuh"
 #include "opcore.cuh"
 
@@ -758,7 +758,7 @@ constexpr int kPushWarpsQ = 4;
 
 template <typename T>
 __global__ void __launch_bounds__(32 * kPushWarpsQ)
-k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int32_t* __restrict__ key,
+k_push_q(PArrays<T> src, PRecords<T> dst, const int32_t* __restrict__ start, int32_t* __restrict__ key,
          int32_t* __restrict__ rank, int32_t* __restrict__ count, const T* __restrict__ Eth, const T* __restrict__ B,
          GridP g, T beta, T qdt, T m, double* __restrict__ lsum, int uw)
 {
@@ -864,12 +864,8 @@ k_push_q(PArrays<T> src, PArrays<T> dst, const int32_t* __restrict__ start, int3
                     }
                     cnew[a] = q;
                 }
-                dst.fx[p] = fn[0];
-                dst.fy[p] = fn[1];
-                dst.ux[p] = u1x;
-                dst.uy[p] = u1y;
-                dst.uz[p] = u1z;
-                dst.w[p] = w;
+                dst.a[p] = PRecA<T>{fn[0], fn[1], u1x, u1y};
+                dst.b[p] = PRecB<T>{u1z, w};
                 if (dst.id) dst.id[p] = src.id[p];
                 newkey = cnew[1] * g.nx + cnew[0];
                 key[p] = newkey;
@@ -966,7 +962,7 @@ int push_blocks_q(GridP g, int cap)
 }
 
 template <typename T>
-cudaError_t push_q(PArrays<T> src, PArrays<T> dst, const int32_t* start, int32_t* key, int32_t* rank,
+cudaError_t push_q(PArrays<T> src, PRecords<T> dst, const int32_t* start, int32_t* key, int32_t* rank,
                    int32_t* count, const T* Eth, const T* B, GridP g, SpeciesConst sc, double* lsum, int nblocks,
                    cudaStream_t st)
 {
@@ -985,7 +981,7 @@ cudaError_t push_q(PArrays<T> src, PArrays<T> dst, const int32_t* start, int32_t
     template cudaError_t deposit_q<T>(const DepositSpecies<T>&, const T*, T*, T*, GridP, cudaStream_t, int);           \
     template cudaError_t field_update_q<T>(const double*, const T*, const T*, T*, T*, const T*, T*, GridP,        \
                                            double*, int, cudaStream_t);                                           \
-    template cudaError_t push_q<T>(PArrays<T>, PArrays<T>, const int32_t*, int32_t*, int32_t*, int32_t*,         \
+    template cudaError_t push_q<T>(PArrays<T>, PRecords<T>, const int32_t*, int32_t*, int32_t*, int32_t*,        \
                                    const T*, const T*, GridP, SpeciesConst, double*, int, cudaStream_t);          \
     RELSIM_Q_OP(T, 0, false) RELSIM_Q_OP(T, 1, false) RELSIM_Q_OP(T, 2, false)                                   \
     RELSIM_Q_OP(T, 0, true) RELSIM_Q_OP(T, 1, true) RELSIM_Q_OP(T, 2, true)

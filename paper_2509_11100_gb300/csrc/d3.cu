@@ -670,26 +670,36 @@ __device__ __forceinline__ void curl_cell3(F f, T rx, T ry, T rz, T (&C)[3])
     C[2] = d[0][1] - d[1][0];
 }
 
-// The operator's tiles: 32 x 2 x 2 nodes (FP64: 32 x 2 x 1), one thread a
-// node. The tile's own mass-matrix rows (16 KB a row of 32 nodes in FP32) come
+// The operator's tiles: 32 x 2 x 2 nodes (FP64: 32 x 2 x 1). The tile's own mass-matrix rows (16 KB a row of 32 nodes in FP32) come
 // into shared memory by asynchronous copies, all in flight together, while
 // the input is staged; read straight from global memory (504 bytes from lane
 // to lane) every load of a block touched 32 lines, and the operator was bound
 // by their latency: 1.28 ms an application on 256x128x128 (FP32 form).
+// Three tiles fit an SM's shared memory, and with a thread a node their twelve
+// warps left it waiting (a third of the issue slots used, no unit above 45%):
+// two threads share a node, one for its own blocks, one for its neighbours',
+// and take the products with the basis in turn. 6.99 -> 6.5 ms for a step's
+// seven applications, FP64 at 64x32x32 1.28 -> 1.05 ms a step. The field
+// update keeps one thread a node: its neighbours' blocks need the registers
+// (1.15 ms, with two 1.42). The neighbours' blocks from outside the tile,
+// copied to shared memory like its own, leave two tiles an SM: slower, 8.1 ms.
 template <typename T>
 struct Op3 {
-    static constexpr int X = 32, Y = 2, Z = sizeof(T) == 4 ? 2 : 1, threads = X * Y * Z;
+    static constexpr int X = 32, Y = 2, Z = sizeof(T) == 4 ? 2 : 1, nodes = X * Y * Z;
+    static constexpr int share = 2;   // threads of a node in the operator (one in the field update)
     struct Shared {
         T Mm[Z * Y][X * kMBlock3];              // own blocks, row z Y + y
         T v[3][Z + 2][Y + 2][X + 2];            // the input on the 1-node halo
         T C[3][Z + 1][Y + 1][X + 1];            // its curl on the cells around the tile's nodes
+        T part[3][nodes];                       // the neighbours' share of M v
     };
-    static_assert(sizeof(Shared) >= sizeof(double) * kOpChunk3 * threads, "the dot products reuse it");
+    static_assert(sizeof(Shared) >= sizeof(double) * (kOpChunk3 + 3) * nodes, "the dot products reuse it");
 };
 // a block's tile and this thread's node
 template <typename T>
 struct At3 {
-    int i0, j0, k0, tw, th, td, tx, ty, tz, i, j, k;
+    int i0, j0, k0, tw, th, td, tx, ty, tz, i, j, k, node;
+    bool second;   // the node's second thread
     bool active;
     int64_t gidx;
     __device__ __forceinline__ explicit At3(const GridP& g)
@@ -705,7 +715,9 @@ struct At3 {
         td = min(O::Z, g.nz - k0);
         tx = threadIdx.x % O::X;
         ty = (threadIdx.x / O::X) % O::Y;
-        tz = threadIdx.x / (O::X * O::Y);
+        node = threadIdx.x % O::nodes;
+        second = threadIdx.x >= O::nodes;
+        tz = node / (O::X * O::Y);
         i = i0 + tx;
         j = j0 + ty;
         k = k0 + tz;
@@ -730,9 +742,9 @@ __device__ __forceinline__ void fetch_rows3(typename Op3<T>::Shared& S, const T*
         const char* src = reinterpret_cast<const char*>(M + node3(t.i0, t.j0 + y, t.k0 + z, g) * kMBlock3);
         char* dst = reinterpret_cast<char*>(&S.Mm[r][0]);
         if (wide)
-            for (int q = threadIdx.x; q < n; q += O::threads) cp_async16(dst + 16 * q, src + 16 * q);
+            for (int q = threadIdx.x; q < n; q += blockDim.x) cp_async16(dst + 16 * q, src + 16 * q);
         else
-            for (int q = threadIdx.x; q < n; q += O::threads) cp_async8(dst + 8 * q, src + 8 * q);
+            for (int q = threadIdx.x; q < n; q += blockDim.x) cp_async8(dst + 8 * q, src + 8 * q);
     }
     asm volatile("cp.async.commit_group;" ::: "memory");
 }
@@ -750,7 +762,8 @@ __device__ __forceinline__ void stage_input3(typename Op3<T>::Shared& S, const d
     const int ga = wrap1(min(t.i0 - 1 + lane, 2 * g.nx - 1), g.nx), gb = wrap1(min(t.i0 + 31 + lane, 2 * g.nx - 1), g.nx);
     // a warp a row of 34 (a lane a column, the last two by two lanes), four
     // rows of loads in flight
-    constexpr int rows = 3 * HZ * HY, W = O::threads / 32;
+    constexpr int rows = 3 * HZ * HY;
+    const int W = blockDim.x / 32;
     for (int r0 = wid; r0 < rows; r0 += 4 * W) {
         double a[4], b[4];
 #pragma unroll
@@ -778,7 +791,7 @@ __device__ __forceinline__ void stage_input3(typename Op3<T>::Shared& S, const d
     }
     __syncthreads();
     const T rx = gc<T>(g).qdx, ry = gc<T>(g).qdy, rz = gc<T>(g).qdz;
-    for (int q = threadIdx.x; q < (O::Z + 1) * (O::Y + 1) * (O::X + 1); q += O::threads) {
+    for (int q = threadIdx.x; q < (O::Z + 1) * (O::Y + 1) * (O::X + 1); q += blockDim.x) {
         const int c = q % (O::X + 1), y = (q / (O::X + 1)) % (O::Y + 1), z = q / ((O::X + 1) * (O::Y + 1));
         T C[3];
         curl_cell3<T>([&](int comp, int p, int o, int w) { return S.v[comp][z + w][y + o][c + p]; }, rx, ry, rz, C);
@@ -827,9 +840,10 @@ __device__ __forceinline__ void block3(const double* p, int, double (&m)[9])
 // (M v) at the thread's node: its own 14 stored blocks times v at g + d(h),
 // and the 13 neighbours' blocks M[g - d(h)][h] times v at g - d(h) (from the
 // tile where they lie in it, else from global memory); with TR each block
-// applied transposed
-template <typename T, bool TR>
-__device__ __forceinline__ void mv3(const typename Op3<T>::Shared& S, const T* __restrict__ M, const At3<T>& t,
+// applied transposed. With SHARE 2 a node's two threads take one sum each and the first
+// gets both (every thread of the block calls)
+template <typename T, bool TR, int SHARE>
+__device__ __forceinline__ void mv3(typename Op3<T>::Shared& S, const T* __restrict__ M, const At3<T>& t,
                                     const GridP& g, T (&out)[3])
 {
     using O = Op3<T>;
@@ -856,32 +870,56 @@ __device__ __forceinline__ void mv3(const typename Op3<T>::Shared& S, const T* _
     // the neighbours' blocks three at a time (h = 2..4, 5..7, 8..10, 11..13),
     // each three on their way while the blocks before them are added
     T nb[2][3][9];
+    auto begin = [&]() {
 #pragma unroll
-    for (int q = 0; q < 3; ++q) neighbour(2 + q, nb[0][q]);
+        for (int q = 0; q < 3; ++q) neighbour(2 + q, nb[0][q]);
+    };
+    auto others = [&]() {
 #pragma unroll
-    for (int h = 0; h < kHalf3; ++h) {
-        int di, dj, dk;
-        half_offset3(h, di, dj, dk);
-        T m[9];
-        block3(Mg + h * 9, h, m);
-        add(m, di, dj, dk);
-    }
+        for (int n = 0; n < 4; ++n) {
 #pragma unroll
-    for (int n = 0; n < 4; ++n) {
+            for (int q = 0; q < 3; ++q)
+                if (n < 3) neighbour(2 + 3 * (n + 1) + q, nb[(n + 1) & 1][q]);
 #pragma unroll
-        for (int q = 0; q < 3; ++q)
-            if (n < 3) neighbour(2 + 3 * (n + 1) + q, nb[(n + 1) & 1][q]);
-#pragma unroll
-        for (int q = 0; q < 3; ++q) {
-            int di, dj, dk;
-            half_offset3(2 + 3 * n + q, di, dj, dk);
-            add(nb[n & 1][q], -di, -dj, -dk);
+            for (int q = 0; q < 3; ++q) {
+                int di, dj, dk;
+                half_offset3(2 + 3 * n + q, di, dj, dk);
+                add(nb[n & 1][q], -di, -dj, -dk);
+            }
         }
-    }
-    {
         T m[9];
         neighbour(1, m);
         add(m, -1, 0, 0);
+    };
+    auto mine = [&]() {
+#pragma unroll
+        for (int h = 0; h < kHalf3; ++h) {
+            int di, dj, dk;
+            half_offset3(h, di, dj, dk);
+            T m[9];
+            block3(Mg + h * 9, h, m);
+            add(m, di, dj, dk);
+        }
+    };
+    if (SHARE == 1) {
+        if (t.active) {
+            begin();
+            mine();
+            others();
+        }
+    } else {
+        if (t.second && t.active) {
+            begin();
+            others();
+#pragma unroll
+            for (int c = 0; c < 3; ++c) S.part[c][t.node] = r[c];
+        } else if (t.active) {
+            mine();
+        }
+        __syncthreads();
+        if (t.active && !t.second)
+#pragma unroll
+            for (int c = 0; c < 3; ++c) r[c] += S.part[c][t.node];
     }
     out[0] = r[0];
     out[1] = r[1];
@@ -895,7 +933,7 @@ __device__ __forceinline__ void mv3(const typename Op3<T>::Shared& S, const T* _
 //   Arnoldi:  v = s in (to vj when vj is not null), out = B v, partials
 //             <out, V_q> (q < nv), <out, v>, <out, out>
 template <typename T, int MODE, bool TR>
-__global__ void __launch_bounds__(Op3<T>::threads, 3)
+__global__ void __launch_bounds__(Op3<T>::share * Op3<T>::nodes, 3)
 k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const double* __restrict__ b,
       double* __restrict__ out, double* __restrict__ vj, const double* __restrict__ V, int64_t ldv, int nv, GridP g,
       double* __restrict__ partial, const GmDyn* __restrict__ dyn)
@@ -916,7 +954,8 @@ k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const do
     const int tid = threadIdx.x;
     fetch_rows3<T>(S, M, t, g);
     double own[3] = {0.0, 0.0, 0.0}, wv[3] = {0.0, 0.0, 0.0};
-    if (t.active) {
+    const bool owner = t.active && !t.second;
+    if (owner) {
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             own[c] = __ldg(in + c * nc + t.gidx);
@@ -925,11 +964,12 @@ k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const do
     }
     if (MODE == k3Arnoldi) stage_input3<T, true>(S, in, (T)s, t, g);
     else stage_input3<T, false>(S, in, T(1), t, g);
-    if (t.active) {
-        T cc3[3], mv[3];
+    T mv[3];
+    mv3<T, TR, O::share>(S, M, t, g, mv);
+    if (owner) {
+        T cc3[3];
         curl_cell3<T>([&](int comp, int p, int o, int w) { return S.C[comp][t.tz + w][t.ty + o][t.tx + p]; },
                       gc<T>(g).qdx, gc<T>(g).qdy, gc<T>(g).qdz, cc3);
-        mv3<T, TR>(S, M, t, g, mv);
         const T td = gc<T>(g).td;
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
@@ -944,12 +984,22 @@ k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const do
     if (MODE == k3A) return;
     const int nq = MODE == k3Residual ? 1 : nv + 2;
     const int lane = tid & 31, wid = tid >> 5;
-    double* buf = reinterpret_cast<double*>(op3_smem);   // [kOpChunk3][threads]
+    double* buf = reinterpret_cast<double*>(op3_smem);   // [kOpChunk3][nodes]
     __syncthreads();   // the tile is no longer read
+    if (MODE == k3Arnoldi && O::share == 2) {   // a node's threads take the products with the basis in turn
+        double* const sw = buf + kOpChunk3 * O::nodes;
+#pragma unroll
+        for (int c = 0; c < 3; ++c)
+            if (!t.second) sw[c * O::nodes + t.node] = wv[c];
+        __syncthreads();
+#pragma unroll
+        for (int c = 0; c < 3; ++c) wv[c] = sw[c * O::nodes + t.node];
+    }
     for (int q0 = 0; q0 < nq; q0 += kOpChunk3) {
         const int kc = min(kOpChunk3, nq - q0);
         for (int c = 0; c < kc; ++c) {
             const int q = q0 + c;
+            if (O::share == 2 && t.second != (MODE == k3Arnoldi && q < nv && (q & 1))) continue;
             double d = 0.0;
             if (t.active) {
                 if (MODE == k3Residual || q == nv + 1) d = wv[0] * wv[0] + wv[1] * wv[1] + wv[2] * wv[2];
@@ -959,13 +1009,13 @@ k_op3(const T* __restrict__ M, const double* __restrict__ in, double s, const do
                     d = wv[0] * __ldg(Vq) + wv[1] * __ldg(Vq + nc) + wv[2] * __ldg(Vq + 2 * nc);
                 }
             }
-            buf[c * O::threads + tid] = d;
+            buf[c * O::nodes + t.node] = d;
         }
         __syncthreads();
-        for (int c = wid; c < kc; c += O::threads / 32) {
+        for (int c = wid; c < kc; c += O::share * O::nodes / 32) {
             double sum = 0.0;
 #pragma unroll
-            for (int m = 0; m < O::threads / 32; ++m) sum += buf[c * O::threads + m * 32 + lane];
+            for (int m = 0; m < O::nodes / 32; ++m) sum += buf[c * O::nodes + m * 32 + lane];
             sum = warp_sum(sum);
             if (lane == 0) partial[(int64_t)blockIdx.x * nq + q0 + c] = sum;
         }
@@ -1016,7 +1066,7 @@ constexpr int kFieldLedger3 = 6;
 // global memory: 1.7 ms on 256x128x128, FP32 form). Term 5 is the work
 // dt dV (Jhat + M E^{n+theta}) . E^{n+theta}.
 template <typename T>
-__global__ void __launch_bounds__(Op3<T>::threads, 3)
+__global__ void __launch_bounds__(Op3<T>::nodes, 3)
 k_field_update3(const double* __restrict__ x, const T* __restrict__ M, const T* __restrict__ J, T* __restrict__ Eth,
                 T* __restrict__ E, const T* __restrict__ B0, T* __restrict__ B1, GridP g, double* __restrict__ partial)
 {
@@ -1031,7 +1081,7 @@ k_field_update3(const double* __restrict__ x, const T* __restrict__ M, const T* 
     if (t.active) {
         const T th = gc<T>(g).theta, hdV = gc<T>(g).hdV, dt = gc<T>(g).dt;
         T mv[3], wk = T(0);
-        mv3<T, false>(S, M, t, g, mv);
+        mv3<T, false, 1>(S, M, t, g, mv);
 #pragma unroll
         for (int c = 0; c < 3; ++c) {
             const T et = S.v[c][t.tz + 1][t.ty + 1][t.tx + 1];
@@ -1352,7 +1402,7 @@ cudaError_t launch_op3(const T* M, const double* in, double sc, const double* b,
     const cudaError_t e = cudaFuncSetAttribute(k_op3<T, MODE, TR>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_op3<T, MODE, TR><<<tiles3<T>(g), Op3<T>::threads, smem, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial, dyn);
+    k_op3<T, MODE, TR><<<tiles3<T>(g), Op3<T>::share * Op3<T>::nodes, smem, st>>>(M, in, sc, b, out, vj, V, ldv, nv, g, partial, dyn);
     return cudaGetLastError();
 }
 
@@ -1372,7 +1422,7 @@ cudaError_t field_update3(const double* x, const T* M, const T* J, T* Eth, T* E,
     const cudaError_t e = cudaFuncSetAttribute(k_field_update3<T>, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (e != cudaSuccess) return e;
     count_launches(1);
-    k_field_update3<T><<<nblocks, Op3<T>::threads, smem, st>>>(x, M, J, Eth, E, B0, B1, g, partial);
+    k_field_update3<T><<<nblocks, Op3<T>::nodes, smem, st>>>(x, M, J, Eth, E, B0, B1, g, partial);
     return cudaGetLastError();
 }
 

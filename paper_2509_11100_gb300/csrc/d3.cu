@@ -300,56 +300,78 @@ __device__ __forceinline__ void load_pairs3(PairTile3<T>& tl, const T* __restric
 // full whatever the cells hold); then the warp runs over the staged particles,
 // and lane k adds to the 9 sums of one of the cell's 27 moments
 //   S[xx][yy][zz][e] = sum_p XX YY ZZ c_p alpha_e,   XX in (X0^2, X0 X1, X1^2), ..
-// (the 36 corner pairs take 27 distinct weight products), two particles per
+// (the 36 corner pairs take 27 distinct weight products), two moments per
 // paired FP32 FMA. When a cell is done, its 36 blocks go to M from shared
 // memory in address order, so that a warp's additions fall in few sectors, and
 // the moments of the cell's upper x face start the next cell's lower face
 // instead of being added to memory twice.
 //
-// Bound by issue. Before, each lane owned one or two of the 36 pairs, a cell's
-// own batches were often half empty, and each lane added its blocks by itself:
-// 61 warp instructions a particle, 11.5 ms on 256x128x128 with 32 particles a
-// cell (FP32 form), 0.23 ms on 64x32x32.
+// Bound by shared memory (FP32: three quarters of its cycles) and issue. A
+// particle is staged in 24 words, written and read 16 bytes at a time, and the
+// current comes from the moments of a fourth column, c' alpha u beside alpha's
+// three (a corner weight is the sum of eight products: X0 = XX0 + XX1, ..),
+// with a batch's particles loaded while the batch before is added up: 7.4 ms
+// on 256x128x128 with 32 particles a cell (four blocks of 128 registers an SM;
+// five with spills 10.8, three 9.3). With 36 words in 4-byte stores of two
+// particles side by side 9.1, 13.6 shared wavefronts a particle; with each
+// lane owning one or two of the 36 pairs and batches per cell 11.5.
 template <typename T>
 struct DepCfg3 {
     static constexpr int warps = sizeof(T) == 4 ? 4 : 2;   // static shared memory < 48 KB
+    static constexpr int blocks = 4;                       // an SM
 };
-constexpr int kMom3 = 27;
 constexpr int kItems3 = 36 * 9;        // a cell's additions to M
 constexpr int kFace3 = 26 * 9;         // those not on the upper x face
-// staged values of a particle: c alpha (rows of four), XX YY, corner weights
-// (lower, upper z face), ZZ, current
+constexpr int kMomZ3 = 86, kMomG3 = 255;   // words from ZZ to ZZ and from group to group (no bank conflicts)
+// staged values of a particle, FP64: c alpha (rows of four), XX YY, corner
+// weights (lower, upper z face), ZZ, current
 enum { kS3E = 0, kS3XY = 12, kS3W = 22, kS3Z = 30, kS3V = 33, kS3N = 36 };
 
-// the staged particles of a warp: FP32 two by two, (value of particle 2r,
-// value of particle 2r + 1), rows 16-byte aligned
+// the staged particles of a warp
 template <typename T>
 struct Stage3 {
     T v[32][kS3N + 1];
-    __device__ __forceinline__ void put(int t, int k, T a) { v[t][k] = a; }
+    __device__ __forceinline__ void put(int t, const T (&W)[8], const T (&XY)[9], const T (&Z)[3], const T (&ca)[9],
+                                        const T (&cu)[3])
+    {
+        T* r = v[t];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) r[kS3E + 4 * (e / 3) + e % 3] = ca[e];
+#pragma unroll
+        for (int e = 0; e < 9; ++e) r[kS3XY + e] = XY[e];
+#pragma unroll
+        for (int a = 0; a < 8; ++a) r[kS3W + a] = W[a];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r[kS3Z + e] = Z[e];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r[kS3V + e] = cu[e];
+    }
 };
+// FP32: six pieces of 16 bytes (c alpha's rows with the current's component,
+// XX YY, the ninth of them with ZZ) in a row of seven
 template <>
 struct Stage3<float> {
-    static constexpr int row = 2 * kS3N + 4;   // (an odd number of 16-byte pieces)
-    float v[16][row];
-    __device__ __forceinline__ void put(int t, int k, float a) { v[t >> 1][2 * k + (t & 1)] = a; }
-    __device__ __forceinline__ float2 get2(int r, int k) const { return *reinterpret_cast<const float2*>(&v[r][2 * k]); }
-    // two neighbouring values (k even)
-    __device__ __forceinline__ void get4(int r, int k, float2& a, float2& b) const
+    float4 v[32][7];
+    __device__ __forceinline__ void put(int t, const float (&)[8], const float (&XY)[9], const float (&Z)[3],
+                                        const float (&ca)[9], const float (&cu)[3])
     {
-        const float4 q = *reinterpret_cast<const float4*>(&v[r][2 * k]);
-        a = make_float2(q.x, q.y);
-        b = make_float2(q.z, q.w);
+        float4* r = v[t];
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r[e] = make_float4(ca[3 * e], ca[3 * e + 1], ca[3 * e + 2], cu[e]);
+        r[3] = make_float4(XY[0], XY[1], XY[2], XY[3]);
+        r[4] = make_float4(XY[4], XY[5], XY[6], XY[7]);
+        r[5] = make_float4(XY[8], Z[0], Z[1], Z[2]);
     }
 };
 
 // A lane's sums over a cell: lanes 0..26 are three groups of nine that take
-// the staged rows in turn; a group's lane (zz, er) sums the nine moments
-// (XX, YY) of its ZZ for row er of alpha, and at zz = 0 and 2 component er of
-// the current at the four corners of the lower and upper z face. (What a
-// staged row costs is the bytes a lane loads, also where all lanes load the
-// same ones: a tile of 9 products x 3 entries takes a third of the shared-
-// memory traffic of one product x 9 entries in each lane.)
+// the staged particles in turn; a group's lane (zz, er) sums the nine moments
+// (XX, YY) of its ZZ for row er of alpha and, FP64 at zz = 0 and 2, component
+// er of the current at the four corners of the lower and upper z face, FP32
+// the moments of that component. (What a staged particle costs is the bytes a
+// lane loads, also where all lanes load the same ones: a tile of 9 products x
+// 3 or 4 entries takes a third of the shared-memory traffic of one product x 9
+// entries in each lane.)
 template <typename T>
 struct Acc3 {
     T m[9][3], j[4];
@@ -383,7 +405,14 @@ struct Acc3 {
         }
     }
     __device__ __forceinline__ T moment(int k, int e) const { return m[k][e]; }
-    __device__ __forceinline__ T current(int c) const { return j[c]; }
+    // corner c of the ZZ's z face (zz = 1 has none)
+    __device__ __forceinline__ void currents(T (&o)[4]) const
+    {
+#pragma unroll
+        for (int c = 0; c < 4; ++c) o[c] = j[c];
+    }
+    // a corner's current from what the lanes of a group left: value [zz][c]
+    static __device__ __forceinline__ T corner(const T* o, int z, int at) { return o[24 * z + at]; }
     // the upper x face's sums become the next cell's lower face's
     __device__ __forceinline__ void carry()
     {
@@ -397,57 +426,67 @@ struct Acc3 {
 };
 template <>
 struct Acc3<float> {
-    float2 m[9][3], j[4];   // even and odd staged particles apart
+    float2 m[4][4];   // moments 2 k and 2 k + 1 of alpha's three entries and the current
+    float m8[4];
     __device__ __forceinline__ void clear()
     {
 #pragma unroll
-        for (int k = 0; k < 9; ++k)
+        for (int e = 0; e < 4; ++e) {
 #pragma unroll
-            for (int e = 0; e < 3; ++e) m[k][e] = make_float2(0.f, 0.f);
-#pragma unroll
-        for (int c = 0; c < 4; ++c) j[c] = make_float2(0.f, 0.f);
+            for (int k = 0; k < 4; ++k) m[k][e] = make_float2(0.f, 0.f);
+            m8[e] = 0.f;
+        }
     }
     __device__ __forceinline__ void add(const Stage3<float>& st, int t0, int t1, int grp, int zz, int er)
     {
-        const int r0 = t0 >> 1, r1 = (t1 + 1) >> 1;
-        for (int r = r0 + (grp + 3 - r0 % 3) % 3; r < r1; r += 3) {
-            float2 z = st.get2(r, kS3Z + zz), v = st.get2(r, kS3V + er);
-            // a row at the cell's ends may hold a particle of another cell
-            if (2 * r < t0) z.x = v.x = 0.f;
-            if (2 * r + 1 >= t1) z.y = v.y = 0.f;
-            float2 e[3], a, b;
-            st.get4(r, kS3E + 4 * er, a, b);
-            e[0] = __fmul2_rn(z, a);
-            e[1] = __fmul2_rn(z, b);
-            e[2] = __fmul2_rn(z, st.get2(r, kS3E + 4 * er + 2));
+#pragma unroll 2
+        for (int t = t0 + (grp + 3 - t0 % 3) % 3; t < t1; t += 3) {
+            const float4* r = st.v[t];
+            const float4 a = r[er], w0 = r[3], w1 = r[4];
+            const float* s = reinterpret_cast<const float*>(r + 5);
+            const float w8 = s[0], z = s[1 + zz];
+            const float2 w[4] = {make_float2(w0.x, w0.y), make_float2(w0.z, w0.w), make_float2(w1.x, w1.y),
+                                 make_float2(w1.z, w1.w)};
+            const float e[4] = {z * a.x, z * a.y, z * a.z, z * a.w};
 #pragma unroll
-            for (int k = 0; k < 9; k += 2) {
-                if (k < 8) st.get4(r, kS3XY + k, a, b);
-                else a = st.get2(r, kS3XY + k);
+            for (int q = 0; q < 4; ++q) {
+                const float2 ee = make_float2(e[q], e[q]);
 #pragma unroll
-                for (int q = 0; q < 3; ++q) {
-                    m[k][q] = __ffma2_rn(a, e[q], m[k][q]);
-                    if (k < 8) m[k + 1][q] = __ffma2_rn(b, e[q], m[k + 1][q]);
-                }
-            }
-#pragma unroll
-            for (int c = 0; c < 4; c += 2) {
-                st.get4(r, kS3W + 2 * zz + c, a, b);
-                j[c] = __ffma2_rn(a, v, j[c]);
-                j[c + 1] = __ffma2_rn(b, v, j[c + 1]);
+                for (int k = 0; k < 4; ++k) m[k][q] = __ffma2_rn(w[k], ee, m[k][q]);
+                m8[q] += w8 * e[q];
             }
         }
     }
-    __device__ __forceinline__ float moment(int k, int e) const { return m[k][e].x + m[k][e].y; }
-    __device__ __forceinline__ float current(int c) const { return j[c].x + j[c].y; }
-    __device__ __forceinline__ void carry()
+    __device__ __forceinline__ float moment(int k, int e) const
+    {
+        return k == 8 ? m8[e] : ((k & 1) ? m[(k >> 1) & 3][e].y : m[(k >> 1) & 3][e].x);
+    }
+    __device__ __forceinline__ void currents(float (&o)[4]) const
     {
 #pragma unroll
-        for (int k = 0; k < 9; ++k)
+        for (int c = 0; c < 4; ++c) {
+            const int k = (c & 1) * 3 + (c >> 1);
+            o[c] = (moment(k, 3) + moment(k + 1, 3)) + (moment(k + 3, 3) + moment(k + 4, 3));
+        }
+    }
+    static __device__ __forceinline__ float corner(const float* o, int z, int at)
+    {
+        return o[12 * z + at] + o[12 * z + 12 + at];
+    }
+    __device__ __forceinline__ void carry()
+    {
+        // (the current's: the upper face's corner takes XX1 + XX2)
+        float n[3][4];
 #pragma unroll
-            for (int e = 0; e < 3; ++e) m[k][e] = k < 3 ? m[k + 6][e] : make_float2(0.f, 0.f);
+        for (int y = 0; y < 3; ++y)
 #pragma unroll
-        for (int c = 0; c < 4; ++c) j[c] = (c & 1) == 0 ? j[c + 1] : make_float2(0.f, 0.f);
+            for (int e = 0; e < 4; ++e) n[y][e] = e < 3 ? moment(6 + y, e) : moment(3 + y, e) + moment(6 + y, e);
+        clear();
+#pragma unroll
+        for (int e = 0; e < 4; ++e) {
+            m[0][e] = make_float2(n[0][e], n[1][e]);
+            m[1][e] = make_float2(n[2][e], 0.f);
+        }
     }
 };
 
@@ -482,7 +521,7 @@ __device__ __forceinline__ void pair_block(int q, int& at, int& hs, int& mom, in
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * DepCfg3<T>::warps)
+__global__ void __launch_bounds__(32 * DepCfg3<T>::warps, DepCfg3<T>::blocks)
 k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__ FzArrays<T> fz,
            const T* __restrict__ B, T* __restrict__ M, T* __restrict__ J,
            GridP g, int uw)
@@ -490,9 +529,9 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
     constexpr int kW = DepCfg3<T>::warps;
     __shared__ __align__(16) Stage3<T> sst[kW];
     __shared__ Tile3B<T> stl[kW];
-    __shared__ T smom[kW][3][kMom3 * 9];   // a cell's moments (the three groups'), for the additions
-    __shared__ T scur[kW][3][24];          // and its currents: corner, component
-    __shared__ int64_t snode[kW][8];    // its corners' nodes
+    __shared__ T smom[kW][3 * kMomG3];   // a cell's moments (the three groups'), for the additions
+    __shared__ T scur[kW][3][36];        // and its currents: ZZ, corner of the z face, component
+    __shared__ int snode[kW][8];         // its corners' nodes
     __shared__ unsigned item[kItems3];  // an addition: corner << 16 | place in the node's blocks << 8 | moment value
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;
     for (int q = threadIdx.x; q < 36; q += blockDim.x) {
@@ -504,7 +543,7 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
             rank += place2 < place ? 1 : 0;
         }
         for (int e = 0; e < 9; ++e)
-            item[rank * 9 + e] = (unsigned)at << 16 | (unsigned)(hs * 9 + e) << 8 | (unsigned)(mom * 9 + e);
+            item[rank * 9 + e] = (unsigned)at << 16 | (unsigned)(hs * 9 + e) << 8 | (unsigned)(mom / 9 * kMomZ3 + mom % 9 * 9 + e);
     }
     __syncthreads();
     const int warp = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
@@ -546,42 +585,54 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
             const int base = first - (incl - cnt);   // particle = base + list index
             int cl = 0;                              // the cell the warp is adding up
             int cend = __shfl_sync(0xffffffffu, incl, nsp - 1);
-            for (int w0 = 0; cl < gc0; w0 += 32) {   // (every pass ends cells or takes 32 particles)
-                const int t = w0 + lane;
+            // a batch's particles are loaded while the batch before is added up
+            int nsg = 0;
+            T nfx = T(0), nfy = T(0), nfz = T(0), nux = T(0), nuy = T(0), nuz = T(0), nwt = T(0);
+            auto fetch = [&](int t) {
                 // the range the lane's particle lies in (all lanes search)
                 int seg = 0;
 #pragma unroll
                 for (int o = 16; o > 0; o >>= 1)
                     if (__shfl_sync(0xffffffffu, incl, seg + o - 1) <= t) seg += o;
                 const int p = __shfl_sync(0xffffffffu, base, seg) + t;
+                nsg = seg;
+                if (t < total) {
+                    const int s = seg % nsp;
+                    nfx = ld(ds.fx[s] + p);
+                    nfy = ld(ds.fy[s] + p);
+                    nfz = ld(fz.fz[s] + p);
+                    nux = ld(ds.ux[s] + p);
+                    nuy = ld(ds.uy[s] + p);
+                    nuz = ld(ds.uz[s] + p);
+                    nwt = ld(ds.w[s] + p);
+                }
+            };
+            fetch(lane);
+            for (int w0 = 0; cl < gc0; w0 += 32) {   // (every pass ends cells or takes 32 particles)
+                const int t = w0 + lane;
+                const int seg = nsg;
+                const T fx = nfx, fy = nfy, fzz = nfz, ux = nux, uy = nuy, uz = nuz, wt = nwt;
+                if (w0 + 32 < total) fetch(t + 32);
                 if (t < total) {
                     const int s = seg % nsp, pc = cg + seg / nsp;
-                    const T fx = ld(ds.fx[s] + p), fy = ld(ds.fy[s] + p), fzz = ld(fz.fz[s] + p);
-                    const T ux = ld(ds.ux[s] + p), uy = ld(ds.uy[s] + p), uz = ld(ds.uz[s] + p);
-                    const T wt = ld(ds.w[s] + p);
-                    T W[8], Bp[3], al[9];
-                    corner_weights(fx, fy, fzz, W);
+                    T W[8] = {}, Bp[3], al[9];
+                    if (sizeof(T) == 8) corner_weights(fx, fy, fzz, W);
                     tile_B3(stl[wib].B, pc, fx, fy, fzz, Bp);
                     const T ig = T(1) / sqrt(T(1) + ux * ux + uy * uy + uz * uz);
                     alpha3(Bp, ds.beta[s] * ig, al);
                     const T cM = wt * ds.cM[s] * ig, cJ = wt * ds.cJ[s] * ig;
                     const T X[3] = {(T(1) - fx) * (T(1) - fx), (T(1) - fx) * fx, fx * fx};
                     const T Y[3] = {(T(1) - fy) * (T(1) - fy), (T(1) - fy) * fy, fy * fy};
+                    const T Z[3] = {(T(1) - fzz) * (T(1) - fzz), (T(1) - fzz) * fzz, fzz * fzz};
+                    T XY[9], ca[9], cu[3];
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) st.put(lane, kS3E + 4 * (e / 3) + e % 3, cM * al[e]);
+                    for (int e = 0; e < 9; ++e) {
+                        ca[e] = cM * al[e];
+                        XY[e] = X[e / 3] * Y[e % 3];
+                    }
 #pragma unroll
-                    for (int e = 0; e < 9; ++e) st.put(lane, kS3XY + e, X[e / 3] * Y[e % 3]);
-                    st.put(lane, kS3Z, (T(1) - fzz) * (T(1) - fzz));
-                    st.put(lane, kS3Z + 1, (T(1) - fzz) * fzz);
-                    st.put(lane, kS3Z + 2, fzz * fzz);
-#pragma unroll
-                    for (int a = 0; a < 8; ++a) st.put(lane, kS3W + a, W[a]);
-#pragma unroll
-                    for (int r = 0; r < 3; ++r)
-                        st.put(lane, kS3V + r, cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz));
-                } else {
-#pragma unroll
-                    for (int q = 0; q < kS3N; ++q) st.put(lane, q, T(0));
+                    for (int r = 0; r < 3; ++r) cu[r] = cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz);
+                    st.put(lane, W, XY, Z, ca, cu);
                 }
                 __syncwarp();
                 const int wend = min(w0 + 32, total);
@@ -596,32 +647,40 @@ k_deposit3(const __grid_constant__ DepositSpecies<T> ds, const __grid_constant__
                     const bool last = cg + cl == cn - 1;
                     if (carry || cend > before) {
                         if (own) {
-                            T* const o = smom[wib][grp] + zz * 81 + er * 3;
+                            T* const o = smom[wib] + grp * kMomG3 + zz * kMomZ3 + er * 3;
 #pragma unroll
                             for (int k = 0; k < 9; ++k)
                                 if (k < 6 || last)
 #pragma unroll
                                     for (int e = 0; e < 3; ++e) o[k * 9 + e] = acc.moment(k, e);
-                            if (zz != 1)
+                            T cur[4];
+                            acc.currents(cur);
 #pragma unroll
-                                for (int c = 0; c < 4; ++c) scur[wib][grp][(zz * 2 + c) * 3 + er] = acc.current(c);
+                            for (int c = 0; c < 4; ++c) scur[wib][grp][(zz * 4 + c) * 3 + er] = cur[c];
                         }
                         const int i = i0 + cg + cl;
                         const int64_t nd = node3(wrap1(i + (lane & 1), g.nx), wrap1(j + ((lane >> 1) & 1), g.ny),
                                                  wrap1(k + ((lane >> 2) & 1), g.nz), g);
-                        if (lane < 8) snode[wib][lane] = nd;
+                        if (lane < 8) snode[wib][lane] = (int)nd;
                         __syncwarp();
-                        const int nit = last ? kItems3 : kFace3;
-                        const T* sm = &smom[wib][0][0];
-                        for (int it = lane; it < nit; it += 32) {
-                            const unsigned q = item[it], v = q & 255u;
-                            atomicAdd(M + snode[wib][q >> 16] * kMBlock3 + ((q >> 8) & 255u),
-                                      sm[v] + sm[kMom3 * 9 + v] + sm[2 * kMom3 * 9 + v]);
-                        }
+                        const T* sm = &smom[wib][0];
+                        auto give = [&](unsigned q) {
+                            const unsigned v = q & 255u;
+                            atomicAdd(M + (int64_t)snode[wib][q >> 16] * kMBlock3 + ((q >> 8) & 255u),
+                                      sm[v] + sm[kMomG3 + v] + sm[2 * kMomG3 + v]);
+                        };
+#pragma unroll
+                        for (int v = 0; v < (kFace3 + 31) / 32; ++v)
+                            if (lane + 32 * v < kFace3) give(item[lane + 32 * v]);
+                        if (last)
+                            for (int it = kFace3 + lane; it < kItems3; it += 32) give(item[it]);
                         const int ja = lane / 3, jc = lane % 3;
-                        if (lane < 24 && (last || (ja & 1) == 0))
+                        if (lane < 24 && (last || (ja & 1) == 0)) {
+                            const int at = (ja & 3) * 3 + jc, z = ja >> 2;
                             atomicAdd(J + (int64_t)jc * g.ncell + snode[wib][ja],
-                                      scur[wib][0][lane] + scur[wib][1][lane] + scur[wib][2][lane]);
+                                      Acc3<T>::corner(scur[wib][0], z, at) + Acc3<T>::corner(scur[wib][1], z, at) +
+                                          Acc3<T>::corner(scur[wib][2], z, at));
+                        }
                         __syncwarp();
                         carry = !last;
                     }

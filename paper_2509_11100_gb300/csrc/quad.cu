@@ -140,63 +140,122 @@ __device__ __forceinline__ void alphaq(const T (&Bp)[3], T bg, T (&al)[9])   // 
 // a group touches the same 3 x 3 frame of the cell's 4 x 4 nodes. Along an
 // axis the frame's node pairs have six weight products, so a particle adds
 // c alpha_e to 36 products; 27 lanes each sum 2 x 2 of them for one row of
-// alpha (4 products x 3 entries, two particles per paired FP32 FMA), per
+// alpha (4 products x 3 entries, two products per paired FP32 FMA), per
 // group in registers over the cell. A cell's sums then go to the union's
 // products in shared memory, held by the column of their left node in a ring
 // of four columns: the next cell's union is this one's moved by a column, so
 // only the column that falls out is added to M, its 37 blocks in address
 // order (the sums of the others grow on).
 //
-// Bound by issue. Before, each lane owned node pairs (45 a group, 106 a
-// cell), a group's sums went through shared memory every 32 particles and
-// all 106 blocks of every cell went to M: 81 warp instructions a particle,
-// 1.85 ms on 512x256 with 128 particles a cell (FP32 form).
+// Bound by shared memory (FP32: 81% of its cycles when a particle's 36 values
+// were stored 4 bytes at a time, two particles side by side: 1.25 ms on
+// 512x256 with 128 particles a cell). A particle is staged in nine 16-byte
+// pieces and a batch's particles are loaded while the batch before is added
+// up: 1.02 ms (1.12 without the early loads; at five blocks an SM the spills
+// make it 1.6). With each lane owning node pairs (45 a group, 106 a cell) and
+// all 106 blocks of every cell added to M it took 1.85.
 template <typename T>
 struct DepCfgQ {
     static constexpr int warps = sizeof(T) == 4 ? 4 : 2;   // static shared memory below 48 KB
-};
-
-// what a lane adds at once: FP32 two particles, FP64 one
-template <typename T>
-struct Pk;
-template <>
-struct Pk<float> {
-    using V = float2;
-    static constexpr int n = 2;
-    static __device__ __forceinline__ V zero() { return make_float2(0.f, 0.f); }
-    static __device__ __forceinline__ V mul(V a, V b) { return __fmul2_rn(a, b); }
-    static __device__ __forceinline__ V fma(V a, V b, V c) { return __ffma2_rn(a, b, c); }
-    static __device__ __forceinline__ float sum(V a) { return a.x + a.y; }
-    // two neighbouring staged values (16-byte aligned)
-    static __device__ __forceinline__ void two(const V* p, V& a, V& b)
-    {
-        const float4 q = *reinterpret_cast<const float4*>(p);
-        a = make_float2(q.x, q.y);
-        b = make_float2(q.z, q.w);
-    }
-};
-template <>
-struct Pk<double> {
-    using V = double;
-    static constexpr int n = 1;
-    static __device__ __forceinline__ V zero() { return 0.0; }
-    static __device__ __forceinline__ V mul(V a, V b) { return a * b; }
-    static __device__ __forceinline__ V fma(V a, V b, V c) { return a * b + c; }
-    static __device__ __forceinline__ double sum(V a) { return a; }
-    static __device__ __forceinline__ void two(const V* p, V& a, V& b)
-    {
-        a = p[0];
-        b = p[1];
-    }
+    static constexpr int blocks = 4;                       // an SM
 };
 
 // staged values of a particle: the six x and six y products, c alpha (rows of
-// four), the frame's nine weights, the current
-enum { kQXX = 0, kQYY = 6, kQE = 12, kQW = 24, kQV = 33, kQN = 36, kQRow = 38 };
+// four, FP32 with the current's component as the fourth), the frame's nine
+// weights, FP64 the current
+enum { kQXX = 0, kQYY = 6, kQE = 12, kQW = 24, kQV = 33, kQRow = 38 };
 template <typename T>
 struct StageQ {
-    typename Pk<T>::V v[32 / Pk<T>::n + 4][kQRow];   // a group starts on a row of its own
-    __device__ __forceinline__ void put(int row, int at, int k, T a) { reinterpret_cast<T*>(&v[row][k])[at] = a; }
+    T v[32][kQRow];
+    __device__ __forceinline__ void put(int row, const T (&xx)[6], const T (&yy)[6], const T (&ca)[9], const T (&W)[9],
+                                        const T (&cu)[3])
+    {
+        T* r = v[row];
+#pragma unroll
+        for (int e = 0; e < 6; ++e) {
+            r[kQXX + e] = xx[e];
+            r[kQYY + e] = yy[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 9; ++e) {
+            r[kQE + 4 * (e / 3) + e % 3] = ca[e];
+            r[kQW + e] = W[e];
+        }
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r[kQV + e] = cu[e];
+    }
+};
+template <>
+struct StageQ<float> {
+    float4 v[32][9];   // (an odd number of 16-byte pieces: rows start on different banks)
+    __device__ __forceinline__ void put(int row, const float (&xx)[6], const float (&yy)[6], const float (&ca)[9],
+                                        const float (&W)[9], const float (&cu)[3])
+    {
+        float4* r = v[row];
+        r[0] = make_float4(xx[0], xx[1], xx[2], xx[3]);
+        r[1] = make_float4(xx[4], xx[5], yy[0], yy[1]);
+        r[2] = make_float4(yy[2], yy[3], yy[4], yy[5]);
+#pragma unroll
+        for (int e = 0; e < 3; ++e) r[3 + e] = make_float4(ca[3 * e], ca[3 * e + 1], ca[3 * e + 2], cu[e]);
+        r[6] = make_float4(W[0], W[1], W[2], W[3]);
+        r[7] = make_float4(W[4], W[5], W[6], W[7]);
+        reinterpret_cast<float*>(r + 8)[0] = W[8];
+    }
+};
+
+// a lane's sums over staged particles: product (x type 2 xg + (q & 1), y type
+// 2 yg + (q >> 1)), entry e of its row of alpha, and its current
+template <typename T>
+struct SumQ {
+    T a[12], j;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int e = 0; e < 12; ++e) a[e] = T(0);
+        j = T(0);
+    }
+    __device__ __forceinline__ void add(const StageQ<T>& st, int row, int xg, int yg, int er, int jf)
+    {
+        const T* r = st.v[row];
+        const T x0 = r[kQXX + 2 * xg], x1 = r[kQXX + 2 * xg + 1], y0 = r[kQYY + 2 * yg], y1 = r[kQYY + 2 * yg + 1];
+        const T w[4] = {x0 * y0, x1 * y0, x0 * y1, x1 * y1};
+#pragma unroll
+        for (int q = 0; q < 4; ++q)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) a[3 * q + e] += w[q] * r[kQE + 4 * er + e];
+        j += r[kQW + jf] * r[kQV + er];
+    }
+    __device__ __forceinline__ T value(int q, int e) const { return a[3 * q + e]; }
+};
+template <>
+struct SumQ<float> {
+    float2 a[2][3];   // [y type][entry], both x types
+    float j;
+    __device__ __forceinline__ void clear()
+    {
+#pragma unroll
+        for (int y = 0; y < 2; ++y)
+#pragma unroll
+            for (int e = 0; e < 3; ++e) a[y][e] = make_float2(0.f, 0.f);
+        j = 0.f;
+    }
+    __device__ __forceinline__ void add(const StageQ<float>& st, int row, int xg, int yg, int er, int jf)
+    {
+        const float* r = reinterpret_cast<const float*>(st.v[row]);
+        const float2 x = *reinterpret_cast<const float2*>(r + kQXX + 2 * xg);
+        const float2 y = *reinterpret_cast<const float2*>(r + kQYY + 2 * yg);
+        const float4 e = *reinterpret_cast<const float4*>(r + kQE + 4 * er);
+        const float2 w0 = make_float2(x.x * y.x, x.y * y.x), w1 = make_float2(x.x * y.y, x.y * y.y);
+        const float2 e0 = make_float2(e.x, e.x), e1 = make_float2(e.y, e.y), e2 = make_float2(e.z, e.z);
+        a[0][0] = __ffma2_rn(w0, e0, a[0][0]);
+        a[0][1] = __ffma2_rn(w0, e1, a[0][1]);
+        a[0][2] = __ffma2_rn(w0, e2, a[0][2]);
+        a[1][0] = __ffma2_rn(w1, e0, a[1][0]);
+        a[1][1] = __ffma2_rn(w1, e1, a[1][1]);
+        a[1][2] = __ffma2_rn(w1, e2, a[1][2]);
+        j += r[kQW + jf] * e.w;
+    }
+    __device__ __forceinline__ float value(int q, int e) const { return (q & 1) ? a[q >> 1][e].y : a[q >> 1][e].x; }
 };
 
 // the union's products: [column of the left node, a ring of four][dx][row c,
@@ -227,13 +286,11 @@ __device__ __forceinline__ void column_block(int q, int& col, int& row, int& hs,
 }
 
 template <typename T>
-__global__ void __launch_bounds__(32 * DepCfgQ<T>::warps)
+__global__ void __launch_bounds__(32 * DepCfgQ<T>::warps, DepCfgQ<T>::blocks)
 k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ B, T* __restrict__ M,
             T* __restrict__ J, GridP g, int uw)
 {
     constexpr int kW = DepCfgQ<T>::warps;
-    using P = Pk<T>;
-    using V = typename P::V;
     __shared__ __align__(16) StageQ<T> sst[kW];
     __shared__ T sum_[kW][4 * kUCol];
     __shared__ T sumj[kW][4][12];       // currents: [column][3 row + component]
@@ -301,43 +358,44 @@ k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ 
 #pragma unroll
                     for (int e = 0; e < 12; ++e) acc[gq][e] = T(0);
                 }
-                for (int q0 = 0; q0 < total; q0 += 32) {
-                    const int t = q0 + lane;
-                    const bool act = t < total;
-                    T fx = T(0), fy = T(0);
+                // a batch's particles are loaded while the batch before is added up
+                int ns = 0;
+                T nfx = T(0), nfy = T(0), nux = T(0), nuy = T(0), nuz = T(0), nwt = T(0);
+                auto fetch = [&](int t) {
+                    if (t >= total) return;
                     int s = 0, p = pst[0] + t;
-                    if (act) {
 #pragma unroll
-                        for (int q = 1; q < kMaxSpecies; ++q)
-                            if (t >= cum[q] && cum[q + 1] > cum[q]) {
-                                s = q;
-                                p = pst[q] + (t - cum[q]);
-                            }
-                        fx = ld(ds.fx[s] + p);
-                        fy = ld(ds.fy[s] + p);
-                    }
+                    for (int q = 1; q < kMaxSpecies; ++q)
+                        if (t >= cum[q] && cum[q + 1] > cum[q]) {
+                            s = q;
+                            p = pst[q] + (t - cum[q]);
+                        }
+                    ns = s;
+                    nfx = ld(ds.fx[s] + p);
+                    nfy = ld(ds.fy[s] + p);
+                    nux = ld(ds.ux[s] + p);
+                    nuy = ld(ds.uy[s] + p);
+                    nuz = ld(ds.uz[s] + p);
+                    nwt = ld(ds.w[s] + p);
+                };
+                fetch(lane);
+                for (int q0 = 0; q0 < total; q0 += 32) {
+                    const int t = q0 + lane, s = ns;
+                    const bool act = t < total;
+                    const T fx = nfx, fy = nfy, ux = nux, uy = nuy, uz = nuz, wt = nwt;
+                    fetch(t + 32);
                     const int hx = fx >= T(0.5), hy = fy >= T(0.5);
                     const int grp = act ? 2 * hy + hx : -1;
                     // rows of the groups, and this particle's place
-                    int gr[5], row = 0, at = 0;
+                    int gr[5], row = 0;
                     gr[0] = 0;
 #pragma unroll
                     for (int gq = 0; gq < 4; ++gq) {
                         const unsigned bal = __ballot_sync(0xffffffffu, grp == gq);
-                        const int cnt = __popc(bal), place = __popc(bal & ((1u << lane) - 1u));
-                        gr[gq + 1] = gr[gq] + (cnt + P::n - 1) / P::n;
-                        if (grp == gq) {
-                            row = gr[gq] + place / P::n;
-                            at = place % P::n;
-                        }
-                        if (P::n == 2 && (cnt & 1)) {   // the row's other half
-                            st.put(gr[gq + 1] - 1, 1, lane, T(0));
-                            if (lane < kQN - 32) st.put(gr[gq + 1] - 1, 1, 32 + lane, T(0));
-                        }
+                        gr[gq + 1] = gr[gq] + __popc(bal);
+                        if (grp == gq) row = gr[gq] + __popc(bal & ((1u << lane) - 1u));
                     }
                     if (act) {
-                        const T ux = ld(ds.ux[s] + p), uy = ld(ds.uy[s] + p), uz = ld(ds.uz[s] + p);
-                        const T wt = ld(ds.w[s] + p);
                         T wx[3], wy[3], Bp[3], al[9];
                         quad3(hx ? fx - T(1) : fx, wx);
                         quad3(hy ? fy - T(1) : fy, wy);
@@ -345,52 +403,39 @@ k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ 
                         const T ig = T(1) / sqrt(T(1) + ux * ux + uy * uy + uz * uz);
                         alphaq(Bp, ds.beta[s] * ig, al);
                         const T cM = wt * ds.cM[s] * ig, cJ = wt * ds.cJ[s] * ig;
+                        T xx[6], yy[6], W[9], cu[3];
                         int n = 0;
 #pragma unroll
                         for (int a = 0; a < 3; ++a)
 #pragma unroll
                             for (int b2 = a; b2 < 3; ++b2) {
-                                st.put(row, at, kQXX + n, wx[a] * wx[b2]);
-                                st.put(row, at, kQYY + n, wy[a] * wy[b2]);
+                                xx[n] = wx[a] * wx[b2];
+                                yy[n] = wy[a] * wy[b2];
                                 ++n;
                             }
 #pragma unroll
-                        for (int e = 0; e < 9; ++e) st.put(row, at, kQE + 4 * (e / 3) + e % 3, cM * al[e]);
+                        for (int r = 0; r < 3; ++r) {
 #pragma unroll
-                        for (int r = 0; r < 3; ++r)
+                            for (int c2 = 0; c2 < 3; ++c2) W[3 * r + c2] = wy[r] * wx[c2];
+                            cu[r] = cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz);
+                        }
 #pragma unroll
-                            for (int c2 = 0; c2 < 3; ++c2) st.put(row, at, kQW + 3 * r + c2, wy[r] * wx[c2]);
-#pragma unroll
-                        for (int r = 0; r < 3; ++r)
-                            st.put(row, at, kQV + r,
-                                   cJ * (al[3 * r] * ux + al[3 * r + 1] * uy + al[3 * r + 2] * uz));
+                        for (int e = 0; e < 9; ++e) al[e] *= cM;
+                        st.put(row, xx, yy, al, W, cu);
                     }
                     __syncwarp();
 #pragma unroll
                     for (int gq = 0; gq < 4; ++gq) {
                         if (gr[gq + 1] == gr[gq]) continue;   // warp-uniform
-                        V a[12], aj = P::zero();
+                        SumQ<T> a;
+                        a.clear();
+                        #pragma unroll 2
+                        for (int r = gr[gq]; r < gr[gq + 1]; ++r) a.add(st, r, xg, yg, er, jf);
 #pragma unroll
-                        for (int e = 0; e < 12; ++e) a[e] = P::zero();
-                        for (int r = gr[gq]; r < gr[gq + 1]; ++r) {
-                            const V* rw = st.v[r];
-                            V x0, x1, y0, y1, e0, e1;
-                            P::two(rw + kQXX + 2 * xg, x0, x1);
-                            P::two(rw + kQYY + 2 * yg, y0, y1);
-                            P::two(rw + kQE + 4 * er, e0, e1);
-                            const V e2 = rw[kQE + 4 * er + 2];
-                            const V w[4] = {P::mul(x0, y0), P::mul(x1, y0), P::mul(x0, y1), P::mul(x1, y1)};
+                        for (int q = 0; q < 4; ++q)
 #pragma unroll
-                            for (int q = 0; q < 4; ++q) {
-                                a[3 * q] = P::fma(w[q], e0, a[3 * q]);
-                                a[3 * q + 1] = P::fma(w[q], e1, a[3 * q + 1]);
-                                a[3 * q + 2] = P::fma(w[q], e2, a[3 * q + 2]);
-                            }
-                            aj = P::fma(rw[kQW + jf], rw[kQV + jc], aj);
-                        }
-#pragma unroll
-                        for (int e = 0; e < 12; ++e) acc[gq][e] += P::sum(a[e]);
-                        accj[gq] += P::sum(aj);
+                            for (int e = 0; e < 3; ++e) acc[gq][3 * q + e] += a.value(q, e);
+                        accj[gq] += a.j;
                     }
                     __syncwarp();
                 }

@@ -1234,6 +1234,7 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PRecords<T> dst,
         int cl = 0;
         // the next batch is loaded while this one is pushed
         T nfx = T(0), nfy = T(0), nfz = T(0), nux = T(0), nuy = T(0), nuz = T(0), nw = T(0);
+        int nid = 0;
         auto fetch = [&](int q) {
             if (q < P1) {
                 nfx = ld(src.fx + q);
@@ -1243,6 +1244,7 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PRecords<T> dst,
                 nuy = ld(src.uy + q);
                 nuz = ld(src.uz + q);
                 nw = ld(src.w + q);
+                if (src.id) nid = ld(src.id + q);
             }
         };
         fetch(P0 + lane);
@@ -1250,6 +1252,7 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PRecords<T> dst,
             const int p = p0 + lane;
             const bool act = p < P1;
             const T fx = nfx, fy = nfy, fz = nfz, ux = nux, uy = nuy, uz = nuz, w = nw;
+            const int pid = nid;
             fetch(p + 32);
             int newkey = -1 - lane;   // distinct for idle lanes
             if (act) {
@@ -1290,7 +1293,7 @@ k_push3(PArrays<T> src, const T* __restrict__ sfz, PRecords<T> dst,
                 dst.a[p] = PRecA<T>{fn[0], fn[1], u1x, u1y};
                 dst.b[p] = PRecB<T>{u1z, w};
                 dst.fz[p] = fn[2];
-                if (dst.id) dst.id[p] = src.id[p];
+                if (dst.id) dst.id[p] = pid;
                 newkey = (int32_t)node3(cnew[0], cnew[1], cnew[2], g);
                 key[p] = newkey;
                 // ledger: g0 - g1 = (u0 - u1).(u0 + u1)/(g0 + g1)

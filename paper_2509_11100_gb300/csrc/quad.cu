@@ -840,6 +840,7 @@ k_push_q(PArrays<T> src, PRecords<T> dst, const int32_t* __restrict__ start, int
         int cl = 0;
         // the next batch is loaded while this one is pushed
         T nfx = T(0), nfy = T(0), nux = T(0), nuy = T(0), nuz = T(0), nw = T(0);
+        int nid = 0;
         auto fetch = [&](int q) {
             if (q < P1) {
                 nfx = ld(src.fx + q);
@@ -848,6 +849,7 @@ k_push_q(PArrays<T> src, PRecords<T> dst, const int32_t* __restrict__ start, int
                 nuy = ld(src.uy + q);
                 nuz = ld(src.uz + q);
                 nw = ld(src.w + q);
+                if (src.id) nid = ld(src.id + q);
             }
         };
         fetch(P0 + lane);
@@ -855,6 +857,7 @@ k_push_q(PArrays<T> src, PRecords<T> dst, const int32_t* __restrict__ start, int
             const int p = p0 + lane;
             const bool act = p < P1;
             const T fx = nfx, fy = nfy, ux = nux, uy = nuy, uz = nuz, w = nw;
+            const int pid = nid;
             fetch(p + 32);
             int newkey = -1 - lane;
             if (act) {
@@ -911,7 +914,7 @@ k_push_q(PArrays<T> src, PRecords<T> dst, const int32_t* __restrict__ start, int
                 }
                 dst.a[p] = PRecA<T>{fn[0], fn[1], u1x, u1y};
                 dst.b[p] = PRecB<T>{u1z, w};
-                if (dst.id) dst.id[p] = src.id[p];
+                if (dst.id) dst.id[p] = pid;
                 newkey = cnew[1] * g.nx + cnew[0];
                 key[p] = newkey;
                 const T ue = ubx * E[0] + uby * E[1] + ubz * E[2];

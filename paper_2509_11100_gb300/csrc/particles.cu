@@ -1034,7 +1034,6 @@ struct PushTile {
 template <typename T, int C>
 struct PushStage {
     T fx[C], fy[C], ux[C], uy[C], uz[C], w[C];
-    int32_t id[C];
     uint8_t dir[C], rank[C], inv[C], cell[C];
     int doff[kGroupMax * (kNDir + 1)];
     int run[kGroupMax * kNDir];
@@ -1290,7 +1289,6 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
                     st.uy[e] = o.u1y;
                     st.uz[e] = o.u1z;
                     st.w[e] = o.w;
-                    if (ids) st.id[e] = src.id[p];
                     st.dir[e] = (uint8_t)o.dir;
                     st.rank[e] = (uint8_t)rank;
                     st.cell[e] = (uint8_t)ci;
@@ -1320,8 +1318,12 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
                 dst.uy[s0 + qq] = st.uy[e];
                 dst.uz[s0 + qq] = st.uz[e];
                 dst.w[s0 + qq] = st.w[e];
-                if (ids) dst.id[s0 + qq] = st.id[e];
             }
+            // (ids move only here: loaded with the batch they would hold registers
+            // or make the warp wait)
+            if (ids)
+#pragma unroll 4
+                for (int qq = lane; qq < tot; qq += 32) dst.id[s0 + qq] = ld(src.id + s0 + st.inv[qq]);
             // the runs of the group's cells: counts and starts per direction
             for (int i = lane; i < gsz * kNDir; i += 32) {
                 const int gi = i / kNDir, d = i - gi * kNDir;

@@ -926,10 +926,10 @@ template <typename T> struct PushCfg {
     static constexpr int warps = 4;                        // static shared memory < 48 KB
     static constexpr int threads = 32 * warps;
     static constexpr int min_blocks = sizeof(T) == 4 ? 5 : 2;
-    static constexpr int cap = sizeof(T) == 4 ? 256 : 128;   // particles of a cell group staged per warp
-    // with the E^n tile of the predicted gamma (3 KB more per block in
-    // FP32) a smaller group keeps five blocks on an SM
-    static constexpr int cap_pred = sizeof(T) == 4 ? 224 : 128;
+    // particles of a cell group staged per warp (uint8 indices; five blocks on
+    // an SM, also with the E^n tile of the predicted gamma: with 224 there
+    // 1304 and 73.3 us a step at 1024x512 and 251x99, now 1296 and 72.4)
+    static constexpr int cap = sizeof(T) == 4 ? 256 : 128;
 };
 constexpr int kGroupMax = 8;    // cells staged together at most
 constexpr int kLedger = 4;      // dK, work, mismatch, K1 (K0 is the previous K1)
@@ -1038,9 +1038,7 @@ struct PushStage {
     int doff[kGroupMax * (kNDir + 1)];
     int run[kGroupMax * kNDir];
 };
-static_assert(PushCfg<float>::cap <= 256 && PushCfg<double>::cap <= 256 && PushCfg<float>::cap_pred <= 256 &&
-                  PushCfg<double>::cap_pred <= 256,
-              "uint8 staging indices");
+static_assert(PushCfg<float>::cap <= 256 && PushCfg<double>::cap <= 256, "uint8 staging indices");
 
 template <typename T>
 __device__ __forceinline__ void block_ledger(const T (&acc)[kLedger], double* red, double* __restrict__ lsum)
@@ -1118,7 +1116,7 @@ __device__ __forceinline__ void push_sort_core(PArrays<T> src, PArrays<T> dst, c
     __shared__ int sstart[W][kUnitW + 1];
     __shared__ PushTile<T> stile[W];
     __shared__ PredTile<T, PRED> sen[W];
-    constexpr int CAP = PRED ? PushCfg<T>::cap_pred : PushCfg<T>::cap;
+    constexpr int CAP = PushCfg<T>::cap;
     __shared__ PushStage<T, CAP> sstage[W];
     __shared__ double red[32 * kLedger];
     const int lane = threadIdx.x & 31, wib = threadIdx.x >> 5;

@@ -108,6 +108,15 @@ __host__ __device__ __forceinline__ int wrap1(int i, int n)
     return i < 0 ? i + n : (i >= n ? i - n : i);
 }
 
+// node `place` (4 columns to the right + rows down) of the 3 columns x 4 rows
+// that the quadratic deposit's column left of cell (i, j) adds to. i runs up
+// to three cells past its row segment (the columns left over), so the index
+// reaches nx + 3: one wrap more than wrap1 where the grid is three cells wide.
+__host__ __device__ __forceinline__ int column_node_q(int i, int j, int place, int nx, int ny)
+{
+    return wrap1(j - 1 + (place & 3), ny) * nx + wrap1(wrap1(i - 1 + (place >> 2), nx), nx);
+}
+
 template <typename T>
 __device__ __forceinline__ T ld(const T* p) { return __ldg(p); }
 

@@ -459,8 +459,7 @@ k_deposit_q(const __grid_constant__ DepositSpecies<T> ds, const T* __restrict__ 
             }
             // the column of nodes i - 1 is complete
             if (live > 0) {
-                if (lane < 12)
-                    snode[wib][lane] = wrap1(j - 1 + (lane & 3), g.ny) * g.nx + wrap1(i - 1 + (lane >> 2), g.nx);
+                if (lane < 12) snode[wib][lane] = column_node_q(i, j, lane, g.nx, g.ny);
                 __syncwarp();
                 T* const C = U + (cl & 3) * kUCol;
                 for (int it = lane; it < kItemsQ; it += 32) {

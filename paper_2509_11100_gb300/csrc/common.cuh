@@ -231,18 +231,29 @@ template <> __device__ __forceinline__ float narrow<float>(double a)
 
 __device__ __forceinline__ bool finite_bits(double v) { return (__double2hiint(v) & 0x7ff00000) != 0x7ff00000; }
 
+// A finite lattice coordinate wrapped into [0, n). One pass does up to 2^53
+// boxes away; beyond, the quotient holds 53 bits and the remainder (exact: one
+// multiply-add) may be far outside still, so the passes go on until it is
+// inside (20 from the largest coordinate). What stays outside is a negative
+// subnormal whose quotient rounds to zero: as every coordinate that rounds to
+// the box's length it lies at the box's beginning.
+__host__ __device__ __forceinline__ double wrap_coord(double xs, int n)
+{
+    for (int t = 0; t < 40 && !(xs >= 0.0 && xs < (double)n); ++t) xs = fma(-(double)n, floor(xs / n), xs);
+    return xs >= 0.0 && xs < (double)n ? xs : 0.0;
+}
+
 // A finite lattice coordinate into its cell (wrapped into [0, n)) and the
 // offset within it, rounded toward zero in FP32
 template <typename T>
 __device__ __noinline__ void split_cell_wrap(double xs, int n, int& i, T& f)
 {
-    if (xs < 0.0 || xs >= (double)n) xs -= n * floor(xs / n);
+    xs = wrap_coord(xs, n);
     const double fi = floor(xs);
-    i = (int)fi;
-    if (i >= n) i -= n;
-    if (i < 0) i = 0;
+    i = min(max((int)fi, 0), n - 1);
     f = from_double_rz<T>(xs - fi);
 }
+
 template <typename T>
 __device__ __forceinline__ void split_cell(double xs, int n, int& i, T& f)
 {

@@ -255,39 +255,6 @@ __device__ __forceinline__ T gbar_u2(T ux, T uy, T uz, T beta, const T (*sEn)[2]
     return sx * sx + sy * sy + sz * sz;
 }
 
-// reciprocal square root and reciprocal: the hardware approximations in the
-// FP32 form (a few ulp). In the FP64 form Newton's iteration from the
-// hardware's FP64 approximations (a relative error e becomes 1.5 e^2 or e^2: two
-// steps from about 2^-20 end at the rounding of the last one): the FP64 pipe
-// takes a warp's operation in about 64 cycles and bounds the FP64 push and
-// deposit, and a square root and a division took it three times as many
-// operations. Values near the ends of the range go the long way.
-__device__ __forceinline__ bool mid_range(double x)   // 2^-900 <= x < 2^900
-{
-    return (unsigned)__double2hiint(x) - ((1023u - 900u) << 20) < (1800u << 20);
-}
-__device__ __forceinline__ float rsqrt_t(float x) { return rsqrtf(x); }
-__device__ __forceinline__ double rsqrt_t(double x)
-{
-    if (!mid_range(x)) return 1.0 / sqrt(x);
-    double y;
-    asm("rsqrt.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-    const double h = -0.5 * x;
-#pragma unroll
-    for (int k = 0; k < 2; ++k) y = fma(y, fma(h, y * y, 0.5), y);
-    return y;
-}
-__device__ __forceinline__ float rcp_t(float x) { return __fdividef(1.0f, x); }
-__device__ __forceinline__ double rcp_t(double x)
-{
-    if (!mid_range(x)) return 1.0 / x;
-    double y;
-    asm("rcp.approx.ftz.f64 %0, %1;" : "=d"(y) : "d"(x));
-#pragma unroll
-    for (int k = 0; k < 2; ++k) y = fma(y, fma(-x, y, 1.0), y);
-    return y;
-}
-
 // The rotation of one particle, shared by the deposit and the push so both
 // see the same alpha: 1/gbar, a = beta B/gbar and 1/(1 + |a|^2).
 template <typename T>

@@ -611,7 +611,10 @@ RELSIM_API void relsim_batch_destroy(relsim_batch* b);
    operator (the 3D and quadratic operators have one): its tile height
    (32-node-wide tiles of 8 or 4 rows in the FP32 form, 4 or 2 in FP64; an
    Arnoldi-mode application with 8 dot products on the deposited mass
-   matrix). Each candidate runs once untimed and three times timed (CUDA events;
+   matrix). Grids whose tiles all fit on the GPU at once are solved in one
+   launch with tiles of its own: there no height is tried (op_nrows 0) and
+   the one that relsim_set_launch_shapes set is kept (relsim_apply_operator
+   uses it). Each candidate runs once untimed and three times timed (CUDA events;
    the least counts). Call it on a loaded state before a build (the trials
    overwrite only what the next step recomputes); later steps use the
    choice (captured step graphs are recaptured). out (may be NULL) receives
@@ -624,7 +627,7 @@ typedef struct {
     int push_blocks[8];
     float push_ms[8];
     int deposit_choice, push_choice;   /* indices into the candidates */
-    int op_nrows;                      /* tile heights tried for the 2D operator */
+    int op_nrows;                      /* tile heights tried for the 2D operator (0: none) */
     int op_rows[4];                    /* rows per operator tile (32 nodes wide)  */
     float op_ms[4];                    /* an Arnoldi-mode application, 8 dots    */
     int op_choice;

@@ -818,11 +818,14 @@ int autotune_impl(relsim_ctx* c, relsim_tuning* out)
             &t.push_ms[k]);
     }
     // the operator's tile height (a compile-time shape with two instances):
-    // an Arnoldi-mode application with 8 dot products on the deposited M
+    // an Arnoldi-mode application with 8 dot products on the deposited M. Not
+    // where the solve is one launch, which has its own tiles, and not for the
+    // 3D and quadratic operators, which have one tile shape
     const int alt = c->prec == 32 ? 4 : 2;
     const int rows_c[2] = {0, alt};
-    t.op_nrows = lin2 ? 2 : 0;   // the 3D and quadratic operators have one tile shape
-    if (r == RELSIM_OK && lin2) {
+    const bool op_shapes = lin2 && !c->solve_rows;
+    t.op_nrows = op_shapes ? 2 : 0;
+    if (r == RELSIM_OK && op_shapes) {
         const int jdots = 8;
         int64_t most = 0;
         for (int k = 0; k < 2; ++k) {
@@ -852,8 +855,8 @@ int autotune_impl(relsim_ctx* c, relsim_tuning* out)
     cudaEventDestroy(e0);
     cudaEventDestroy(e1);
     if (r != RELSIM_OK) return r;
-    t.op_choice = lin2 && t.op_ms[1] < t.op_ms[0] ? 1 : 0;
-    c->g.op_y = rows_c[t.op_choice];
+    t.op_choice = op_shapes && t.op_ms[1] < t.op_ms[0] ? 1 : 0;
+    if (op_shapes) c->g.op_y = rows_c[t.op_choice];
     int bd = 0, bp = 0;
     for (int k = 1; k < ncand; ++k) {
         if (t.deposit_ms[k] < t.deposit_ms[bd]) bd = k;

@@ -330,7 +330,8 @@ RELSIM_API int relsim_field_adjoint(relsim_ctx* ctx, const double* gE1, const do
    <gJ, Jhat> + <gM, M> per unit weight), in the current order, and
    overwrites gB = dL/dB^n (centre field, 3*ncell) with this species'
    contribution. Per particle from the stored values, in the form's
-   precision. Call it after relsim_build_mass_matrix and before
+   precision (FP32: gJ and gM are converted once, into device scratch of 24
+   ncell doubles that the context keeps). Call it after relsim_build_mass_matrix and before
    relsim_push. Synchronises the stream. Errors: INVALID_ARG (including a
    gamma_pred context: relsim_step_adjoint covers that reading), BAD_STATE,
    OOM, CUDA.
@@ -353,8 +354,8 @@ RELSIM_API int relsim_deposit_adjoint(relsim_ctx* ctx, int species, const double
    push), it returns gu0 = dL/du^n (3n), gx0 = dL/dx^{n+1/2} (2n), and
    overwrites gE = dL/dE^{n+theta} (node field, 3*ncell) and gB = dL/dB^n
    (centre field, 3*ncell) with this species' contribution (sum the species
-   yourself). The push is replayed per particle in FP64 from the stored
-   values; the gathers' transposes are scatters with the same weights.
+   yourself). The push is replayed per particle in the form's precision from
+   the stored values; the gathers' transposes are scatters with the same weights.
    Call it between relsim_field_solve and relsim_push. Synchronises the
    stream. Errors: INVALID_ARG (including a gamma_pred context), BAD_STATE,
    OOM, CUDA. */
@@ -658,12 +659,14 @@ RELSIM_API int relsim_version(void);
                                       by move direction; ledger sums          */
 #define RELSIM_PROF_SORT_TABLES 2  /* new-cell counts and their scan           */
 #define RELSIM_PROF_PERMUTE 3      /* the pushed particles into new-cell order */
-#define RELSIM_PROF_GMRES_APPLY 4  /* operator applications in GMRES           */
+#define RELSIM_PROF_GMRES_APPLY 4  /* operator applications in GMRES; the whole
+                                      solve where it is one launch (2D grids
+                                      whose tiles fit on the GPU at once)      */
 #define RELSIM_PROF_GMRES_ORTHO 5  /* Gram-Schmidt, norms, basis updates       */
 #define RELSIM_PROF_FIELD_UPDATE 6 /* E^{n+1}, B^{n+1}, field ledger terms     */
 #define RELSIM_PROF_RHS 7          /* right-hand side of the field equation    */
-#define RELSIM_PROF_LOAD 8         /* load conversion + radix sort + gather    */
-#define RELSIM_PROF_GENERAL_SORT 9 /* long-move push path (radix sort)         */
+#define RELSIM_PROF_LOAD 8         /* load conversion, sort by cell, gather    */
+#define RELSIM_PROF_GENERAL_SORT 9 /* 3D, quadratic and long-move push + sort  */
 #define RELSIM_PROF_NSLOTS 10
 
 typedef struct {

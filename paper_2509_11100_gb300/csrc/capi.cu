@@ -2034,9 +2034,10 @@ int shared_outcome(relsim_shared* sb, int i, const void* head, int* iters, bool 
     memcpy(&h, head, kGmHead);
     if (first) count_launches((int)sb->k_static[0]);
     count_launches((int)(sb->k_cycle[i] * h.restarts + sb->k_iter[i] * h.total));
-    // the shared deposit reports its staging timeouts on the first instance
+    // the shared deposit reports its staging timeouts on the first instance,
+    // whose own solve raises the same flag
     if (i != 0 && (*sb->c[0]->hpush & 2))
-        return fail(c, RELSIM_ERR_TIMEOUT, "a shared-memory staging wait of the shared deposit gave up");
+        return fail(c, RELSIM_ERR_TIMEOUT, "a bounded wait gave up (staging of the shared deposit, or the first instance's solve)");
     TRY(check_push(c));
     return solve_outcome(c, &h, iters, nullptr);
 }
@@ -2197,7 +2198,7 @@ int mode_grad_impl(relsim_ctx* c, int comp, int mode, double* energy, double* gB
 int check_push(relsim_ctx* c)
 {
     if (*c->hpush & 2)
-        return fail(c, RELSIM_ERR_TIMEOUT, "a shared-memory staging wait gave up (deposit, push or operator)");
+        return fail(c, RELSIM_ERR_TIMEOUT, "a bounded wait gave up (staging of the deposit or the operator, or the solve's grid barrier)");
     if (*c->hpush)
         return fail(c, RELSIM_ERR_INTERNAL, "particle sort: the moves counted and the new cell starts disagreed");
     return RELSIM_OK;

@@ -215,10 +215,10 @@ cudaError_t gather_grad(const int32_t* id, const double* gu, const double* gx, d
 // gu[id[i]] = lu[i], gx[id[i]] = lx[i] (or += with add)
 cudaError_t scatter_grad(const int32_t* id, const double* lu, const double* lx, double* gu, double* gx, int64_t n,
                          bool add, cudaStream_t st);
-// gw[id[i]] += lw[i]
 // out = in in the form's precision
 template <typename T>
 cudaError_t narrow_array(const double* in, T* out, int64_t n, cudaStream_t st);
+// gw[id[i]] += lw[i]
 cudaError_t scatter_add_w(const int32_t* id, const double* lw, double* gw, int64_t n, cudaStream_t st);
 // bit 0 of *bad if id[i] or ids[i] is outside [0, n) (flag accumulates)
 cudaError_t check_ids(const int32_t* id, const int32_t* ids, int64_t n, int* bad, cudaStream_t st);

@@ -370,8 +370,9 @@ struct Moments<float> {
 // distances 4, 2, 1): afterwards lane gl holds the group sums of the 12
 // flat values 12 gl .. 12 gl + 11, where lane L's block is S[L][0..8]
 // followed by S[8][3L..3L+2] (L < 3), Jm[3(L-3)..3(L-3)+2] (3 <= L < 7)
-// or zeros (L = 7). Each sum pairs the lanes' values in the order the
-// butterfly of group_reduce does, so the results are the same.
+// or zeros (L = 7). A sum adds the lanes' values in a fixed order: lanes four
+// apart first, then two, then one, the lane that keeps it on the left (an
+// addition commutes, so it is the same for every lane that keeps one).
 template <typename T>
 __device__ __forceinline__ void reduce_scatter8(const Moments<T>& m, int gl, T (&r)[12])
 {

@@ -15,8 +15,8 @@
 // separate what the tiles exchange (the partial dot products, and v_{j+1} for
 // the halos). Every block adds up all partial sums itself, in one fixed
 // order, so all take the same decisions without a further exchange; the
-// Hessenberg column, its Givens rotations and the stop test (gmres.cu's) run
-// on one thread of block 0 while the others update the basis. Same
+// Hessenberg column, its Givens rotations and the stop test (gmtail.cuh) run
+// on one warp of block 0 while the others update the basis. Same
 // iteration, stop tests, restart rule and arithmetic per vector element as
 // the launches it replaces; only the order of the dot products' partial
 // sums differs.

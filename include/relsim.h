@@ -187,6 +187,8 @@ RELSIM_API const char* relsim_last_error(const relsim_ctx* ctx);
    order). Ids (if tracked) are the input indices 0..n-1. n = 0 empties the
    species. Errors: INVALID_ARG (species out of range, n < 0 or > 2^31-1,
    NULL arrays with n > 0), NONFINITE (NaN/Inf in the input), OOM, CUDA.
+   After NONFINITE the species is as it was, or empty where the record has
+   taken its room (the species had been loaded in cell order, or had to grow).
    Resets the step state: the next call must be relsim_build_mass_matrix. */
 RELSIM_API int relsim_load_particles(relsim_ctx* ctx, int species, int64_t n, const double* x,
                           const double* u, const double* w, int where);

@@ -364,6 +364,18 @@ void free_arrays(Species& sp, int b)
     dfree(sp.id[b]);
 }
 
+// no particles (and none of their kinetic energy in the ledger)
+int empty_species(relsim_ctx* c, int s)
+{
+    Species& sp = c->sp[s];
+    sp.n = 0;
+    sp.cur = 0;
+    CK(cudaMemsetAsync(sp.start, 0, sizeof(int32_t) * (size_t)(c->g.ncell + 1), c->st));
+    CK(cudaMemsetAsync(c->dled + kLedgerField + kLedgerSpecies * s, 0, sizeof(double) * kLedgerSpecies, c->st));
+    return RELSIM_OK;
+}
+
+// room for n particles; a species that has to grow for it is empty afterwards
 int ensure_species(relsim_ctx* c, int s, int64_t n)
 {
     Species& sp = c->sp[s];
@@ -372,6 +384,7 @@ int ensure_species(relsim_ctx* c, int s, int64_t n)
         TRY(dalloc(c, &sp.start_alt, sizeof(int32_t) * (size_t)(c->g.ncell + 1)));
     }
     if (n <= sp.cap) return RELSIM_OK;
+    TRY(empty_species(c, s));
     for (int b = 0; b < 2; ++b) free_arrays(sp, b);
     sp.cap = 0;
     const int narr = c->g.dim == 3 ? 7 : 6;
@@ -427,10 +440,8 @@ int load_impl(relsim_ctx* c, int s, int64_t n, const double* x, const double* u,
 {
     Species& sp = c->sp[s];
     TRY(ensure_species(c, s, n));
-    sp.n = n;
-    sp.cur = 0;
     if (n == 0) {
-        CK(cudaMemsetAsync(sp.start, 0, sizeof(int32_t) * (size_t)(c->g.ncell + 1), c->st));
+        TRY(empty_species(c, s));
     } else {
         const double *dx, *du, *dw;
         const int D = c->g.dim;   // x holds D coordinates per particle
@@ -449,13 +460,20 @@ int load_impl(relsim_ctx* c, int s, int64_t n, const double* x, const double* u,
         CK(keys_unsorted(c->rk[0], n, c->dflag, c->st));
         CK(histogram_keys(c->rk[0], n, c->count_new, c->g.ncell, c->st));
         CK(cells_above(c->count_new, c->g.ncell, c->dflag, c->st));
-        CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp,
-                              c->st));
         PROF_END();
         CK(cudaMemcpyAsync(c->hflag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
         CK(cudaStreamSynchronize(c->st));
-        if (*c->hflag & 1) return fail(c, RELSIM_ERR_NONFINITE, "non-finite value in particles");
+        if (*c->hflag & 1) {
+            // the species' own particles are still there, with their cell
+            // starts, unless they lay in the buffer of the conversion
+            if (sp.cur == 1) TRY(empty_species(c, s));
+            return fail(c, RELSIM_ERR_NONFINITE, "non-finite value in particles");
+        }
         PROF_BEGIN(RELSIM_PROF_LOAD);
+        sp.n = n;
+        sp.cur = 0;
+        CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp,
+                              c->st));
         if (*c->hflag & 2) {
             // the stable sort by cell, then the particles gathered in that order
             const int32_t* perm = c->rv[1];

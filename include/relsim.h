@@ -566,8 +566,10 @@ RELSIM_API int relsim_batch_create(relsim_ctx* const* ctxs, int count, int nwork
    (host, may be NULL). status[b] (host, required) receives RELSIM_OK, the
    first error of instance b (its later steps are skipped), or
    RELSIM_ERR_NOT_CONVERGED if a solve hit gmres_maxit (the steps go on).
-   Returns RELSIM_OK when every status is OK, otherwise the first non-OK
-   status in instance order. Errors of the call itself: INVALID_ARG, OOM,
+   Instances whose one-launch solves would want the same SMs solve by
+   launches during the run (the same iteration, in another order of its
+   sums). Returns RELSIM_OK when every status is OK, otherwise the first
+   non-OK status in instance order. Errors of the call itself: INVALID_ARG, OOM,
    CUDA. */
 RELSIM_API int relsim_batch_run(relsim_batch* b, int nsteps, int component, int nmodes, double* modes,
                                 int* status, int* iters);
@@ -617,7 +619,7 @@ RELSIM_API void relsim_batch_destroy(relsim_batch* b);
    matrix). Grids whose tiles all fit on the GPU at once are solved in one
    launch with tiles of its own: there no height is tried (op_nrows 0) and
    the one that relsim_set_launch_shapes set is kept (relsim_apply_operator
-   uses it). Each candidate runs once untimed and three times timed (CUDA events;
+   uses it, and a batch's run where it solves by launches). Each candidate runs once untimed and three times timed (CUDA events;
    the least counts). Call it on a loaded state before a build (the trials
    overwrite only what the next step recomputes); later steps use the
    choice (captured step graphs are recaptured). out (may be NULL) receives

@@ -342,6 +342,37 @@ int run_shared(relsim_batch* b, int nsteps, int first, int component, int nmodes
     return rc;
 }
 
+// How the instances solve while a batch runs them side by side. The one-launch
+// solve starts only when all its blocks fit on the GPU at once, so next to
+// others it waits for their kernels and holds the SMs while it waits at its
+// grid barriers. An instance whose solve takes more than a third of the blocks
+// that can be resident solves by launches (gmres.cu) where the batch's solves
+// together want more than 7/4 of them. Microseconds a step of a batch, one
+// launch | launches, 32 particles a cell, FP32: eight of 384x192 (share 0.95)
+// 3693 | 2990, three 1370 | 1162, two 954 | 863; eight of 320x160 (0.66) 2489 |
+// 2195; eight of 256x128 (0.42) 1640 | 1594, two 485 | 540; eight of 224x112
+// (0.32) 1263 | 1316, of 192x96 (0.24) 1047 | 1123, of 128x64 (0.21) 661 | 809.
+// FP64, 8 a cell: eight of 128x64 (0.84) 2946 | 2660, two 793 | 830; four of
+// 192x96 (0.47) 2227 | 2187; eight of 64x32 (0.21) 792 | 1113. With shared
+// launches eight of 384x192 take 4200 | 3560. (Where all the solves together
+// want less than 7/4, e.g. 384x192 beside 256x128, 1.37, 690 | 704, the two ways
+// are within 3% or one launch is the faster.)
+constexpr double kSolveWide = 1.0 / 3.0, kSolveMost = 1.75;
+struct SolveWays {
+    const std::vector<relsim_ctx*>& ctx;
+    explicit SolveWays(const std::vector<relsim_ctx*>& c) : ctx(c)
+    {
+        double want = 0.0;
+        for (const relsim_ctx* i : ctx) want += ctx_solve_share(i);
+        if (want > kSolveMost)
+            for (relsim_ctx* i : ctx) ctx_solve_beside(i, ctx_solve_share(i) > kSolveWide);
+    }
+    ~SolveWays()
+    {
+        for (relsim_ctx* i : ctx) ctx_solve_beside(i, false);
+    }
+};
+
 }  // namespace
 
 extern "C" {
@@ -373,6 +404,7 @@ int relsim_batch_run(relsim_batch* b, int nsteps, int component, int nmodes, dou
     for (int i = 0; i < count; ++i) status[i] = RELSIM_OK;
     if (nsteps == 0) return RELSIM_OK;
     if (cudaSetDevice(b->device) != cudaSuccess) return RELSIM_ERR_CUDA;
+    const SolveWays ways(b->ctx);
 
     // device slots for the mode energies: (instance, step, mode); one
     // call per context first, on the loaded state, sizes the context's

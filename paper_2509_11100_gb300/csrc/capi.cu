@@ -110,6 +110,8 @@ struct relsim_ctx {
     // GMRES
     int mrest = 30;
     int solve_rows = 0;        // tile height of the one-launch solve (0: the launches of gmres.cu)
+    double solve_share = 0.0;  // its blocks, of those that can be resident on the GPU at once
+    bool beside = false;       // solve by launches: a batch has other solves wait for the same SMs
     int64_t nvec = 0;
     double* V = nullptr;
     double* gw = nullptr;
@@ -126,8 +128,9 @@ struct relsim_ctx {
     cudaEvent_t gev[2] = {nullptr, nullptr};   // read-back events of the host-driven Arnoldi loop
     GmState* gms = nullptr;    // device-side GMRES control state
     GmState* ghead = nullptr;  // pinned host, two read-back slots (heads only)
-    // step graphs (two layouts alternate from step to step)
-    StepGraph sg[2];
+    // step graphs (two layouts alternate from step to step), then those of a
+    // batch's run that solves by launches
+    StepGraph sg[4];
     uint64_t gen = 1;          // bumped whenever a buffer or a launch shape changes
     bool graph_off = false;    // a capture failed: host-driven steps from then on
     std::string graph_why;     // why
@@ -943,6 +946,8 @@ int solve_rhs(relsim_ctx* c, const GmSetup& S, cudaStream_t s)
     return RELSIM_OK;
 }
 
+bool one_launch(const relsim_ctx* c) { return c->solve_rows && !c->beside; }
+
 // the whole solve in one launch (grids that fit: solve.cu)
 template <typename T>
 int solve_launch(relsim_ctx* c, const GmSetup& S, cudaStream_t s, bool tr)
@@ -1100,7 +1105,7 @@ int solve_impl(relsim_ctx* c, int* iters_out, double* relres_out)
 {
     const GmSetup S = gm_setup(c);
     TRY(solve_reserve(c, S));
-    if (c->solve_rows) {
+    if (one_launch(c)) {
         TRY(solve_rhs<T>(c, S, c->st));
         TRY(solve_launch<T>(c, S, c->st, false));
         TRY(solve_read(c));
@@ -1302,7 +1307,7 @@ int capture_into(relsim_ctx* c, cudaStream_t s, cudaGraph_t body, long long* tal
 template <typename T>
 int capture_solve(relsim_ctx* c, const GmSetup& S, StepGraph& G)
 {
-    if (c->solve_rows) {
+    if (one_launch(c)) {
         TRY(solve_rhs<T>(c, S, c->st));
         TRY(solve_launch<T>(c, S, c->st, false));
         return solve_epilogue<T>(c, c->st);
@@ -1378,6 +1383,9 @@ int capture_step(relsim_ctx* c, StepGraph& G)
     return RELSIM_OK;
 }
 
+// the context's two graphs of the way it solves now
+StepGraph* graphs(relsim_ctx* c) { return c->sg + (c->beside ? 2 : 0); }
+
 // captured on the context's buffers and counts (of either step parity). A
 // load of as many particles into the same buffers leaves them as they are, so
 // a run that reloads states (the segments of a differentiable window) keeps
@@ -1403,12 +1411,12 @@ bool graph_matches(const relsim_ctx* c, const StepGraph& G)
 template <typename T>
 int step_graph(relsim_ctx* c, relsim_energy* ledger, int* status)
 {
-    StepGraph* G = nullptr;
-    for (StepGraph& g : c->sg)
-        if (graph_matches(c, g)) G = &g;
+    StepGraph *G = nullptr, *const sg = graphs(c);
+    for (int k = 0; k < 2; ++k)
+        if (graph_matches(c, sg[k])) G = &sg[k];
     if (!G) {
         // replace the slot not matching the other parity's layout
-        G = &c->sg[graph_current(c, c->sg[0]) && c->sg[0].bcur != c->bcur ? 1 : 0];
+        G = &sg[graph_current(c, sg[0]) && sg[0].bcur != c->bcur ? 1 : 0];
         if (capture_step<T>(c, *G) != RELSIM_OK) {
             c->graph_off = true;
             c->graph_why = c->err;
@@ -1462,7 +1470,7 @@ int adjoint_impl(relsim_ctx* c, const double* gE1, const double* gB1, const doub
     TRY(solve_reserve(c, S));
     CK(adjoint_pre(d1, d2, d3, c->gb, c->g, c->st));
     CK(cudaMemsetAsync(c->gx, 0, sizeof(double) * (size_t)n, c->st));
-    if (c->solve_rows) {
+    if (one_launch(c)) {
         TRY(solve_launch<T>(c, S, c->st, true));
         TRY(solve_read(c));
     } else {
@@ -1684,8 +1692,8 @@ bool graph_eligible(const relsim_ctx* c)
 
 StepGraph* graph_for_layout(relsim_ctx* c)
 {
-    for (StepGraph& g : c->sg)
-        if (graph_matches(c, g)) return &g;
+    for (int k = 0; k < 2; ++k)
+        if (graph_matches(c, graphs(c)[k])) return &graphs(c)[k];
     return nullptr;
 }
 
@@ -2071,7 +2079,8 @@ int ctx_graph_prepare(relsim_ctx* c)
     push_commit(c);
     if (have_a && have_b) return 1;
     for (int k = 0; k < 2; ++k) {
-        const int r = c->prec == 32 ? capture_step<float>(c, c->sg[k]) : capture_step<double>(c, c->sg[k]);
+        StepGraph& G = graphs(c)[k];
+        const int r = c->prec == 32 ? capture_step<float>(c, G) : capture_step<double>(c, G);
         if (r != RELSIM_OK) {
             if (k == 1) push_commit(c);
             c->graph_off = true;
@@ -2102,7 +2111,7 @@ int ctx_graph_outcome(relsim_ctx* c, const void* head, int* iters)
 {
     GmState h;
     memcpy(&h, head, kGmHead);
-    const StepGraph& G = c->sg[0];
+    const StepGraph& G = graphs(c)[0];
     count_launches((int)(G.k_static + G.k_cycle * h.restarts + G.k_iter * h.total));
     TRY(check_push(c));
     return solve_outcome(c, &h, iters, nullptr);
@@ -2310,6 +2319,9 @@ int validate(const relsim_config* cfg, std::string* why)
 namespace relsim {
 cudaStream_t ctx_stream(const relsim_ctx* c) { return c->st; }
 int ctx_last_iters(const relsim_ctx* c) { return c->last_iters; }
+double ctx_solve_share(const relsim_ctx* c) { return c->solve_share; }
+void ctx_solve_beside(relsim_ctx* c, bool on) { c->beside = on; }
+
 int64_t ctx_particles(const relsim_ctx* c)
 {
     int64_t n = 0;
@@ -2393,8 +2405,8 @@ int relsim_init(const relsim_config* cfg, void* cuda_stream, relsim_ctx** out)
     A(dalloc(c, &c->gms, sizeof(GmState)));
     // (the grid barrier counts its arrivals in 32 bits)
     if (c->cfg.gmres_maxit <= 1 << 20 &&
-        (cfg->precision == 32 ? gm_solve_rows<float>(c->g, &c->solve_rows)
-                              : gm_solve_rows<double>(c->g, &c->solve_rows)) != cudaSuccess) {
+        (cfg->precision == 32 ? gm_solve_rows<float>(c->g, &c->solve_rows, &c->solve_share)
+                              : gm_solve_rows<double>(c->g, &c->solve_rows, &c->solve_share)) != cudaSuccess) {
         r = fail(c, RELSIM_ERR_CUDA, "sizing the solve's launch failed");
         goto fail_init;
     }

@@ -422,9 +422,10 @@ cudaError_t gm_update_scale_dyn(GmState* st, const GmPtrs& p, const GmParams& q,
                                 int df);
 
 // ----- solve.cu: the solve in one cooperative launch -----
-// *rows: the tile height to use, 0 if the grid does not fit
+// *rows: the tile height to use, 0 if the grid does not fit; *share: its
+// blocks, of those that can be resident on the GPU at once
 template <typename T>
-cudaError_t gm_solve_rows(GridP g, int* rows);
+cudaError_t gm_solve_rows(GridP g, int* rows, double* share);
 // doubles of partial sums it needs (m: the restart length)
 int64_t gm_solve_partials(GridP g, int rows, int m);
 // from b and the first iterate x (GMRES vectors): x, and the outcome in st;
@@ -456,6 +457,10 @@ namespace relsim {
 cudaStream_t ctx_stream(const relsim_ctx* c);
 int ctx_last_iters(const relsim_ctx* c);
 int64_t ctx_particles(const relsim_ctx* c);
+// the GPU's share that the context's one-launch solve takes (0: it has none),
+// and whether the context solves by launches instead
+double ctx_solve_share(const relsim_ctx* c);
+void ctx_solve_beside(relsim_ctx* c, bool on);
 // graph steps enqueued without waiting: prepare captures both buffer layouts
 // (1: ready; 0: this context steps from the host); enqueue launches one
 // step and copies its solve outcome (head_bytes) to the pinned host buffer

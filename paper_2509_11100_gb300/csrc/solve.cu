@@ -596,9 +596,10 @@ cudaError_t solve_resident(int Y, int nsm, int* blocks)
 // flight) that leaves at most one block per SM, else the form's largest if
 // its blocks are all resident together, else 0 (the launches of gmres.cu).
 template <typename T>
-cudaError_t gm_solve_rows(GridP g, int* rows)
+cudaError_t gm_solve_rows(GridP g, int* rows, double* share)
 {
     *rows = 0;
+    *share = 0.0;
     if (g.dim != 2 || g.shape != 1) return cudaSuccess;
     int dev = 0, nsm = 0, coop = 0;
     cudaError_t e = cudaGetDevice(&dev);
@@ -619,7 +620,10 @@ cudaError_t gm_solve_rows(GridP g, int* rows)
         e = solve_resident<T, false, false>(Y, nsm, &most);
         if (e == cudaSuccess) e = solve_resident<T, false, true>(Y, nsm, &most);
     }
-    if (e == cudaSuccess && solve_tiles(g, Y) <= most) *rows = Y;
+    if (e == cudaSuccess && solve_tiles(g, Y) <= most) {
+        *rows = Y;
+        *share = (double)solve_tiles(g, Y) / (double)most;
+    }
     return e;
 }
 
@@ -651,8 +655,8 @@ cudaError_t gm_solve(const T* M, const double* b, double* x, const GmPtrs& p, co
     return tr ? launch_solve<T, false, true>(a, blocks, s) : launch_solve<T, false, false>(a, blocks, s);
 }
 
-template cudaError_t gm_solve_rows<float>(GridP, int*);
-template cudaError_t gm_solve_rows<double>(GridP, int*);
+template cudaError_t gm_solve_rows<float>(GridP, int*, double*);
+template cudaError_t gm_solve_rows<double>(GridP, int*, double*);
 template cudaError_t gm_solve<float>(const float*, const double*, double*, const GmPtrs&, const GmParams&, GridP, int,
                                      double*, GmState*, int*, bool, cudaStream_t);
 template cudaError_t gm_solve<double>(const double*, const double*, double*, const GmPtrs&, const GmParams&, GridP, int,

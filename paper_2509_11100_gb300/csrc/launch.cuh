@@ -126,8 +126,10 @@ cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32
 size_t radix_tmp_ints(int64_t n);
 cudaError_t radix_sort_pairs(int32_t* k0, int32_t* v0, int32_t* k1, int32_t* v1, int64_t n,
                              int key_bits, int32_t* tmp, bool* result_in_1, cudaStream_t st);
-// bit 3 (8) of *flag if a cell holds more particles than stable_cell_order takes
-cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, cudaStream_t st);
+// bit 3 (8) of *flag if a cell holds more particles than stable_cell_order
+// takes; the cell starts start[0 .. ncell] into keep, if keep is not null
+cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, const int32_t* start, int32_t* keep,
+                        cudaStream_t st);
 // perm = the stable order of keys by cell (cells' first places in start; taken
 // and tmp: scratch of ncell and n)
 cudaError_t stable_cell_order(const int32_t* keys, int64_t n, const int32_t* start, int ncell, int32_t* taken,

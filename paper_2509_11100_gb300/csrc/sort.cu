@@ -207,11 +207,15 @@ __global__ void k_iota(int32_t* a, int64_t n)
 // 305 for five passes of the radix sort; cells are bounded by kRankMost (the
 // work grows with the square of a cell's particles), larger ones leave the
 // load to the radix sort.
-__global__ void k_cell_above(const int32_t* __restrict__ counts, int n, int most, int* flag)
+// (and start[0 .. n] into keep, where that is not null)
+__global__ void k_cell_above(const int32_t* __restrict__ counts, int n, int most, int* flag,
+                             const int32_t* __restrict__ start, int32_t* __restrict__ keep)
 {
     bool above = false;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c < n; c += gridDim.x * blockDim.x)
-        above = above || counts[c] > most;
+    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= n; c += gridDim.x * blockDim.x) {
+        if (keep) keep[c] = start[c];
+        above = above || (c < n && counts[c] > most);
+    }
     if (__syncthreads_or(above) && threadIdx.x == 0) atomicOr(flag, 8);
 }
 
@@ -369,11 +373,12 @@ cudaError_t histogram_keys(const int32_t* keys, int64_t n, int32_t* counts, int 
     return cudaGetLastError();
 }
 
-cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, cudaStream_t st)
+cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, const int32_t* start, int32_t* keep,
+                        cudaStream_t st)
 {
     count_launches(1);
     const int b = (ncell + 1023) / 1024;
-    k_cell_above<<<b < 152 ? b : 152, 1024, 0, st>>>(counts, ncell, kRankMost, flag);
+    k_cell_above<<<b < 152 ? b : 152, 1024, 0, st>>>(counts, ncell, kRankMost, flag, start, keep);
     return cudaGetLastError();
 }
 

@@ -460,16 +460,13 @@ int load_impl(relsim_ctx* c, int s, int64_t n, const double* x, const double* u,
             CK(load_convert3<T>(dx, du, dw, n, c->g, tmp, (T*)sp.a[1][6], c->rk[0], c->rv[0], c->dflag, c->st));
         else
             CK(load_convert<T>(dx, du, dw, n, c->g, tmp, c->rk[0], c->rv[0], c->dflag, c->st));
-        CK(keys_unsorted(c->rk[0], n, c->dflag, c->st));
-        CK(histogram_keys(c->rk[0], n, c->count_new, c->g.ncell, c->st));
+        CK(histogram_keys(c->rk[0], n, c->count_new, c->g.ncell, c->st, c->dflag));
         // the cell starts come before the check's read-back (after it they made
         // two loads of 4.2 million particles 1% longer); those of the species'
         // own particles go to the side until the record has passed, unless the
         // conversion has just overwritten the particles
         const bool keep = sp.n > 0 && sp.cur == 0;
-        CK(cells_above(c->count_new, c->g.ncell, c->dflag, sp.start, keep ? sp.start_alt : nullptr, c->st));
-        CK(scan_exclusive_i32(c->count_new, sp.start, c->g.ncell, sp.start + c->g.ncell, c->scan_tmp,
-                              c->st));
+        CK(scan_cells(c->count_new, sp.start, c->g.ncell, c->scan_tmp, c->dflag, keep ? sp.start_alt : nullptr, c->st));
         PROF_END();
         CK(cudaMemcpyAsync(c->hflag, c->dflag, sizeof(int), cudaMemcpyDeviceToHost, c->st));
         CK(cudaStreamSynchronize(c->st));

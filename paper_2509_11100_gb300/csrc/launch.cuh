@@ -126,17 +126,19 @@ cudaError_t scan_exclusive_i32(const int32_t* in, int32_t* out, int64_t n, int32
 size_t radix_tmp_ints(int64_t n);
 cudaError_t radix_sort_pairs(int32_t* k0, int32_t* v0, int32_t* k1, int32_t* v1, int64_t n,
                              int key_bits, int32_t* tmp, bool* result_in_1, cudaStream_t st);
-// bit 3 (8) of *flag if a cell holds more particles than stable_cell_order
-// takes; the cell starts start[0 .. ncell] into keep, if keep is not null
-cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, const int32_t* start, int32_t* keep,
-                        cudaStream_t st);
+// a load's cell starts start[0 .. ncell] from its counts; bit 3 (8) of *flag if
+// a cell holds more particles than stable_cell_order takes; the starts that
+// were there into keep, if keep is not null
+cudaError_t scan_cells(const int32_t* counts, int32_t* start, int ncell, int32_t* tmp, int* flag, int32_t* keep,
+                       cudaStream_t st);
 // perm = the stable order of keys by cell (cells' first places in start; taken
 // and tmp: scratch of ncell and n)
 cudaError_t stable_cell_order(const int32_t* keys, int64_t n, const int32_t* start, int ncell, int32_t* taken,
                               int32_t* tmp, int32_t* perm, cudaStream_t st);
-// counts[k] = #keys equal to k (counts zeroed inside)
+// counts[k] = #keys equal to k (counts zeroed inside); bit 1 (2) of *unsorted
+// (not null) if a key is above the one after it (the flag accumulates)
 cudaError_t histogram_keys(const int32_t* keys, int64_t n, int32_t* counts, int nkeys,
-                           cudaStream_t st);
+                           cudaStream_t st, int* unsorted = nullptr);
 // new-cell counts of the neighbour-move sort
 cudaError_t move_counts(const int32_t* n9, int32_t* count_new, GridP g, cudaStream_t st);
 // zero `bytes` (a multiple of 4) from p (16-byte aligned) with a kernel
@@ -230,8 +232,6 @@ cudaError_t relabel_ids(int32_t* id, const int32_t* ids, int64_t n, cudaStream_t
 cudaError_t add_fields(const double* a, const double* b, double* out, int64_t n, cudaStream_t st);
 
 // ----- particles.cu -----
-// bit 2 of *flag if keys[0..n) is not non-decreasing (flag accumulates)
-cudaError_t keys_unsorted(const int32_t* keys, int64_t n, int* flag, cudaStream_t st);
 template <typename T>
 cudaError_t load_convert(const double* x, const double* u, const double* w, int64_t n, GridP g,
                          PArrays<T> out, int32_t* key, int32_t* val, int* bad, cudaStream_t st);

@@ -62,15 +62,6 @@ __global__ void k_load_convert(const double* __restrict__ x, const double* __res
     }
 }
 
-// sets bit 2 of flag if keys[] is not non-decreasing
-__global__ void k_keys_unsorted(const int32_t* __restrict__ keys, int64_t n, int* flag)
-{
-    bool bad = false;
-    for (int64_t p = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; p + 1 < n; p += (int64_t)gridDim.x * blockDim.x)
-        bad = bad || keys[p] > keys[p + 1];
-    if (__syncthreads_or(bad) && threadIdx.x == 0) atomicOr(flag, 2);
-}
-
 template <typename T>
 __global__ void k_gather(const int32_t* __restrict__ perm, PArrays<T> src, PArrays<T> dst, int64_t n,
                          bool ids_from_perm)
@@ -2164,14 +2155,6 @@ cudaError_t load_convert(const double* x, const double* u, const double* w, int6
     if (n <= 0) return cudaSuccess;
     count_launches(1);
     k_load_convert<T><<<blocks_for(n, 256, 152 * 32), 256, 0, st>>>(x, u, w, n, g, out, key, val, bad);
-    return cudaGetLastError();
-}
-
-cudaError_t keys_unsorted(const int32_t* keys, int64_t n, int* flag, cudaStream_t st)
-{
-    if (n <= 1) return cudaSuccess;
-    count_launches(1);
-    k_keys_unsorted<<<blocks_for(n, 256, 152 * 8), 256, 0, st>>>(keys, n, flag);
     return cudaGetLastError();
 }
 

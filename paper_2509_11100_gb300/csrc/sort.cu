@@ -60,6 +60,31 @@ __global__ void k_scan_reduce(const int32_t* __restrict__ in, int64_t n, int32_t
     if (threadIdx.x == 0) partial[blockIdx.x] = tot;
 }
 
+// the same over a load's counts by cell: bit 3 (8) of *flag if one is above
+// most, and start[0 .. n], which the scan is about to overwrite, into keep where
+// that is not null (as a launch of its own this made small loads 6% longer)
+__global__ void k_scan_reduce_cells(const int32_t* __restrict__ in, int64_t n, int32_t* __restrict__ partial, int most,
+                                    int* flag, const int32_t* __restrict__ start, int32_t* __restrict__ keep)
+{
+    __shared__ int smem[32];
+    int64_t base = (int64_t)blockIdx.x * kScanTile + threadIdx.x * kScanItems;
+    int s = 0;
+    bool above = false;
+#pragma unroll
+    for (int r = 0; r < kScanItems; ++r)
+        if (base + r < n) {
+            const int c = in[base + r];
+            s += c;
+            above = above || c > most;
+            if (keep) keep[base + r] = start[base + r];
+        }
+    if (keep && blockIdx.x == 0 && threadIdx.x == 0) keep[n] = start[n];
+    if (__syncthreads_or(above) && threadIdx.x == 0) atomicOr(flag, 8);
+    int tot;
+    block_scan_excl(s, smem, &tot);
+    if (threadIdx.x == 0) partial[blockIdx.x] = tot;
+}
+
 __global__ void k_scan_partials(int32_t* partial, int nb, int32_t* total)
 {
     __shared__ int smem[32];
@@ -178,19 +203,23 @@ k_radix_down(const int32_t* __restrict__ kin, const int32_t* __restrict__ vin, i
     }
 }
 
-__global__ void k_hist(const int32_t* __restrict__ keys, int64_t n, int32_t* counts)
+// (with unsorted not null, bit 1 (2) of it is set if the keys are not ascending)
+__global__ void k_hist(const int32_t* __restrict__ keys, int64_t n, int32_t* counts, int* unsorted)
 {
+    bool bad = false;
     int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
     int64_t stride = (int64_t)gridDim.x * blockDim.x;
     for (; i - threadIdx.x < n; i += stride) {
         bool ok = i < n;
         int key = ok ? keys[i] : -1;
+        if (unsorted && i + 1 < n) bad = bad || key > keys[i + 1];
         unsigned act = __ballot_sync(0xffffffffu, ok);
         if (!ok) continue;
         unsigned peers = __match_any_sync(act, key);
         int leader = __ffs(peers) - 1;
         if ((threadIdx.x & 31) == leader) atomicAdd(&counts[key], __popc(peers));
     }
+    if (unsorted && __syncthreads_or(bad) && threadIdx.x == 0) atomicOr(unsorted, 2);
 }
 
 __global__ void k_iota(int32_t* a, int64_t n)
@@ -207,18 +236,6 @@ __global__ void k_iota(int32_t* a, int64_t n)
 // 305 for five passes of the radix sort; cells are bounded by kRankMost (the
 // work grows with the square of a cell's particles), larger ones leave the
 // load to the radix sort.
-// (and start[0 .. n] into keep, where that is not null)
-__global__ void k_cell_above(const int32_t* __restrict__ counts, int n, int most, int* flag,
-                             const int32_t* __restrict__ start, int32_t* __restrict__ keep)
-{
-    bool above = false;
-    for (int c = blockIdx.x * blockDim.x + threadIdx.x; c <= n; c += gridDim.x * blockDim.x) {
-        if (keep) keep[c] = start[c];
-        above = above || (c < n && counts[c] > most);
-    }
-    if (__syncthreads_or(above) && threadIdx.x == 0) atomicOr(flag, 8);
-}
-
 __global__ void k_take_places(const int32_t* __restrict__ keys, int64_t n, const int32_t* __restrict__ start,
                               int32_t* __restrict__ taken, int32_t* __restrict__ out)
 {
@@ -362,23 +379,26 @@ cudaError_t radix_sort_pairs(int32_t* k0, int32_t* v0, int32_t* k1, int32_t* v1,
 }
 
 cudaError_t histogram_keys(const int32_t* keys, int64_t n, int32_t* counts, int nkeys,
-                           cudaStream_t st)
+                           cudaStream_t st, int* unsorted)
 {
     cudaError_t e = cudaMemsetAsync(counts, 0, sizeof(int32_t) * (size_t)nkeys, st);
     if (e != cudaSuccess || n <= 0) return e;
     int64_t blocks = (n + 255) / 256;
     if (blocks > 152 * 64) blocks = 152 * 64;
     count_launches(1);
-    k_hist<<<(unsigned)blocks, 256, 0, st>>>(keys, n, counts);
+    k_hist<<<(unsigned)blocks, 256, 0, st>>>(keys, n, counts, unsorted);
     return cudaGetLastError();
 }
 
-cudaError_t cells_above(const int32_t* counts, int ncell, int* flag, const int32_t* start, int32_t* keep,
-                        cudaStream_t st)
+cudaError_t scan_cells(const int32_t* counts, int32_t* start, int ncell, int32_t* tmp, int* flag, int32_t* keep,
+                       cudaStream_t st)
 {
-    count_launches(1);
-    const int b = (ncell + 1023) / 1024;
-    k_cell_above<<<b < 152 ? b : 152, 1024, 0, st>>>(counts, ncell, kRankMost, flag, start, keep);
+    const int64_t nb = ((int64_t)ncell + kScanTile - 1) / kScanTile;
+    if (nb < 1 || nb > kMaxScanBlocks) return cudaErrorInvalidValue;
+    count_launches(3);
+    k_scan_reduce_cells<<<(unsigned)nb, kScanThreads, 0, st>>>(counts, ncell, tmp, kRankMost, flag, start, keep);
+    k_scan_partials<<<1, kScanThreads, 0, st>>>(tmp, (int)nb, start + ncell);
+    k_scan_apply<<<(unsigned)nb, kScanThreads, 0, st>>>(counts, start, ncell, tmp);
     return cudaGetLastError();
 }
 
